@@ -441,12 +441,10 @@ Plan make_plan(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max, int
                int32_t rows_hint) {
   Plan p;
   p.tc = attention_tc_supported(Hq, Hkv, d, min(D_max, rows_hint));
-  if (p.tc) {
-    const TcPlan t = attention_tc_plan(B, Hq, Hkv, D_max, L_max);
-    p.nwarps = 0;
-    p.mtiles = t.mtiles;
-    p.splits = t.splits;
-    p.kps = t.kps;
+  if (p.tc) {  // plans on the device, merges its splits itself
+    p.nwarps = p.mtiles = 0;
+    p.splits = 1;
+    p.kps = L_max;
     return p;
   }
   const int32_t G = Hq / Hkv;
@@ -513,13 +511,13 @@ int32_t attention_rows_hint(const ssd_grid& g, int32_t D_max) {
   return n < D_max ? (int32_t)n : D_max;
 }
 
-// Large enough for the plan of either kernel, so that the kernel choice (which
-// depends on the grid) never outgrows a workspace sized without it.
+// Sized for the mma.sync kernel's plan whichever kernel runs (the tcgen05 kernel
+// needs none), so that the kernel choice (which depends on the grid) never
+// outgrows a workspace sized without it.
 size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
                            int32_t L_max) {
   size_t bytes = align256((size_t)B * sizeof(int32_t));
-  int32_t splits = 1;
-  for (int32_t hint : {D_max, 0}) splits = max(splits, make_plan(B, Hq, Hkv, d, D_max, L_max, hint).splits);
+  const int32_t splits = make_plan(B, Hq, Hkv, d, D_max, L_max, /*rows_hint=*/0).splits;
   if (splits > 1) {
     const size_t prow = (size_t)B * Hq * D_max * splits;
     bytes += align256(prow * d * sizeof(float)) + align256(prow * sizeof(float));
@@ -571,14 +569,9 @@ cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaS
   if (a.B == 0) return cudaSuccess;
   const Plan p = make_plan(a.B, a.Hq, a.Hkv, a.d, a.D_max, a.L_max,
                            attention_rows_hint(a.grid, a.D_max));
+  if (p.tc) return launch_attention_tc(a, stream, pdl);
   const AttnLaunch L = carve(a, p, ws);
   cudaError_t e;
-  if (p.tc) {
-    e = launch_attention_tc(a, TcPlan{p.splits, p.kps, p.mtiles}, L.seq_ok, L.part_o, L.part_lse,
-                            stream, pdl);
-    if (e != cudaSuccess) return e;
-    return (p.splits == 1 || defer_combine) ? cudaSuccess : launch_combine(a, L, stream);
-  }
   CUtensorMap tmK, tmV;
   const int64_t rows = (int64_t)a.B * a.Hkv * a.L_max;
   if (!make_kv_map(&tmK, a.k, rows, a.d) || !make_kv_map(&tmV, a.v, rows, a.d))

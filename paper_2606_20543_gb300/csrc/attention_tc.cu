@@ -5,48 +5,63 @@
 // drafts before it in raster order):
 //   O[b][j][h] = softmax_s(scale * Q[b][j][h] . K[b][g][s] + M(s, j)) V[b][g][s]
 //
-// Design (GB300, tcgen05 + TMEM): a persistent kernel, one CTA per SM, that
-// walks work items (KV split, sequence, KV head, tile of 128 query rows =
-// drafts x the Hq/Hkv heads sharing the KV head; 64-row tiles with M = 64
-// products when a KV head's query rows fit in 64).  Sequences are taken
-// longest first and the items are dealt to the CTAs in snake order, so the
-// long items start early and every CTA gets a similar share.
-//  * warp 8 (producer): decodes the next item, checks and converts its draft
-//    positions into an item slot (two slots), loads Q into one of two Q
-//    buffers through a 3D tensor map, then the item's K tiles of 128 keys;
-//    warp 10 streams its V tiles (TMA, 128-byte swizzle, one copy per tile,
-//    issued by two threads because one thread issues only a few million copies
-//    per second).  The producers run ahead of the other warps by up to two
-//    items, so the next item's loads overlap the current item's last tiles
-//    and its epilogue;
-//  * warp 9 issues S_t = Q K_t^T (N = 128 keys) into one of two TMEM S/P
-//    buffers; warp 11, once the softmax has written P_t, O += P_t V_t with P
+// Design (GB300, tcgen05 + TMEM): a persistent kernel, two CTAs per SM in
+// clusters of kCluster, that walks work items (sequence, KV head, tile of 128
+// query rows = drafts x the Hq/Hkv heads sharing the KV head; 64-row tiles
+// with M = 64 products when a KV head's query rows fit in 64).  The kernel is
+// bound by the K/V stream when its items fill the GPU and by the serial chain
+// of one item (load, S, softmax, PV per tile) when they do not, hence:
+//  * two CTAs per SM: one CTA's start-up, item boundaries and tile chain
+//    overlap the other's (one 202 KB CTA per SM with 128-key tiles before: the
+//    24x24 sweep's step 62.6 us, the 16 x 32x32 GQA step 51.6 us, 8 x 64x64 at
+//    2300-3800 keys 75.5 us; now 49.4, 40.9 and 73.2 us, the last 5.75 TB/s);
+//  * the producer warp alone sets up, plans and issues its first item's five
+//    copies, a lane each in one instruction, before the block's barrier.  What
+//    an SM waits for between that and the first P is instruction fetch once
+//    other kernels ran in between: code is rolled wherever it runs once per
+//    item (the kernel is 64 KB; at 107 KB the sweep's CTAs spent 2.4 us on
+//    their first softmax tile instead of 0.4);
+//  * every CTA computes the same plan from the cache lengths: the sequences
+//    longest first, only the items that have drafts, dealt in snake order.
+//    When the live items fit more than once into the CTAs (small batches, or
+//    the last passes of a batch whose other images are complete, which only
+//    the device knows), 2 or kCluster CTAs of a cluster share an item, each
+//    streaming a part of its keys, and merge their partial rows through
+//    distributed shared memory at the end: no partials in global memory and
+//    no second kernel (one image left of 8 x 64x64: the attention 40 -> 27 us;
+//    two rounds on 8 x 24x24: 86.5 -> 67.8 us with no combine launch).
+//  * warp 4 (producer): decodes the next item, checks and converts its draft
+//    positions into an item slot (two slots), loads Q through a 3D tensor map
+//    and the item's K tiles of 64 keys; warp 5 streams its V tiles (TMA,
+//    128-byte swizzle, one copy per tile, issued by two threads because one
+//    thread issues only a few million copies per second).  The producers run
+//    ahead of the other warps, so the next item's loads overlap the current
+//    item's last tiles and its epilogue;
+//  * warp 6 issues S_t = Q K_t^T (N = 64 keys) into one of two TMEM S/P
+//    buffers; warp 7, once the softmax has written P_t, O += P_t V_t with P
 //    read from TMEM (the A operand of a tcgen05.mma may live in tensor
-//    memory) into the item's TMEM O buffer (two buffers, so an item's
-//    epilogue overlaps the next item's products);
-//  * warps 0-7 (softmax; query row = TMEM lane, warp w owns lane quarter w % 4
-//    and the half w / 4 of every row's columns): tcgen05.ld of its half of the
-//    row of S_t, the spatial mask (a per-row bitmask of the visible drafts,
-//    built once per item), the partial maxima of the two halves exchanged
-//    through a named barrier per warp pair, the running max and sum, and P_t
-//    as bf16 pairs stored with tcgen05.st over the first half of the same
-//    TMEM buffer; then the item's epilogue.  Warps whose rows are all padding
-//    skip the math.  The running max is only moved (and O in TMEM rescaled
-//    with tcgen05.ld/st) when it grows by more than 2^8; otherwise the
-//    exponentials use the stale max, which the final sum shares, so the
-//    result is exact.
+//    memory);
+//  * warps 0-3 (softmax; query row = TMEM lane, warp w owns lane quarter w):
+//    tcgen05.ld of the row of S_t, the spatial mask (a per-row bitmask of the
+//    visible drafts, built once per item), the running max and sum, and P_t as
+//    bf16 pairs stored with tcgen05.st over the first half of the same TMEM
+//    buffer; then the item's epilogue.  Warps whose rows are all padding skip
+//    the math.  The running max is only moved (and O in TMEM rescaled with
+//    tcgen05.ld/st) when it grows by more than 2^8; otherwise the exponentials
+//    use the stale max, which the final sum shares, so the result is exact.
 // K stages, V stages and S/P buffers form rings of two indexed by tile t mod
 // 2, and one barrier per ring slot covers several conditions: "K_t loaded and
 // S/P buffer free (PV of tile t - 2 done)" and "V_t loaded and P_t written".
 // An mbarrier poll costs a few hundred cycles even when the phase is complete
 // and a tcgen05.mma tens of cycles to issue, so each issuing thread has one
-// wait, one group of products and one commit per 128-key tile.  Code that
-// runs once per item (mask, bitmask, epilogue) is kept small: unrolled cold
-// paths cost instruction-cache misses of thousands of cycles.
+// wait, one group of products and one commit per tile.  Code that runs once
+// per item (mask, bitmask, epilogue) is kept small: unrolled cold paths cost
+// instruction-cache misses of thousands of cycles.
 // Every barrier a thread waits on is at most one phase ahead of it (tile
 // barriers are per tile parity, item barriers per item slot), so parity
 // waits are unambiguous.
 #include <algorithm>
+#include <atomic>
 
 #include "kernels.cuh"
 
@@ -54,12 +69,17 @@ namespace ssd {
 
 namespace {
 
-constexpr int kBM = 128;          // query rows per CTA (TMEM lanes)
-constexpr int KTC = 128;          // keys per tile
+constexpr int kBM = 128;          // most query rows per CTA (TMEM lanes)
+constexpr int KTC = 64;           // keys per tile
 constexpr int kNB = 2;            // ring depth: K stages, V stages, TMEM S/P buffers
-constexpr uint32_t kTmemCols = 512;  // S/P x 2 (128 columns each), O x 2 (128 columns each) at 256
-constexpr int kSoftWarps = 8;     // two per TMEM lane quarter, each taking half of every row
-constexpr int kThreadsTC = (kSoftWarps + 4) * 32;  // + K/Q producer, S, V producer, PV
+constexpr uint32_t kTmemCols = 256;  // S/P x 2 (64 columns each), O (up to 128 columns) at 128
+constexpr int kSoftWarps = 4;     // one per TMEM lane quarter
+constexpr int kThreadsTC = (kSoftWarps + 4) * 32;  // + K/Q producer, V producer, S, PV
+constexpr int kCtasPerSmTC = 2;   // 2 x 256 TMEM columns, 2 x ~107 KB of shared memory
+#ifndef SSD_ATTN_CLUSTER
+#define SSD_ATTN_CLUSTER 4
+#endif
+constexpr int kCluster = SSD_ATTN_CLUSTER;  // CTAs that can share one item
 constexpr float kLog2eTC = 1.4426950408889634f;
 constexpr float kRescale = 8.0f;  // log2 growth of the running max that forces a rescale
 
@@ -98,24 +118,6 @@ __device__ __forceinline__ void tld16x256_x4(uint32_t taddr, float* v) {
 #pragma unroll
   for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
-__device__ __forceinline__ void tst16x256_x8(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
-      "%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32};" ::"r"(taddr),
-      "r"(__float_as_uint(v[0])), "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])),
-      "r"(__float_as_uint(v[3])), "r"(__float_as_uint(v[4])), "r"(__float_as_uint(v[5])),
-      "r"(__float_as_uint(v[6])), "r"(__float_as_uint(v[7])), "r"(__float_as_uint(v[8])),
-      "r"(__float_as_uint(v[9])), "r"(__float_as_uint(v[10])), "r"(__float_as_uint(v[11])),
-      "r"(__float_as_uint(v[12])), "r"(__float_as_uint(v[13])), "r"(__float_as_uint(v[14])),
-      "r"(__float_as_uint(v[15])), "r"(__float_as_uint(v[16])), "r"(__float_as_uint(v[17])),
-      "r"(__float_as_uint(v[18])), "r"(__float_as_uint(v[19])), "r"(__float_as_uint(v[20])),
-      "r"(__float_as_uint(v[21])), "r"(__float_as_uint(v[22])), "r"(__float_as_uint(v[23])),
-      "r"(__float_as_uint(v[24])), "r"(__float_as_uint(v[25])), "r"(__float_as_uint(v[26])),
-      "r"(__float_as_uint(v[27])), "r"(__float_as_uint(v[28])), "r"(__float_as_uint(v[29])),
-      "r"(__float_as_uint(v[30])), "r"(__float_as_uint(v[31]))
-      : "memory");
-  asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void tst16x256_x4(uint32_t taddr, const float* v) {
   asm volatile(
       "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
@@ -144,38 +146,145 @@ __host__ __device__ constexpr uint32_t idesc_f16(int n, bool b_mn_major, int m =
   return idesc_bf16(m, n, false, b_mn_major);
 }
 
+// 64 consecutive 32-bit columns of this thread's TMEM lane (warp-collective).
+__device__ __forceinline__ void tmem_ld64(uint32_t taddr, float* v) {
+  uint32_t r[64];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x64.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,"
+      "%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31,%32,%33,%34,%35,%36,"
+      "%37,%38,%39,%40,%41,%42,%43,%44,%45,%46,%47,%48,%49,%50,%51,%52,%53,%54,%55,%56,%57,%58,"
+      "%59,%60,%61,%62,%63}, [%64];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
+        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
+        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+        "=r"(r[32]), "=r"(r[33]), "=r"(r[34]), "=r"(r[35]), "=r"(r[36]), "=r"(r[37]),
+        "=r"(r[38]), "=r"(r[39]), "=r"(r[40]), "=r"(r[41]), "=r"(r[42]), "=r"(r[43]),
+        "=r"(r[44]), "=r"(r[45]), "=r"(r[46]), "=r"(r[47]), "=r"(r[48]), "=r"(r[49]),
+        "=r"(r[50]), "=r"(r[51]), "=r"(r[52]), "=r"(r[53]), "=r"(r[54]), "=r"(r[55]),
+        "=r"(r[56]), "=r"(r[57]), "=r"(r[58]), "=r"(r[59]), "=r"(r[60]), "=r"(r[61]),
+        "=r"(r[62]), "=r"(r[63])
+      : "r"(taddr)
+      : "memory");
+#pragma unroll
+  for (int i = 0; i < 64; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+// ------------------------------------------------ cluster (distributed smem)
+__device__ __forceinline__ uint32_t cluster_size() {
+  uint32_t n;
+  asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
+  return n;
+}
+// Every thread of every CTA of the cluster; orders shared-memory accesses.
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The address of this CTA's shared-memory location `saddr` in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, uint32_t rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float4 ld_peer4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+__device__ __forceinline__ float2 ld_peer2(uint32_t a) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];"
+               : "=f"(v.x), "=f"(v.y)
+               : "r"(a)
+               : "memory");
+  return v;
+}
+
 struct TcLaunch {
-  int32_t splits, kps, mtiles;
-  float* part_o;
-  float* part_lse;
-  int32_t* seq_ok;
+  int32_t mtiles;   // query tiles of a KV head with D_max drafts
 };
 
-// One work item (KV split, sequence, KV head, query tile) as the producer
-// hands it to the MMA and softmax warps; ntiles < 0 ends the CTA's work.
+// One work item (sequence, KV head, query tile, part of the keys) as the
+// producer hands it to the MMA and softmax warps; ntiles < 0 ends the CTA's
+// work.
 struct TcItem {
-  int32_t b, g, split, row0, rows_total, cache, Lk, k_lo, k_hi, ntiles, direct;
-  int32_t increasing;  // kflat strictly increasing (the raster frontier): draft j sees draft j' iff j' <= j
-  int32_t pad[4];
+  int32_t b, g, row0, rows_total, cache, Lk, k_lo, k_hi, ntiles;
+  int32_t order;       // kOrder*: how the drafts' positions are ordered
+  int32_t pad[2];
   int32_t kflat[128];  // raster position of each draft of b
 };
 
+// The drafts' raster positions: in any order (kflat), strictly increasing
+// (kflat; draft j sees draft j' iff j' <= j), or the flat positions right after
+// the cache (the step's frontier: cache + j, kflat unused).
+constexpr int32_t kOrderAny = 0, kOrderIncreasing = 1, kOrderFlat = 2;
+
+// A sequence of the plan, in longest-first order; its items are off .. off +
+// (items of the sequence) - 1.
+struct TcSeq {
+  int32_t b, cache, nd, off;
+};
+
+// Q buffers: the next item's Q loads while the current one is in use where
+// two fit beside the rings (64-row tiles).
+template <int BM>
+constexpr int kQBufs = BM == 64 ? 2 : 1;
 template <int D, int BM>
 constexpr size_t tc_smem_bytes() {
-  return 1024 + (size_t)2 * BM * D * 2 + (size_t)2 * kNB * KTC * D * 2 + 320 +
-         2 * sizeof(TcItem) + (size_t)6 * kBM * 4;
+  return 1024 + (size_t)kQBufs<BM> * BM * D * 2 + (size_t)2 * kNB * KTC * D * 2 + 256 +
+         2 * sizeof(TcItem) + (size_t)kBM * 8;
 }
 
-// One K or V tile of KTC keys in the MMA's layout [d / 64][KTC rows][128 B]
-// (128-byte swizzle) with one copy: for d = 128 the tensor map is the 3D view
-// {64, rows, 2} whose last dimension steps 128 B inside a row.
+// One Q, K or V tile in the MMA's layout [d / 64][rows][128 B] (128-byte
+// swizzle) with one copy: every map is a 4D view whose dimension of extent d /
+// 64 steps 128 B inside a row, so that one instruction (with a lane per tile)
+// can issue the copies of all three.
+__device__ __forceinline__ void load_tile(void* dst, const CUtensorMap* map, int32_t c1, int32_t c2,
+                                          uint64_t* bar, uint64_t policy) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(0), "r"(smem_u32(bar)),
+      "l"(policy)
+      : "memory");
+}
+
+// Byte offset of 16-byte chunk ch of row r of a CTA's partial O [rows][D] fp32
+// in shared memory: chunks permuted by the row so that a warp's stores of one
+// column by 32 rows spread over the banks.
 template <int D>
-__device__ __forceinline__ void load_kv_tile(void* dst, const CUtensorMap* map, int32_t row,
-                                             uint64_t* bar, uint64_t pol) {
-  if constexpr (D == 128)
-    tma_load_3d(dst, map, 0, row, 0, bar, pol);
-  else
-    tma_load_2d(dst, map, 0, row, bar, pol);
+__device__ __forceinline__ uint32_t part_off(int32_t r, int32_t ch) {
+  return (uint32_t)r * (D * 4) + (uint32_t)((ch ^ (r & 7)) << 4);
+}
+
+// The keys c0 .. c0 + 63 a row may see, as a bit mask: cache keys are a prefix
+// of the window (visible up to qpos), draft keys come from the row's
+// visibility bits (vhi:vlo), keys past the part are dropped.
+__device__ __forceinline__ uint64_t keep_mask(int32_t c0, int32_t cache, int32_t k_hi, int32_t qpos,
+                                              uint64_t vlo, uint64_t vhi) {
+  auto low = [](int32_t n) -> uint64_t {
+    return n <= 0 ? 0ull : (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
+  };
+  const int32_t base = c0 - cache;  // draft index of column 0
+  uint64_t win;                     // bit jj: draft base + jj is visible
+  if (base >= 128 || base <= -64) win = 0;
+  else if (base >= 64) win = vhi >> (base - 64);
+  else if (base > 0) win = (vlo >> base) | (vhi << (64 - base));
+  else if (base == 0) win = vlo;
+  else win = vlo << (-base);
+  const int32_t seen_end = qpos < cache ? qpos + 1 : cache;
+  return (low(seen_end - c0) | (win & ~low(cache - c0))) & low(k_hi - c0);
+}
+// Visibility bits of drafts 0 .. n - 1.
+__device__ __forceinline__ void first_bits(int32_t n, uint64_t& lo, uint64_t& hi) {  // 1 <= n <= 128
+  lo = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
+  hi = n <= 64 ? 0ull : (n >= 128 ? ~0ull : ((1ull << (n - 64)) - 1ull));
 }
 
 // BM = 128: query tiles of 128 rows, row m in TMEM lane m.  BM = 64 (items of
@@ -183,206 +292,316 @@ __device__ __forceinline__ void load_kv_tile(void* dst, const CUtensorMap* map, 
 // so the rows spread over the four lane quarters and their softmax over all
 // four SM sub-partitions.
 template <int D, int BM>
-__global__ void __launch_bounds__(kThreadsTC, 1)
+__global__ void __launch_bounds__(kThreadsTC, kCtasPerSmTC)
 frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, AttnArgs a, TcLaunch L) {
   static_assert(BM == 64 || BM == 128, "query tile");
-  constexpr int NSUB = D / 64;
+  static_assert(kLptMax <= kThreadsTC, "one thread per planned sequence");
+  constexpr int NQ = kQBufs<BM>;
   constexpr int Q_BYTES = BM * D * 2;
   constexpr int KV_BYTES = KTC * D * 2;      // one K (or V) tile
   constexpr uint32_t kIdescS = idesc_f16(KTC, false, BM);
   constexpr uint32_t kIdescO = idesc_f16(D, true, BM);
-  constexpr int HC = KTC / 2;                // S columns per softmax thread (P: HC / 2)
-  constexpr int HD = D / 2;                  // O columns per softmax thread
+  static_assert(BM * D * 4 <= 2 * kNB * KV_BYTES, "a partial O fits in the K and V rings");
 
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ int32_t s_order[kLptMax];
-  __shared__ int32_t s_key[kLptMax];
+  __shared__ TcSeq s_seq[kLptMax];     // the plan: sequences longest first
+  __shared__ int2 s_key[kLptMax];      // (keys, items) of each sequence
+  __shared__ int32_t s_plan[2];        // live items, most keys
+  __shared__ TcItem* s_merge;          // the item this CTA shares with its group (split mode)
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  unsigned char* sQ = smem;                         // [2][Q_BYTES]
-  unsigned char* sK = sQ + 2 * Q_BYTES;             // [kNB][KV_BYTES]
+  unsigned char* sQ = smem;                         // [NQ][Q_BYTES]
+  unsigned char* sK = sQ + NQ * Q_BYTES;            // [kNB][KV_BYTES]
   unsigned char* sV = sK + kNB * KV_BYTES;          // [kNB][KV_BYTES]
   uint64_t* bar = reinterpret_cast<uint64_t*>(sV + kNB * KV_BYTES);
-  uint64_t* q_full = bar;                           // [2] per item slot
-  uint64_t* q_empty = q_full + 2;                   // [2]
-  uint64_t* it_full = q_empty + 2;                  // [2]
+  uint64_t* q_full = bar;                           // [NQ] per Q buffer
+  uint64_t* q_empty = q_full + 2;                   // [NQ]
+  uint64_t* it_full = q_empty + 2;                  // [2] per item slot
   uint64_t* it_empty = it_full + 2;                 // [2]
-  uint64_t* o_empty = it_empty + 2;                 // [2]
+  uint64_t* o_empty = it_empty + 2;                 // O read by the epilogue
   // per ring slot t % kNB: k_ready = K_t loaded and the TMEM S/P buffer free
   // (PV_{t-kNB} done); s_full = S_t done (K stage free); v_ready = V_t loaded
   // and P_t written; pv_done = PV_t done (V stage free)
-  uint64_t* k_ready = o_empty + 2;                  // [kNB]
+  uint64_t* k_ready = o_empty + 1;                  // [kNB]
   uint64_t* s_full = k_ready + kNB;                 // [kNB]
   uint64_t* v_ready = s_full + kNB;                 // [kNB]
   uint64_t* pv_done = v_ready + kNB;                // [kNB]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pv_done + kNB);
-  TcItem* items = reinterpret_cast<TcItem*>(bar + 40);  // [2]
-  float* xch = reinterpret_cast<float*>(items + 2);     // [3 slots][2 halves][128 rows]
+  TcItem* items = reinterpret_cast<TcItem*>(bar + 32);  // [2]
+  float2* s_ml = reinterpret_cast<float2*>(items + 2);  // [128] split mode: (max, sum) of each row
 
   const int32_t G = a.Hq / a.Hkv;
   const int32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int32_t per_b = a.Hkv * L.splits * L.mtiles;
-  const int64_t n_items = (int64_t)a.B * per_b;
+  const bool planned = a.B <= kLptMax;
 
-  // ---- set-up: barriers, TMEM, the longest-first order of the sequences
-  if (tid == 0) {
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&q_full[i], 1);
-      mbar_init(&q_empty[i], 1);
-      mbar_init(&it_full[i], 1);
-      mbar_init(&it_empty[i], kSoftWarps);
-      mbar_init(&o_empty[i], kSoftWarps);
+  // ---- set-up.  The first copies are the start-up's critical path, so the
+  // producer warp alone initialises the barriers, makes the plan (of up to 32
+  // sequences, a lane each) and issues its first item's copies before the
+  // block's barrier; larger batches are planned by the whole block.
+  const float c2 = (a.scale != 0.f ? a.scale : rsqrtf((float)D)) * kLog2eTC;
+  const uint64_t pol = policy_evict_first(), polq = policy_evict_last();
+  const int32_t per_b = a.Hkv * L.mtiles;
+  // this thread's sequence: (keys, items), cache length and drafts; a lane of
+  // the producer warp each, or a thread of the block each for larger batches
+  const bool small = a.B <= 32;
+  const int32_t seq = small ? (warp == kSoftWarps ? lane : a.B) : tid;
+  int2 key = make_int2(0, 0);
+  int32_t c = 0, n = 0;
+  if (planned && seq < a.B) {
+    c = a.cache_len[seq];
+    n = attn_drafts(a, seq);
+    if (n < 0 || n > a.D_max || c < 0 || c > a.L_max - n) {
+      if (blockIdx.x == 0) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
+    } else if (n > 0) {
+      key = make_int2(c + n, a.Hkv * ((n * G + BM - 1) / BM));
     }
-    for (int s = 0; s < kNB; ++s) {
-      mbar_init(&k_ready[s], 2);
-      mbar_init(&s_full[s], 1);
-      mbar_init(&v_ready[s], 1 + kSoftWarps);
-      mbar_init(&pv_done[s], 1);
-    }
-    fence_barrier_init();
-    // every S/P buffer starts free: the PV arrivals of the first round
-    for (int s = 0; s < kNB; ++s) mbar_arrive(&k_ready[s]);
   }
-  if (warp == kSoftWarps && lane < 3)  // the first copies need the descriptors
-    prefetch_tensormap(lane == 0 ? &tmQ : (lane == 1 ? &tmK : &tmV));
-  if (warp == 0) {
+  TcSeq mine{0, 0, 0, 0x7fffffff};  // producer warp: this lane's sequence and first item (B <= 32)
+  if (warp == kSoftWarps) {
+    if (lane == 0) {
+      for (int i = 0; i < NQ; ++i) {
+        mbar_init(&q_full[i], 1);
+        mbar_init(&q_empty[i], 1);
+      }
+      for (int i = 0; i < 2; ++i) {
+        mbar_init(&it_full[i], 1);
+        mbar_init(&it_empty[i], kSoftWarps);
+      }
+      mbar_init(o_empty, kSoftWarps);
+#pragma unroll 1
+      for (int s = 0; s < kNB; ++s) {
+        mbar_init(&k_ready[s], 2);
+        mbar_init(&s_full[s], 1);
+        mbar_init(&v_ready[s], 1 + kSoftWarps);
+        mbar_init(&pv_done[s], 1);
+      }
+      fence_barrier_init();
+      // every S/P buffer starts free: the PV arrivals of the first round
+#pragma unroll 1
+      for (int s = 0; s < kNB; ++s) mbar_arrive(&k_ready[s]);
+      s_merge = nullptr;
+    }
+    if (small) {
+      // sequences longest first (ties by index), those without drafts last
+      int32_t off = 0;
+#pragma unroll 2
+      for (int32_t j = 0; j < a.B; ++j) {
+        const int32_t kj = __shfl_sync(0xffffffffu, key.x, j), cj = __shfl_sync(0xffffffffu, key.y, j);
+        off += (kj > key.x || (kj == key.x && j < lane)) ? cj : 0;
+      }
+      if (key.y > 0) mine = TcSeq{lane, c, n, off};
+      const int32_t total = __reduce_add_sync(0xffffffffu, key.y);
+      const int32_t most = __reduce_max_sync(0xffffffffu, key.x);
+      if (lane == 0) {
+        s_plan[0] = total;
+        s_plan[1] = most;
+      }
+    }
+    __syncwarp();
+  } else if (warp == kSoftWarps + 1) {
+    if (lane < 3)  // the first copies need the descriptors
+      prefetch_tensormap(lane == 0 ? &tmQ : (lane == 1 ? &tmK : &tmV));
+  } else if (warp == kSoftWarps + 3) {
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
-  if (a.B <= kLptMax) {
-    // s_order[rank] = the sequence with the rank-th most keys (ties by index);
-    // a sequence with no drafts ranks last (its items are empty)
-    for (int32_t i = tid; i < a.B; i += blockDim.x) {
-      const int32_t c = a.cache_len[i], n = attn_drafts(a, i);
-      s_key[i] = (c >= 0 && n > 0 && c <= a.L_max && n <= a.D_max) ? c + n : 0;
+  if (planned && !small) {
+    if (tid < a.B) s_key[tid] = key;
+    __syncthreads();
+    if (tid < a.B) {
+      int32_t r = 0, off = 0, total = 0, most = 0;
+#pragma unroll 1
+      for (int32_t j = 0; j < a.B; ++j) {
+        const int2 kj = s_key[j];
+        const bool ahead = kj.x > key.x || (kj.x == key.x && j < tid);
+        r += ahead ? 1 : 0;
+        off += ahead ? kj.y : 0;
+        total += kj.y;
+        most = max(most, kj.x);
+      }
+      s_seq[r] = TcSeq{tid, c, n, off};
+      if (tid == 0) {
+        s_plan[0] = total;
+        s_plan[1] = most;
+      }
     }
     __syncthreads();
-    for (int32_t i = tid; i < a.B; i += blockDim.x) {
-      const int32_t key = s_key[i];
-      int32_t r = 0;
-      for (int32_t j = 0; j < a.B; ++j) {
-        const int32_t kj = s_key[j];
-        r += (kj > key) || (kj == key && j < i);
-      }
-      s_order[r] = i;
-    }
   }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-  const uint32_t tS = tmem;            // [kNB] x KTC columns: S_t in fp32, then P_t in bf16
-  const uint32_t tO0 = tmem + 256;     // [2] x 128 columns
 
-  const float c2 = (a.scale != 0.f ? a.scale : rsqrtf((float)D)) * kLog2eTC;
+  // CTAs per item: as many of a cluster (a power of two) as leave one item or
+  // none per group of them, but no more than the longest item has tiles
+  int32_t n_items = 0, ns_log = 0;
+  auto read_plan = [&]() {
+    n_items = planned ? s_plan[0] : a.B * per_b;
+    if (planned) {
+      const int32_t cs = (int32_t)cluster_size(), most_tiles = (s_plan[1] + KTC - 1) / KTC;
+      while ((2 << ns_log) <= cs && ((2 << ns_log) * n_items) <= (int32_t)gridDim.x &&
+             (2 << ns_log) <= most_tiles)
+        ++ns_log;
+    }
+  };
+  uint32_t tmem = 0, tS = 0, tO = 0;
+  auto block_start = [&]() {  // every warp: the set-up is done
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    tmem = *tmem_slot;
+    tS = tmem;          // [kNB] x KTC columns: S_t in fp32, then P_t in bf16
+    tO = tmem + 128;    // up to 128 columns
+  };
+  if (warp != kSoftWarps) {
+    block_start();
+    read_plan();
+  }
 
   if (warp == kSoftWarps) {
     // ------------------------------------------------------------ producer
     // Items in snake order over the longest-first list: round k takes items
-    // k * gridDim.x + (blockIdx.x, or its mirror on odd rounds).
-    const uint64_t pol = policy_evict_first();
-    const uint64_t polq = policy_evict_last();
+    // k * ngroups + (group, or its mirror on odd rounds).
     const int32_t HW = a.grid.grid_h * a.grid.grid_w;
-    bool ok = true;
+    bool ok = true, started = false;
     int32_t k = 0;        // items handed out
-    uint32_t T = 0;       // K/V tiles issued
-    for (int64_t round = 0; ok; ++round) {
-      const int64_t base = round * gridDim.x;
+    uint32_t T = 0;       // K tiles issued
+    read_plan();
+    const int32_t ns = 1 << ns_log;
+    const int32_t part = (int32_t)blockIdx.x & (ns - 1), group = (int32_t)blockIdx.x >> ns_log;
+    const int32_t ngroups = (int32_t)gridDim.x >> ns_log;
+#pragma unroll 1
+    for (int32_t round = 0; ok; ++round) {
+      const int32_t base = round * ngroups;
       if (base >= n_items) break;
-      const int64_t i = base + ((round & 1) ? (gridDim.x - 1 - blockIdx.x) : blockIdx.x);
+      const int32_t i = base + ((round & 1) ? (ngroups - 1 - group) : group);
       if (i >= n_items) continue;
-      const int32_t rank_b = (int32_t)(i / per_b);
-      int32_t rem = (int32_t)(i - (int64_t)rank_b * per_b);
-      const int32_t mtile = rem % L.mtiles;
-      rem /= L.mtiles;
-      const int32_t split = rem % L.splits, g = rem / L.splits;
-      const int32_t b = (a.B <= kLptMax) ? s_order[rank_b] : rank_b;
-      const int32_t cache = a.cache_len[b], nd = attn_drafts(a, b);
-      const bool shape_ok = nd >= 0 && nd <= a.D_max && cache >= 0 && cache <= a.L_max - nd;
-      // draft positions (validity is identical in every item of b)
-      int32_t kfv[4];
-      bool bad = !shape_ok;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int32_t j = lane + 32 * u;
-        kfv[u] = 0;
-        if (shape_ok && j < nd) {
-          const int32_t gidx = attn_draft_pos(a, b, j);
-          if (gidx < 0 || gidx >= HW) {
-            bad = true;
-          } else {
-            const int32_t y = gidx / a.grid.grid_w, x = gidx - y * a.grid.grid_w;
-            kfv[u] = a.grid.prefix_len + y * a.grid.row_stride + x;
-          }
+      TcSeq q;
+      int32_t mt = 1;
+      if (small) {
+        // the sequence with the last first item at or before i
+        const int32_t first = __reduce_max_sync(0xffffffffu, mine.off <= i ? mine.off : -1);
+        const int src = __ffs(__ballot_sync(0xffffffffu, mine.off == first)) - 1;
+        q.b = src;
+        q.cache = __shfl_sync(0xffffffffu, mine.cache, src);
+        q.nd = __shfl_sync(0xffffffffu, mine.nd, src);
+        q.off = first;
+      } else if (planned) {
+        // (sequences without items come last, at off == n_items)
+        int32_t r = -1;
+#pragma unroll 1
+        for (int32_t r0 = 0; r0 < a.B; r0 += 32) {
+          const bool le = r0 + lane < a.B && s_seq[r0 + lane].off <= i;
+          const uint32_t m = __ballot_sync(0xffffffffu, le);
+          if (m == 0) break;
+          r = r0 + 31 - __clz(m);
         }
+        q = s_seq[r];
+      } else {
+        q.b = i / per_b;
+        q.off = q.b * per_b;
+        q.cache = a.cache_len[q.b];
+        q.nd = attn_drafts(a, q.b);
+        mt = L.mtiles;
       }
-      const bool valid = !__any_sync(0xffffffffu, bad);
-      // strictly increasing positions? (the previous draft of j = lane + 32 u is
-      // lane - 1 of the same u, or lane 31 of u - 1)
-      bool dec = false;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int32_t up = __shfl_up_sync(0xffffffffu, kfv[u], 1);
-        const int32_t prev_hi = __shfl_sync(0xffffffffu, u > 0 ? kfv[u > 0 ? u - 1 : 0] : 0, 31);
-        const int32_t prev = lane > 0 ? up : prev_hi;
-        const int32_t j = lane + 32 * u;
-        if (j >= 1 && j < nd && kfv[u] <= prev) dec = true;
+      const int32_t b = q.b, cache = q.cache, nd = q.nd;
+      if (planned && L.mtiles > 1) mt = (nd * G + BM - 1) / BM;
+      int32_t g = i - q.off, mtile = 0;
+      if (mt > 1) {
+        const int32_t rem = g;
+        g = rem / mt;
+        mtile = rem - g * mt;
       }
-      const bool increasing = !__any_sync(0xffffffffu, dec);
-      if (split == 0 && g == 0 && mtile == 0 && lane == 0) {
-        L.seq_ok[b] = valid ? 1 : 0;
-        if (!valid) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
-      }
-      const int32_t Lk = valid ? cache + nd : 0;
-      const int32_t rows_total = valid ? nd * G : 0;
-      const int32_t row0 = mtile * BM;
-      const int32_t k_lo = split * L.kps;
-      const int32_t k_hi = min(Lk, k_lo + L.kps);
-      if (!valid || nd == 0 || row0 >= rows_total || k_lo >= Lk) continue;
-      const int32_t ntiles = (k_hi - k_lo + KTC - 1) / KTC;
       const int s = k & 1;
+      TcItem& it = items[s];
+      // (a slot is rewritten once the softmax is done with its item before)
       if (k >= 2 && lane == 0) ok = mbar_wait(&it_empty[s], ((k >> 1) - 1) & 1, a.status);
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
-      TcItem& it = items[s];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (lane + 32 * u < nd) it.kflat[lane + 32 * u] = kfv[u];
+      bool valid = planned || (nd >= 0 && nd <= a.D_max && cache >= 0 && cache <= a.L_max - nd);
+      int32_t order = kOrderFlat;
+      if (!(a.raster && a.grid.row_stride == a.grid.grid_w) && valid) {
+        // draft positions (validity is identical in every item of b); strictly
+        // increasing ones?  (The draft before j is lane - 1's, or the last lane's
+        // of the 32 before.)
+        bool bad = false, dec = false;
+        int32_t last = -1;
+#pragma unroll 1
+        for (int32_t j = lane; j - lane < nd; j += 32) {
+          int32_t kf = 0x7fffffff;
+          if (j < nd) {
+            const int32_t gidx = attn_draft_pos(a, b, j);
+            if (gidx < 0 || gidx >= HW) {
+              bad = true;
+            } else {
+              const int32_t y = gidx / a.grid.grid_w, x = gidx - y * a.grid.grid_w;
+              kf = a.grid.prefix_len + y * a.grid.row_stride + x;
+            }
+            it.kflat[j] = kf;
+          }
+          const int32_t up = __shfl_up_sync(0xffffffffu, kf, 1);
+          if (j < nd && kf <= (lane > 0 ? up : last)) dec = true;
+          last = __shfl_sync(0xffffffffu, kf, 31);
+        }
+        valid = !__any_sync(0xffffffffu, bad);
+        order = __any_sync(0xffffffffu, dec) ? kOrderAny : kOrderIncreasing;
+      }
+      if (!valid && i == q.off && part == 0 && lane == 0)
+        record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
+      const int32_t Lk = cache + nd, rows_total = nd * G, row0 = mtile * BM;
+      if (!valid || nd == 0 || row0 >= rows_total) continue;
+      const int32_t tiles = (Lk + KTC - 1) / KTC;
+      const int32_t t_lo = (tiles * part) >> ns_log, t_hi = (tiles * (part + 1)) >> ns_log;
+      const int32_t ntiles = t_hi - t_lo;
+      const int32_t kvrow0 = (b * a.Hkv + g) * a.L_max + t_lo * KTC;  // 2D row of the first key
+      const int32_t qrow = b * a.D_max + row0 / G;
+      const int sq = k % NQ;
+      int t = 0;
       if (lane == 0) {
         it.b = b;
         it.g = g;
-        it.split = split;
         it.row0 = row0;
         it.rows_total = rows_total;
         it.cache = cache;
         it.Lk = Lk;
-        it.k_lo = k_lo;
-        it.k_hi = k_hi;
+        it.k_lo = t_lo * KTC;
+        it.k_hi = min(Lk, t_hi * KTC);
         it.ntiles = ntiles;
-        it.direct = ((Lk + L.kps - 1) / L.kps) == 1;
-        it.increasing = increasing ? 1 : 0;
+        it.order = order;
+        if (ns > 1) s_merge = &it;
       }
+      if (ntiles == 0) continue;  // split mode: fewer tiles than CTAs in the group
       __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&it_full[s]);
-        // Q of this item into slot s once the S products of item k - 2 are done
-        if (k >= 2) ok = mbar_wait(&q_empty[s], ((k >> 1) - 1) & 1, a.status);
-        if (ok) {
-          mbar_arrive_expect_tx(&q_full[s], Q_BYTES);
-          for (int c = 0; c < NSUB; ++c) {
-            // 3D Q view {d, Hq, B * D_max}: box {64, G, BM / G} -> rows (j, hg)
-            asm volatile(
-                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
-                " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(
-                    smem_u32(sQ + s * Q_BYTES + c * (BM * 128))),
-                "l"(reinterpret_cast<uint64_t>(&tmQ)), "r"(c * 64), "r"(g * G),
-                "r"(b * a.D_max + row0 / G), "r"(smem_u32(&q_full[s])), "l"(polq)
-                : "memory");
+      if (k == 0) {
+        // the CTA's first item: every ring slot is free, so its first K, Q and V
+        // copies go out at once, one lane each
+        t = min(ntiles, kNB);
+        if (lane < 1 + 2 * kNB) {
+          const bool is_q = lane == 1, is_k = lane == 0 || (lane > 1 && (lane & 1));
+          const int st = is_q ? 0 : (lane == 0 ? 0 : (lane - 1) >> 1);  // lanes 0 K0, 1 Q, 2 V0, 3 K1, 4 V1
+          if (is_q || st < ntiles) {
+            uint64_t* bar1 = is_q ? &q_full[0] : (is_k ? &k_ready[st] : &v_ready[st]);
+            unsigned char* dst = is_q ? sQ : (is_k ? sK : sV) + st * KV_BYTES;
+            mbar_arrive_expect_tx(bar1, is_q ? Q_BYTES : KV_BYTES);
+            load_tile(dst, is_q ? &tmQ : (is_k ? &tmK : &tmV), is_q ? g * G : kvrow0 + st * KTC,
+                      is_q ? qrow : 0, bar1, is_q ? polq : pol);
           }
         }
-        const int32_t kvrow0 = (b * a.Hkv + g) * a.L_max + k_lo;  // 2D row of the first key
-        for (int t = 0; t < ntiles && ok; ++t, ++T) {
+        T = t;
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&it_full[0]);
+        block_start();
+        started = true;
+      } else if (lane == 0) {
+        mbar_arrive(&it_full[s]);
+        // Q of this item into its buffer once the S products of the item before
+        // that used it are done
+        if (k >= NQ) ok = mbar_wait(&q_empty[sq], ((k / NQ) - 1) & 1, a.status);
+        if (ok) {
+          mbar_arrive_expect_tx(&q_full[sq], Q_BYTES);
+          load_tile(sQ + sq * Q_BYTES, &tmQ, g * G, qrow, &q_full[sq], polq);
+        }
+      }
+      if (lane == 0) {
+#pragma unroll 1
+        for (; t < ntiles && ok; ++t, ++T) {
           const int sb = T % kNB;
           // K stage sb is free once S_{T-kNB} is done
           if (T >= (uint32_t)kNB && !mbar_wait(&s_full[sb], ((T / kNB) - 1) & 1, a.status)) {
@@ -390,7 +609,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             break;
           }
           mbar_arrive_expect_tx(&k_ready[sb], KV_BYTES);
-          load_kv_tile<D>(sK + sb * KV_BYTES, &tmK, kvrow0 + t * KTC, &k_ready[sb], pol);
+          load_tile(sK + sb * KV_BYTES, &tmK, kvrow0 + t * KTC, 0, &k_ready[sb], pol);
         }
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -402,12 +621,14 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const int s = k & 1;
       if (k >= 2 && lane == 0) ok = mbar_wait(&it_empty[s], ((k >> 1) - 1) & 1, a.status);
       if (lane == 0 && ok) {
+        // (split mode: at most one item, in slot 0, which the merge still reads)
         items[s].ntiles = -1;
         mbar_arrive(&it_full[s]);
       }
     }
     __syncwarp();
-  } else if (warp == kSoftWarps + 2) {
+    if (!started) block_start();
+  } else if (warp == kSoftWarps + 1) {
     // ---------------------------------------------------------- V producer
     // Follows the item slots like the MMA warp; a slot is not rewritten before
     // the softmax has finished its item, which needs every V tile of it.
@@ -422,7 +643,6 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // other branch of the V loop's lane test, so that lane 0 never waits at
     // the reconvergence point of a block of its own.
     if (lane == 0) {
-      const uint64_t pol = policy_evict_first();
       uint32_t T = 0;
       bool ok = true;
       for (int32_t k = 0; ok; ++k) {
@@ -432,7 +652,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const int32_t ntiles = it.ntiles;
         if (ntiles < 0) break;
         const int32_t kvrow0 = (it.b * a.Hkv + it.g) * a.L_max + it.k_lo;
-        for (int t = 0; t < ntiles; ++t, ++T) {
+        int t = 0;
+        if (k == 0) T = t = min(ntiles, kNB);  // issued by the producer with the first K tiles
+#pragma unroll 1
+        for (; t < ntiles; ++t, ++T) {
           const int sb = T % kNB;
           // V stage sb is free once PV_{T-kNB} is done
           if (T >= (uint32_t)kNB && !mbar_wait(&pv_done[sb], ((T / kNB) - 1) & 1, a.status)) {
@@ -440,7 +663,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             break;
           }
           mbar_arrive_expect_tx(&v_ready[sb], KV_BYTES);
-          load_kv_tile<D>(sV + sb * KV_BYTES, &tmV, kvrow0 + t * KTC, &v_ready[sb], pol);
+          load_tile(sV + sb * KV_BYTES, &tmV, kvrow0 + t * KTC, 0, &v_ready[sb], pol);
         }
       }
     } else if (lane == 1) {
@@ -448,19 +671,20 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       pdl_launch_dependents();
     }
     __syncwarp();
-  } else if (warp == kSoftWarps + 1) {
+  } else if (warp == kSoftWarps + 2) {
     // ----------------------------------------------------------- S products
     if (lane == 0) {
       uint32_t T = 0;
       for (int32_t k = 0;; ++k) {
-        const int s = k & 1;
+        const int s = k & 1, sq = k % NQ;
         if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) break;
         const int32_t ntiles = items[s].ntiles;
         if (ntiles < 0) break;
-        if (!mbar_wait(&q_full[s], (k >> 1) & 1, a.status)) break;
+        if (!mbar_wait(&q_full[sq], (k / NQ) & 1, a.status)) break;
         tc_fence_after();
-        const uint64_t dq = smem_desc(smem_u32(sQ + s * Q_BYTES), 16, 1024);
+        const uint64_t dq = smem_desc(smem_u32(sQ + sq * Q_BYTES), 16, 1024);
         bool ok = true;
+#pragma unroll 1
         for (int t = 0; t < ntiles; ++t, ++T) {
           const int sb = T % kNB;
           if (!mbar_wait(&k_ready[sb], (T / kNB) & 1, a.status)) { ok = false; break; }
@@ -473,7 +697,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                  smem_desc_at(dk, sub * (KTC * 128) + kin), kIdescS, ks > 0 ? 1u : 0u);
           }
           mma_commit(&s_full[sb]);
-          if (t == ntiles - 1) mma_commit(&q_empty[s]);
+          if (t == ntiles - 1) mma_commit(&q_empty[sq]);
         }
         if (!ok) break;
       }
@@ -491,9 +715,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) break;
         const int32_t ntiles = items[s].ntiles;
         if (ntiles < 0) break;
-        // the first product of the item overwrites O[s]: the epilogue of item k - 2 must be done
-        if (k >= 2 && !mbar_wait(&o_empty[s], ((k >> 1) - 1) & 1, a.status)) break;
+        // the first product of the item overwrites O: the epilogue of the item before must be done
+        if (k >= 1 && !mbar_wait(o_empty, (k - 1) & 1, a.status)) break;
         bool ok = true;
+#pragma unroll 1
         for (int t = 0; t < ntiles; ++t, ++T) {
           const int sb = T % kNB;
           if (!mbar_wait(&v_ready[sb], (T / kNB) & 1, a.status)) { ok = false; break; }
@@ -503,7 +728,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           const uint64_t dv = smem_desc(smem_u32(sV + sb * KV_BYTES), KTC * 128, 1024);
 #pragma unroll
           for (int kk = 0; kk < KTC / 16; ++kk)
-            mma_ts(tO0 + s * 128, tS + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
+            mma_ts(tO, tS + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
                     (t == 0 && kk == 0) ? 0u : 1u);
           mma_commit(&pv_done[sb]);
           mma_commit(&k_ready[sb]);  // S_{T+kNB} may start: the S/P buffer is free again
@@ -512,290 +737,18 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       }
     }
     __syncwarp();
-  } else if constexpr (BM == 64) {
-    // ------------------------------------------------ softmax, M = 64 items
-    // Item row m sits in TMEM lane 32 (m / 16) + m % 16, so lane quarter q
-    // holds item rows 16q .. 16q + 15.  Warp w takes quarter w % 4 and half
-    // w / 4 of every row's columns; with 16-lane accesses each thread holds two
-    // rows (t / 4 and t / 4 + 8 of the quarter) x 16 columns of its half, and
-    // the four threads t % 4 of a row finish its maxima and sums by shuffles.
-    const int quarter = warp & 3, half = warp >> 2;
-    const int cq = lane & 3;
-    const int32_t rlA = quarter * 16 + (lane >> 2), rlB = rlA + 8;  // item rows of this thread
-    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-    auto xs = [&](int slot, int hf, int32_t rl) -> float& {
-      return xch[(slot * 2 + hf) * kBM + rl];
-    };
-    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory"); };
-    auto low = [](int32_t n) -> uint64_t {
-      return n <= 0 ? 0ull : (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
-    };
-    bool ok = true;
-    uint32_t T = 0;
-    for (int32_t k = 0; ok; ++k) {
-      const int s = k & 1;
-      if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) { ok = false; break; }
-      const TcItem& it = items[s];
-      const int32_t ntiles = it.ntiles;
-      if (ntiles < 0) break;
-      const int32_t b = it.b, g = it.g, split = it.split, row0 = it.row0;
-      const int32_t rows_total = it.rows_total, cache = it.cache, Lk = it.Lk;
-      const int32_t k_lo = it.k_lo, k_hi = it.k_hi;
-      const bool direct = it.direct != 0;
-      const int32_t* kflat = it.kflat;
-      const uint32_t tO = tO0 + s * 128;
-      const int32_t rA = row0 + rlA, rB = row0 + rlB;
-      const bool liveA = rA < rows_total, liveB = rB < rows_total;
-      const bool warp_live = row0 + quarter * 16 < rows_total;  // same for both warps of a pair
-      const int32_t jqA = liveA ? rA / G : 0, hA = g * G + (liveA ? rA - jqA * G : 0);
-      const int32_t jqB = liveB ? rB / G : 0, hB = g * G + (liveB ? rB - jqB * G : 0);
-      const int32_t qposA = liveA ? kflat[jqA] : 0x7fffffff;
-      const int32_t qposB = liveB ? kflat[jqB] : 0x7fffffff;
-      const bool increasing = it.increasing != 0;
-      int32_t minq = 0x7fffffff;
-      const int32_t j_lo = row0 / G;
-      if (increasing) {
-        minq = kflat[j_lo];
-      } else {
-        const int32_t j_end = (min(rows_total, row0 + BM) + G - 1) / G;
-        for (int32_t j = j_lo + lane; j < j_end; j += 32) minq = min(minq, kflat[j]);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) minq = min(minq, __shfl_xor_sync(0xffffffffu, minq, o));
-      }
-      const int32_t mask_from = min(cache, minq + 1);
-      // visibility of the item's drafts to rows A and B (bit j: draft j visible)
-      uint64_t vAlo = 0, vAhi = 0, vBlo = 0, vBhi = 0;
-      if (warp_live && increasing) {
-        const int32_t nA = jqA + 1, nB = jqB + 1;  // 1 .. 128
-        vAlo = nA >= 64 ? ~0ull : ((1ull << nA) - 1ull);
-        vAhi = nA <= 64 ? 0ull : (nA >= 128 ? ~0ull : ((1ull << (nA - 64)) - 1ull));
-        vBlo = nB >= 64 ? ~0ull : ((1ull << nB) - 1ull);
-        vBhi = nB <= 64 ? 0ull : (nB >= 128 ? ~0ull : ((1ull << (nB - 64)) - 1ull));
-      } else if (warp_live) {
-        const int32_t nd = Lk - cache;
-#pragma unroll 1
-        for (int j = 0; j < nd; j += 4) {
-          const int4 kf = *reinterpret_cast<const int4*>(kflat + j);
-          const uint64_t bA = (uint64_t)((uint32_t)(kf.x <= qposA) | ((uint32_t)(kf.y <= qposA) << 1) |
-                                         ((uint32_t)(kf.z <= qposA) << 2) |
-                                         ((uint32_t)(kf.w <= qposA) << 3));
-          const uint64_t bB = (uint64_t)((uint32_t)(kf.x <= qposB) | ((uint32_t)(kf.y <= qposB) << 1) |
-                                         ((uint32_t)(kf.z <= qposB) << 2) |
-                                         ((uint32_t)(kf.w <= qposB) << 3));
-          if (j < 64) {
-            vAlo |= bA << j;
-            vBlo |= bB << j;
-          } else {
-            vAhi |= bA << (j - 64);
-            vBhi |= bB << (j - 64);
-          }
-        }
-      }
-      // keep mask of one row over keys c0 .. c0 + 63 (as in the M = 128 path)
-      auto keep_of = [&](int32_t c0, int32_t qpos, uint64_t vlo, uint64_t vhi) -> uint64_t {
-        const int32_t base = c0 - cache;  // draft index of column 0
-        uint64_t win;
-        if (base >= 128 || base <= -64) win = 0;
-        else if (base >= 64) win = vhi >> (base - 64);
-        else if (base > 0) win = (vlo >> base) | (vhi << (64 - base));
-        else if (base == 0) win = vlo;
-        else win = vlo << (-base);
-        const int32_t seen_end = qpos < cache ? qpos + 1 : cache;
-        return (low(seen_end - c0) | (win & ~low(cache - c0))) & low(k_hi - c0);
-      };
-      float m_runA = -INFINITY, m_runB = -INFINITY, l_runA = 0.f, l_runB = 0.f;
-      for (int t = 0; t < ntiles; ++t, ++T) {
-        const int bb = T & 1, sb = T % kNB;
-        if (!mbar_wait(&s_full[sb], (T / kNB) & 1, a.status)) ok = false;
-        tc_fence_after();
-        float sv[32];
-        if (warp_live) tld16x256_x8(tS + lane_off + sb * KTC + half * HC, sv);
-        bool movedA = false, movedB = false;
-        float alphaA = 1.f, alphaB = 1.f;
-        uint32_t pk[16];
-        if (warp_live) {
-          const int32_t c0 = k_lo + t * KTC + half * HC;
-          if (c0 + HC > k_hi || c0 + HC > mask_from) {
-            const uint64_t keepA = keep_of(c0, qposA, vAlo, vAhi);
-            const uint64_t keepB = keep_of(c0, qposB, vBlo, vBhi);
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int jj = 8 * u + 2 * cq + e;
-                if (!((keepA >> jj) & 1ull)) sv[4 * u + e] = -INFINITY;
-                if (!((keepB >> jj) & 1ull)) sv[4 * u + 2 + e] = -INFINITY;
-              }
-          }
-          float a4[4], b4[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            a4[i] = fmaxf(fmaxf(sv[8 * i], sv[8 * i + 1]), fmaxf(sv[8 * i + 4], sv[8 * i + 5]));
-            b4[i] = fmaxf(fmaxf(sv[8 * i + 2], sv[8 * i + 3]), fmaxf(sv[8 * i + 6], sv[8 * i + 7]));
-          }
-          float mxA = fmaxf(fmaxf(a4[0], a4[1]), fmaxf(a4[2], a4[3]));
-          float mxB = fmaxf(fmaxf(b4[0], b4[1]), fmaxf(b4[2], b4[3]));
-          mxA = fmaxf(mxA, __shfl_xor_sync(0xffffffffu, mxA, 1));
-          mxB = fmaxf(mxB, __shfl_xor_sync(0xffffffffu, mxB, 1));
-          mxA = fmaxf(mxA, __shfl_xor_sync(0xffffffffu, mxA, 2));
-          mxB = fmaxf(mxB, __shfl_xor_sync(0xffffffffu, mxB, 2));
-          // (the pair barrier also orders the partner's tcgen05.ld of S before
-          // this warp overwrites the buffer with P)
-          if (cq == 0) {
-            xs(bb, half, rlA) = mxA;
-            xs(bb, half, rlB) = mxB;
-          }
-          pair_sync();
-          mxA = fmaxf(mxA, xs(bb, half ^ 1, rlA));
-          mxB = fmaxf(mxB, xs(bb, half ^ 1, rlB));
-          // move a running max only when it grows by more than 2^kRescale
-          if (mxA != -INFINITY && (m_runA == -INFINITY || (mxA - m_runA) * c2 > kRescale)) {
-            alphaA = (m_runA == -INFINITY) ? 0.f : ex2_approx((m_runA - mxA) * c2);
-            m_runA = mxA;
-            movedA = true;
-          }
-          if (mxB != -INFINITY && (m_runB == -INFINITY || (mxB - m_runB) * c2 > kRescale)) {
-            alphaB = (m_runB == -INFINITY) ? 0.f : ex2_approx((m_runB - mxB) * c2);
-            m_runB = mxB;
-            movedB = true;
-          }
-          const float moffA = (m_runA == -INFINITY) ? 0.f : m_runA * c2;
-          const float moffB = (m_runB == -INFINITY) ? 0.f : m_runB * c2;
-          float sA[4] = {0.f, 0.f, 0.f, 0.f}, sB[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const float eA0 = ex2_approx(fmaf(sv[4 * u], c2, -moffA));
-            const float eA1 = ex2_approx(fmaf(sv[4 * u + 1], c2, -moffA));
-            const float eB0 = ex2_approx(fmaf(sv[4 * u + 2], c2, -moffB));
-            const float eB1 = ex2_approx(fmaf(sv[4 * u + 3], c2, -moffB));
-            sA[u & 3] += eA0 + eA1;
-            sB[u & 3] += eB0 + eB1;
-            pk[2 * u] = pack_bf16x2(eA0, eA1);
-            pk[2 * u + 1] = pack_bf16x2(eB0, eB1);
-          }
-          l_runA = l_runA * alphaA + ((sA[0] + sA[1]) + (sA[2] + sA[3]));
-          l_runB = l_runB * alphaB + ((sB[0] + sB[1]) + (sB[2] + sB[3]));
-        }
-        if (warp_live) {
-          // O may be rescaled once PV_{T-1} is done
-          if (__any_sync(0xffffffffu, (movedA || movedB) && t > 0)) {
-            if (!mbar_wait(&pv_done[(T - 1) % kNB], ((T - 1) / kNB) & 1, a.status)) ok = false;
-            tc_fence_after();
-            float ov[HD / 2];
-            const uint32_t ta = tO + lane_off + half * HD;
-            if constexpr (HD == 64) tld16x256_x8(ta, ov);
-            else tld16x256_x4(ta, ov);
-#pragma unroll
-            for (int u = 0; u < HD / 8; ++u) {
-              ov[4 * u] *= alphaA;
-              ov[4 * u + 1] *= alphaA;
-              ov[4 * u + 2] *= alphaB;
-              ov[4 * u + 3] *= alphaB;
-            }
-            if constexpr (HD == 64) tst16x256_x8(ta, ov);
-            else tst16x256_x4(ta, ov);
-          }
-          // P_T as bf16 pairs over the first half of its S buffer: this half's
-          // keys are word columns [half * HC / 2, (half + 1) * HC / 2)
-          tst16x128_x8(tS + lane_off + sb * KTC + half * (HC / 2), pk);
-        }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&v_ready[sb]);
-      }
-      // ---- epilogue: wait for the item's last PV product, normalise, write this half
-      const uint32_t Tl = T - 1;
-      if (!mbar_wait(&pv_done[Tl % kNB], (Tl / kNB) & 1, a.status)) ok = false;
-      tc_fence_after();
-      if (warp_live) {
-        float lA = l_runA, lB = l_runB;
-        lA += __shfl_xor_sync(0xffffffffu, lA, 1);
-        lB += __shfl_xor_sync(0xffffffffu, lB, 1);
-        lA += __shfl_xor_sync(0xffffffffu, lA, 2);
-        lB += __shfl_xor_sync(0xffffffffu, lB, 2);
-        if (cq == 0) {
-          xs(2, half, rlA) = lA;
-          xs(2, half, rlB) = lB;
-        }
-        pair_sync();
-        const float ltA = lA + xs(2, half ^ 1, rlA), ltB = lB + xs(2, half ^ 1, rlB);
-        const float invA = ltA > 0.f ? __fdividef(1.0f, ltA) : 0.f;
-        const float invB = ltB > 0.f ? __fdividef(1.0f, ltB) : 0.f;
-        float ov[HD / 2];
-        const uint32_t ta = tO + lane_off + half * HD;
-        if constexpr (HD == 64) tld16x256_x8(ta, ov);
-        else tld16x256_x4(ta, ov);
-        // (debug builds: the rows' store indexes against their buffers)
-        const int64_t n_rows_o = (int64_t)a.B * a.D_max * a.Hq;
-        const int64_t n_rows_p = (int64_t)a.B * a.Hq * a.D_max * L.splits;
-        const bool sA = liveA && (direct ? dbg_in(((int64_t)b * a.D_max + jqA) * a.Hq + hA, n_rows_o, a.status)
-                                         : dbg_in((((int64_t)b * a.Hq + hA) * a.D_max + jqA) * L.splits + split, n_rows_p, a.status));
-        const bool sB = liveB && (direct ? dbg_in(((int64_t)b * a.D_max + jqB) * a.Hq + hB, n_rows_o, a.status)
-                                         : dbg_in((((int64_t)b * a.Hq + hB) * a.D_max + jqB) * L.splits + split, n_rows_p, a.status));
-        if (ok) {
-          const int colb = half * HD + 2 * cq;
-          if (direct) {
-            __nv_bfloat16* oA = reinterpret_cast<__nv_bfloat16*>(a.o) +
-                                (((int64_t)b * a.D_max + jqA) * a.Hq + hA) * D + colb;
-            __nv_bfloat16* oB = reinterpret_cast<__nv_bfloat16*>(a.o) +
-                                (((int64_t)b * a.D_max + jqB) * a.Hq + hB) * D + colb;
-#pragma unroll
-            for (int u = 0; u < HD / 8; ++u) {
-              if (sA)
-                *reinterpret_cast<uint32_t*>(oA + 8 * u) =
-                    pack_bf16x2(ov[4 * u] * invA, ov[4 * u + 1] * invA);
-              if (sB)
-                *reinterpret_cast<uint32_t*>(oB + 8 * u) =
-                    pack_bf16x2(ov[4 * u + 2] * invB, ov[4 * u + 3] * invB);
-            }
-          } else {
-            float* pA = L.part_o +
-                        ((((int64_t)b * a.Hq + hA) * a.D_max + jqA) * L.splits + split) * D + colb;
-            float* pB = L.part_o +
-                        ((((int64_t)b * a.Hq + hB) * a.D_max + jqB) * L.splits + split) * D + colb;
-#pragma unroll
-            for (int u = 0; u < HD / 8; ++u) {
-              if (sA)
-                *reinterpret_cast<float2*>(pA + 8 * u) =
-                    make_float2(ov[4 * u] * invA, ov[4 * u + 1] * invA);
-              if (sB)
-                *reinterpret_cast<float2*>(pB + 8 * u) =
-                    make_float2(ov[4 * u + 2] * invB, ov[4 * u + 3] * invB);
-            }
-          }
-          if (half == 0 && cq == 0) {
-            const float lseA =
-                ltA > 0.f ? (m_runA * (c2 / kLog2eTC) + __logf(ltA)) : -INFINITY;
-            const float lseB =
-                ltB > 0.f ? (m_runB * (c2 / kLog2eTC) + __logf(ltB)) : -INFINITY;
-            if (direct) {
-              if (a.lse != nullptr && sA) a.lse[((int64_t)b * a.Hq + hA) * a.D_max + jqA] = lseA;
-              if (a.lse != nullptr && sB) a.lse[((int64_t)b * a.Hq + hB) * a.D_max + jqB] = lseB;
-            } else {
-              if (sA)
-                L.part_lse[(((int64_t)b * a.Hq + hA) * a.D_max + jqA) * L.splits + split] = lseA;
-              if (sB)
-                L.part_lse[(((int64_t)b * a.Hq + hB) * a.D_max + jqB) * L.splits + split] = lseB;
-            }
-          }
-        }
-      }
-      // O[s] and the item slot are free for item k + 2
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {
-        mbar_arrive(&o_empty[s]);
-        mbar_arrive(&it_empty[s]);
-      }
-    }
   } else {
     // ------------------------------------------------------------- softmax
-    const int quarter = warp & 3, half = warp >> 2;
-    const int32_t rl = quarter * 32 + lane;   // row inside the tile = TMEM lane
-    const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-    // partial values of the two halves of a row: slots 0 / 1 by tile parity, 2 for the epilogue
-    auto xslot = [&](int slot, int hf) -> float& { return xch[(slot * 2 + hf) * kBM + rl]; };
-    auto pair_sync = [&]() { asm volatile("bar.sync %0, 64;" ::"r"(1 + quarter) : "memory"); };
+    // BM = 128: thread = query row = TMEM lane.  BM = 64: item row m sits in
+    // TMEM lane 32 (m / 16) + m % 16, so lane quarter q holds item rows 16q ..
+    // 16q + 15; with 16-lane accesses each thread holds two rows (t / 4 and
+    // t / 4 + 8 of the quarter) x 16 of the 64 columns, and the four threads
+    // t % 4 of a row finish its maxima and sums by shuffles.
+    constexpr int NR = BM == 64 ? 2 : 1;      // rows per thread
+    const bool split = ns_log > 0;
+    if (split && tid < kBM) s_ml[tid] = make_float2(-INFINITY, 0.f);  // rows of a part without keys
+    const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+    const int cq = lane & 3;
     bool ok = true;
     uint32_t T = 0;
     for (int32_t k = 0; ok; ++k) {
@@ -804,216 +757,342 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const TcItem& it = items[s];
       const int32_t ntiles = it.ntiles;
       if (ntiles < 0) break;
-      const int32_t b = it.b, g = it.g, split = it.split, row0 = it.row0;
-      const int32_t rows_total = it.rows_total, cache = it.cache, Lk = it.Lk;
+      const int32_t row0 = it.row0, rows_total = it.rows_total, cache = it.cache, Lk = it.Lk;
       const int32_t k_lo = it.k_lo, k_hi = it.k_hi;
-      const bool direct = it.direct != 0;
       const int32_t* kflat = it.kflat;
-      const uint32_t tO = tO0 + s * 128;
-      const int32_t r = row0 + rl;              // this thread's query row
-      const bool live = r < rows_total;
-      const bool warp_live = row0 + quarter * 32 < rows_total;  // same for both warps of a pair
-      // this row's draft and query head (computed once per item)
-      const int32_t jq = live ? r / G : 0, h = g * G + (live ? r - (r / G) * G : 0);
-      const int32_t qpos = live ? kflat[jq] : 0x7fffffff;
-      const bool increasing = it.increasing != 0;
+      const bool warp_live = row0 + warp * (BM / 4) < rows_total;
+      // this thread's query rows: item row, draft and position
+      const int32_t order = it.order;
+      int32_t rl[NR], jq[NR], qpos[NR];
+#pragma unroll
+      for (int e = 0; e < NR; ++e) {
+        rl[e] = BM == 64 ? warp * 16 + (lane >> 2) + 8 * e : warp * 32 + lane;
+        const int32_t r = row0 + rl[e];
+        jq[e] = r < rows_total ? r / G : 0;
+        qpos[e] = r >= rows_total ? 0x7fffffff : (order == kOrderFlat ? cache + jq[e] : kflat[jq[e]]);
+      }
       // cache slots below every query position of this item are visible to all rows
       int32_t minq = 0x7fffffff;
       const int32_t j_lo = row0 / G;
-      if (increasing) {
+      if (order == kOrderFlat) {
+        minq = cache;
+      } else if (order == kOrderIncreasing) {
         minq = kflat[j_lo];
       } else {
-        const int32_t j_end = (min(rows_total, row0 + kBM) + G - 1) / G;
+        const int32_t j_end = (min(rows_total, row0 + BM) + G - 1) / G;
+#pragma unroll 1
         for (int32_t j = j_lo + lane; j < j_end; j += 32) minq = min(minq, kflat[j]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) minq = min(minq, __shfl_xor_sync(0xffffffffu, minq, o));
       }
       const int32_t mask_from = min(cache, minq + 1);
-      // visibility of the item's drafts to this row: bit j of (vis_hi:vis_lo) is
+      // visibility of the item's drafts to each row: bit j of (vhi:vlo) is
       // kflat[j] <= qpos, that is j <= jq for increasing positions.  Runs once
       // per item, so the general loop is kept rolled (small code: a cold
       // unrolled path costs instruction-cache misses).
-      uint64_t vis_lo = 0, vis_hi = 0;
-      if (warp_live && increasing) {
-        const int32_t n = jq + 1;  // 1 .. 128
-        vis_lo = n >= 64 ? ~0ull : ((1ull << n) - 1ull);
-        vis_hi = n <= 64 ? 0ull : (n >= 128 ? ~0ull : ((1ull << (n - 64)) - 1ull));
+      uint64_t vlo[NR], vhi[NR];
+#pragma unroll
+      for (int e = 0; e < NR; ++e) vlo[e] = vhi[e] = 0;
+      if (warp_live && order != kOrderAny) {
+#pragma unroll
+        for (int e = 0; e < NR; ++e) first_bits(jq[e] + 1, vlo[e], vhi[e]);
       } else if (warp_live) {
         const int32_t nd = Lk - cache;
 #pragma unroll 1
         for (int j = 0; j < nd; j += 4) {
           const int4 kf = *reinterpret_cast<const int4*>(kflat + j);
-          const uint64_t bits = (uint64_t)((uint32_t)(kf.x <= qpos) | ((uint32_t)(kf.y <= qpos) << 1) |
-                                           ((uint32_t)(kf.z <= qpos) << 2) |
-                                           ((uint32_t)(kf.w <= qpos) << 3));
-          if (j < 64) vis_lo |= bits << j;
-          else vis_hi |= bits << (j - 64);
+#pragma unroll
+          for (int e = 0; e < NR; ++e) {
+            const uint64_t bits =
+                (uint64_t)((uint32_t)(kf.x <= qpos[e]) | ((uint32_t)(kf.y <= qpos[e]) << 1) |
+                           ((uint32_t)(kf.z <= qpos[e]) << 2) | ((uint32_t)(kf.w <= qpos[e]) << 3));
+            if (j < 64) vlo[e] |= bits << j;
+            else vhi[e] |= bits << (j - 64);
+          }
         }
       }
-      float m_run = -INFINITY, l_run = 0.f;  // l_run: this half's partial sum
+      float m_run[NR], l_run[NR];  // l_run: BM = 64: this thread's columns only, until the epilogue
+#pragma unroll
+      for (int e = 0; e < NR; ++e) {
+        m_run[e] = -INFINITY;
+        l_run[e] = 0.f;
+      }
+#pragma unroll 1
       for (int t = 0; t < ntiles; ++t, ++T) {
-        const int bb = T & 1, sb = T % kNB;
+        const int sb = T % kNB;
         if (!mbar_wait(&s_full[sb], (T / kNB) & 1, a.status)) ok = false;
         tc_fence_after();
-        float sv[HC];
         if (warp_live) {
-          tmem_ld32(tS + lane_off + sb * KTC + half * HC, sv);
-          tmem_ld32(tS + lane_off + sb * KTC + half * HC + 32, sv + 32);
-        }
-        bool moved = false;
-        float alpha = 1.f;
-        uint32_t pk[HC / 2];
-        if (warp_live) {
-          // mask: keys past this split / the sequence, and the spatial predicate
-          const int32_t c0 = k_lo + t * KTC + half * HC;
-          if (c0 + HC > k_hi || c0 + HC > mask_from) {
-            // keep bit jj: key c0 + jj is visible to this row.  Cache keys are a
-            // prefix of the window (visible up to qpos), draft keys come from the
-            // visibility bits, keys past the split are dropped.
-            auto low = [](int32_t n) -> uint64_t {
-              return n <= 0 ? 0ull : (n >= 64 ? ~0ull : ((1ull << n) - 1ull));
-            };
-            const int32_t base = c0 - cache;  // draft index of column 0
-            uint64_t win;                     // bit jj: draft base + jj is visible
-            if (base >= 128 || base <= -64) win = 0;
-            else if (base >= 64) win = vis_hi >> (base - 64);
-            else if (base > 0) win = (vis_lo >> base) | (vis_hi << (64 - base));
-            else if (base == 0) win = vis_lo;
-            else win = vis_lo << (-base);
-            const int32_t seen_end = qpos < cache ? qpos + 1 : cache;
-            const uint64_t keep =
-                (low(seen_end - c0) | (win & ~low(cache - c0))) & low(k_hi - c0);
+          const int32_t c0 = k_lo + t * KTC;
+          const bool masked = c0 + KTC > k_hi || c0 + KTC > mask_from;
+          float alpha[NR];
+          bool moved = false;
+          // the running max moves only when it grows by more than 2^kRescale
+          auto move_max = [&](int e, float mx) {
+            alpha[e] = 1.f;
+            if (mx != -INFINITY && (m_run[e] == -INFINITY || (mx - m_run[e]) * c2 > kRescale)) {
+              alpha[e] = (m_run[e] == -INFINITY) ? 0.f : ex2_approx((m_run[e] - mx) * c2);
+              m_run[e] = mx;
+              moved = true;
+            }
+            return (m_run[e] == -INFINITY) ? 0.f : m_run[e] * c2;
+          };
+          uint32_t pk[32 / NR];
+          if constexpr (BM == 128) {
+            float sv[64];
+            tmem_ld64(tS + lane_off + sb * KTC, sv);
+            if (masked) {
+              const uint64_t keep = keep_mask(c0, cache, k_hi, qpos[0], vlo[0], vhi[0]);
 #pragma unroll
-            for (int jj = 0; jj < HC; ++jj)
-              if (!((keep >> jj) & 1ull)) sv[jj] = -INFINITY;
+              for (int jj = 0; jj < 64; ++jj)
+                if (!((keep >> jj) & 1ull)) sv[jj] = -INFINITY;
+            }
+            float m4[4];  // four chains of three-input maxima
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              m4[w] = fmax3(sv[16 * w], sv[16 * w + 1], sv[16 * w + 2]);
+#pragma unroll
+              for (int i = 3; i < 15; i += 2) m4[w] = fmax3(m4[w], sv[16 * w + i], sv[16 * w + i + 1]);
+              m4[w] = fmaxf(m4[w], sv[16 * w + 15]);
+            }
+            const float moff = move_max(0, fmaxf(fmax3(m4[0], m4[1], m4[2]), m4[3]));
+            const float2 cc = make_float2(c2, c2), nm = make_float2(-moff, -moff);
+            float2 s4[4];
+#pragma unroll
+            for (int i = 0; i < 32; ++i) {
+              const float2 x = ffma2(make_float2(sv[2 * i], sv[2 * i + 1]), cc, nm);
+              const float2 e = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+              s4[i & 3] = i < 4 ? e : fadd2(s4[i & 3], e);
+              pk[i] = pack_bf16x2(e.x, e.y);
+            }
+            const float2 ss = fadd2(fadd2(s4[0], s4[1]), fadd2(s4[2], s4[3]));
+            l_run[0] = l_run[0] * alpha[0] + (ss.x + ss.y);
+          } else {
+            float sv[32];
+            tld16x256_x8(tS + lane_off + sb * KTC, sv);
+            if (masked) {
+#pragma unroll
+              for (int e = 0; e < 2; ++e) {
+                const uint64_t keep = keep_mask(c0, cache, k_hi, qpos[e], vlo[e], vhi[e]) >> (2 * cq);
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+#pragma unroll
+                  for (int x = 0; x < 2; ++x)
+                    if (!((keep >> (8 * u + x)) & 1ull)) sv[4 * u + 2 * e + x] = -INFINITY;
+              }
+            }
+            float mx[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              float m0 = fmax3(sv[2 * e], sv[2 * e + 1], sv[4 + 2 * e]);
+              float m1 = fmax3(sv[4 + 2 * e + 1], sv[8 + 2 * e], sv[8 + 2 * e + 1]);
+              m0 = fmax3(m0, sv[12 + 2 * e], sv[12 + 2 * e + 1]);
+              m1 = fmax3(m1, sv[16 + 2 * e], sv[16 + 2 * e + 1]);
+              m0 = fmax3(m0, sv[20 + 2 * e], sv[20 + 2 * e + 1]);
+              m1 = fmax3(m1, sv[24 + 2 * e], sv[24 + 2 * e + 1]);
+              mx[e] = fmaxf(fmax3(m0, sv[28 + 2 * e], sv[28 + 2 * e + 1]), m1);
+              mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 1));
+              mx[e] = fmaxf(mx[e], __shfl_xor_sync(0xffffffffu, mx[e], 2));
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float moff = move_max(e, mx[e]);
+              const float2 cc = make_float2(c2, c2), nm = make_float2(-moff, -moff);
+              float2 s2[2];
+#pragma unroll
+              for (int u = 0; u < 8; ++u) {
+                const float2 x = ffma2(make_float2(sv[4 * u + 2 * e], sv[4 * u + 2 * e + 1]), cc, nm);
+                const float2 p = make_float2(ex2_approx(x.x), ex2_approx(x.y));
+                s2[u & 1] = u < 2 ? p : fadd2(s2[u & 1], p);
+                pk[2 * u + e] = pack_bf16x2(p.x, p.y);
+              }
+              const float2 ss = fadd2(s2[0], s2[1]);
+              l_run[e] = l_run[e] * alpha[e] + (ss.x + ss.y);
+            }
           }
-          // tree reductions: short dependency chains
-          float m8[HC / 4];
-#pragma unroll
-          for (int i = 0; i < HC / 4; ++i)
-            m8[i] = fmaxf(fmaxf(sv[4 * i], sv[4 * i + 1]), fmaxf(sv[4 * i + 2], sv[4 * i + 3]));
-#pragma unroll
-          for (int w = HC / 8; w >= 1; w >>= 1)
-#pragma unroll
-            for (int i = 0; i < w; ++i) m8[i] = fmaxf(m8[i], m8[i + w]);
-          float mx = m8[0];
-          // (the pair barrier also orders the partner's tcgen05.ld of S before
-          // this warp overwrites the buffer with P)
-          xslot(bb, half) = mx;
-          pair_sync();
-          mx = fmaxf(mx, xslot(bb, half ^ 1));
-          // move the running max only when it grows by more than 2^kRescale
-          if (mx != -INFINITY && (m_run == -INFINITY || (mx - m_run) * c2 > kRescale)) {
-            alpha = (m_run == -INFINITY) ? 0.f : ex2_approx((m_run - mx) * c2);
-            m_run = mx;
-            moved = true;
-          }
-          const float moff = (m_run == -INFINITY) ? 0.f : m_run * c2;
-          float r8[HC / 4];
-#pragma unroll
-          for (int i = 0; i < HC / 4; ++i) {
-            const float e0 = ex2_approx(fmaf(sv[4 * i], c2, -moff));
-            const float e1 = ex2_approx(fmaf(sv[4 * i + 1], c2, -moff));
-            const float e2 = ex2_approx(fmaf(sv[4 * i + 2], c2, -moff));
-            const float e3 = ex2_approx(fmaf(sv[4 * i + 3], c2, -moff));
-            r8[i] = (e0 + e1) + (e2 + e3);
-            pk[2 * i] = pack_bf16x2(e0, e1);
-            pk[2 * i + 1] = pack_bf16x2(e2, e3);
-          }
-#pragma unroll
-          for (int w = HC / 8; w >= 1; w >>= 1)
-#pragma unroll
-            for (int i = 0; i < w; ++i) r8[i] += r8[i + w];
-          l_run = l_run * alpha + r8[0];
-        }
-        // O may be rescaled once PV_{T-1} is done
-        if (warp_live) {
+          // O may be rescaled once PV_{T-1} is done
           if (__any_sync(0xffffffffu, moved && t > 0)) {
             if (!mbar_wait(&pv_done[(T - 1) % kNB], ((T - 1) / kNB) & 1, a.status)) ok = false;
             tc_fence_after();
-            float ov[32];
 #pragma unroll 1
-            for (int cc = 0; cc < HD / 32; ++cc) {
-              const uint32_t ta = tO + lane_off + half * HD + cc * 32;
-              tmem_ld32(ta, ov);
+            for (int cc = 0; cc < D / 32; ++cc) {
+              const uint32_t ta = tO + lane_off + cc * 32;
+              if constexpr (BM == 128) {
+                float ov[32];
+                tmem_ld32(ta, ov);
 #pragma unroll
-              for (int i = 0; i < 32; ++i) ov[i] *= alpha;
-              tmem_st32(ta, ov);
+                for (int i = 0; i < 32; ++i) ov[i] *= alpha[0];
+                tmem_st32(ta, ov);
+              } else {
+                float ov[16];
+                tld16x256_x4(ta, ov);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) ov[i] *= alpha[(i >> 1) & 1 ? NR - 1 : 0];
+                tst16x256_x4(ta, ov);
+              }
             }
           }
-          // P_T as bf16 pairs over the first half of its S buffer: this half's keys
-          // are columns [half * HC / 2, (half + 1) * HC / 2)
-          tmem_st32(tS + lane_off + sb * KTC + half * (HC / 2), pk);
+          // P_T as bf16 pairs over the first half of its S buffer
+          if constexpr (BM == 128) tmem_st32(tS + lane_off + sb * KTC, pk);
+          else tst16x128_x8(tS + lane_off + sb * KTC, pk);
         }
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&v_ready[sb]);
       }
-      // ---- epilogue: wait for the item's last PV product, normalise, write this half
+      // ---- epilogue: wait for the item's last PV product; normalise and write
+      // the rows, or (split mode) leave them for the merge
       const uint32_t Tl = T - 1;
       if (!mbar_wait(&pv_done[Tl % kNB], (Tl / kNB) & 1, a.status)) ok = false;
       tc_fence_after();
       if (warp_live) {
-        xslot(2, half) = l_run;
-        pair_sync();
-        const float l_tot = l_run + xslot(2, half ^ 1);
-        // fast reciprocal and logarithm: the epilogue runs once per item, and
-        // its instruction count is its cost
-        const float inv_l = l_tot > 0.f ? __fdividef(1.0f, l_tot) : 0.f;
-        const float lse = (l_tot > 0.f) ? (m_run * (c2 / kLog2eTC) + __logf(l_tot)) : -INFINITY;
-        // (debug builds: the row's store index against its buffer)
-        const bool sL = live && (direct ? dbg_in(((int64_t)b * a.D_max + jq) * a.Hq + h,
-                                                 (int64_t)a.B * a.D_max * a.Hq, a.status)
-                                        : dbg_in((((int64_t)b * a.Hq + h) * a.D_max + jq) * L.splits + split,
-                                                 (int64_t)a.B * a.Hq * a.D_max * L.splits, a.status));
-#pragma unroll 1
-        for (int cc = 0; cc < HD / 32; ++cc) {
-          float ov[32];
-          tmem_ld32(tO + lane_off + half * HD + cc * 32, ov);
-          if (!sL || !ok) continue;
-          const int col = half * HD + cc * 32;
-          if (direct) {
-            __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(a.o) +
-                                (((int64_t)b * a.D_max + jq) * a.Hq + h) * D + col;
+        if constexpr (BM == 64) {
 #pragma unroll
-            for (int i = 0; i < 32; i += 8) {
-              uint4 w;
-              w.x = pack_bf16x2(ov[i] * inv_l, ov[i + 1] * inv_l);
-              w.y = pack_bf16x2(ov[i + 2] * inv_l, ov[i + 3] * inv_l);
-              w.z = pack_bf16x2(ov[i + 4] * inv_l, ov[i + 5] * inv_l);
-              w.w = pack_bf16x2(ov[i + 6] * inv_l, ov[i + 7] * inv_l);
-              *reinterpret_cast<uint4*>(ob + i) = w;
-            }
-          } else {
-            const int64_t prow = (((int64_t)b * a.Hq + h) * a.D_max + jq) * L.splits + split;
-            float* po = L.part_o + prow * D + col;
-#pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              *reinterpret_cast<float4*>(po + i) = make_float4(
-                  ov[i] * inv_l, ov[i + 1] * inv_l, ov[i + 2] * inv_l, ov[i + 3] * inv_l);
+          for (int e = 0; e < NR; ++e) {
+            l_run[e] += __shfl_xor_sync(0xffffffffu, l_run[e], 1);
+            l_run[e] += __shfl_xor_sync(0xffffffffu, l_run[e], 2);
           }
         }
-        if (sL && ok && half == 0) {
-          if (direct) {
-            if (a.lse != nullptr) a.lse[((int64_t)b * a.Hq + h) * a.D_max + jq] = lse;
+        const int32_t b = it.b, g = it.g;
+        bool live[NR];
+        float inv[NR];
+        int64_t orow[NR];
+#pragma unroll
+        for (int e = 0; e < NR; ++e) {
+          const int32_t r = row0 + rl[e], h = g * G + r - jq[e] * G;
+          orow[e] = ((int64_t)b * a.D_max + jq[e]) * a.Hq + h;
+          // (debug builds: the row's store index against its buffer)
+          live[e] = r < rows_total && ok && dbg_in(orow[e], (int64_t)a.B * a.D_max * a.Hq, a.status);
+          // fast reciprocal and logarithm: the epilogue runs once per item, and
+          // its instruction count is its cost
+          inv[e] = l_run[e] > 0.f ? __fdividef(1.0f, l_run[e]) : 0.f;
+          if (live[e] && (BM == 128 || cq == 0)) {
+            if (split)
+              s_ml[rl[e]] = make_float2(m_run[e], l_run[e]);
+            else if (a.lse != nullptr)
+              a.lse[((int64_t)b * a.Hq + h) * a.D_max + jq[e]] =
+                  l_run[e] > 0.f ? (m_run[e] * (c2 / kLog2eTC) + __logf(l_run[e])) : -INFINITY;
+          }
+        }
+#pragma unroll 1
+        for (int cc = 0; cc < D / 32; ++cc) {
+          if constexpr (BM == 128) {
+            float ov[32];
+            tmem_ld32(tO + lane_off + cc * 32, ov);
+            if (!live[0]) continue;
+            if (split) {  // the partial row over the K and V rings, which are done
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                *reinterpret_cast<float4*>(sK + part_off<D>(rl[0], cc * 8 + i)) =
+                    make_float4(ov[4 * i], ov[4 * i + 1], ov[4 * i + 2], ov[4 * i + 3]);
+            } else {
+              __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(a.o) + orow[0] * D + cc * 32;
+#pragma unroll
+              for (int i = 0; i < 32; i += 8) {
+                uint4 w;
+                w.x = pack_bf16x2(ov[i] * inv[0], ov[i + 1] * inv[0]);
+                w.y = pack_bf16x2(ov[i + 2] * inv[0], ov[i + 3] * inv[0]);
+                w.z = pack_bf16x2(ov[i + 4] * inv[0], ov[i + 5] * inv[0]);
+                w.w = pack_bf16x2(ov[i + 6] * inv[0], ov[i + 7] * inv[0]);
+                *reinterpret_cast<uint4*>(ob + i) = w;
+              }
+            }
           } else {
-            L.part_lse[(((int64_t)b * a.Hq + h) * a.D_max + jq) * L.splits + split] = lse;
+            float ov[16];
+            tld16x256_x4(tO + lane_off + cc * 32, ov);
+#pragma unroll
+            for (int e = 0; e < NR; ++e) {
+              if (!live[e]) continue;
+              // columns cc * 32 + 8 u + 2 cq + {0, 1}
+              if (split) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  *reinterpret_cast<float2*>(sK + part_off<D>(rl[e], cc * 8 + 2 * u + (cq >> 1)) +
+                                             (cq & 1) * 8) =
+                      make_float2(ov[4 * u + 2 * e], ov[4 * u + 2 * e + 1]);
+              } else {
+                __nv_bfloat16* ob =
+                    reinterpret_cast<__nv_bfloat16*>(a.o) + orow[e] * D + cc * 32 + 2 * cq;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                  *reinterpret_cast<uint32_t*>(ob + 8 * u) =
+                      pack_bf16x2(ov[4 * u + 2 * e] * inv[e], ov[4 * u + 2 * e + 1] * inv[e]);
+              }
+            }
           }
         }
       }
-      // O[s] and the item slot are free for item k + 2
+      // O and the item slot are free for the next items
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(&o_empty[s]);
+        mbar_arrive(o_empty);
         mbar_arrive(&it_empty[s]);
       }
     }
   }
+  // ---- split mode: merge the group's partial rows.  Every CTA of the grid
+  // takes the same branch (the plan is the same in all of them).
+  if (ns_log > 0) {
+    const int32_t ns = 1 << ns_log, part = (int32_t)blockIdx.x & (ns - 1);
+    __syncwarp();
+    cluster_sync_all();  // every partial row and its (max, sum) written
+    const TcItem* it = s_merge;
+    if (it != nullptr) {
+      const int32_t row0 = it->row0, rows = min(BM, it->rows_total - row0);
+      const int32_t cs = (int32_t)cluster_size();
+      const uint32_t rank0 = (uint32_t)((int32_t)blockIdx.x % cs - part);  // the group's first CTA
+      const uint32_t base_o = smem_u32(sK), base_ml = smem_u32(s_ml);
+      constexpr int LPR = D / 4;              // lanes per row (a float4 each)
+      constexpr int RPW = 32 / LPR;           // rows per warp and step
+      const int sub = lane / LPR, ch = lane % LPR;
+      // the group's CTAs take every ns-th row
+#pragma unroll 1
+      for (int32_t r = part + ns * (warp * RPW + sub); r < rows; r += ns * (kThreadsTC / 32) * RPW) {
+        float2 ml[kCluster];
+        float4 x[kCluster];
+        float M = -INFINITY;
+#pragma unroll
+        for (int p = 0; p < kCluster; ++p)
+          if (p < ns) {
+            ml[p] = ld_peer2(peer_addr(base_ml + r * 8, rank0 + p));
+            x[p] = ld_peer4(peer_addr(base_o + part_off<D>(r, ch), rank0 + p));
+          }
+#pragma unroll
+        for (int p = 0; p < kCluster; ++p)
+          if (p < ns && ml[p].y > 0.f) M = fmaxf(M, ml[p].x);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+        float l = 0.f;
+#pragma unroll
+        for (int p = 0; p < kCluster; ++p)
+          if (p < ns && ml[p].y > 0.f) {  // (a part whose keys the row does not see has no sum)
+            const float w = ex2_approx((ml[p].x - M) * c2);
+            l = fmaf(w, ml[p].y, l);
+            acc.x = fmaf(w, x[p].x, acc.x);
+            acc.y = fmaf(w, x[p].y, acc.y);
+            acc.z = fmaf(w, x[p].z, acc.z);
+            acc.w = fmaf(w, x[p].w, acc.w);
+          }
+        const int32_t jq = (row0 + r) / G, h = it->g * G + row0 + r - jq * G;
+        const int64_t orow = ((int64_t)it->b * a.D_max + jq) * a.Hq + h;
+        if (!dbg_in(orow, (int64_t)a.B * a.D_max * a.Hq, a.status)) continue;
+        const float inv = l > 0.f ? __fdividef(1.0f, l) : 0.f;
+        uint2 w;
+        w.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+        w.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.o) + orow * D + 4 * ch) = w;
+        if (a.lse != nullptr && ch == 0)
+          a.lse[((int64_t)it->b * a.Hq + h) * a.D_max + jq] =
+              l > 0.f ? (M * (c2 / kLog2eTC) + __logf(l)) : -INFINITY;
+      }
+    }
+    __syncwarp();
+    cluster_sync_all();  // the peers have read this CTA's rows
+  }
   // ---- teardown
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) {
+  if (warp == kSoftWarps + 3) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
@@ -1035,73 +1114,72 @@ namespace {
 // Query rows per tile: 64 when a KV group's rows fit (M = 64 products, their
 // softmax spread over the four lane quarters), else 128.
 int32_t tc_tile_rows(int32_t D_max, int32_t G) { return D_max * G <= 64 ? 64 : kBM; }
+
+// Clusters of the kernel that the current device can hold at once (a device
+// constant, queried once per device and kernel), at least one.  The occupancy
+// calculator counts one CTA per SM for any kernel that allocates tensor
+// memory; kCtasPerSmTC of this kernel's CTAs, which share the 512 columns, do
+// run on an SM (304 of 304 CTAs of a probe started at once).
+constexpr int kMaxDevicesTC = 64;
+template <typename K>
+int resident_clusters(K kernel, size_t smem) {
+  static std::atomic<int> known[kMaxDevicesTC];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  const bool slot = dev >= 0 && dev < kMaxDevicesTC;
+  int n = slot ? known[dev].load(std::memory_order_relaxed) : 0;
+  if (n > 0) return n;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(kCluster);
+  cfg.blockDim = dim3(kThreadsTC);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kCluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
+    cudaGetLastError();
+    n = std::max(1, device_sm_count() / kCluster / 2);
+  }
+  n *= kCtasPerSmTC;
+  if (slot) known[dev].store(n, std::memory_order_relaxed);
+  return n;
+}
 }  // namespace
 
-TcPlan attention_tc_plan(int32_t B, int32_t Hq, int32_t Hkv, int32_t D_max, int32_t L_max) {
-  TcPlan p;
-  const int32_t G = Hq / Hkv;
-  const int32_t bm = tc_tile_rows(D_max, G);
-  p.mtiles = (D_max * G + bm - 1) / bm;
-  const int64_t base = (int64_t)B * Hkv * p.mtiles;
-  const int32_t target = device_sm_count();  // one CTA per SM
-  const int32_t max_splits = max(1, (L_max + 2 * KTC - 1) / (2 * KTC));  // >= 2 tiles each
-  int32_t splits = (int32_t)((target + base - 1) / base);
-  splits = max(1, min(splits, max_splits));
-  int32_t kps = (L_max + splits - 1) / splits;
-  kps = ((kps + KTC - 1) / KTC) * KTC;
-  p.splits = (L_max + kps - 1) / kps;
-  p.kps = kps;
-  return p;
-}
-
-cudaError_t launch_attention_tc(const AttnArgs& a, const TcPlan& p, int32_t* seq_ok, float* part_o,
-                                float* part_lse, cudaStream_t stream, bool pdl) {
-  EncodeTiledFn fn = tensor_map_encoder();
-  if (fn == nullptr) return cudaErrorInvalidValue;
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl) {
   const int32_t G = a.Hq / a.Hkv;
   const int32_t bm = tc_tile_rows(a.D_max, G);
   CUtensorMap tq, tk, tv;
-  {
-    cuuint64_t dims[3] = {(cuuint64_t)a.d, (cuuint64_t)a.Hq, (cuuint64_t)a.B * a.D_max};
-    cuuint64_t strides[2] = {(cuuint64_t)a.d * 2, (cuuint64_t)a.Hq * a.d * 2};
-    cuuint32_t box[3] = {64, (cuuint32_t)G, (cuuint32_t)(bm / G)};
-    cuuint32_t estr[3] = {1, 1, 1};
-    if (fn(&tq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(a.q), dims, strides, box,
-           estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
+  bool ok;
+  const uint64_t row = (uint64_t)a.d * 2, halves = (uint64_t)a.d / 64;
+  {  // {64 columns, Hq, B * D_max, d / 64}, box {64, G, bm / G, d / 64}: rows (draft, head of the group)
+    const uint64_t dims[4] = {64, (uint64_t)a.Hq, (uint64_t)a.B * a.D_max, halves};
+    const uint64_t strides[3] = {row, (uint64_t)a.Hq * row, 128};
+    const uint32_t box[4] = {64, (uint32_t)G, (uint32_t)(bm / G), (uint32_t)halves};
+    ok = bf16_tensor_map(&tq, a.q, 4, dims, strides, box);
   }
-  const int64_t rows = (int64_t)a.B * a.Hkv * a.L_max;
-  for (int w = 0; w < 2; ++w) {
-    // d = 128: {64 columns, rows, 2 halves}, the halves 128 B apart inside a row,
-    // so one box {64, KTC, 2} is a whole tile; d = 64: {64, rows}, box {64, KTC}
-    const cuuint32_t rank = a.d == 128 ? 3 : 2;
-    cuuint64_t dims[3] = {64, (cuuint64_t)rows, 2};
-    cuuint64_t strides[2] = {(cuuint64_t)a.d * 2, 128};
-    cuuint32_t box[3] = {64, KTC, 2};
-    cuuint32_t estr[3] = {1, 1, 1};
-    if (fn(w == 0 ? &tk : &tv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, rank,
-           const_cast<void*>(w == 0 ? a.k : a.v), dims, strides, box, estr,
-           CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-           CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return cudaErrorInvalidValue;
+  {  // {64 columns, rows, 1, d / 64}, box {64, KTC, 1, d / 64}
+    const uint64_t dims[4] = {64, (uint64_t)a.B * a.Hkv * a.L_max, 1, halves};
+    const uint64_t strides[3] = {row, row, 128};
+    const uint32_t box[4] = {64, KTC, 1, (uint32_t)halves};
+    ok = ok && bf16_tensor_map(&tk, a.k, 4, dims, strides, box) &&
+         bf16_tensor_map(&tv, a.v, 4, dims, strides, box);
   }
+  if (!ok) return cudaErrorInvalidValue;
   TcLaunch L;
-  L.splits = p.splits;
-  L.kps = p.kps;
-  L.mtiles = p.mtiles;
-  L.part_o = part_o;
-  L.part_lse = part_lse;
-  L.seq_ok = seq_ok;
-  // persistent: one CTA per SM (at most one per work item)
-  const int64_t n_items = (int64_t)a.B * a.Hkv * p.mtiles * p.splits;
-  const dim3 grid((unsigned)std::min<int64_t>(n_items, device_sm_count()));
-  const dim3 block(kThreadsTC);
+  L.mtiles = (a.D_max * G + bm - 1) / bm;
+  // persistent: whole clusters, as many as are resident, at most one per item
+  const int64_t n_items = (int64_t)a.B * a.Hkv * L.mtiles;
   auto launch = [&](auto kernel, size_t smem) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_kernel(kernel, grid, block, smem, stream, pdl, tq, tk, tv, a, L);
+    const int64_t clusters = std::min<int64_t>(n_items, resident_clusters(kernel, smem));
+    return launch_clusters(kernel, dim3((unsigned)(clusters * kCluster)), dim3(kThreadsTC), smem,
+                           stream, pdl, kCluster, tq, tk, tv, a, L);
   };
   if (a.d == 128)
     return bm == 64 ? launch(frontier_attn_tc_kernel<128, 64>, tc_smem_bytes<128, 64>())

@@ -121,8 +121,11 @@ __device__ __forceinline__ bool give_up(uint32_t poll, const int32_t* status) {
 
 // Bounded wait on an mbarrier phase.  Returns false (and records
 // SSD_ERR_TIMEOUT) if the phase did not complete within max_polls polls.
+// (Rolled: the kernels wait in many places, and code that other kernels
+// evicted is fetched cold.)
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int32_t* status,
                                           uint32_t max_polls = kMaxPolls) {
+#pragma unroll 1
   for (uint32_t i = 0; i < max_polls; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (i > 4096) {
@@ -399,7 +402,7 @@ struct Philox4 {
 __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
                                                  uint32_t k0, uint32_t k1) {
   const uint32_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u, W0 = 0x9E3779B9u, W1 = 0xBB67AE85u;
-#pragma unroll
+#pragma unroll 1
   for (int r = 0; r < 10; ++r) {
     const uint32_t hi0 = __umulhi(M0, c0), lo0 = M0 * c0;
     const uint32_t hi1 = __umulhi(M1, c2), lo1 = M1 * c2;

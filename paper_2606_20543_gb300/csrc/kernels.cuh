@@ -48,6 +48,26 @@ cudaError_t launch_kernel(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
 }
 
+// The same with clusters of `cluster` CTAs (the grid's x extent a multiple of it).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_clusters(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t stream, bool pdl, int cluster, Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cluster;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Args&&>(args)...);
+}
+
 // ---- frontier.cu
 cudaError_t launch_record_commit(int32_t B, int32_t D_max, int32_t prefix_len, int32_t hw,
                                  const int32_t* cache_len, const int32_t* next_cache_len,
@@ -170,9 +190,7 @@ struct AcceptArgs {
   int32_t* tickets = nullptr;
   // Under a programmatic launch of a kernel that reads none of this pass's
   // results (the step's attention): let it be scheduled at once, on the SMs
-  // this pass leaves idle, instead of after the pass's last CTA.  0: never,
-  // 1: always, 2: when the frontiers (cache_len non-null) hold at most one
-  // row per two CTAs.
+  // this pass leaves idle, instead of after the pass's last CTA.
   int32_t early_dependents = 0;
 };
 bool accept_supported(int32_t V);
@@ -280,14 +298,9 @@ int attention_launches(const ssd_grid& g, int32_t B, int32_t Hq, int32_t Hkv, in
 int32_t attention_rows_hint(const ssd_grid& g, int32_t D_max);
 
 // ---- attention_tc.cu (tcgen05 frontier attention: query groups dividing 128,
-// more than 64 query rows per KV group)
-struct TcPlan {
-  int32_t splits, kps, mtiles;
-};
+// more than 16 query rows per KV group); one launch, no workspace
 bool attention_tc_supported(int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max);
-TcPlan attention_tc_plan(int32_t B, int32_t Hq, int32_t Hkv, int32_t D_max, int32_t L_max);
-cudaError_t launch_attention_tc(const AttnArgs& a, const TcPlan& p, int32_t* seq_ok, float* part_o,
-                                float* part_lse, cudaStream_t stream, bool pdl = false);
+cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl = false);
 // Same as launch_attention with the library's static device scratch as the
 // workspace (ssd_verify_attention_noalloc); cudaErrorMemoryAllocation if the
 // problem needs more than SSD_NOALLOC_SCRATCH_BYTES.

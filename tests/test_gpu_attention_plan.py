@@ -1,0 +1,32 @@
+"""The tcgen05 attention's device-side plan (which CTA takes which item, and how
+many CTAs of a cluster share one) at the sizes where it changes shape, against
+the oracle: attention within 2e-2, log-sum-exp within 2e-2 absolute."""
+import pytest
+
+import synth
+from tests.test_gpu_attention import check_case, ssd  # noqa: F401 (ssd: the fixture)
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("name,B,heads,d,grid,prefix,cache", [
+    # few live items: 4 CTAs of a cluster share each; the second sequence has
+    # fewer key tiles (one) than CTAs, so some of them have no keys
+    ("parts_without_keys", 2, (4, 4), 128, 24, 0, [24 * 20 + 5, 0]),
+    # 64-row tiles, d = 64, each part one or two tiles
+    ("short_parts", 1, (8, 8), 64, 16, 32, [200]),
+    # 128-row tiles (GQA): two query tiles for the first sequence's 256 rows, one
+    # for the second's last grid row; every other image complete
+    ("tail_gqa", 8, (32, 8), 128, 32, 64, [64 + 1024] * 5 + [64 + 300, 64 + 1024, 64 + 31 * 32 + 4]),
+    # exactly as many live items as half the CTAs and fewer: 2 CTAs per item
+    ("two_way", 8, (16, 16), 128, 24, 120, [120 + 72 * k for k in range(8)]),
+    # more than 32 sequences: planned by the block (empty frontiers among them)
+    ("block_plan", 40, (4, 4), 64, 16, 7, [7 + (37 * k) % 257 for k in range(40)]),
+    # more sequences than the plan holds: dealt in their order
+    ("unplanned", 260, (1, 1), 64, 10, 3, [3 + (7 * k) % 101 for k in range(260)]),
+])
+def test_plan_shapes(ssd, name, B, heads, d, grid, prefix, cache):  # noqa: F811
+    c = synth.make_case(name, grid_h=grid, grid_w=grid, prefix_len=prefix, cache_len=cache,
+                        Hq=heads[0], Hkv=heads[1], d=d, V=64, seed=23, with_logits=False)
+    assert c.B == B
+    check_case(ssd, c)
