@@ -130,9 +130,9 @@ struct Shared {
 // (kind 0) and, in the horizontal stage, the bonus row after a sequence's
 // last draft (kind 3).  Producer and consumers walk the same rows and skip
 // the same ones.
-__device__ __forceinline__ int row_kind(const AcceptArgs& a, int64_t r) {
+__device__ __forceinline__ int row_kind(const AcceptArgs& a, int32_t r) {
   if (a.cache_len != nullptr || a.n_drafts != nullptr) {
-    const int32_t b = (int32_t)(r / a.D_max), j = (int32_t)(r % a.D_max);
+    const int32_t b = r / a.D_max, j = r - b * a.D_max;
     const int32_t n = a.cache_len != nullptr ? frontier_drafts(a.grid, a.cache_len[b], a.D_max)
                                              : a.n_drafts[b];
     if (j >= n) return (a.bonus && j == n && n > 0) ? 3 : 1;  // bonus row / padding slot
@@ -159,6 +159,7 @@ __device__ __forceinline__ int32_t find_block(const float* mass, int32_t nblocks
                                               float* t_in_block, int lane) {
   const int32_t per = (nblocks + 31) / 32;
   float ls = 0.f;
+#pragma unroll 1
   for (int32_t q = 0; q < per; ++q) {
     const int32_t bk = lane * per + q;
     ls += (bk < nblocks) ? mass[bk] : 0.f;
@@ -181,6 +182,7 @@ __device__ __forceinline__ int32_t find_block(const float* mass, int32_t nblocks
   float tb = INFINITY;
   if (lane == ls_star) {
     float cum = 0.f;
+#pragma unroll 1
     for (int32_t q = 0; q < per; ++q) {
       const int32_t bk = lane * per + q;
       const float m = (bk < nblocks) ? mass[bk] : 0.f;
@@ -263,7 +265,11 @@ __device__ __forceinline__ int32_t walk_block(const float4* tp, const float4* dp
   return last_pos;  // rounding ran past the end of the block
 }
 
-template <int STRATEGY>
+// LAZY: strategy (C) with the draws left to resolve_kernel.  A kernel of its
+// own: the one-pass kernel is the one that runs in every step, and what it
+// does not contain need not stay in the instruction caches beside the
+// attention's code.
+template <int STRATEGY, bool LAZY>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   float* ring = reinterpret_cast<float*>(smem_raw);                  // [kStages][2][kChunk]
@@ -271,21 +277,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
   __shared__ Shared sh;
   const int32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int32_t nch = (a.V + kChunk - 1) / kChunk;
-  __shared__ int32_t s_early;
-  if (warp == 0) {
-    // mode 1: always; mode 2: when the step's frontiers leave at most half of
-    // the CTAs a row (most SMs idle while the busy CTAs stream their rows)
-    bool early = a.early_dependents == 1;
-    if (a.early_dependents == 2 && a.cache_len != nullptr) {
-      int32_t live = 0;
-      for (int32_t b = lane; b < a.rows / a.D_max; b += 32)
-        live += frontier_drafts(a.grid, a.cache_len[b], a.D_max);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) live += __shfl_xor_sync(0xffffffffu, live, o);
-      early = 2 * live <= (int32_t)gridDim.x;
-    }
-    if (lane == 0) s_early = early ? 1 : 0;
-  }
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
       mbar_init(&sh.full[s], 1);
@@ -294,36 +285,39 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
     fence_barrier_init();
   }
   __syncthreads();
-  if (s_early) pdl_launch_dependents();
+  if (a.early_dependents) pdl_launch_dependents();
 
   // (A) never draws and lazy (C) leaves its draws to launch_resolve: one pass
-  const int32_t passes = (STRATEGY == SSD_STRATEGY_GREEDY || a.lazy) ? 1 : 2;
+  constexpr int32_t passes = (STRATEGY == SSD_STRATEGY_GREEDY || LAZY) ? 1 : 2;
 
   // ------------------------------------------------------------ producer warp
   if (warp == kCWarps) {
     if (lane == 0) {
       uint32_t g = 0;  // chunks issued by this CTA
-      for (int64_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
+#pragma unroll 1
+      for (int32_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
         const int kind = row_kind(a, r);
         if (kind == 1 || kind == 2) continue;
         // the row's reference is read once: the consumers may redirect it for
         // the next round while this row's second pass is still being issued
         const float* drow =
-            (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + r * a.ld;
+            (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + (int64_t)r * a.ld;
+#pragma unroll 1
         for (int32_t cc = 0; cc < passes * nch; ++cc, ++g) {  // one or two passes over the row
-          const int32_t ch = cc % nch;
+          const int32_t ch = passes > 1 && cc >= nch ? cc - nch : cc;
           const int s = g % kStages;
           if (g >= kStages) mbar_wait(&sh.empty[s], ((g / kStages) - 1) & 1, a.status);
           const uint32_t bytes = (uint32_t)min(kChunk, a.V - ch * kChunk) * 4u;
           float* dst = ring + s * 2 * kChunk;
           mbar_arrive_expect_tx(&sh.full[s], 2u * bytes);
-          bulk_g2s(dst, a.tgt + r * a.ld + (int64_t)ch * kChunk, bytes, &sh.full[s]);
+          bulk_g2s(dst, a.tgt + (int64_t)r * a.ld + (int64_t)ch * kChunk, bytes, &sh.full[s]);
           bulk_g2s(dst + kChunk, drow + (int64_t)ch * kChunk, bytes, &sh.full[s]);
         }
       }
     } else if (a.cache_len != nullptr) {
       // lanes 1-31: write the frontier of sequences blockIdx.x, + gridDim.x, ...
       const int32_t B = (int32_t)(a.rows / a.D_max);
+#pragma unroll 1
       for (int32_t b = blockIdx.x; b < B; b += gridDim.x) {
         const int32_t n = frontier_drafts(a.grid, a.cache_len[b], a.D_max);
         const int32_t n_c = a.cache_len[b] - a.grid.prefix_len;
@@ -332,6 +326,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
           if (a.tickets != nullptr) a.tickets[b] = 0;
           if (n < 0) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
         }
+#pragma unroll 1
         for (int32_t j = lane - 1; j < a.D_max; j += 31)
           a.draft_pos[(int64_t)b * a.D_max + j] = j < n ? n_c + j : -1;
       }
@@ -349,7 +344,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
   const int32_t nblocks = nch * kBlocksPerChunk;
   const float4 ninf = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   uint32_t g = 0;  // chunks consumed
-  for (int64_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
+#pragma unroll 1
+  for (int32_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
     const int kind = row_kind(a, r);
     if (kind == 1 || kind == 2) {
       if (tid == 0) {
@@ -358,8 +354,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
         if (a.ratio) a.ratio[r] = 0.f;
         if (kind == 1 && a.lse) { a.lse[2 * r] = 0.f; a.lse[2 * r + 1] = 0.f; }
         if (kind == 2) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
-        if (a.ref_rows != nullptr && a.ref_init) a.ref_rows[r] = a.drf + r * a.ld;
-        if (a.lazy) a.stats[r] = make_float2(NAN, NAN);
+        if (a.ref_rows != nullptr && a.ref_init) a.ref_rows[r] = a.drf + (int64_t)r * a.ld;
+        if (LAZY) a.stats[r] = make_float2(NAN, NAN);
       }
       continue;
     }
@@ -377,6 +373,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
     float mp = kLowest, mq = kLowest, xpa = 0.f;
     float2 sp2 = make_float2(0.f, 0.f), sq2 = sp2;
     int32_t iq = 0x7fffffff, ip = 0x7fffffff;
+#pragma unroll 1
     for (int32_t ch = 0; ch < nch; ++ch, ++g) {
       const int s = g % kStages;
       mbar_wait(&sh.full[s], (g / kStages) & 1, a.status);
@@ -437,7 +434,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
     // the row's reference (draft) row: read here, before the barrier after
     // which this row's decision may redirect it for the next round
     const float* drow =
-        (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + r * a.ld;
+        (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + (int64_t)r * a.ld;
     if (greedy) {  // first argmax of p over the CTA (warp tree, then the warps in order)
       float pm = mp;
 #pragma unroll
@@ -452,8 +449,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
       }
     }
     // block reduction in a fixed order: xor tree in each warp, then a
-    // three-level xor tree over the warps' results in warp 0
-#pragma unroll
+    // three-level xor tree over the warps' results in warp 0 (rolled: once per
+    // row, so its instructions are fetched rather than reused)
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) {
       merge(mp, sp, __shfl_xor_sync(0xffffffffu, mp, o), __shfl_xor_sync(0xffffffffu, sp, o), c);
       const float om = __shfl_xor_sync(0xffffffffu, mq, o);
@@ -479,7 +477,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
       float Mq = have ? sh.red[lane][2] : kLowest, Sq = have ? sh.red[lane][3] : 0.f;
       float xp_t = have ? sh.red[lane][4] : 0.f;
       int32_t t = have ? sh.red_i[lane] : 0x7fffffff;
-#pragma unroll
+#pragma unroll 1
       for (int o = kCWarps / 2; o > 0; o >>= 1) {
         merge(Mp, Sp, __shfl_xor_sync(0xffffffffu, Mp, o), __shfl_xor_sync(0xffffffffu, Sp, o), c);
         const float om = __shfl_xor_sync(0xffffffffu, Mq, o);
@@ -506,7 +504,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
         sh.u_res = u.y;
         sh.Cp = Mp * c + lsp;
         sh.Cq = 0.f;
-        if (a.lazy) {  // drawn by launch_resolve if every draft is accepted
+        if (LAZY) {  // drawn by launch_resolve if every draft is accepted
           a.out_tok[r] = -1;
           a.stats[r] = make_float2(sh.Cp, 0.f);
         }
@@ -557,14 +555,14 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
           a.accepted[r] = acc ? 1 : 0;
           if (acc || greedy) a.out_tok[r] = out;
           // the next round's reference of a row this round did not accept
-          if (a.ref_rows != nullptr && valid_t && !acc) a.ref_rows[r] = a.tgt + r * a.ld;
+          if (a.ref_rows != nullptr && valid_t && !acc) a.ref_rows[r] = a.tgt + (int64_t)r * a.ld;
           else if (a.ref_rows != nullptr && a.ref_init) a.ref_rows[r] = drow;
         }
         if (!valid_t) {
           a.accepted[r] = 0;
           a.out_tok[r] = -1;
         }
-        if (a.lazy) {  // a rejected row's token is drawn by launch_resolve if committed
+        if (LAZY) {  // a rejected row's token is drawn by launch_resolve if committed
           if (sh.accept == 0) a.out_tok[r] = -1;
           a.stats[r] = valid_t ? make_float2(sh.Cp, sh.Cq) : make_float2(NAN, NAN);
         }
@@ -576,11 +574,12 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
       }
     }
     consumers_sync();
-    if (passes == 1) continue;  // uniform; sh is rewritten only after the next row's pass A
+    if constexpr (passes == 1) continue;  // sh is rewritten only after the next row's pass A
     const bool draw = (sh.accept == 0);
     const float2 ncp = make_float2(-sh.Cp, -sh.Cp), ncq = make_float2(-sh.Cq, -sh.Cq);
 
     // ---- pass B: second-pass chunks; residual mass of every 256-entry block
+#pragma unroll 1
     for (int32_t ch = 0; ch < nch; ++ch, ++g) {
       const int s = g % kStages;
       mbar_wait(&sh.full[s], (g / kStages) & 1, a.status);
@@ -600,15 +599,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
     }
     if (!draw) continue;  // uniform
     consumers_sync();
-    const float4* tp = reinterpret_cast<const float4*>(a.tgt + r * a.ld);
+    const float4* tp = reinterpret_cast<const float4*>(a.tgt + (int64_t)r * a.ld);
     const float4* dp = reinterpret_cast<const float4*>(drow);
     if (warp == 0) {
       float tb;
-      int32_t bk = find_block(block_mass, nblocks, sh.u_res, &tb, lane);
+      int32_t bk;
       bool from_p = row_p;
-      if (bk < 0 && !row_p) {
+#pragma unroll 1
+      for (;;) {
+        bk = find_block(block_mass, nblocks, sh.u_res, &tb, lane);
+        if (bk >= 0 || from_p) break;
         // zero residual mass: the same draw from p (block masses of p itself)
         from_p = true;
+#pragma unroll 1
+#pragma unroll 1
         for (int32_t b0 = 0; b0 < nblocks; ++b0) {
           const int32_t i0 = b0 * 64 + lane, i1 = i0 + 32;
           float4 w0 = make_float4(0.f, 0.f, 0.f, 0.f), w1 = w0;
@@ -618,7 +622,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
           if (lane == 0) block_mass[b0] = m;
         }
         __syncwarp();
-        bk = find_block(block_mass, nblocks, sh.u_res, &tb, lane);
       }
       if (bk < 0) {
         if (lane == 0) {  // no positive mass at all (non-finite logits)
@@ -632,7 +635,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
           a.out_tok[r] = pick;
           if (sample && !is_bonus) {
             a.accepted[r] = pick == sh.t_hat ? 1 : 0;
-            if (a.ref_rows != nullptr && pick != sh.t_hat) a.ref_rows[r] = a.tgt + r * a.ld;
+            if (a.ref_rows != nullptr && pick != sh.t_hat) a.ref_rows[r] = a.tgt + (int64_t)r * a.ld;
             else if (a.ref_rows != nullptr && a.ref_init) a.ref_rows[r] = drow;
           }
         }
@@ -659,6 +662,7 @@ constexpr int kRBlocks = 2;  // blocks per part: one batch of loads
 __device__ __forceinline__ void resolve_part_masses(const float4* tp, const float4* dp, int32_t bk0,
                                                     int32_t bk1, int32_t nv, float2 cc, float2 ncp,
                                                     float2 ncq, bool from_p, float* mass, int lane) {
+#pragma unroll 1
   for (int32_t b0 = bk0; b0 < bk1; b0 += 2) {
     float4 xp[2][2], xq[2][2];
 #pragma unroll
@@ -733,8 +737,8 @@ __global__ void __launch_bounds__(32, 32) resolve_kernel(ResolveArgs a) {
   const float c = kLog2e / a.temperature;
   const float2 cc = make_float2(c, c);
   const float2 ncp = make_float2(-st.x, -st.x), ncq = make_float2(-st.y, -st.y);
-  const float4* tp = reinterpret_cast<const float4*>(a.tgt + r * a.ld);
-  const float4* dp = reinterpret_cast<const float4*>(a.drf + r * a.ld);
+  const float4* tp = reinterpret_cast<const float4*>(a.tgt + (int64_t)r * a.ld);
+  const float4* dp = reinterpret_cast<const float4*>(a.drf + (int64_t)r * a.ld);
   float* gmass = a.mass + (int64_t)b * nblocks;
   if (j != 0) load_part(tp, dp, is_bonus);  // the speculative rows were not the committed one
   // this part's block masses, with the arithmetic of resolve_part_masses
@@ -762,15 +766,17 @@ __global__ void __launch_bounds__(32, 32) resolve_kernel(ResolveArgs a) {
   __syncwarp();
   const float u_res = row_uniforms(a.rng, r).y;
   float tb = 0.f;
-  int32_t bk = find_block(rmass, nblocks, u_res, &tb, lane);
+  int32_t bk;
   bool from_p = is_bonus;
-  if (bk < 0 && !is_bonus) {
+#pragma unroll 1
+  for (;;) {
+    bk = find_block(rmass, nblocks, u_res, &tb, lane);
+    if (bk >= 0 || from_p) break;
     // zero residual mass: the same draw from p (block masses of p itself)
     from_p = true;
     __syncwarp();
     resolve_part_masses(tp, tp, 0, nblocks, nv, cc, ncp, ncq, true, rmass, lane);
     __syncwarp();
-    bk = find_block(rmass, nblocks, u_res, &tb, lane);
   }
   if (bk < 0) {
     if (lane == 0) {  // no positive mass at all (non-finite logits)
@@ -806,9 +812,11 @@ cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t stream) {
     return cudaGetLastError();
   };
   switch (a.strategy) {
-    case SSD_STRATEGY_GREEDY: return launch(accept_kernel<SSD_STRATEGY_GREEDY>);
-    case SSD_STRATEGY_SAMPLE: return launch(accept_kernel<SSD_STRATEGY_SAMPLE>);
-    default: return launch(accept_kernel<SSD_STRATEGY_ACCEPT_REJECT>);
+    case SSD_STRATEGY_GREEDY: return launch(accept_kernel<SSD_STRATEGY_GREEDY, false>);
+    case SSD_STRATEGY_SAMPLE: return launch(accept_kernel<SSD_STRATEGY_SAMPLE, false>);
+    default:
+      return a.lazy ? launch(accept_kernel<SSD_STRATEGY_ACCEPT_REJECT, true>)
+                    : launch(accept_kernel<SSD_STRATEGY_ACCEPT_REJECT, false>);
   }
 }
 
