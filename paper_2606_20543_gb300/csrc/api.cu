@@ -33,8 +33,9 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Side stream of ssd_verify_step: acceptance runs on it, concurrently with the
-// attention of the same step on the caller's stream (they share no data).
+// Side stream of ssd_verify_step on the fused path and beside the mma.sync
+// attention: acceptance runs on it, concurrently with the attention of the
+// same step on the caller's stream (they share no data).
 // One per device and host thread, created on first use and kept until exit.
 struct SideStream {
   cudaStream_t stream = nullptr;
@@ -504,10 +505,6 @@ ssd_status check_accept_part(const ssd_verify_args* x, const ssd_verify_out* y) 
 
 // Logits path, a1 + a3-a5: the acceptance pass, which computes the frontier
 // itself and writes it out (n_drafts, draft_pos).
-#ifndef SSD_ACCEPT_EARLY_PDL
-#define SSD_ACCEPT_EARLY_PDL 1
-#endif
-
 cudaError_t launch_accept_phase(const ssd_verify_args* x, const ssd_verify_out* y, void* ws,
                                 cudaStream_t stream, int early_dependents = 0) {
   const bool lazy = lazy_draws(x);
@@ -625,7 +622,7 @@ int32_t ssd_verify_step_launches(const ssd_verify_args* x) {
   // logits: acceptance (with the frontier) + attention (+ split combine) + counts/draws;
   // fused: frontier + attention (+ combine) + lm_head acceptance + counts
   const int fixed = x->tgt_logits != nullptr ? 2 : 3;
-  return fixed + attention_launches(x->grid, x->B, x->Hq, x->Hkv, x->d, x->D_max, x->L_max);
+  return fixed + attention_launches(x->B, x->Hq, x->Hkv, x->d, x->D_max, x->L_max);
 }
 
 ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, void* workspace,
@@ -678,34 +675,27 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
     // out (a1 + a3-a5); the attention computes the same frontier from
     // cache_len (a2), so the two need no frontier launch before them.
     a.raster = 1;
-    // Rows that can hold a draft: the frontier bound per sequence (+ the bonus row).
-    const int64_t live_rows =
-        (int64_t)x->B * std::min<int32_t>(x->D_max, attention_rows_hint(x->grid, x->D_max) +
-                                                        (x->commit == SSD_COMMIT_PREFIX_BONUS));
-    // Measured on GB300: lazy (C) gains from hiding its draws under the attention; greedy,
-    // which has nothing to hide, gains from this order only when its pass is short (few
-    // live rows, e.g. the horizontal stage: 33.4 -> 31.5 us), and loses on the sweep.
-    const bool serial =
-        x->B * x->D_max >= 2 * device_sm_count() &&
-        (lazy_draws(x) || (x->strategy == SSD_STRATEGY_GREEDY && live_rows <= device_sm_count()));
+    // One stream whenever the tcgen05 attention runs: as a programmatic dependent
+    // of the acceptance it starts on the SMs that the acceptance leaves, at
+    // once when there are few rows, with no fork and join of a second stream
+    // (16x16 step 17.0 -> 13.9 us, two rounds on 8 x 24x24 72 -> 62 us; 24x24
+    // sweep under (A) 53.1 -> 50.8, GQA batch under (A) 45.4 -> 39.5 and (B)
+    // 52.3 -> 46.4).
+    const bool serial = attention_tc_supported(x->Hq, x->Hkv, x->d);
     if (serial) {
       // On `stream` alone: the acceptance; the attention, which reads none of
-      // its results, as a programmatic dependent (the tcgen05 kernel starts
-      // as the acceptance's CTAs retire and lets the next kernel be scheduled
-      // only once the acceptance has completed; the mma.sync kernel starts
-      // after it); then a7 (the counts, with the committed draws when lazy) as
-      // a programmatic dependent of the attention: its small CTAs run beside
-      // the attention, in the registers it leaves free.
-      e = launch_accept_phase(x, y, ws + attn_ws, stream, /*early_dependents=*/SSD_ACCEPT_EARLY_PDL);
+      // its results, as a programmatic dependent that lets the next kernel be
+      // scheduled only once the acceptance has completed; then a7 (the counts,
+      // with the committed draws when lazy) as a programmatic dependent of the
+      // attention: its small CTAs run beside the attention's.
+      e = launch_accept_phase(x, y, ws + attn_ws, stream, /*early_dependents=*/1);
       if (e != cudaSuccess) return SSD_ERR_CUDA;
-      e = launch_attention(a, ws, attn_ws, stream, /*defer_combine=*/true, /*pdl=*/true);
+      e = launch_attention(a, ws, attn_ws, stream, /*pdl=*/true);
       if (e != cudaSuccess) return SSD_ERR_CUDA;
-      e = launch_finish_phase(x, y, ws + attn_ws, /*pdl=*/true, stream);
-      if (e != cudaSuccess) return SSD_ERR_CUDA;
-      return from_cuda(launch_attention_combine(a, ws, stream));
+      return from_cuda(launch_finish_phase(x, y, ws + attn_ws, /*pdl=*/true, stream));
     }
-    // Otherwise the acceptance and a7 on a side stream beside the attention:
-    // kernels that do not fill the GPU, or that draw every row, overlap.
+    // Otherwise (the mma.sync attention, a plain launch) the acceptance and a7
+    // on a side stream beside the attention.
     if (side_stream(&side) != cudaSuccess) return SSD_ERR_CUDA;
     if (cudaEventRecord(side->fork, stream) != cudaSuccess ||
         cudaStreamWaitEvent(side->stream, side->fork, 0) != cudaSuccess)

@@ -92,16 +92,6 @@ __device__ __forceinline__ bool load_draft_positions(const AttnArgs& a, int32_t 
   return *bad == 0;
 }
 
-// Launched as a programmatic dependent (the step's schedule): block 0 exits
-// only after the kernel before it, and lets the next kernel be scheduled
-// then, so that stream order holds.
-__device__ __forceinline__ void pdl_exit() {
-  if (pdl_first_block()) {
-    pdl_wait();
-    pdl_launch_dependents();
-  }
-}
-
 template <int D>
 __global__ void __launch_bounds__(kMaxWarps * 32, 1)
 frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
@@ -110,9 +100,6 @@ frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   constexpr int TILE_BYTES = KT * D * 2;       // one K (or V) tile
   constexpr int KSTEPS = D / 16;               // k16 steps of QK^T
   constexpr int NT_O = D / 8;                  // n8 tiles of O
-  // as in the tcgen05 kernel: a dependent may start beside it once block 0
-  // has seen the kernel before this one complete (block 0 triggers on exit)
-  if (!pdl_first_block()) pdl_launch_dependents();
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   // 1024-byte alignment for the swizzle atoms
   unsigned char* smem = reinterpret_cast<unsigned char*>(
@@ -181,7 +168,6 @@ frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
   if (!seq_valid || !has_work) {
     // never leave with copies in flight into this CTA's shared memory
     for (int t = 0; t < n_pre; ++t) mbar_wait(&full[t % kStages], 0, a.status);
-    pdl_exit();
     return;
   }
 
@@ -324,10 +310,7 @@ frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     // stage s is free for the producer; a timed-out wait anywhere stops every thread
     if (!__syncthreads_and(ok)) { ok = false; break; }
   }
-  if (!ok || !warp_active) {
-    pdl_exit();
-    return;
-  }
+  if (!ok || !warp_active) return;
 
   // ---- epilogue: normalise, write O (bf16) or the split partial (fp32)
   const bool direct = (n_active == 1);
@@ -366,7 +349,6 @@ frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
       if ((lane & 3) == 0) L.part_lse[prow] = lse;
     }
   }
-  pdl_exit();
 }
 
 // One warp per (b, j, h) row: merge the active splits by log-sum-exp.
@@ -431,22 +413,11 @@ bool make_kv_map(CUtensorMap* map, const void* base, int64_t rows, int32_t d) {
 
 struct Plan {
   int32_t nwarps, mtiles, splits, kps;
-  bool tc;  // tcgen05 kernel (attention_tc.cu)
 };
 
-// `rows_hint` (<= D_max) bounds the drafts a sequence can have in this launch;
-// it chooses between the two kernels only, both of which size their work by
-// D_max, so a wrong hint costs time, never correctness.
-Plan make_plan(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max, int32_t L_max,
-               int32_t rows_hint) {
+// The mma.sync kernel's plan.
+Plan make_plan(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max, int32_t L_max) {
   Plan p;
-  p.tc = attention_tc_supported(Hq, Hkv, d, min(D_max, rows_hint));
-  if (p.tc) {  // plans on the device, merges its splits itself
-    p.nwarps = p.mtiles = 0;
-    p.splits = 1;
-    p.kps = L_max;
-    return p;
-  }
   const int32_t G = Hq / Hkv;
   const int32_t rows = D_max * G;
   p.nwarps = min(kMaxWarps, (rows + 15) / 16);
@@ -511,13 +482,13 @@ int32_t attention_rows_hint(const ssd_grid& g, int32_t D_max) {
   return n < D_max ? (int32_t)n : D_max;
 }
 
-// Sized for the mma.sync kernel's plan whichever kernel runs (the tcgen05 kernel
-// needs none), so that the kernel choice (which depends on the grid) never
-// outgrows a workspace sized without it.
+// The mma.sync kernel's plan whichever kernel runs (the tcgen05 kernel needs
+// none): callers' sizes, and what the no-allocation entry point refuses, do
+// not depend on the kernel.
 size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
                            int32_t L_max) {
   size_t bytes = align256((size_t)B * sizeof(int32_t));
-  const int32_t splits = make_plan(B, Hq, Hkv, d, D_max, L_max, /*rows_hint=*/0).splits;
+  const int32_t splits = make_plan(B, Hq, Hkv, d, D_max, L_max).splits;
   if (splits > 1) {
     const size_t prow = (size_t)B * Hq * D_max * splits;
     bytes += align256(prow * d * sizeof(float)) + align256(prow * sizeof(float));
@@ -527,10 +498,11 @@ size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_
 
 static cudaError_t launch_combine(const AttnArgs& a, const AttnLaunch& L, cudaStream_t stream);
 
-int attention_launches(const ssd_grid& g, int32_t B, int32_t Hq, int32_t Hkv, int32_t d,
-                       int32_t D_max, int32_t L_max) {
+int attention_launches(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
+                       int32_t L_max) {
   if (B == 0) return 0;
-  return make_plan(B, Hq, Hkv, d, D_max, L_max, attention_rows_hint(g, D_max)).splits > 1 ? 2 : 1;
+  if (attention_tc_supported(Hq, Hkv, d)) return 1;
+  return make_plan(B, Hq, Hkv, d, D_max, L_max).splits > 1 ? 2 : 1;
 }
 
 namespace {
@@ -557,19 +529,11 @@ AttnLaunch carve(const AttnArgs& a, const Plan& p, void* ws) {
 
 }  // namespace
 
-cudaError_t launch_attention_combine(const AttnArgs& a, void* ws, cudaStream_t stream) {
-  if (a.B == 0) return cudaSuccess;
-  const Plan p = make_plan(a.B, a.Hq, a.Hkv, a.d, a.D_max, a.L_max,
-                           attention_rows_hint(a.grid, a.D_max));
-  return p.splits == 1 ? cudaSuccess : launch_combine(a, carve(a, p, ws), stream);
-}
-
 cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream,
-                             bool defer_combine, bool pdl) {
+                             bool pdl) {
   if (a.B == 0) return cudaSuccess;
-  const Plan p = make_plan(a.B, a.Hq, a.Hkv, a.d, a.D_max, a.L_max,
-                           attention_rows_hint(a.grid, a.D_max));
-  if (p.tc) return launch_attention_tc(a, stream, pdl);
+  if (attention_tc_supported(a.Hq, a.Hkv, a.d)) return launch_attention_tc(a, stream, pdl);
+  const Plan p = make_plan(a.B, a.Hq, a.Hkv, a.d, a.D_max, a.L_max);
   const AttnLaunch L = carve(a, p, ws);
   cudaError_t e;
   CUtensorMap tmK, tmV;
@@ -594,7 +558,7 @@ cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaS
     if (e != cudaSuccess) return e;
   }
   e = cudaGetLastError();
-  if (e != cudaSuccess || p.splits == 1 || defer_combine) return e;
+  if (e != cudaSuccess || p.splits == 1) return e;
   return launch_combine(a, L, stream);
 }
 

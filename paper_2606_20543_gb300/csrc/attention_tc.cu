@@ -7,8 +7,10 @@
 //
 // Design (GB300, tcgen05 + TMEM): a persistent kernel, two CTAs per SM in
 // clusters of kCluster, that walks work items (sequence, KV head, tile of 128
-// query rows = drafts x the Hq/Hkv heads sharing the KV head; 64-row tiles
-// with M = 64 products when a KV head's query rows fit in 64).  The kernel is
+// query rows = drafts x the Hq/Hkv heads sharing the KV head, up to 128 heads;
+// 64-row tiles with M = 64 products when a KV head's query rows fit in 64).
+// The horizontal stage's 6 rows per head run here too (20 images: 28.9 -> 20.7
+// us per step against the mma.sync kernel).  The kernel is
 // bound by the K/V stream when its items fill the GPU and by the serial chain
 // of one item (load, S, softmax, PV per tile) when they do not, hence:
 //  * two CTAs per SM: one CTA's start-up, item boundaries and tile chain
@@ -207,14 +209,17 @@ __device__ __forceinline__ float2 ld_peer2(uint32_t a) {
 }
 
 struct TcLaunch {
-  int32_t mtiles;   // query tiles of a KV head with D_max drafts
+  int32_t mtiles;    // query tiles of a KV head with D_max drafts
+  int32_t drafts;    // drafts per query tile (BM / G): its rows are drafts * G <= BM
+  int32_t order;     // leading CTAs that only order the launches (programmatic launch), else 0
+  int32_t q_copies;  // copies per Q tile: 1, or one per 64 columns if the tile has fewer than BM rows
 };
 
 // One work item (sequence, KV head, query tile, part of the keys) as the
 // producer hands it to the MMA and softmax warps; ntiles < 0 ends the CTA's
 // work.
 struct TcItem {
-  int32_t b, g, row0, rows_total, cache, Lk, k_lo, k_hi, ntiles;
+  int32_t b, g, row0, row_end, cache, Lk, k_lo, k_hi, ntiles;  // query rows row0 .. row_end - 1
   int32_t order;       // kOrder*: how the drafts' positions are ordered
   int32_t pad[2];
   int32_t kflat[128];  // raster position of each draft of b
@@ -246,11 +251,11 @@ constexpr size_t tc_smem_bytes() {
 // 64 steps 128 B inside a row, so that one instruction (with a lane per tile)
 // can issue the copies of all three.
 __device__ __forceinline__ void load_tile(void* dst, const CUtensorMap* map, int32_t c1, int32_t c2,
-                                          uint64_t* bar, uint64_t policy) {
+                                          int32_t c3, uint64_t* bar, uint64_t policy) {
   asm volatile(
       "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
       " [%0], [%1, {%2, %3, %4, %5}], [%6], %7;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(0), "r"(smem_u32(bar)),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(c1), "r"(c2), "r"(c3), "r"(smem_u32(bar)),
       "l"(policy)
       : "memory");
 }
@@ -304,6 +309,23 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   constexpr uint32_t kIdescO = idesc_f16(D, true, BM);
   static_assert(BM * D * 4 <= 2 * kNB * KV_BYTES, "a partial O fits in the K and V rings");
 
+  // Launch ordering (programmatic dependent launch): launched as a dependent of
+  // the step's acceptance pass, whose results it does not read, the kernel
+  // starts as the acceptance's CTAs retire.  The first cluster has no items:
+  // its block 0 waits for the acceptance to complete and only then lets the
+  // kernel queued after this one (the counts and draws, which read them) be
+  // scheduled beside this one; the other blocks let it be scheduled at once
+  // (it is scheduled when every block has).  A thread of a working CTA holds up
+  // its whole warp in that wait: with the wait in a V producer's idle lane the
+  // CTA stood still until the acceptance's end (one image left of 8 x 64x64
+  // 44.0 -> 36.9 us per step, GQA batch 41.1 -> 39.1 without it).
+  if ((int32_t)blockIdx.x < L.order) {
+    if (pdl_first_block()) pdl_wait();
+    pdl_launch_dependents();
+    return;
+  }
+  pdl_launch_dependents();
+  const int32_t cta = (int32_t)blockIdx.x - L.order, ncta = (int32_t)gridDim.x - L.order;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ TcSeq s_seq[kLptMax];     // the plan: sequences longest first
   __shared__ int2 s_key[kLptMax];      // (keys, items) of each sequence
@@ -352,21 +374,21 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     c = a.cache_len[seq];
     n = attn_drafts(a, seq);
     if (n < 0 || n > a.D_max || c < 0 || c > a.L_max - n) {
-      if (blockIdx.x == 0) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
+      if (cta == 0) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
     } else if (n > 0) {
-      key = make_int2(c + n, a.Hkv * ((n * G + BM - 1) / BM));
+      key = make_int2(c + n, a.Hkv * (L.mtiles == 1 ? 1 : (n + L.drafts - 1) / L.drafts));
     }
   }
   TcSeq mine{0, 0, 0, 0x7fffffff};  // producer warp: this lane's sequence and first item (B <= 32)
   if (warp == kSoftWarps) {
     if (lane == 0) {
       for (int i = 0; i < NQ; ++i) {
-        mbar_init(&q_full[i], 1);
+        mbar_init(&q_full[i], L.q_copies);
         mbar_init(&q_empty[i], 1);
       }
       for (int i = 0; i < 2; ++i) {
         mbar_init(&it_full[i], 1);
-        mbar_init(&it_empty[i], kSoftWarps);
+        mbar_init(&it_empty[i], kSoftWarps + 1);  // and the V producer
       }
       mbar_init(o_empty, kSoftWarps);
 #pragma unroll 1
@@ -436,7 +458,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     n_items = planned ? s_plan[0] : a.B * per_b;
     if (planned) {
       const int32_t cs = (int32_t)cluster_size(), most_tiles = (s_plan[1] + KTC - 1) / KTC;
-      while ((2 << ns_log) <= cs && ((2 << ns_log) * n_items) <= (int32_t)gridDim.x &&
+      while ((2 << ns_log) <= cs && ((2 << ns_log) * n_items) <= ncta &&
              (2 << ns_log) <= most_tiles)
         ++ns_log;
     }
@@ -463,10 +485,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     bool ok = true, started = false;
     int32_t k = 0;        // items handed out
     uint32_t T = 0;       // K tiles issued
+    const uint32_t q_bytes = (uint32_t)(L.drafts * G * 128) * (L.q_copies == 1 ? D / 64 : 1);  // per copy
     read_plan();
     const int32_t ns = 1 << ns_log;
-    const int32_t part = (int32_t)blockIdx.x & (ns - 1), group = (int32_t)blockIdx.x >> ns_log;
-    const int32_t ngroups = (int32_t)gridDim.x >> ns_log;
+    const int32_t part = cta & (ns - 1), group = cta >> ns_log, ngroups = ncta >> ns_log;
 #pragma unroll 1
     for (int32_t round = 0; ok; ++round) {
       const int32_t base = round * ngroups;
@@ -502,7 +524,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         mt = L.mtiles;
       }
       const int32_t b = q.b, cache = q.cache, nd = q.nd;
-      if (planned && L.mtiles > 1) mt = (nd * G + BM - 1) / BM;
+      if (planned && L.mtiles > 1) mt = (nd + L.drafts - 1) / L.drafts;
       int32_t g = i - q.off, mtile = 0;
       if (mt > 1) {
         const int32_t rem = g;
@@ -545,20 +567,20 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       }
       if (!valid && i == q.off && part == 0 && lane == 0)
         record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
-      const int32_t Lk = cache + nd, rows_total = nd * G, row0 = mtile * BM;
-      if (!valid || nd == 0 || row0 >= rows_total) continue;
+      const int32_t Lk = cache + nd, draft0 = mtile * L.drafts;
+      if (!valid || draft0 >= nd) continue;
       const int32_t tiles = (Lk + KTC - 1) / KTC;
       const int32_t t_lo = (tiles * part) >> ns_log, t_hi = (tiles * (part + 1)) >> ns_log;
       const int32_t ntiles = t_hi - t_lo;
       const int32_t kvrow0 = (b * a.Hkv + g) * a.L_max + t_lo * KTC;  // 2D row of the first key
-      const int32_t qrow = b * a.D_max + row0 / G;
+      const int32_t qrow = b * a.D_max + draft0;
       const int sq = k % NQ;
       int t = 0;
       if (lane == 0) {
         it.b = b;
         it.g = g;
-        it.row0 = row0;
-        it.rows_total = rows_total;
+        it.row0 = draft0 * G;
+        it.row_end = min(nd, draft0 + L.drafts) * G;
         it.cache = cache;
         it.Lk = Lk;
         it.k_lo = t_lo * KTC;
@@ -573,16 +595,15 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // the CTA's first item: every ring slot is free, so its first K, Q and V
         // copies go out at once, one lane each
         t = min(ntiles, kNB);
-        if (lane < 1 + 2 * kNB) {
-          const bool is_q = lane == 1, is_k = lane == 0 || (lane > 1 && (lane & 1));
-          const int st = is_q ? 0 : (lane == 0 ? 0 : (lane - 1) >> 1);  // lanes 0 K0, 1 Q, 2 V0, 3 K1, 4 V1
-          if (is_q || st < ntiles) {
-            uint64_t* bar1 = is_q ? &q_full[0] : (is_k ? &k_ready[st] : &v_ready[st]);
-            unsigned char* dst = is_q ? sQ : (is_k ? sK : sV) + st * KV_BYTES;
-            mbar_arrive_expect_tx(bar1, is_q ? Q_BYTES : KV_BYTES);
-            load_tile(dst, is_q ? &tmQ : (is_k ? &tmK : &tmV), is_q ? g * G : kvrow0 + st * KTC,
-                      is_q ? qrow : 0, bar1, is_q ? polq : pol);
-          }
+        // lanes 0 K0, 1 Q, 2 V0, 3 K1, 4 V1, 5 (q_copies = 2) Q's second half
+        const bool is_q = lane == 1 || lane == 5, is_k = lane == 0 || lane == 3;
+        const int st = lane >= 3 ? 1 : 0;  // ring slot; Q: half
+        if (is_q ? st < L.q_copies : (lane < 5 && st < ntiles)) {
+          uint64_t* bar1 = is_q ? &q_full[0] : (is_k ? &k_ready[st] : &v_ready[st]);
+          unsigned char* dst = is_q ? sQ + st * (BM * 128) : (is_k ? sK : sV) + st * KV_BYTES;
+          mbar_arrive_expect_tx(bar1, is_q ? q_bytes : KV_BYTES);
+          load_tile(dst, is_q ? &tmQ : (is_k ? &tmK : &tmV), is_q ? g * G : kvrow0 + st * KTC,
+                    is_q ? qrow : 0, is_q ? st : 0, bar1, is_q ? polq : pol);
         }
         T = t;
         __syncwarp();
@@ -595,8 +616,11 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // that used it are done
         if (k >= NQ) ok = mbar_wait(&q_empty[sq], ((k / NQ) - 1) & 1, a.status);
         if (ok) {
-          mbar_arrive_expect_tx(&q_full[sq], Q_BYTES);
-          load_tile(sQ + sq * Q_BYTES, &tmQ, g * G, qrow, &q_full[sq], polq);
+#pragma unroll 1
+          for (int h = 0; h < L.q_copies; ++h) {
+            mbar_arrive_expect_tx(&q_full[sq], q_bytes);
+            load_tile(sQ + sq * Q_BYTES + h * (BM * 128), &tmQ, g * G, qrow, h, &q_full[sq], polq);
+          }
         }
       }
       if (lane == 0) {
@@ -609,7 +633,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             break;
           }
           mbar_arrive_expect_tx(&k_ready[sb], KV_BYTES);
-          load_tile(sK + sb * KV_BYTES, &tmK, kvrow0 + t * KTC, 0, &k_ready[sb], pol);
+          load_tile(sK + sb * KV_BYTES, &tmK, kvrow0 + t * KTC, 0, 0, &k_ready[sb], pol);
         }
       }
       ok = __shfl_sync(0xffffffffu, ok, 0);
@@ -631,17 +655,8 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   } else if (warp == kSoftWarps + 1) {
     // ---------------------------------------------------------- V producer
     // Follows the item slots like the MMA warp; a slot is not rewritten before
-    // the softmax has finished its item, which needs every V tile of it.
-    // Launch ordering (programmatic dependent launch): launched as a dependent
-    // of the step's acceptance pass, whose results it does not read, the
-    // kernel starts as the acceptance's CTAs retire; lane 1 of block 0 waits
-    // for the acceptance to complete and only then lets the kernel queued
-    // after this one (the counts and draws, which read them) be scheduled
-    // beside it; lane 1 of the other blocks lets it be scheduled at once (it
-    // is scheduled when every block has).  Under a plain launch the wait
-    // returns at once.  The wait sits in the
-    // other branch of the V loop's lane test, so that lane 0 never waits at
-    // the reconvergence point of a block of its own.
+    // the softmax and this warp are done with its item (an item whose V tiles
+    // are all among the first copies can finish without this warp).
     if (lane == 0) {
       uint32_t T = 0;
       bool ok = true;
@@ -663,12 +678,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             break;
           }
           mbar_arrive_expect_tx(&v_ready[sb], KV_BYTES);
-          load_tile(sV + sb * KV_BYTES, &tmV, kvrow0 + t * KTC, 0, &v_ready[sb], pol);
+          load_tile(sV + sb * KV_BYTES, &tmV, kvrow0 + t * KTC, 0, 0, &v_ready[sb], pol);
         }
+        if (ok) mbar_arrive(&it_empty[s]);
       }
-    } else if (lane == 1) {
-      if (pdl_first_block()) pdl_wait();
-      pdl_launch_dependents();
     }
     __syncwarp();
   } else if (warp == kSoftWarps + 2) {
@@ -757,10 +770,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const TcItem& it = items[s];
       const int32_t ntiles = it.ntiles;
       if (ntiles < 0) break;
-      const int32_t row0 = it.row0, rows_total = it.rows_total, cache = it.cache, Lk = it.Lk;
+      const int32_t row0 = it.row0, row_end = it.row_end, cache = it.cache, Lk = it.Lk;
       const int32_t k_lo = it.k_lo, k_hi = it.k_hi;
       const int32_t* kflat = it.kflat;
-      const bool warp_live = row0 + warp * (BM / 4) < rows_total;
+      const bool warp_live = row0 + warp * (BM / 4) < row_end;
       // this thread's query rows: item row, draft and position
       const int32_t order = it.order;
       int32_t rl[NR], jq[NR], qpos[NR];
@@ -768,8 +781,8 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       for (int e = 0; e < NR; ++e) {
         rl[e] = BM == 64 ? warp * 16 + (lane >> 2) + 8 * e : warp * 32 + lane;
         const int32_t r = row0 + rl[e];
-        jq[e] = r < rows_total ? r / G : 0;
-        qpos[e] = r >= rows_total ? 0x7fffffff : (order == kOrderFlat ? cache + jq[e] : kflat[jq[e]]);
+        jq[e] = r < row_end ? r / G : 0;
+        qpos[e] = r >= row_end ? 0x7fffffff : (order == kOrderFlat ? cache + jq[e] : kflat[jq[e]]);
       }
       // cache slots below every query position of this item are visible to all rows
       int32_t minq = 0x7fffffff;
@@ -779,7 +792,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       } else if (order == kOrderIncreasing) {
         minq = kflat[j_lo];
       } else {
-        const int32_t j_end = (min(rows_total, row0 + BM) + G - 1) / G;
+        const int32_t j_end = row_end / G;
 #pragma unroll 1
         for (int32_t j = j_lo + lane; j < j_end; j += 32) minq = min(minq, kflat[j]);
 #pragma unroll
@@ -962,7 +975,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           const int32_t r = row0 + rl[e], h = g * G + r - jq[e] * G;
           orow[e] = ((int64_t)b * a.D_max + jq[e]) * a.Hq + h;
           // (debug builds: the row's store index against its buffer)
-          live[e] = r < rows_total && ok && dbg_in(orow[e], (int64_t)a.B * a.D_max * a.Hq, a.status);
+          live[e] = r < row_end && ok && dbg_in(orow[e], (int64_t)a.B * a.D_max * a.Hq, a.status);
           // fast reciprocal and logarithm: the epilogue runs once per item, and
           // its instruction count is its cost
           inv[e] = l_run[e] > 0.f ? __fdividef(1.0f, l_run[e]) : 0.f;
@@ -1034,14 +1047,14 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   // ---- split mode: merge the group's partial rows.  Every CTA of the grid
   // takes the same branch (the plan is the same in all of them).
   if (ns_log > 0) {
-    const int32_t ns = 1 << ns_log, part = (int32_t)blockIdx.x & (ns - 1);
+    const int32_t ns = 1 << ns_log, part = cta & (ns - 1);
     __syncwarp();
     cluster_sync_all();  // every partial row and its (max, sum) written
     const TcItem* it = s_merge;
     if (it != nullptr) {
-      const int32_t row0 = it->row0, rows = min(BM, it->rows_total - row0);
+      const int32_t row0 = it->row0, rows = it->row_end - row0;
       const int32_t cs = (int32_t)cluster_size();
-      const uint32_t rank0 = (uint32_t)((int32_t)blockIdx.x % cs - part);  // the group's first CTA
+      const uint32_t rank0 = (uint32_t)(cta % cs - part);  // the group's first CTA
       const uint32_t base_o = smem_u32(sK), base_ml = smem_u32(s_ml);
       constexpr int LPR = D / 4;              // lanes per row (a float4 each)
       constexpr int RPW = 32 / LPR;           // rows per warp and step
@@ -1100,20 +1113,18 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
 }  // namespace
 
-#ifndef SSD_ATTN_TC_MIN_ROWS
-#define SSD_ATTN_TC_MIN_ROWS 16  // query rows per KV group above which the tcgen05 kernel runs
-#endif
-
-bool attention_tc_supported(int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max) {
+bool attention_tc_supported(int32_t Hq, int32_t Hkv, int32_t d) {
   const int32_t G = Hq / Hkv;
-  return (d == 64 || d == 128) && G >= 1 && G <= kBM && (kBM % G) == 0 &&
-         D_max * G > SSD_ATTN_TC_MIN_ROWS;
+  return (d == 64 || d == 128) && G >= 1 && G <= kBM;
 }
 
 namespace {
-// Query rows per tile: 64 when a KV group's rows fit (M = 64 products, their
-// softmax spread over the four lane quarters), else 128.
-int32_t tc_tile_rows(int32_t D_max, int32_t G) { return D_max * G <= 64 ? 64 : kBM; }
+// Query rows per tile: 64 when a KV group's rows under this grid's frontier fit
+// (M = 64 products, their softmax spread over the four lane quarters), else
+// 128.  Frontiers above the hint take more tiles.
+int32_t tc_tile_rows(const AttnArgs& a) {
+  return attention_rows_hint(a.grid, a.D_max) * (a.Hq / a.Hkv) <= 64 ? 64 : kBM;
+}
 
 // Clusters of the kernel that the current device can hold at once (a device
 // constant, queried once per device and kernel), at least one.  The occupancy
@@ -1151,14 +1162,22 @@ int resident_clusters(K kernel, size_t smem) {
 
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl) {
   const int32_t G = a.Hq / a.Hkv;
-  const int32_t bm = tc_tile_rows(a.D_max, G);
+  const int32_t bm = tc_tile_rows(a);
   CUtensorMap tq, tk, tv;
   bool ok;
   const uint64_t row = (uint64_t)a.d * 2, halves = (uint64_t)a.d / 64;
-  {  // {64 columns, Hq, B * D_max, d / 64}, box {64, G, bm / G, d / 64}: rows (draft, head of the group)
+  // Rows (draft, head of the group): a tile of bm / G drafts.  When G divides bm
+  // its d / 64 column blocks of bm rows are one copy; a tile of fewer rows takes
+  // a copy per block, so that every block starts on a swizzle atom (the rows
+  // past it are never read back).
+  TcLaunch L;
+  L.drafts = bm / G;
+  L.mtiles = (a.D_max + L.drafts - 1) / L.drafts;
+  L.q_copies = bm % G == 0 ? 1 : (int32_t)halves;
+  {  // {64 columns, Hq, B * D_max, d / 64}, box {64, G, bm / G, d / 64 or 1}
     const uint64_t dims[4] = {64, (uint64_t)a.Hq, (uint64_t)a.B * a.D_max, halves};
     const uint64_t strides[3] = {row, (uint64_t)a.Hq * row, 128};
-    const uint32_t box[4] = {64, (uint32_t)G, (uint32_t)(bm / G), (uint32_t)halves};
+    const uint32_t box[4] = {64, (uint32_t)G, (uint32_t)L.drafts, L.q_copies == 1 ? (uint32_t)halves : 1u};
     ok = bf16_tensor_map(&tq, a.q, 4, dims, strides, box);
   }
   {  // {64 columns, rows, 1, d / 64}, box {64, KTC, 1, d / 64}
@@ -1169,8 +1188,6 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
          bf16_tensor_map(&tv, a.v, 4, dims, strides, box);
   }
   if (!ok) return cudaErrorInvalidValue;
-  TcLaunch L;
-  L.mtiles = (a.D_max * G + bm - 1) / bm;
   // persistent: whole clusters, as many as are resident, at most one per item
   const int64_t n_items = (int64_t)a.B * a.Hkv * L.mtiles;
   auto launch = [&](auto kernel, size_t smem) {
@@ -1178,8 +1195,9 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
                                          (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t clusters = std::min<int64_t>(n_items, resident_clusters(kernel, smem));
-    return launch_clusters(kernel, dim3((unsigned)(clusters * kCluster)), dim3(kThreadsTC), smem,
-                           stream, pdl, kCluster, tq, tk, tv, a, L);
+    L.order = pdl ? kCluster : 0;
+    return launch_clusters(kernel, dim3((unsigned)(clusters * kCluster + L.order)),
+                           dim3(kThreadsTC), smem, stream, pdl, kCluster, tq, tk, tv, a, L);
   };
   if (a.d == 128)
     return bm == 64 ? launch(frontier_attn_tc_kernel<128, 64>, tc_smem_bytes<128, 64>())

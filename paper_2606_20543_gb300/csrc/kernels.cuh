@@ -281,25 +281,22 @@ __device__ __forceinline__ int32_t longest_first(const AttnArgs& a, int32_t rank
 }
 size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
                            int32_t L_max);
-// defer_combine: leave the split-KV combine (if the plan has splits) to
-// launch_attention_combine, so that another kernel can be queued between.
 // pdl: the tcgen05 kernel is launched as a programmatic dependent of the kernel
 // before it (it reads none of that kernel's results, starts as its CTAs retire,
 // and lets the kernel after it be scheduled only once that kernel completed);
 // the mma.sync kernel is always launched plainly.
 cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream,
-                             bool defer_combine = false, bool pdl = false);
-cudaError_t launch_attention_combine(const AttnArgs& a, void* ws, cudaStream_t stream);
-int attention_launches(const ssd_grid& g, int32_t B, int32_t Hq, int32_t Hkv, int32_t d,
-                       int32_t D_max, int32_t L_max);
+                             bool pdl = false);
+int attention_launches(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
+                       int32_t L_max);
 // Most drafts one sequence can have under grid `g` (Sec. 3.3 frontier: at most
 // min(k_h, W) horizontal positions, or W - c with k_h = 0, then k_v rows of W),
 // clipped to D_max.
 int32_t attention_rows_hint(const ssd_grid& g, int32_t D_max);
 
-// ---- attention_tc.cu (tcgen05 frontier attention: query groups dividing 128,
-// more than 16 query rows per KV group); one launch, no workspace
-bool attention_tc_supported(int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max);
+// ---- attention_tc.cu (tcgen05 frontier attention: at most 128 query heads per
+// KV head); one launch, no workspace
+bool attention_tc_supported(int32_t Hq, int32_t Hkv, int32_t d);
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl = false);
 // Same as launch_attention with the library's static device scratch as the
 // workspace (ssd_verify_attention_noalloc); cudaErrorMemoryAllocation if the

@@ -22,11 +22,22 @@ pytestmark = pytest.mark.gpu
     ("two_way", 8, (16, 16), 128, 24, 120, [120 + 72 * k for k in range(8)]),
     # more than 32 sequences: planned by the block (empty frontiers among them)
     ("block_plan", 40, (4, 4), 64, 16, 7, [7 + (37 * k) % 257 for k in range(40)]),
+    # 3 and 20 query heads per KV head: tiles of 126 and 120 rows (42 and 6 drafts),
+    # 63 of a 64-row tile with d = 64
+    ("group_of_3", 3, (12, 4), 128, 24, 120, [120, 409, 120 + 23 * 24 + 1]),
+    ("group_of_20", 2, (20, 1), 128, 12, 9, [9 + 30, 9 + 140]),
+    ("group_of_3_64_rows", 4, (9, 3), 64, 10, 3, [3, 40, 77, 99]),
+    # more than 128 query heads per KV head: the mma.sync kernel, splits merged
+    # by its combine kernel
+    ("group_of_150", 2, (150, 1), 64, 1, 300, [300, 301]),
     # more sequences than the plan holds: dealt in their order
     ("unplanned", 260, (1, 1), 64, 10, 3, [3 + (7 * k) % 101 for k in range(260)]),
+    # five items per CTA of one to three key tiles, 64- and 128-row tiles
+    ("many_items", 100, (16, 16), 64, 10, 3, [3 + (7 * k) % 101 for k in range(100)]),
+    ("many_items_128", 24, (32, 8), 128, 16, 9, [9 + (31 * k) % 240 for k in range(24)]),
 ])
 def test_plan_shapes(ssd, name, B, heads, d, grid, prefix, cache):  # noqa: F811
-    c = synth.make_case(name, grid_h=grid, grid_w=grid, prefix_len=prefix, cache_len=cache,
+    c = synth.make_case(name, grid_h=max(grid, 3), grid_w=grid, prefix_len=prefix, cache_len=cache,
                         Hq=heads[0], Hkv=heads[1], d=d, V=64, seed=23, with_logits=False)
     assert c.B == B
     check_case(ssd, c)
