@@ -354,7 +354,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   float2* s_ml = reinterpret_cast<float2*>(items + 2);  // [128] split mode: (max, sum) of each row
 
   const int32_t G = a.Hq / a.Hkv;
-  const int32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int32_t tid = threadIdx.x, lane = tid & 31, warp = (int32_t)warp_uniform(tid >> 5);
   const bool planned = a.B <= kLptMax;
 
   // ---- set-up.  The first copies are the start-up's critical path, so the
@@ -686,67 +686,76 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     __syncwarp();
   } else if (warp == kSoftWarps + 2) {
     // ----------------------------------------------------------- S products
-    if (lane == 0) {
-      uint32_t T = 0;
-      for (int32_t k = 0;; ++k) {
-        const int s = k & 1, sq = k % NQ;
-        if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) break;
-        const int32_t ntiles = items[s].ntiles;
-        if (ntiles < 0) break;
-        if (!mbar_wait(&q_full[sq], (k / NQ) & 1, a.status)) break;
-        tc_fence_after();
-        const uint64_t dq = smem_desc(smem_u32(sQ + sq * Q_BYTES), 16, 1024);
-        bool ok = true;
+    // (every lane in the loop, one elected around the products: elect_one())
+    const uint32_t tSu = warp_uniform(tS), aQ = warp_uniform(smem_u32(sQ)), aK = warp_uniform(smem_u32(sK));
+    const bool leader = elect_one();
+    bool ok = true;
+    uint32_t T = 0;
 #pragma unroll 1
-        for (int t = 0; t < ntiles; ++t, ++T) {
-          const int sb = T % kNB;
-          if (!mbar_wait(&k_ready[sb], (T / kNB) & 1, a.status)) { ok = false; break; }
-          tc_fence_after();
-          const uint64_t dk = smem_desc(smem_u32(sK + sb * KV_BYTES), 16, 1024);
+    for (int32_t k = 0; ok; ++k) {
+      const int s = k & 1, sq = k % NQ;
+      if (!mbar_wait_warp(&it_full[s], (k >> 1) & 1, a.status)) break;
+      const int32_t ntiles = (int32_t)warp_uniform((uint32_t)items[s].ntiles);
+      if (ntiles < 0) break;
+      if (!mbar_wait_warp(&q_full[sq], (k / NQ) & 1, a.status)) break;
+      tc_fence_after();
+      const uint64_t dq = smem_desc(aQ + sq * Q_BYTES, 16, 1024);
+#pragma unroll 1
+      for (int t = 0; t < ntiles; ++t, ++T) {
+        const int sb = T % kNB;
+        ok = mbar_wait_warp(&k_ready[sb], (T / kNB) & 1, a.status);
+        if (!ok) break;
+        tc_fence_after();
+        const uint64_t dk = smem_desc(aK + sb * KV_BYTES, 16, 1024);
+        if (leader) {
 #pragma unroll
           for (int ks = 0; ks < D / 16; ++ks) {
             const int sub = ks >> 2, kin = (ks & 3) * 32;
-            mma_ss(tS + sb * KTC, smem_desc_at(dq, sub * (BM * 128) + kin),
+            mma_ss(tSu + sb * KTC, smem_desc_at(dq, sub * (BM * 128) + kin),
                  smem_desc_at(dk, sub * (KTC * 128) + kin), kIdescS, ks > 0 ? 1u : 0u);
           }
           mma_commit(&s_full[sb]);
           if (t == ntiles - 1) mma_commit(&q_empty[sq]);
         }
-        if (!ok) break;
+        __syncwarp();
       }
     }
     __syncwarp();
   } else if (warp == kSoftWarps + 3) {
     // ---------------------------------------------------------- PV products
-    // Issued by a thread of its own: a tcgen05.mma takes tens of cycles to
-    // issue and an mbarrier poll a few hundred, so one thread issuing both
-    // products would be the slowest stage of the tile loop.
-    if (lane == 0) {
-      uint32_t T = 0;
-      for (int32_t k = 0;; ++k) {
-        const int s = k & 1;
-        if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) break;
-        const int32_t ntiles = items[s].ntiles;
-        if (ntiles < 0) break;
-        // the first product of the item overwrites O: the epilogue of the item before must be done
-        if (k >= 1 && !mbar_wait(o_empty, (k - 1) & 1, a.status)) break;
-        bool ok = true;
+    // Issued by a warp of its own: an mbarrier poll takes a few hundred cycles,
+    // so one warp issuing both products would be the slowest stage of the tile
+    // loop.
+    const uint32_t tSu = warp_uniform(tS), tOu = warp_uniform(tO), aV = warp_uniform(smem_u32(sV));
+    const bool leader = elect_one();
+    bool ok = true;
+    uint32_t T = 0;
 #pragma unroll 1
-        for (int t = 0; t < ntiles; ++t, ++T) {
-          const int sb = T % kNB;
-          if (!mbar_wait(&v_ready[sb], (T / kNB) & 1, a.status)) { ok = false; break; }
-          tc_fence_after();
-          // A = P in TMEM (16 keys = 8 columns per step), B = V (MN-major: d
-          // atoms KTC*128 bytes apart, 8-key groups 1 KB apart; 16 keys = 2 KB)
-          const uint64_t dv = smem_desc(smem_u32(sV + sb * KV_BYTES), KTC * 128, 1024);
+    for (int32_t k = 0; ok; ++k) {
+      const int s = k & 1;
+      if (!mbar_wait_warp(&it_full[s], (k >> 1) & 1, a.status)) break;
+      const int32_t ntiles = (int32_t)warp_uniform((uint32_t)items[s].ntiles);
+      if (ntiles < 0) break;
+      // the first product of the item overwrites O: the epilogue of the item before must be done
+      if (k >= 1 && !mbar_wait_warp(o_empty, (k - 1) & 1, a.status)) break;
+#pragma unroll 1
+      for (int t = 0; t < ntiles; ++t, ++T) {
+        const int sb = T % kNB;
+        ok = mbar_wait_warp(&v_ready[sb], (T / kNB) & 1, a.status);
+        if (!ok) break;
+        tc_fence_after();
+        // A = P in TMEM (16 keys = 8 columns per step), B = V (MN-major: d
+        // atoms KTC*128 bytes apart, 8-key groups 1 KB apart; 16 keys = 2 KB)
+        const uint64_t dv = smem_desc(aV + sb * KV_BYTES, KTC * 128, 1024);
+        if (leader) {
 #pragma unroll
           for (int kk = 0; kk < KTC / 16; ++kk)
-            mma_ts(tO, tS + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
+            mma_ts(tOu, tSu + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
                     (t == 0 && kk == 0) ? 0u : 1u);
           mma_commit(&pv_done[sb]);
           mma_commit(&k_ready[sb]);  // S_{T+kNB} may start: the S/P buffer is free again
         }
-        if (!ok) break;
+        __syncwarp();
       }
     }
     __syncwarp();

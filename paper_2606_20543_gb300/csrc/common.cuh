@@ -137,6 +137,12 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int32_
   return false;
 }
 
+// The same for a whole converged warp: every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, int32_t* status,
+                                               uint32_t max_polls = kMaxPolls) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, max_polls)) != 0;
+}
+
 __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -283,6 +289,20 @@ __device__ __forceinline__ void tc_fence_before() {
 }
 __device__ __forceinline__ void tc_fence_after() {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+}
+// One lane of a converged warp.  The issuing warps run their loops with every
+// lane and elect one only around the products: the descriptors and addresses
+// then stay in uniform registers, where a loop inside `if (lane == 0)` moves
+// each operand of each tcgen05.mma over.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}"
+               : "=r"(p));
+  return p != 0;
+}
+// A value that is the same in every lane, as the compiler can tell.
+__device__ __forceinline__ uint32_t warp_uniform(uint32_t x) {
+  return __shfl_sync(0xffffffffu, x, 0);
 }
 // D[tmem] (+)= A[smem] * B[smem], kind::f16 (bf16 inputs here), fp32 accumulation.
 __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,

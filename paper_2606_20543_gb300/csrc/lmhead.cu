@@ -35,7 +35,7 @@ namespace {
 
 constexpr int kBM = 128;        // rows per MMA tile (TMEM lanes)
 constexpr int kBN = 128;        // vocabulary entries per CTA
-constexpr int kBK = 64;         // K per stage: one 128-byte swizzle atom of bf16
+constexpr int kBK = 64;         // K of one 128-byte swizzle atom of bf16
 constexpr int kMMAK = 16;       // K per tcgen05.mma (kind::f16)
 constexpr int kThreadsL = 512;  // warps 0-3 own the 128 TMEM lanes; all 16 share the combines
 constexpr int kTmemWarps = 4;
@@ -45,8 +45,6 @@ constexpr int kMaxRowTiles = 2; // rows <= 256
 constexpr float kLog2eL = 1.4426950408889634f;
 constexpr float kLn2L = 0.6931471805599453f;
 
-constexpr int kTileA = kBM * kBK * 2;   // 16 KB: [128 rows x 64 K] bf16
-constexpr int kTileB = kBK * kBN * 2;   // 16 KB: [64 K x 128 vocab] bf16 (two 64-wide boxes)
 
 struct LmPartial {  // one row, one vocabulary tile (32 bytes)
   float max_p, sum_p, max_q, sum_q;
@@ -124,6 +122,8 @@ struct LmRowRec {   // one row's combine, for every CTA after the second barrier
 
 struct LmLaunch {
   int32_t ncta, mt, stages;
+  int32_t ku;           // K per stage (64 or 128)
+  int32_t rpad;         // staged rows: the rows in swizzle groups of 8
   LmPartial* part;      // [rows][ncta]
   float* mass;          // [rows][ncta]
   LmRowRec* rec;        // [rows] each row's decision, written by the CTA that combined it
@@ -140,7 +140,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int mt = L.mt, S = L.stages;
-  const int stage_bytes = 2 * mt * kTileA + 2 * kTileB;
+  const int a_bytes = L.rpad * L.ku * 2, w_bytes = L.ku * kBN * 2;
+  const int stage_bytes = a_bytes + w_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
   uint64_t* empty = full + S;
   uint64_t* done = empty + S;
@@ -149,16 +150,16 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   int32_t* fail = flag + 1;
   LmSmemRow* rowinfo = reinterpret_cast<LmSmemRow*>(fail + 2);  // [mt * 128]
 
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, warp = (int)warp_uniform(tid >> 5);
   const int cta = blockIdx.x;
   const int32_t v0 = cta * kBN;
-  const int32_t nkb = a.K / kBK;
+  const int32_t nunits = 2 * (a.K / L.ku);  // ring units: K step u / 2 of the target (even u) or draft head
   const uint32_t ncols = (uint32_t)(mt * 2 * kBN);  // target + draft accumulators per row tile
 
   // ---- set-up: barriers, TMEM
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
-      mbar_init(&full[s], 1);
+      mbar_init(&full[s], 2);  // the weight and the hidden-state producer
       mbar_init(&empty[s], 1);
     }
     mbar_init(done, 1);
@@ -174,79 +175,85 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // ---- main loop: warp 0 lane 0 produces, warp 1 lane 0 issues the MMAs.
-  // The other lanes of those two warps park at __syncwarp: spinning on an
-  // mbarrier in the same warp would let a suspended try_wait of theirs hold
-  // up the lane that drives the pipeline.
-  if (warp == 0) {
-    // Lane 0 issues the hidden-state tiles, lane 1 the two weight tiles (one
-    // copy each through the 3D view {64, K, V / 64}): one thread issues only a
-    // few million copies per second.
-    if (lane < 2) {
-    const uint64_t pol = policy_evict_first();     // weights: read once
-    const uint64_t pol_h = policy_evict_last();    // hidden states: read by every CTA
-    const uint32_t bytes = (uint32_t)stage_bytes;
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % S;
-      int stop = 0;
-      if (lane == 0) {
-        if (kb >= S && !mbar_wait(&empty[s], ((kb / S) - 1) & 1, a.status, L.max_polls)) {
+  // ---- main loop: warp 0 lane 0 copies the weights, warp 2 lane 0 the hidden
+  // states, warp 1 lane 0 issues the MMAs; the other threads wait at the
+  // block's barrier (not polling beside them).  The loop is bound by the copies'
+  // issue unless there are few of them: one thread issues a copy every ~0.37 us
+  // (several lanes of a warp in one instruction ~0.17 us each), so a unit of
+  // one head takes two copies of up to 32 KB, from two warps.  With four 16 KB
+  // copies per 64 K the loop took 0.75 us per step whatever the vocabulary.
+  if (warp == 0 || warp == 2) {
+    if (lane == 0) {
+      const bool w = warp == 0;
+      const uint64_t pol = w ? policy_evict_first()   // weights: read once
+                             : policy_evict_last();   // hidden states: read by every CTA
+#pragma unroll 1
+      for (int u = 0; u < nunits; ++u) {
+        const int s = u % S, k0 = (u >> 1) * L.ku;
+        if (u >= S && !mbar_wait(&empty[s], ((u / S) - 1) & 1, a.status, L.max_polls)) {
           *fail = 1;
-          stop = 1;
-        } else {
-          mbar_arrive_expect_tx(&full[s], bytes);
+          break;
         }
+        unsigned char* st = smem + s * stage_bytes;
+        mbar_arrive_expect_tx(&full[s], (uint32_t)(w ? w_bytes : a_bytes));
+        // weights: 3D view {64, K, V / 64}; hidden states: {64, rows, K / 64}
+        tma_load_3d(w ? st + a_bytes : st, w ? ((u & 1) ? &tmWd : &tmWt) : ((u & 1) ? &tmHd : &tmHt), 0,
+                    w ? k0 : 0, w ? v0 / 64 : k0 / kBK, &full[s], pol);
       }
-      stop = __shfl_sync(0x3u, stop, 0);  // the stage is free and its bytes expected
-      if (stop) break;
-      unsigned char* st = smem + s * stage_bytes;
-      if (lane == 0) {
-        for (int m = 0; m < mt; ++m) {
-          tma_load_2d(st + m * kTileA, &tmHt, kb * kBK, m * kBM, &full[s], pol_h);
-          tma_load_2d(st + (mt + m) * kTileA, &tmHd, kb * kBK, m * kBM, &full[s], pol_h);
-        }
-      } else {
-        unsigned char* bt = st + 2 * mt * kTileA;
-        tma_load_3d(bt, &tmWt, 0, kb * kBK, v0 / 64, &full[s], pol);
-        tma_load_3d(bt + kTileB, &tmWd, 0, kb * kBK, v0 / 64, &full[s], pol);
-      }
-    }
     }
     __syncwarp();
   } else if (warp == 1) {
-    if (lane == 0) {
-    for (int kb = 0; kb < nkb; ++kb) {
-      const int s = kb % S;
-      if (!mbar_wait(&full[s], (kb / S) & 1, a.status, L.max_polls)) { *fail = 1; break; }
+    const uint32_t base = warp_uniform(smem_u32(smem)), tm = warp_uniform(tmem);
+    const bool leader = elect_one();
+    int s = 0;
+    uint32_t ph = 0;
+    bool good = true;
+#pragma unroll 1
+    for (int u = 0; u < nunits && good; ++u) {
+      good = mbar_wait_warp(&full[s], ph, a.status, L.max_polls);
+      if (!good) break;
       tc_fence_after();
-      const uint32_t st = smem_u32(smem + s * stage_bytes);
-      const uint32_t bt = st + 2 * mt * kTileA, bd = bt + kTileB;
+      const uint32_t st = base + s * stage_bytes;
+      // B (MN-major): 64-wide vocabulary atoms ku * 128 bytes apart (LBO), 8-row K
+      // groups 1 KB apart (SBO); one MMA's K = 16 rows = 2 KB further per step.
+      // A (K-major): 8-row groups 1 KB apart (SBO); K = 16 is 32 bytes along the
+      // row, 64 K a [rpad][128 B] block.  (A row tile is read to 128 rows, past
+      // the staged ones: those rows of the accumulators are never used.)
+      const uint64_t db0 = smem_desc(st + a_bytes, L.ku * 128, 1024), da0 = smem_desc(st, 16, 1024);
+      const uint32_t d = tm + (u & 1) * kBN;
+      const uint32_t acc0 = u > 1 ? 1u : 0u;
+      if (leader) {
+#pragma unroll 1
+        for (int sub = 0; sub < L.ku / kBK; ++sub) {
+          const uint64_t da = smem_desc_at(da0, sub * L.rpad * 128), db = smem_desc_at(db0, sub * 8192);
 #pragma unroll
-      for (int kk = 0; kk < kBK / kMMAK; ++kk) {
-        // B (MN-major): 64-wide vocabulary atoms 8 KB apart (LBO), 8-row K groups
-        // 1 KB apart (SBO); one MMA's K = 16 rows = 2 KB further per step.
-        const uint64_t db_t = smem_desc(bt + kk * 2048, 8192, 1024);
-        const uint64_t db_d = smem_desc(bd + kk * 2048, 8192, 1024);
-        for (int m = 0; m < mt; ++m) {
-          // A (K-major): 8-row groups 1 KB apart (SBO); K = 16 is 32 bytes along the row.
-          const uint64_t da_t = smem_desc(st + m * kTileA + kk * 32, 16, 1024);
-          const uint64_t da_d = smem_desc(st + (mt + m) * kTileA + kk * 32, 16, 1024);
-          const uint32_t acc = (kb > 0 || kk > 0) ? 1u : 0u;
-          mma_ss(tmem + m * 2 * kBN, da_t, db_t, kIdesc, acc);
-          mma_ss(tmem + m * 2 * kBN + kBN, da_d, db_d, kIdesc, acc);
+          for (int kk = 0; kk < kBK / kMMAK; ++kk)
+            mma_ss(d, smem_desc_at(da, kk * 32), smem_desc_at(db, kk * 2048), kIdesc,
+                   kk > 0 || sub > 0 ? 1u : acc0);
+          if (mt > 1) {
+#pragma unroll
+            for (int kk = 0; kk < kBK / kMMAK; ++kk)
+              mma_ss(d + 2 * kBN, smem_desc_at(da, kBM * 128 + kk * 32), smem_desc_at(db, kk * 2048),
+                     kIdesc, kk > 0 || sub > 0 ? 1u : acc0);
+          }
         }
+        mma_commit(&empty[s]);
       }
-      mma_commit(&empty[s]);
+      __syncwarp();
+      if (++s == S) {
+        s = 0;
+        ph ^= 1u;
+      }
     }
-    mma_commit(done);
-    }
+    if (leader) mma_commit(done);
+    // the accumulators, for every thread at the barrier below
+    if (!good || !mbar_wait_warp(done, 0, a.status, L.max_polls)) *fail = 1;
     __syncwarp();
   }
-  // every thread waits for the accumulators
-  const bool mma_ok = mbar_wait(done, 0, a.status, L.max_polls);
+  tc_fence_before();
+  __syncthreads();
   tc_fence_after();
-  bool ok = __syncthreads_and(mma_ok) != 0;
-  ok = ok && (*fail == 0);
+  bool ok = *fail == 0;
 
   const float c = kLog2eL / a.temperature;
   const int32_t rows = a.rows;
@@ -566,49 +573,45 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   }
 }
 
-// bf16 [outer][inner] matrix, box [box_outer x 64 inner], 128-byte swizzle.
-bool make_map(CUtensorMap* map, const void* base, uint64_t inner, uint64_t outer,
-              uint32_t box_outer) {
-  EncodeTiledFn fn = tensor_map_encoder();
-  if (fn == nullptr) return false;
-  cuuint64_t dims[2] = {inner, outer};
-  cuuint64_t strides[1] = {inner * 2};
-  cuuint32_t box[2] = {64, box_outer};
-  cuuint32_t estr[2] = {1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// bf16 [rows][K] hidden states as {64, rows, K / 64} (the last dimension steps
+// 128 B along a row), box {64, rpad, ku / 64}: every row's next ku entries as
+// [ku / 64][rpad][128 B] in one copy (rows past the matrix read as zero).
+bool make_hidden_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t K, uint32_t rpad,
+                     uint32_t ku) {
+  const uint64_t dims[3] = {64, rows, K / 64}, strides[2] = {K * 2, 128};
+  const uint32_t box[3] = {64, rpad, ku / 64};
+  return bf16_tensor_map(map, base, 3, dims, strides, box);
 }
 
 // bf16 [K][V] weights as the 3D view {64 vocabulary entries, K rows, V / 64
 // column blocks} (the last dimension steps 128 B along a row); a box
-// {64, kBK, 2} is one CTA's [2 blocks][kBK rows][128 B] weight tile in one copy.
-bool make_weight_map(CUtensorMap* map, const void* base, uint64_t V, uint64_t K) {
-  EncodeTiledFn fn = tensor_map_encoder();
-  if (fn == nullptr) return false;
-  cuuint64_t dims[3] = {64, K, V / 64};
-  cuuint64_t strides[2] = {V * 2, 128};
-  cuuint32_t box[3] = {64, kBK, kBN / 64};
-  cuuint32_t estr[3] = {1, 1, 1};
-  return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box,
-            estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+// {64, ku, 2} is one CTA's [2 blocks][ku rows][128 B] weight tile in one copy.
+bool make_weight_map(CUtensorMap* map, const void* base, uint64_t V, uint64_t K, uint32_t ku) {
+  const uint64_t dims[3] = {64, K, V / 64}, strides[2] = {V * 2, 128};
+  const uint32_t box[3] = {64, ku, kBN / 64};
+  return bf16_tensor_map(map, base, 3, dims, strides, box);
 }
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
 int row_tiles(int32_t rows) { return (rows + kBM - 1) / kBM; }
 
-size_t smem_bytes(int mt, int stages) {
+// Staged rows, and K per ring unit: 128 while a unit of all rows leaves room for
+// three stages (fewer, larger copies), else 64.
+int staged_rows(int32_t rows) { return (rows + 7) / 8 * 8; }
+int unit_k(int32_t rows, int32_t K) { return rows <= kBM && K % 128 == 0 ? 128 : kBK; }
+
+size_t smem_bytes(int32_t rows, int ku, int stages) {
+  const int mt = row_tiles(rows);
   // + the first rejected draft of each sequence (at most one per row)
-  return 1024 + (size_t)stages * (2 * mt * kTileA + 2 * kTileB) + (2 * stages + 1) * 8 + 16 +
+  return 1024 + (size_t)stages * (staged_rows(rows) + kBN) * ku * 2 + (2 * stages + 1) * 8 + 16 +
          (size_t)mt * kBM * sizeof(LmSmemRow) + (size_t)mt * kBM * sizeof(int32_t);
 }
 
 // As many stages as the shared memory holds, at most 8.
-int stages_for(int mt) {
+int stages_for(int32_t rows, int ku) {
   int s = 8;
-  while (s > 2 && smem_bytes(mt, s) > 232448) --s;
+  while (s > 2 && smem_bytes(rows, ku, s) > 232448) --s;
   return s;
 }
 
@@ -626,9 +629,9 @@ ssd_status lmhead_check(int32_t rows, int32_t V, int32_t K) {
   if (V <= 0 || V % kBN != 0) return SSD_ERR_UNSUPPORTED;
   if (V / kBN > 32 * kMaxTilesPerLane) return SSD_ERR_UNSUPPORTED;
   // every CTA must be resident at once (one CTA per SM: TMEM and shared memory)
-  const int mt = row_tiles(rows);
   int per_sm = 0;
-  const size_t smem = smem_bytes(mt, stages_for(mt));
+  const int ku = unit_k(rows, K);
+  const size_t smem = smem_bytes(rows, ku, stages_for(rows, ku));
   if (cudaFuncSetAttribute(lmhead_accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem) != cudaSuccess)
     return SSD_ERR_CUDA;
@@ -645,7 +648,9 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
   LmLaunch L;
   L.ncta = a.V / kBN;
   L.mt = mt;
-  L.stages = stages_for(mt);
+  L.ku = unit_k(a.rows, a.K);
+  L.rpad = staged_rows(a.rows);
+  L.stages = stages_for(a.rows, L.ku);
   L.max_polls = wait_poll_limit();
   L.shortfall = barrier_shortfall();
   unsigned char* w = static_cast<unsigned char*>(ws);
@@ -657,19 +662,18 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
   w += al256((size_t)a.rows * L.ncta * sizeof(float));
   L.rec = reinterpret_cast<LmRowRec*>(w);
   CUtensorMap ht, hd, wt, wd;
-  // hidden [rows][K]: boxes of 128 rows (rows past `rows` read as zero);
-  // weights [K][V]: boxes of 64 K-rows x 128 vocabulary entries (3D view)
-  if (!make_map(&ht, a.h_tgt, (uint64_t)a.K, (uint64_t)a.rows, kBM) ||
-      !make_map(&hd, a.h_drf, (uint64_t)a.K, (uint64_t)a.rows, kBM) ||
-      !make_weight_map(&wt, a.w_tgt, (uint64_t)a.V, (uint64_t)a.K) ||
-      !make_weight_map(&wd, a.w_drf, (uint64_t)a.V, (uint64_t)a.K))
+  const uint32_t ku = (uint32_t)L.ku, rpad = (uint32_t)L.rpad;
+  if (!make_hidden_map(&ht, a.h_tgt, (uint64_t)a.rows, (uint64_t)a.K, rpad, ku) ||
+      !make_hidden_map(&hd, a.h_drf, (uint64_t)a.rows, (uint64_t)a.K, rpad, ku) ||
+      !make_weight_map(&wt, a.w_tgt, (uint64_t)a.V, (uint64_t)a.K, ku) ||
+      !make_weight_map(&wd, a.w_drf, (uint64_t)a.V, (uint64_t)a.K, ku))
     return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   if (!a.counters_zeroed) {
     e = cudaMemsetAsync(L.barrier, 0, kLmheadCounters * sizeof(unsigned int), stream);
     if (e != cudaSuccess) return e;
   }
-  const size_t smem = smem_bytes(mt, L.stages);
+  const size_t smem = smem_bytes(a.rows, L.ku, L.stages);
   e = cudaFuncSetAttribute(lmhead_accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)smem);
   if (e != cudaSuccess) return e;

@@ -452,7 +452,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
   uint32_t* bcast = reinterpret_cast<uint32_t*>(tmem_slot + 2);  // [2]
   float* srow = reinterpret_cast<float*>(tmem_slot + 8);          // [128]
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = (int)warp_uniform(threadIdx.x >> 5), lane = tid & 31;
   const int32_t cta = blockIdx.x;
   uint32_t ncols = 32;
   while (ncols < (uint32_t)(4 * L.nc)) ncols <<= 1;
@@ -611,37 +611,44 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
         mbar_wait(&full[x % S], (x / S) & 1, nullptr, L.max_polls);
     __syncwarp();
   } else if (warp == kWarpMma) {
-    // ---- MMA issue: one thread
-    if (lane == 0) {
-      const uint32_t idk = idesc_bf16(128, L.nn, false, false);
-      const uint32_t idmn = idesc_bf16(128, L.nn, true, false);
-      const uint32_t xatom = (uint32_t)L.nn * 128u;  // one 64-wide K atom of the activations
-      uint32_t gu = 0, tc = 0;
-      bool ok = true;
-      for (int p = 0; p < kPhases && ok; ++p) {
-        const PredPhase& ph = L.ph[p];
-        const int64_t lo = unit_start(cta, ph.units, L.ncta), hi = unit_start(cta + 1, ph.units, L.ncta);
-        uint32_t buf = 0;
-        int32_t j = (int32_t)(lo % ph.upt);  // K step of unit u inside its tile
-        for (int64_t u = lo; u < hi; ++u, ++gu, j = (j + 1 == ph.upt) ? 0 : j + 1) {
-          const bool first = (u == lo) || j == 0;
-          const bool last = (u == hi - 1) || j == ph.upt - 1;
-          if (first) {
-            buf = tc & 1u;
-            if (tc >= 2 && !mbar_wait(&acc_empty[buf], ((tc >> 1) - 1) & 1, L.status, L.max_polls)) {
-              ok = false;
-              break;
-            }
-          }
-          if (!mbar_wait(&full[gu % S], (gu / S) & 1, L.status, L.max_polls)) {
+    // ---- MMA issue (every lane in the loop, one elected around the products)
+    const uint32_t idk = idesc_bf16(128, L.nn, false, false);
+    const uint32_t idmn = idesc_bf16(128, L.nn, true, false);
+    const uint32_t xatom = (uint32_t)L.nn * 128u;  // one 64-wide K atom of the activations
+    const uint32_t tm = warp_uniform(tmem), ring0 = warp_uniform(smem_u32(ring));
+    const bool leader = elect_one();
+    uint32_t tc = 0, ph = 0;
+    int s = 0;  // ring slot of the unit, its phase ph
+    bool ok = true;
+#pragma unroll 1
+    for (int p = 0; p < kPhases && ok; ++p) {
+      const PredPhase& pp = L.ph[p];
+      const int64_t lo = unit_start(cta, pp.units, L.ncta), hi = unit_start(cta + 1, pp.units, L.ncta);
+      uint32_t buf = 0;
+      int32_t j = (int32_t)(lo % pp.upt);  // K step of unit u inside its tile
+      const int32_t n = (int32_t)(hi - lo);
+#pragma unroll 1
+      for (int32_t u = 0; u < n; ++u, j = (j + 1 == pp.upt) ? 0 : j + 1) {
+        const bool first = u == 0 || j == 0;
+        const bool last = u == n - 1 || j == pp.upt - 1;
+        if (first) {
+          buf = tc & 1u;
+          if (tc >= 2 &&
+              !mbar_wait_warp(&acc_empty[buf], ((tc >> 1) - 1) & 1, L.status, L.max_polls)) {
             ok = false;
             break;
           }
-          tc_fence_after();
-          const uint32_t wb = smem_u32(ring + (gu % S) * slot_bytes);
-          const uint64_t dx = smem_desc(wb + kUnitBytes, 16, 1024);
-          const uint32_t dacc = tmem + buf * 2u * (uint32_t)L.nc;
-          const uint32_t a0 = first ? 0u : 1u;
+        }
+        if (!mbar_wait_warp(&full[s], ph, L.status, L.max_polls)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t wb = ring0 + s * slot_bytes;
+        const uint64_t dx = smem_desc(wb + kUnitBytes, 16, 1024);
+        const uint32_t dacc = tm + buf * 2u * (uint32_t)L.nc;
+        const uint32_t a0 = first ? 0u : 1u;
+        if (leader) {
           if (p == 1) {  // W1 and W3 tiles of 64 K against one activation atom
             const uint64_t dw = smem_desc(wb, 16, 1024);
 #pragma unroll
@@ -664,16 +671,19 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
               mma_ss(dacc, smem_desc_at(dw, (kk >> 2) * 16384 + (kk & 3) * 32),
                      smem_desc_at(dx, (kk >> 2) * xatom + (kk & 3) * 32), idk, kk > 0 ? 1u : a0);
           }
-          mma_commit(&empty[gu % S]);
-          if (last) {
-            mma_commit(&acc_full[buf]);
-            ++tc;
-          }
+          mma_commit(&empty[s]);
+          if (last) mma_commit(&acc_full[buf]);
+        }
+        if (last) ++tc;
+        __syncwarp();
+        if (++s == S) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-      if (!ok) *fail = 1;
-      mma_commit(mma_done);  // arrives once every MMA issued above has completed
     }
+    if (!ok) *fail = 1;
+    if (leader) mma_commit(mma_done);  // arrives once every MMA issued above has completed
     __syncwarp();
   } else {
     // ---- epilogue (warps 4-7): TMEM lane = feature et of the tile
