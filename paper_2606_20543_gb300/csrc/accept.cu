@@ -275,7 +275,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
   float* ring = reinterpret_cast<float*>(smem_raw);                  // [kStages][2][kChunk]
   float* block_mass = ring + kStages * 2 * kChunk;                   // [nch * 16]
   __shared__ Shared sh;
-  const int32_t tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int32_t tid = threadIdx.x, lane = tid & 31, warp = (int32_t)warp_uniform(tid >> 5);
   const int32_t nch = (a.V + kChunk - 1) / kChunk;
   if (tid == 0) {
     for (int s = 0; s < kStages; ++s) {
@@ -292,46 +292,54 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
 
   // ------------------------------------------------------------ producer warp
   if (warp == kCWarps) {
-    if (lane == 0) {
-      uint32_t g = 0;  // chunks issued by this CTA
+    const uint32_t ring_a = warp_uniform(smem_u32(ring));
+    const bool leader = elect_one();
+    uint32_t g = 0;  // chunks issued by this CTA
+    int s = 0;       // ring slot of chunk g, its next phase ph
+    uint32_t ph = 1;
 #pragma unroll 1
-      for (int32_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
-        const int kind = row_kind(a, r);
-        if (kind == 1 || kind == 2) continue;
-        // the row's reference is read once: the consumers may redirect it for
-        // the next round while this row's second pass is still being issued
-        const float* drow =
-            (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + (int64_t)r * a.ld;
+    for (int32_t r = blockIdx.x; r < a.rows; r += gridDim.x) {
+      const int kind = row_kind(a, r);
+      if (kind == 1 || kind == 2) continue;
+      // the row's reference is read once: the consumers may redirect it for
+      // the next round while this row's second pass is still being issued
+      const float* drow =
+          (a.ref_rows != nullptr && !a.ref_init) ? a.ref_rows[r] : a.drf + (int64_t)r * a.ld;
+      const float* trow = a.tgt + (int64_t)r * a.ld;
 #pragma unroll 1
-        for (int32_t cc = 0; cc < passes * nch; ++cc, ++g) {  // one or two passes over the row
-          const int32_t ch = passes > 1 && cc >= nch ? cc - nch : cc;
-          const int s = g % kStages;
-          if (g >= kStages) mbar_wait(&sh.empty[s], ((g / kStages) - 1) & 1, a.status);
-          const uint32_t bytes = (uint32_t)min(kChunk, a.V - ch * kChunk) * 4u;
-          float* dst = ring + s * 2 * kChunk;
+      for (int32_t cc = 0; cc < passes * nch; ++cc, ++g) {  // one or two passes over the row
+        const int32_t ch = passes > 1 && cc >= nch ? cc - nch : cc;
+        const uint32_t bytes = (uint32_t)min(kChunk, a.V - ch * kChunk) * 4u;
+        if (g >= kStages) mbar_wait(&sh.empty[s], ph, a.status);
+        __syncwarp();
+        if (leader) {
           mbar_arrive_expect_tx(&sh.full[s], 2u * bytes);
-          bulk_g2s(dst, a.tgt + (int64_t)r * a.ld + (int64_t)ch * kChunk, bytes, &sh.full[s]);
-          bulk_g2s(dst + kChunk, drow + (int64_t)ch * kChunk, bytes, &sh.full[s]);
+          bulk_g2s_at(ring_a + s * (2 * kChunk * 4), trow + ch * kChunk, bytes, &sh.full[s]);
+          bulk_g2s_at(ring_a + s * (2 * kChunk * 4) + kChunk * 4, drow + ch * kChunk, bytes, &sh.full[s]);
+        }
+        if (++s == kStages) {
+          s = 0;
+          ph ^= 1u;
         }
       }
-    } else if (a.cache_len != nullptr) {
-      // lanes 1-31: write the frontier of sequences blockIdx.x, + gridDim.x, ...
-      const int32_t B = (int32_t)(a.rows / a.D_max);
+    }
+    if (a.cache_len != nullptr) {
+      // the frontier of sequences blockIdx.x, + gridDim.x, ...
+      const int32_t B = a.rows / a.D_max;
 #pragma unroll 1
       for (int32_t b = blockIdx.x; b < B; b += gridDim.x) {
         const int32_t n = frontier_drafts(a.grid, a.cache_len[b], a.D_max);
         const int32_t n_c = a.cache_len[b] - a.grid.prefix_len;
-        if (lane == 1) {
+        if (lane == 0) {
           a.n_drafts_out[b] = n < 0 ? 0 : n;
           if (a.tickets != nullptr) a.tickets[b] = 0;
           if (n < 0) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
         }
 #pragma unroll 1
-        for (int32_t j = lane - 1; j < a.D_max; j += 31)
+        for (int32_t j = lane; j < a.D_max; j += 32)
           a.draft_pos[(int64_t)b * a.D_max + j] = j < n ? n_c + j : -1;
       }
     }
-    __syncwarp();
     return;
   }
 

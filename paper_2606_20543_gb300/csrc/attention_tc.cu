@@ -483,6 +483,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // k * ngroups + (group, or its mirror on odd rounds).
     const int32_t HW = a.grid.grid_h * a.grid.grid_w;
     bool ok = true, started = false;
+    const bool leader = elect_one();
     int32_t k = 0;        // items handed out
     uint32_t T = 0;       // K tiles issued
     const uint32_t q_bytes = (uint32_t)(L.drafts * G * 128) * (L.q_copies == 1 ? D / 64 : 1);  // per copy
@@ -623,21 +624,19 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           }
         }
       }
-      if (lane == 0) {
+      ok = __shfl_sync(0xffffffffu, ok, 0);
 #pragma unroll 1
-        for (; t < ntiles && ok; ++t, ++T) {
-          const int sb = T % kNB;
-          // K stage sb is free once S_{T-kNB} is done
-          if (T >= (uint32_t)kNB && !mbar_wait(&s_full[sb], ((T / kNB) - 1) & 1, a.status)) {
-            ok = false;
-            break;
-          }
+      for (; t < ntiles && ok; ++t, ++T) {
+        const int sb = T % kNB;
+        // K stage sb is free once S_{T-kNB} is done
+        ok = T < (uint32_t)kNB || mbar_wait_warp(&s_full[sb], ((T / kNB) - 1) & 1, a.status);
+        if (!ok) break;
+        if (leader) {
           mbar_arrive_expect_tx(&k_ready[sb], KV_BYTES);
           load_tile(sK + sb * KV_BYTES, &tmK, kvrow0 + t * KTC, 0, 0, &k_ready[sb], pol);
         }
+        __syncwarp();
       }
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      T = __shfl_sync(0xffffffffu, T, 0);
       ++k;
     }
     if (ok) {
@@ -657,31 +656,33 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // Follows the item slots like the MMA warp; a slot is not rewritten before
     // the softmax and this warp are done with its item (an item whose V tiles
     // are all among the first copies can finish without this warp).
-    if (lane == 0) {
-      uint32_t T = 0;
-      bool ok = true;
-      for (int32_t k = 0; ok; ++k) {
-        const int s = k & 1;
-        if (!mbar_wait(&it_full[s], (k >> 1) & 1, a.status)) break;
-        const TcItem& it = items[s];
-        const int32_t ntiles = it.ntiles;
-        if (ntiles < 0) break;
-        const int32_t kvrow0 = (it.b * a.Hkv + it.g) * a.L_max + it.k_lo;
-        int t = 0;
-        if (k == 0) T = t = min(ntiles, kNB);  // issued by the producer with the first K tiles
+    const bool leader = elect_one();
+    uint32_t T = 0;
+    bool ok = true;
 #pragma unroll 1
-        for (; t < ntiles; ++t, ++T) {
-          const int sb = T % kNB;
-          // V stage sb is free once PV_{T-kNB} is done
-          if (T >= (uint32_t)kNB && !mbar_wait(&pv_done[sb], ((T / kNB) - 1) & 1, a.status)) {
-            ok = false;
-            break;
-          }
+    for (int32_t k = 0; ok; ++k) {
+      const int s = k & 1;
+      if (!mbar_wait_warp(&it_full[s], (k >> 1) & 1, a.status)) break;
+      const TcItem& it = items[s];
+      const int32_t ntiles = (int32_t)warp_uniform((uint32_t)it.ntiles);
+      if (ntiles < 0) break;
+      const int32_t kvrow0 =
+          (int32_t)warp_uniform((uint32_t)((it.b * a.Hkv + it.g) * a.L_max + it.k_lo));
+      int t = 0;
+      if (k == 0) T = t = min(ntiles, kNB);  // issued by the producer with the first K tiles
+#pragma unroll 1
+      for (; t < ntiles; ++t, ++T) {
+        const int sb = T % kNB;
+        // V stage sb is free once PV_{T-kNB} is done
+        ok = T < (uint32_t)kNB || mbar_wait_warp(&pv_done[sb], ((T / kNB) - 1) & 1, a.status);
+        if (!ok) break;
+        if (leader) {
           mbar_arrive_expect_tx(&v_ready[sb], KV_BYTES);
           load_tile(sV + sb * KV_BYTES, &tmV, kvrow0 + t * KTC, 0, 0, &v_ready[sb], pol);
         }
-        if (ok) mbar_arrive(&it_empty[s]);
+        __syncwarp();
       }
+      if (ok && leader) mbar_arrive(&it_empty[s]);
     }
     __syncwarp();
   } else if (warp == kSoftWarps + 2) {

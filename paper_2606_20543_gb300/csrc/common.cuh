@@ -179,11 +179,11 @@ __device__ __forceinline__ bool mbar_wait2(uint64_t* bar1, uint32_t parity1, uin
 // ------------------------------------------------------------- bulk copies
 // Untiled bulk copy global -> shared (TMA engine); both addresses 16-byte
 // aligned, bytes a multiple of 16.  Completion is signalled on `bar`.
-__device__ __forceinline__ void bulk_g2s(void* smem_dst, const void* gmem_src, uint32_t bytes,
-                                         uint64_t* bar) {
+__device__ __forceinline__ void bulk_g2s_at(uint32_t smem_dst, const void* gmem_src, uint32_t bytes,
+                                            uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_u32(smem_dst)),
+          smem_dst),
       "l"(gmem_src), "r"(bytes), "r"(smem_u32(bar))
       : "memory");
 }

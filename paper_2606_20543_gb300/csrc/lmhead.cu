@@ -183,22 +183,33 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // one head takes two copies of up to 32 KB, from two warps.  With four 16 KB
   // copies per 64 K the loop took 0.75 us per step whatever the vocabulary.
   if (warp == 0 || warp == 2) {
-    if (lane == 0) {
-      const bool w = warp == 0;
-      const uint64_t pol = w ? policy_evict_first()   // weights: read once
-                             : policy_evict_last();   // hidden states: read by every CTA
+    const bool w = warp == 0, leader = elect_one();
+    const uint64_t pol = w ? policy_evict_first()   // weights: read once
+                           : policy_evict_last();   // hidden states: read by every CTA
+    int s = 0;
+    uint32_t ph = 1;
 #pragma unroll 1
-      for (int u = 0; u < nunits; ++u) {
-        const int s = u % S, k0 = (u >> 1) * L.ku;
-        if (u >= S && !mbar_wait(&empty[s], ((u / S) - 1) & 1, a.status, L.max_polls)) {
-          *fail = 1;
-          break;
-        }
+    for (int u = 0; u < nunits; ++u) {
+      const int k0 = (u >> 1) * L.ku;
+      if (u >= S && !mbar_wait_warp(&empty[s], ph, a.status, L.max_polls)) {
+        *fail = 1;
+        break;
+      }
+      if (leader) {
         unsigned char* st = smem + s * stage_bytes;
-        mbar_arrive_expect_tx(&full[s], (uint32_t)(w ? w_bytes : a_bytes));
         // weights: 3D view {64, K, V / 64}; hidden states: {64, rows, K / 64}
-        tma_load_3d(w ? st + a_bytes : st, w ? ((u & 1) ? &tmWd : &tmWt) : ((u & 1) ? &tmHd : &tmHt), 0,
-                    w ? k0 : 0, w ? v0 / 64 : k0 / kBK, &full[s], pol);
+        if (w) {
+          mbar_arrive_expect_tx(&full[s], (uint32_t)w_bytes);
+          tma_load_3d(st + a_bytes, (u & 1) ? &tmWd : &tmWt, 0, k0, v0 / 64, &full[s], pol);
+        } else {
+          mbar_arrive_expect_tx(&full[s], (uint32_t)a_bytes);
+          tma_load_3d(st, (u & 1) ? &tmHd : &tmHt, 0, 0, k0 / kBK, &full[s], pol);
+        }
+      }
+      __syncwarp();
+      if (++s == S) {
+        s = 0;
+        ph ^= 1u;
       }
     }
     __syncwarp();
