@@ -148,10 +148,28 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_current_stream = None
+
+
+def _current_stream_getter():
+    """The raw handle of torch's current stream on the current device.  The
+    stream object of torch.cuda.current_stream() costs 3 us of a 14 us call;
+    torch's own raw getter, where it has one, 0.2 us."""
+    global _current_stream
+    import torch
+    torch.cuda.current_stream()  # initialises CUDA in this process
+    device = getattr(torch._C, "_cuda_getDevice", None)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if device is not None and raw is not None:
+        _current_stream = lambda: raw(device())  # noqa: E731
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+    return _current_stream
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return (_current_stream or _current_stream_getter())()
     return getattr(stream, "cuda_stream", stream)
 
 

@@ -834,9 +834,7 @@ cudaError_t launch_resolve(const ResolveArgs& a, bool pdl, cudaStream_t stream) 
   if (a.B == 0) return cudaSuccess;
   const int32_t nblocks = resolve_blocks(a.V);
   const size_t smem = (size_t)nblocks * sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(resolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
+  static_assert(kMaxV / 256 * sizeof(float) <= 48 * 1024, "within the default shared memory limit");
   const dim3 grid((unsigned)((nblocks + kRBlocks - 1) / kRBlocks), (unsigned)a.B);
   return launch_kernel(resolve_kernel, grid, dim3(32), smem, stream, pdl, a);
 }
