@@ -760,19 +760,19 @@ __global__ void __launch_bounds__(32, 32) resolve_kernel(ResolveArgs a) {
     const float m = warp_sum(((w0.x + w0.y) + (w0.z + w0.w)) + ((w1.x + w1.y) + (w1.z + w1.w)));
     if (lane == 0) gmass[bk] = m;
   }
-  // last part to finish: its fence orders every part's masses before its ticket
-  __threadfence();
+  // last part to finish: lane 0 stored this part's masses; its ticket releases
+  // them and, for the last part, acquires the others'
   int32_t last = 0;
-  if (lane == 0) last = atomicAdd(&a.tickets[b], 1) == (int32_t)gridDim.x - 1;
+  if (lane == 0) last = atom_add_acq_rel(&a.tickets[b], 1) == (int32_t)gridDim.x - 1;
+  const float u_res = row_uniforms(a.rng, r).y;
   last = __shfl_sync(0xffffffffu, last, 0);
   if (!last) {
     if (pdl_first_block()) pdl_wait();
     return;
   }
-  __threadfence();
+#pragma unroll 4
   for (int32_t k = lane; k < nblocks; k += 32) rmass[k] = __ldcg(gmass + k);
   __syncwarp();
-  const float u_res = row_uniforms(a.rng, r).y;
   float tb = 0.f;
   int32_t bk;
   bool from_p = is_bonus;

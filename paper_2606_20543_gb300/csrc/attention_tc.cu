@@ -82,6 +82,10 @@ constexpr int kCtasPerSmTC = 2;   // 2 x 256 TMEM columns, 2 x ~107 KB of shared
 #define SSD_ATTN_CLUSTER 4
 #endif
 constexpr int kCluster = SSD_ATTN_CLUSTER;  // CTAs that can share one item
+// Fewest key tiles of a part of the longest item: merging parts takes ~3 us, a
+// tile 0.3-0.5 us (two rounds on 8 x 24x24, at most 11 tiles: 59.5 us with parts
+// of a tile or more, 51.6 whole; 16x16, 4 tiles: 12.3 and 12.0 us).
+constexpr int kMinTiles = 8;
 constexpr float kLog2eTC = 1.4426950408889634f;
 constexpr float kRescale = 8.0f;  // log2 growth of the running max that forces a rescale
 
@@ -459,7 +463,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     if (planned) {
       const int32_t cs = (int32_t)cluster_size(), most_tiles = (s_plan[1] + KTC - 1) / KTC;
       while ((2 << ns_log) <= cs && ((2 << ns_log) * n_items) <= ncta &&
-             (2 << ns_log) <= most_tiles)
+             (2 << ns_log) * kMinTiles <= most_tiles)
         ++ns_log;
     }
   };
@@ -1069,44 +1073,55 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       constexpr int LPR = D / 4;              // lanes per row (a float4 each)
       constexpr int RPW = 32 / LPR;           // rows per warp and step
       const int sub = lane / LPR, ch = lane % LPR;
-      // the group's CTAs take every ns-th row
+      // the group's CTAs take every ns-th row, two rows of a lane at a time (both
+      // rows' remote loads in flight)
+      constexpr int RS = (kThreadsTC / 32) * RPW;  // rows per step of the block
 #pragma unroll 1
-      for (int32_t r = part + ns * (warp * RPW + sub); r < rows; r += ns * (kThreadsTC / 32) * RPW) {
-        float2 ml[kCluster];
-        float4 x[kCluster];
-        float M = -INFINITY;
+      for (int32_t r0 = part + ns * (warp * RPW + sub); r0 < rows; r0 += 2 * ns * RS) {
+        float2 ml[2][kCluster];
+        float4 x[2][kCluster];
 #pragma unroll
-        for (int p = 0; p < kCluster; ++p)
-          if (p < ns) {
-            ml[p] = ld_peer2(peer_addr(base_ml + r * 8, rank0 + p));
-            x[p] = ld_peer4(peer_addr(base_o + part_off<D>(r, ch), rank0 + p));
-          }
+        for (int e = 0; e < 2; ++e) {
+          const int32_t r = min(r0 + e * ns * RS, rows - 1);
 #pragma unroll
-        for (int p = 0; p < kCluster; ++p)
-          if (p < ns && ml[p].y > 0.f) M = fmaxf(M, ml[p].x);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-        float l = 0.f;
+          for (int p = 0; p < kCluster; ++p)
+            if (p < ns) {
+              ml[e][p] = ld_peer2(peer_addr(base_ml + r * 8, rank0 + p));
+              x[e][p] = ld_peer4(peer_addr(base_o + part_off<D>(r, ch), rank0 + p));
+            }
+        }
 #pragma unroll
-        for (int p = 0; p < kCluster; ++p)
-          if (p < ns && ml[p].y > 0.f) {  // (a part whose keys the row does not see has no sum)
-            const float w = ex2_approx((ml[p].x - M) * c2);
-            l = fmaf(w, ml[p].y, l);
-            acc.x = fmaf(w, x[p].x, acc.x);
-            acc.y = fmaf(w, x[p].y, acc.y);
-            acc.z = fmaf(w, x[p].z, acc.z);
-            acc.w = fmaf(w, x[p].w, acc.w);
-          }
-        const int32_t jq = (row0 + r) / G, h = it->g * G + row0 + r - jq * G;
-        const int64_t orow = ((int64_t)it->b * a.D_max + jq) * a.Hq + h;
-        if (!dbg_in(orow, (int64_t)a.B * a.D_max * a.Hq, a.status)) continue;
-        const float inv = l > 0.f ? __fdividef(1.0f, l) : 0.f;
-        uint2 w;
-        w.x = pack_bf16x2(acc.x * inv, acc.y * inv);
-        w.y = pack_bf16x2(acc.z * inv, acc.w * inv);
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.o) + orow * D + 4 * ch) = w;
-        if (a.lse != nullptr && ch == 0)
-          a.lse[((int64_t)it->b * a.Hq + h) * a.D_max + jq] =
-              l > 0.f ? (M * (c2 / kLog2eTC) + __logf(l)) : -INFINITY;
+        for (int e = 0; e < 2; ++e) {
+          const int32_t r = r0 + e * ns * RS;
+          if (r >= rows) break;
+          float M = -INFINITY;
+#pragma unroll
+          for (int p = 0; p < kCluster; ++p)
+            if (p < ns && ml[e][p].y > 0.f) M = fmaxf(M, ml[e][p].x);
+          float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+          float l = 0.f;
+#pragma unroll
+          for (int p = 0; p < kCluster; ++p)
+            if (p < ns && ml[e][p].y > 0.f) {  // (a part whose keys the row does not see has no sum)
+              const float w = ex2_approx((ml[e][p].x - M) * c2);
+              l = fmaf(w, ml[e][p].y, l);
+              acc.x = fmaf(w, x[e][p].x, acc.x);
+              acc.y = fmaf(w, x[e][p].y, acc.y);
+              acc.z = fmaf(w, x[e][p].z, acc.z);
+              acc.w = fmaf(w, x[e][p].w, acc.w);
+            }
+          const int32_t jq = (row0 + r) / G, h = it->g * G + row0 + r - jq * G;
+          const int64_t orow = ((int64_t)it->b * a.D_max + jq) * a.Hq + h;
+          if (!dbg_in(orow, (int64_t)a.B * a.D_max * a.Hq, a.status)) continue;
+          const float inv = l > 0.f ? __fdividef(1.0f, l) : 0.f;
+          uint2 w;
+          w.x = pack_bf16x2(acc.x * inv, acc.y * inv);
+          w.y = pack_bf16x2(acc.z * inv, acc.w * inv);
+          *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.o) + orow * D + 4 * ch) = w;
+          if (a.lse != nullptr && ch == 0)
+            a.lse[((int64_t)it->b * a.Hq + h) * a.D_max + jq] =
+                l > 0.f ? (M * (c2 / kLog2eTC) + __logf(l)) : -INFINITY;
+        }
       }
     }
     __syncwarp();

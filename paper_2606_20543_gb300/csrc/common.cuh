@@ -46,6 +46,14 @@ __device__ __forceinline__ void record_status(int32_t* status, int32_t code) {
   if (status != nullptr) atomicCAS(status, (int32_t)SSD_OK, code);
 }
 
+// A counter that publishes this thread's earlier writes and, for the thread
+// that reads the last count, everyone else's.
+__device__ __forceinline__ int32_t atom_add_acq_rel(int32_t* p, int32_t v) {
+  int32_t old;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
+}
+
 // Debug build (SSD_DEBUG_BOUNDS=1: `python -m paper_2606_20543_gb300.build
 // --debug-bounds` writes libssd_debug.so): the kernels check the indexes of
 // their global stores and of the loads they compute from device data

@@ -113,19 +113,29 @@ __device__ __forceinline__ int32_t sequence_counts(const ssd_grid& g, int32_t co
                                                    bool write = true) {
   int32_t count = 0, prefix = 0;
   bool run = true;  // still inside the leading accepted run
-  for (int32_t j0 = 0; j0 < n; j0 += 32) {
-    const int32_t j = j0 + lane;
-    const bool a = (j < n) && accepted[(int64_t)b * D_max + j] != 0;
-    const uint32_t acc_mask = __ballot_sync(0xffffffffu, a);
-    count += __popc(acc_mask);
-    if (run) {
-      const uint32_t valid = (n - j0 >= 32) ? 0xffffffffu : ((1u << (n - j0)) - 1u);
-      const uint32_t rejected = valid & ~acc_mask;
-      if (rejected) {
-        prefix += __ffs(rejected) - 1;
-        run = false;
-      } else {
-        prefix += __popc(valid);
+#pragma unroll 1
+  for (int32_t j0 = 0; j0 < n; j0 += 128) {
+    bool a[4];  // 128 drafts' flags in flight (every frontier of the attention is one batch)
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int32_t j = j0 + 32 * u + lane;
+      a[u] = (j < n) && accepted[(int64_t)b * D_max + j] != 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int32_t left = n - j0 - 32 * u;
+      if (left <= 0) break;
+      const uint32_t acc_mask = __ballot_sync(0xffffffffu, a[u]);
+      count += __popc(acc_mask);
+      if (run) {
+        const uint32_t valid = left >= 32 ? 0xffffffffu : ((1u << left) - 1u);
+        const uint32_t rejected = valid & ~acc_mask;
+        if (rejected) {
+          prefix += __ffs(rejected) - 1;
+          run = false;
+        } else {
+          prefix += __popc(valid);
+        }
       }
     }
   }
