@@ -81,13 +81,15 @@ __device__ __forceinline__ uint32_t ld_acquire(const unsigned int* p) {
 // slower CTA that later sees the count reached through that CTA's next
 // arrival fails too instead of going on with missing partials.  Returns false
 // in every thread if this CTA gave up or the kernel was aborted.
-__device__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* status,
+__device__ __noinline__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* status,
                              int32_t* flag, uint32_t max_polls) {
   __syncthreads();
   if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(ctr, 1u);
+    // (a release and an acquire, ordered with the block by its barriers, instead of
+    // two full fences: ~1 us per grid barrier)
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
     bool ok = false;
+#pragma unroll 1
     for (uint32_t i = 0; i < max_polls; ++i) {
       if (ld_acquire(ctr) >= target) { ok = true; break; }
       if (i > 256) __nanosleep(64);
@@ -98,7 +100,6 @@ __device__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* st
       atomicExch(ctr + 1, 1u);
       record_status(status, SSD_ERR_TIMEOUT);
     }
-    __threadfence();
     *flag = ok ? 1 : 0;
   }
   __syncthreads();
@@ -452,20 +453,19 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     const LmSmemRow& ri = rowinfo[m * kBM + tid];
     const uint32_t tp = tmem + lane_off + m * 2 * kBN, tq = tp + kBN;
     float mass = 0.f;
-    float v[32], w[32];
     // every lane of the warp takes part in tcgen05.ld; rows that do not draw
     // simply discard the values
     const bool draw = row < rows && ri.state == 1;
     if (!__any_sync(0xffffffffu, draw)) continue;  // warp-uniform: no row of this warp draws
+    const float Cp = ri.Cp, Cq = ri.Cq;
 #pragma unroll 1
-    for (int ch = 0; ch < kBN / 32; ++ch) {
-      tmem_ld32(tp + ch * 32, v);
-      tmem_ld32(tq + ch * 32, w);
-      if (draw) {
+    for (int ch = 0; ch < kBN; ch += 8) {
+      float v[8], w[8];
+      tmem_ld8(tp + ch, v);
+      tmem_ld8(tq + ch, w);
 #pragma unroll
-        for (int i = 0; i < 32; ++i)
-          mass += fmaxf(ex2_approx(fmaf(v[i], c, -ri.Cp)) - ex2_approx(fmaf(w[i], c, -ri.Cq)), 0.f);
-      }
+      for (int i = 0; i < 8; ++i)
+        mass += fmaxf(ex2_approx(fmaf(v[i], c, -Cp)) - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
     }
     if (draw) L.mass[(int64_t)row * L.ncta + cta] = mass;
   }
@@ -552,23 +552,24 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     if (!__any_sync(0xffffffffu, mine)) continue;  // warp-uniform
     const bool from_p = ri.from_p != 0;
     const uint32_t tp = tmem + lane_off + m * 2 * kBN, tq = tp + kBN;
-    float v[32], w[32];
+    const float Cp = ri.Cp, Cq = ri.Cq, tc = ri.tc;
     float cum = 0.f;
     int32_t pick = -1, lastpos = -1;
+    // (8 entries per rolled step: it runs once, and an unrolled tile was fetched
+    // cold, 9.5 us in the CTAs that hold a crossing)
 #pragma unroll 1
-    for (int ch = 0; ch < kBN / 32; ++ch) {
-      tmem_ld32(tp + ch * 32, v);
-      tmem_ld32(tq + ch * 32, w);
-      if (mine && pick < 0) {
+    for (int ch = 0; ch < kBN; ch += 8) {
+      float v[8], w[8];
+      tmem_ld8(tp + ch, v);
+      tmem_ld8(tq + ch, w);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float pv = ex2_approx(fmaf(v[i], c, -ri.Cp));
-          const float wt = from_p ? pv : fmaxf(pv - ex2_approx(fmaf(w[i], c, -ri.Cq)), 0.f);
-          cum += wt;
-          if (wt > 0.f) {
-            lastpos = v0 + ch * 32 + i;
-            if (pick < 0 && cum > ri.tc) pick = lastpos;
-          }
+      for (int i = 0; i < 8; ++i) {
+        const float pv = ex2_approx(fmaf(v[i], c, -Cp));
+        const float wt = from_p ? pv : fmaxf(pv - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
+        cum += wt;
+        if (wt > 0.f) {
+          lastpos = v0 + ch + i;
+          if (pick < 0 && cum > tc) pick = lastpos;
         }
       }
     }
