@@ -390,17 +390,18 @@ ssd_status ssd_lmhead_accept(int32_t rows, int32_t V, int32_t K, const void* h_t
  * with SSD_COMMIT_PREFIX draws likewise only each sequence's first rejected
  * draft.  The other commit rules, ref_rows and strategies (A) and (B) draw
  * every row.
- * Streams: logits path — the acceptance pass computes the frontier itself
+ * Streams: on the logits path the acceptance pass computes the frontier itself
  * (and writes n_drafts and draft_pos) and the attention computes the same
- * frontier from cache_len.  With at most 128 query heads per KV head (the
- * tcgen05 attention) everything runs on `stream`: acceptance, attention, then
- * the counts (and committed draws) as a programmatic dependent of the
+ * frontier from cache_len; on the fused path the frontier comes first.  With at
+ * most 128 query heads per KV head (the tcgen05 attention) everything runs on
+ * `stream`: the acceptance (or the lm_head acceptance); the attention as its
+ * programmatic dependent (it reads none of its results and takes the SMs that
+ * it leaves); then the counts (and committed draws) as one of the
  * attention (they need only the acceptance's results, start once every
  * attention CTA is resident and wait for the attention before they exit, so
- * stream order holds).  Otherwise, and on the fused path (frontier first,
- * lm_head acceptance), the acceptance and counts run on a side stream beside
- * the attention, joined back into `stream`; the library creates that stream
- * once per device and host thread (with two events).  Make the first call on
+ * stream order holds).  Otherwise the acceptance and counts run on a side
+ * stream beside the attention, joined back into `stream`; the library creates
+ * that stream once per device and host thread (with two events).  Make the first call on
  * each device and host thread outside any stream capture; later calls may
  * be captured (the fork and join become graph edges).
  * ------------------------------------------------------------------------- */

@@ -33,9 +33,9 @@ size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
-// Side stream of ssd_verify_step on the fused path and beside the mma.sync
-// attention: acceptance runs on it, concurrently with the attention of the
-// same step on the caller's stream (they share no data).
+// Side stream of ssd_verify_step beside the mma.sync attention: acceptance runs
+// on it, concurrently with the attention of the same step on the caller's
+// stream (they share no data).
 // One per device and host thread, created on first use and kept until exit.
 struct SideStream {
   cudaStream_t stream = nullptr;
@@ -574,9 +574,17 @@ cudaError_t launch_finish_phase(const ssd_verify_args* x, const ssd_verify_out* 
   return launch_resolve(r, pdl, stream);
 }
 
-// Fused path, a1 + a6 + a7 on one stream (the frontier already written).
+// Fused path, a7 after the lm_head acceptance.
+cudaError_t launch_fused_counts(const ssd_verify_args* x, const ssd_verify_out* y, bool pdl,
+                                cudaStream_t stream) {
+  return launch_counts(x->grid, x->commit, x->B, x->D_max, x->cache_len, y->n_drafts, y->accepted,
+                       y->accepted_count, y->accepted_prefix, y->next_cache_len, y->status, pdl,
+                       stream);
+}
+
+// Fused path, a6 (the frontier already written).
 cudaError_t launch_fused_accept(const ssd_verify_args* x, const ssd_verify_out* y, void* ws,
-                                size_t ws_bytes, cudaStream_t stream) {
+                                size_t ws_bytes, cudaStream_t stream, int early_dependents = 0) {
   LmHeadArgs h;
   h.rows = x->B * x->D_max;
   h.V = x->V;
@@ -598,11 +606,8 @@ cudaError_t launch_fused_accept(const ssd_verify_args* x, const ssd_verify_out* 
   // a one-round prefix commit keeps one drawn token per sequence: draw only it
   h.lazy = x->commit == SSD_COMMIT_PREFIX ? 1 : 0;
   h.counters_zeroed = 1;  // by the frontier kernel before it
-  cudaError_t e = launch_lmhead(h, ws, ws_bytes, stream);
-  if (e != cudaSuccess) return e;
-  return launch_counts(x->grid, x->commit, x->B, x->D_max, x->cache_len, y->n_drafts, y->accepted,
-                       y->accepted_count, y->accepted_prefix, y->next_cache_len, y->status,
-                       false, stream);
+  h.early_dependents = early_dependents;
+  return launch_lmhead(h, ws, ws_bytes, stream);
 }
 
 }  // namespace
@@ -713,18 +718,37 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
       return SSD_ERR_CUDA;
     return SSD_OK;
   }
-  // Fused path: a1, then the attention on `stream` beside the lm_head
-  // acceptance and the counts on a side stream, joined back into `stream`.
-  if (side_stream(&side) != cudaSuccess) return SSD_ERR_CUDA;
+  // Fused path.
   e = launch_frontier(x->grid, x->B, x->cache_len, x->D_max, y->n_drafts, y->draft_pos, y->status,
                       stream, lmhead_counters(ws + attn_ws), kLmheadCounters);
   if (e != cudaSuccess) return SSD_ERR_CUDA;
+  if (attention_tc_supported(x->Hq, x->Hkv, x->d)) {
+    // On `stream` alone: a1; the lm_head acceptance, one CTA per 128 vocabulary
+    // entries; the attention as its programmatic dependent, on the SMs that it
+    // leaves idle (24 of 152 with 16384 entries: its CTAs follow one another
+    // there, and what is left runs when the lm_head ends); then the counts.  The
+    // attention first, beside a side stream, held the lm_head's cooperative
+    // launch up until it had ended (five 24x24 images 91.6 -> 82.3 us per step, with
+    // 512 hidden entries 49.9 -> 40.9; two 64x64 images of 4200 keys, most of whose
+    // attention is left when the lm_head ends, 97.9 -> 97.6).
+    e = launch_fused_accept(x, y, ws + attn_ws, workspace_bytes - attn_ws, stream,
+                            /*early_dependents=*/1);
+    if (e != cudaSuccess) return SSD_ERR_CUDA;
+    e = launch_attention(a, ws, attn_ws, stream, /*pdl=*/true);
+    if (e != cudaSuccess) return SSD_ERR_CUDA;
+    return from_cuda(launch_fused_counts(x, y, /*pdl=*/true, stream));
+  }
+  // The mma.sync attention (a plain launch) on `stream`, beside the lm_head
+  // acceptance and the counts on a side stream, joined back into `stream`.
+  if (side_stream(&side) != cudaSuccess) return SSD_ERR_CUDA;
   if (cudaEventRecord(side->fork, stream) != cudaSuccess ||
       cudaStreamWaitEvent(side->stream, side->fork, 0) != cudaSuccess)
     return SSD_ERR_CUDA;
   e = launch_attention(a, ws, attn_ws, stream);
   if (e != cudaSuccess) return SSD_ERR_CUDA;
   e = launch_fused_accept(x, y, ws + attn_ws, workspace_bytes - attn_ws, side->stream);
+  if (e != cudaSuccess) return SSD_ERR_CUDA;
+  e = launch_fused_counts(x, y, /*pdl=*/false, side->stream);
   if (e != cudaSuccess) return SSD_ERR_CUDA;
   if (cudaEventRecord(side->join, side->stream) != cudaSuccess ||
       cudaStreamWaitEvent(stream, side->join, 0) != cudaSuccess)
@@ -751,7 +775,9 @@ ssd_status ssd_verify_accept(const ssd_verify_args* x, const ssd_verify_out* y, 
                                     y->draft_pos, y->status, st, lmhead_counters(workspace),
                                     kLmheadCounters);
     if (e != cudaSuccess) return SSD_ERR_CUDA;
-    return from_cuda(launch_fused_accept(x, y, workspace, workspace_bytes, st));
+    e = launch_fused_accept(x, y, workspace, workspace_bytes, st);
+    if (e != cudaSuccess) return SSD_ERR_CUDA;
+    return from_cuda(launch_fused_counts(x, y, /*pdl=*/false, st));
   }
   cudaError_t e = launch_accept_phase(x, y, workspace, st);
   if (e != cudaSuccess) return SSD_ERR_CUDA;

@@ -336,6 +336,8 @@ struct LmHeadArgs {
   // The barrier words at the start of the workspace were cleared by a kernel
   // earlier on the stream (launch_frontier's `zero`): no memset.
   int32_t counters_zeroed = 0;
+  // The kernel after this one may start on the SMs that it leaves idle.
+  int32_t early_dependents = 0;
 };
 size_t lmhead_workspace(int32_t rows, int32_t V);
 // The grid-barrier words at the start of a workspace and their count.

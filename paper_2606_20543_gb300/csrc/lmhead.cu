@@ -140,6 +140,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  if (a.early_dependents) pdl_launch_dependents();
   const int mt = L.mt, S = L.stages;
   const int a_bytes = L.rpad * L.ku * 2, w_bytes = L.ku * kBN * 2;
   const int stage_bytes = a_bytes + w_bytes;
