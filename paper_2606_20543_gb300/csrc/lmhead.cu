@@ -10,7 +10,7 @@
 // Design (GB300, tcgen05 + TMEM):
 //  * one CTA per tile of 128 vocabulary entries; draft rows on the MMA's M
 //    dimension (TMEM lanes, padded to 128 per row tile), vocabulary on N, so
-//    each epilogue thread owns one row's 128 logits of the tile;
+//    each epilogue thread owns 32 of one row's 128 logits of the tile;
 //  * A = hidden states (K-major), B = weights (MN-major: the vocabulary is
 //    contiguous in W[K][V]); both staged by TMA with the 128-byte swizzle
 //    through a 3-stage mbarrier ring, two threads producing (hidden states;
@@ -25,8 +25,14 @@
 //    rows to draw (every rejected row, or, inside a one-round prefix-commit
 //    step, only each sequence's first rejection: the one token the commit
 //    keeps), their per-tile residual masses, a third barrier, and the CTA
-//    holding the CDF crossing scans its row tile sequentially.  Logits stay
+//    holding the CDF crossing scans the chunk of 32 that holds it.  Logits stay
 //    in TMEM throughout.
+// Bound: the weights' bytes (each read once) in the main loop, then a chain of
+// three grid barriers, each followed by one cold pass over a little code: 48 rows x
+// 16384 x 4096 take 56.8 us, 36 of them the loop (7.4 TB/s), 1.6 the partials, 3 to
+// 4 each the combine, the masses and the search with their barriers, and 5 the
+// cooperative launch.  Small rolled code over all 16 warps took the chain after
+// the loop from 25 to 14 us.
 #include "kernels.cuh"
 
 namespace ssd {
@@ -37,9 +43,9 @@ constexpr int kBM = 128;        // rows per MMA tile (TMEM lanes)
 constexpr int kBN = 128;        // vocabulary entries per CTA
 constexpr int kBK = 64;         // K of one 128-byte swizzle atom of bf16
 constexpr int kMMAK = 16;       // K per tcgen05.mma (kind::f16)
-constexpr int kThreadsL = 512;  // warps 0-3 own the 128 TMEM lanes; all 16 share the combines
-constexpr int kTmemWarps = 4;
+constexpr int kThreadsL = 512;  // 16 warps: 4 TMEM lane quarters x 4 column chunks of a tile
 constexpr int kCombWarps = kThreadsL / 32;
+constexpr int kChunk = kBN / (kCombWarps / 4);  // columns of a tile per warp in the epilogues
 constexpr int kMaxTilesPerLane = 8;  // vocabulary tiles per lane in the combines: V <= 32768
 constexpr int kMaxRowTiles = 2; // rows <= 256
 constexpr float kLog2eL = 1.4426950408889634f;
@@ -106,6 +112,11 @@ __device__ __noinline__ bool grid_barrier(unsigned int* ctr, unsigned int target
   return *flag != 0;
 }
 
+// The 128 threads of one TMEM lane quarter (4 warps).
+__device__ __forceinline__ void quarter_sync(int quarter) {
+  asm volatile("bar.sync %0, 128;" ::"r"(quarter + 1) : "memory");
+}
+
 struct LmSmemRow {  // per-row results of the decision, broadcast inside the CTA
   float Cp, Cq;     // log2-domain normalisers max * c + log2(sum)
   float u_res;
@@ -118,7 +129,7 @@ struct LmSmemRow {  // per-row results of the decision, broadcast inside the CTA
 
 struct LmRowRec {   // one row's combine, for every CTA after the second barrier
   float Cp, Cq, u_res;
-  int32_t state;    // 1: valid and rejected (a draw candidate), else 0
+  int32_t state;    // 0: padding or accepted, 1: rejected (a draw candidate), 2: no draft token
 };
 
 struct LmLaunch {
@@ -270,63 +281,74 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
 
   const float c = kLog2eL / a.temperature;
   const int32_t rows = a.rows;
-  // TMEM lane quarter of this warp: lanes 32*warp .. +31 (row tile m, row m*128 + tid)
-  const uint32_t lane_off = (uint32_t)(warp * 32) << 16;
+  // The epilogues over the accumulators use every warp: warp w reads the TMEM lane
+  // quarter w % 4 (the lanes that the hardware gives it) and columns
+  // [32 (w / 4), + 32) of the tile, and a quarter's four warps merge their
+  // chunks through shared memory (the ring's, free now).
+  const int quarter = warp & 3, chunk = warp >> 2;
+  const int lrow = quarter * 32 + lane;  // row of a row tile
+  const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
+  float4* chunk_part = reinterpret_cast<float4*>(smem);  // [mt][4 chunks][2][128 rows]
+  float* chunk_mass = reinterpret_cast<float*>(chunk_part + mt * 8 * kBM);  // [mt][4 chunks][128]
 
-  // ---- epilogue 1: per-tile softmax partials of every row (TMEM warps)
-  for (int m = 0; m < mt && ok && warp < kTmemWarps; ++m) {
-    const int32_t row = m * kBM + tid;
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN, tq = tp + kBN;
-    float mp = -INFINITY, sp = 0.f, mq = -INFINITY, sq = 0.f;
+  // ---- epilogue 1: per-tile softmax partials of every row (4 warps alone took
+  // 1.7 us per row tile)
+#pragma unroll 1
+  for (int m = 0; m < mt && ok; ++m) {
+    const int32_t row = m * kBM + lrow;
+    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
     float xq_c = -INFINITY, xp_c = 0.f;
     int32_t cand = -1;
     const int32_t given = (a.draft_tok != nullptr && row < rows) ? a.draft_tok[row] : -1;
-    float v[32], w[32];
-#pragma unroll 1
-    for (int ch = 0; ch < kBN / 32; ++ch) {
-      tmem_ld32(tp + ch * 32, v);
-      tmem_ld32(tq + ch * 32, w);
-      float cmp = -INFINITY, cmq = -INFINITY;
+    const int32_t c0 = v0 + chunk * kChunk;
+    float v[kChunk], w[kChunk];
+    tmem_ld32(tp, v);
+    tmem_ld32(tq, w);
+    float cmp = -INFINITY, cmq = -INFINITY;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        cmp = fmaxf(cmp, v[i]);
-        cmq = fmaxf(cmq, w[i]);
-      }
-      if (given < 0 && cmq > xq_c) {  // first maximum of q (ascending scan)
-#pragma unroll
-        for (int i = 31; i >= 0; --i)
-          if (w[i] == cmq) { cand = v0 + ch * 32 + i; xp_c = v[i]; }
-        xq_c = cmq;
-      }
-      if (given >= v0 + ch * 32 && given < v0 + ch * 32 + 32) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-          if (given == v0 + ch * 32 + i) { cand = given; xp_c = v[i]; xq_c = w[i]; }
-      }
-      float lp = 0.f, lq = 0.f;
-      const float cmpc = cmp * c, cmqc = cmq * c;
-#pragma unroll
-      for (int i = 0; i < 32; ++i) {
-        lp += ex2_approx(fmaf(v[i], c, -cmpc));
-        lq += ex2_approx(fmaf(w[i], c, -cmqc));
-      }
-      merge_ms(mp, sp, cmp, lp, c);
-      merge_ms(mq, sq, cmq, lq, c);
+    for (int i = 0; i < kChunk; ++i) {
+      cmp = fmaxf(cmp, v[i]);
+      cmq = fmaxf(cmq, w[i]);
     }
-    if (row < rows) {
-      LmPartial P;
-      P.max_p = mp;
-      P.sum_p = sp;
-      P.max_q = mq;
-      P.sum_q = sq;
-      P.xq_c = cand >= 0 ? xq_c : -INFINITY;
-      P.xp_c = xp_c;
-      P.cand = cand;
-      P.pad = 0.f;
-      reinterpret_cast<float4*>(L.part + (int64_t)row * L.ncta + cta)[0] =
-          make_float4(P.max_p, P.sum_p, P.max_q, P.sum_q);
-      reinterpret_cast<float4*>(L.part + (int64_t)row * L.ncta + cta)[1] =
-          make_float4(P.xq_c, P.xp_c, __int_as_float(P.cand), 0.f);
+    if (given < 0 && cmq > xq_c) {  // first maximum of q
+#pragma unroll
+      for (int i = kChunk - 1; i >= 0; --i)
+        if (w[i] == cmq) { cand = c0 + i; xp_c = v[i]; }
+      xq_c = cmq;
+    }
+    if (given >= c0 && given < c0 + kChunk) {
+#pragma unroll
+      for (int i = 0; i < kChunk; ++i)
+        if (given == c0 + i) { cand = given; xp_c = v[i]; xq_c = w[i]; }
+    }
+    float lp = 0.f, lq = 0.f;
+    const float cmpc = cmp * c, cmqc = cmq * c;
+#pragma unroll
+    for (int i = 0; i < kChunk; ++i) {
+      lp += ex2_approx(fmaf(v[i], c, -cmpc));
+      lq += ex2_approx(fmaf(w[i], c, -cmqc));
+    }
+    float4* part = chunk_part + m * 8 * kBM + lrow;
+    part[(2 * chunk) * kBM] = make_float4(cmp, lp, cmq, lq);
+    part[(2 * chunk + 1) * kBM] = make_float4(xq_c, xp_c, __int_as_float(cand), 0.f);
+    quarter_sync(quarter);
+    if (chunk == 0 && row < rows) {
+      float mp = -INFINITY, sp = 0.f, mq = -INFINITY, sq = 0.f, xq = -INFINITY, xp = 0.f;
+      int32_t t = -1;
+#pragma unroll 1
+      for (int k = 0; k < kCombWarps / 4; ++k) {  // ascending: the first maximum stays
+        const float4 e0 = part[(2 * k) * kBM], e1 = part[(2 * k + 1) * kBM];
+        merge_ms(mp, sp, e0.x, e0.y, c);
+        merge_ms(mq, sq, e0.z, e0.w, c);
+        if (__float_as_int(e1.z) >= 0 && (t < 0 || e1.x > xq)) {
+          xq = e1.x;
+          xp = e1.y;
+          t = __float_as_int(e1.z);
+        }
+      }
+      float4* out = reinterpret_cast<float4*>(L.part + (int64_t)row * L.ncta + cta);
+      out[0] = make_float4(mp, sp, mq, sq);
+      out[1] = make_float4(xq, xp, __int_as_float(t), 0.f);
     }
   }
   ok = grid_barrier(L.barrier, (unsigned)L.ncta + L.shortfall, a.status, flag, L.max_polls) && ok;
@@ -335,6 +357,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // combined by CTA r % ncta alone (one warp per row; lane l merges tiles l,
   // l + 32, ... in order, then a xor tree), which writes its outputs and its
   // record for the other CTAs.  All loads of a row are issued before any merge.
+#pragma unroll 1
   for (int32_t row = cta + L.ncta * warp; row < rows && ok; row += L.ncta * kCombWarps) {
     bool pad = false;
     if (a.n_drafts != nullptr) {
@@ -366,20 +389,32 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
 #pragma unroll
     for (int j = 0; j < kMaxTilesPerLane; ++j) {
       if (lane + 32 * j < L.ncta) {
-        merge_ms(Mp, Sp, q0[j].x, q0[j].y, c);
-        merge_ms(Mq, Sq, q0[j].z, q0[j].w, c);
+        Mp = fmaxf(Mp, q0[j].x);
+        Mq = fmaxf(Mq, q0[j].z);
         const int32_t ck = __float_as_int(q1[j].z);
         if (ck >= 0 && better(q1[j].x, ck, xq, t)) { xq = q1[j].x; xp = q1[j].y; t = ck; }
       }
     }
-#pragma unroll
+#pragma unroll 1
     for (int o = 16; o > 0; o >>= 1) {
-      merge_ms(Mp, Sp, __shfl_xor_sync(0xffffffffu, Mp, o), __shfl_xor_sync(0xffffffffu, Sp, o), c);
-      merge_ms(Mq, Sq, __shfl_xor_sync(0xffffffffu, Mq, o), __shfl_xor_sync(0xffffffffu, Sq, o), c);
+      Mp = fmaxf(Mp, __shfl_xor_sync(0xffffffffu, Mp, o));
+      Mq = fmaxf(Mq, __shfl_xor_sync(0xffffffffu, Mq, o));
       const float oq = __shfl_xor_sync(0xffffffffu, xq, o);
       const float op = __shfl_xor_sync(0xffffffffu, xp, o);
       const int32_t ot = __shfl_xor_sync(0xffffffffu, t, o);
       if (better(oq, ot, xq, t)) { xq = oq; xp = op; t = ot; }
+    }
+#pragma unroll
+    for (int j = 0; j < kMaxTilesPerLane; ++j) {
+      if (lane + 32 * j < L.ncta) {  // (a tile of -inf alone has no sum)
+        if (q0[j].x > -INFINITY) Sp = fmaf(q0[j].y, ex2_approx((q0[j].x - Mp) * c), Sp);
+        if (q0[j].z > -INFINITY) Sq = fmaf(q0[j].w, ex2_approx((q0[j].z - Mq) * c), Sq);
+      }
+    }
+#pragma unroll 1
+    for (int o = 16; o > 0; o >>= 1) {
+      Sp += __shfl_xor_sync(0xffffffffu, Sp, o);
+      Sq += __shfl_xor_sync(0xffffffffu, Sq, o);
     }
     if (lane == 0) {
       const int32_t given = a.draft_tok != nullptr ? a.draft_tok[row] : -1;
@@ -397,7 +432,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       rr.Cp = Mp * c + log2f(Sp);
       rr.Cq = Mq * c + log2f(Sq);
       rr.u_res = u.y;
-      rr.state = (valid_t && !acc) ? 1 : 0;
+      rr.state = acc ? 0 : valid_t ? 1 : 2;
       L.rec[row] = rr;
       if (!valid_t) record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
       a.accepted[row] = acc ? 1 : 0;
@@ -418,49 +453,48 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   int32_t* first = reinterpret_cast<int32_t*>(rowinfo + mt * kBM);  // [rows / D_max]
   const bool lazy = a.lazy != 0 && a.n_drafts != nullptr;
   const int32_t ngroups = lazy ? rows / a.D_max : 0;
+  int32_t* ndraw = first + mt * kBM;     // the rows to draw, in any order, and their count
+  int32_t* drawn = ndraw + 1;            // [mt * 128]
+  if (tid == 0) *ndraw = 0;
   for (int32_t g = tid; g < ngroups; g += kThreadsL) first[g] = 0x7fffffff;
+  // the record of a row, written by another CTA, read from L2 (at most one row
+  // per thread; its state says all that the choice needs)
+  static_assert(kMaxRowTiles * kBM <= kThreadsL, "one row per thread");
+  float4 rv = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (tid < rows && ok) rv = __ldcg(reinterpret_cast<const float4*>(L.rec + tid));
+  const int32_t state = __float_as_int(rv.w);
+  const int32_t group = lazy ? tid / a.D_max : 0;
   __syncthreads();
-  if (lazy && ok) {
-    for (int32_t row = tid; row < rows; row += kThreadsL) {
-      const int32_t b = row / a.D_max, j = row - b * a.D_max;
-      if (j < a.n_drafts[b] && __ldcg(a.accepted + row) == 0) atomicMin(&first[b], j);
-    }
-  }
+  if (lazy && state != 0) atomicMin(&first[group], tid - group * a.D_max);
   __syncthreads();
-  for (int32_t r = tid; r < mt * kBM; r += kThreadsL) {
-    LmSmemRow& ri = rowinfo[r];
-    ri.state = 0;
+  if (tid < mt * kBM) {
+    LmSmemRow& ri = rowinfo[tid];
+    const bool pick = state == 1 && (!lazy || tid - group * a.D_max == first[group]);
+    ri.Cp = rv.x;
+    ri.Cq = rv.y;
+    ri.u_res = rv.z;
+    ri.state = pick ? 1 : 0;
     ri.from_p = 0;
     ri.cstar = -1;
-    if (r < rows && ok) {
-      // the record of another CTA, read from L2
-      const float4 rv = __ldcg(reinterpret_cast<const float4*>(L.rec + r));
-      const bool pick = __float_as_int(rv.w) == 1 &&
-                        (!lazy || r - (r / a.D_max) * a.D_max == first[r / a.D_max]);
-      if (pick) {
-        ri.Cp = rv.x;
-        ri.Cq = rv.y;
-        ri.u_res = rv.z;
-        ri.state = 1;
-      }
-    }
+    if (pick) drawn[atomicAdd(ndraw, 1)] = tid;
   }
   __syncthreads();
 
-  // ---- epilogue 3: residual mass of this tile for every row to draw
-  // (sequential over the tile in vocabulary order; TMEM warps)
-  for (int m = 0; m < mt && ok && warp < kTmemWarps; ++m) {
-    const int32_t row = m * kBM + tid;
-    const LmSmemRow& ri = rowinfo[m * kBM + tid];
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN, tq = tp + kBN;
+  // ---- epilogue 3: residual mass of this tile for every row to draw: chunk sums
+  // in vocabulary order, then their sum
+#pragma unroll 1
+  for (int m = 0; m < mt && ok; ++m) {
+    const int32_t row = m * kBM + lrow;
+    const LmSmemRow& ri = rowinfo[m * kBM + lrow];
+    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
     float mass = 0.f;
     // every lane of the warp takes part in tcgen05.ld; rows that do not draw
     // simply discard the values
     const bool draw = row < rows && ri.state == 1;
-    if (!__any_sync(0xffffffffu, draw)) continue;  // warp-uniform: no row of this warp draws
+    if (!__any_sync(0xffffffffu, draw)) continue;  // no row of this quarter draws
     const float Cp = ri.Cp, Cq = ri.Cq;
 #pragma unroll 1
-    for (int ch = 0; ch < kBN; ch += 8) {
+    for (int ch = 0; ch < kChunk; ch += 8) {
       float v[8], w[8];
       tmem_ld8(tp + ch, v);
       tmem_ld8(tq + ch, w);
@@ -468,7 +502,11 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       for (int i = 0; i < 8; ++i)
         mass += fmaxf(ex2_approx(fmaf(v[i], c, -Cp)) - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
     }
-    if (draw) L.mass[(int64_t)row * L.ncta + cta] = mass;
+    float* cm = chunk_mass + m * 4 * kBM + lrow;
+    cm[chunk * kBM] = mass;
+    quarter_sync(quarter);
+    if (draw && chunk == 0)
+      L.mass[(int64_t)row * L.ncta + cta] = mass + cm[kBM] + cm[2 * kBM] + cm[3 * kBM];
   }
   ok = grid_barrier(L.barrier, 3u * ((unsigned)L.ncta + L.shortfall), a.status, flag,
                     L.max_polls) && ok;
@@ -477,22 +515,38 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // owns tiles [l*per, (l+1)*per) and keeps their masses in registers; the
   // same arithmetic in every CTA)
   const int32_t per = (L.ncta + 31) / 32;  // <= kMaxTilesPerLane
-  for (int m = 0; m < mt && ok; ++m) {
-    for (int rl = warp; rl < kBM; rl += kCombWarps) {
-      LmSmemRow& ri = rowinfo[m * kBM + rl];
-      if (ri.state != 1) continue;
-      const int32_t row = m * kBM + rl;
-      for (int fp = 0; fp < 2; ++fp) {
-        float mk[kMaxTilesPerLane];
+  // (a row takes a warp ~1.1 us: from the list, since by row number the drawn rows
+  // of images of 48 rows fell to one warp, 5 us)
+  if (ok) {
+    const int32_t nd = *ndraw;
+    auto tile_masses = [&](int32_t i, float* mk) {
 #pragma unroll
-        for (int q = 0; q < kMaxTilesPerLane; ++q) {
-          const int k = lane * per + q;
-          mk[q] = 0.f;
-          if (q < per && k < L.ncta) {
-            if (fp == 0) {
-              mk[q] = L.mass[(int64_t)row * L.ncta + k];
-            } else {  // masses of p itself, from the tile partials
-              const float4 p0 = reinterpret_cast<const float4*>(L.part + (int64_t)row * L.ncta + k)[0];
+      for (int q = 0; q < kMaxTilesPerLane; ++q) {
+        const int k = lane * per + q;
+        mk[q] = q < per && k < L.ncta && i < nd
+                    ? __ldcg(L.mass + (int64_t)drawn[i] * L.ncta + k) : 0.f;
+      }
+    };
+    float mnext[kMaxTilesPerLane];  // of the warp's next row, in flight during this one
+    tile_masses(warp, mnext);
+#pragma unroll 1
+    for (int32_t i = warp; i < nd; i += kCombWarps) {
+      const int32_t row = drawn[i];
+      LmSmemRow& ri = rowinfo[row];
+      float mk[kMaxTilesPerLane];
+#pragma unroll
+      for (int q = 0; q < kMaxTilesPerLane; ++q) mk[q] = mnext[q];
+      tile_masses(i + kCombWarps, mnext);
+#pragma unroll 1
+      for (int fp = 0; fp < 2; ++fp) {
+        if (fp == 1) {  // masses of p itself, from the tile partials
+#pragma unroll
+          for (int q = 0; q < kMaxTilesPerLane; ++q) {
+            const int k = lane * per + q;
+            mk[q] = 0.f;
+            if (q < per && k < L.ncta) {
+              const float4 p0 =
+                  __ldcg(reinterpret_cast<const float4*>(L.part + (int64_t)row * L.ncta + k));
               mk[q] = p0.y * ex2_approx(p0.x * c - ri.Cp);
             }
           }
@@ -501,7 +555,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
 #pragma unroll
         for (int q = 0; q < kMaxTilesPerLane; ++q) ls += mk[q];
         float incl = ls;
-#pragma unroll
+#pragma unroll 1
         for (int o = 1; o < 32; o <<= 1) {
           const float y = __shfl_up_sync(0xffffffffu, incl, o);
           if (lane >= o) incl += y;
@@ -545,34 +599,62 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   }
   __syncthreads();
 
-  // ---- epilogue 5: the CTA holding the crossing scans its tile sequentially
-  for (int m = 0; m < mt && ok && warp < kTmemWarps; ++m) {
-    const int32_t row = m * kBM + tid;
-    const LmSmemRow& ri = rowinfo[m * kBM + tid];
-    const bool mine = row < rows && ri.state == 1 && ri.cstar == cta;
+  // ---- epilogue 5: the CTA holding the crossing scans the chunk that holds it
+  // (its chunk masses say which) in order; a row drawn from p, whose chunk
+  // masses are not kept, is scanned whole by the first chunk's warp
+#pragma unroll 1
+  for (int m = 0; m < mt && ok; ++m) {
+    const int32_t row = m * kBM + lrow;
+    const LmSmemRow& ri = rowinfo[m * kBM + lrow];
+    bool mine = row < rows && ri.state == 1 && ri.cstar == cta;
     if (!__any_sync(0xffffffffu, mine)) continue;  // warp-uniform
     const bool from_p = ri.from_p != 0;
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN, tq = tp + kBN;
-    const float Cp = ri.Cp, Cq = ri.Cq, tc = ri.tc;
+    float target = ri.tc;
+    if (mine && !from_p) {
+      const float* cm = chunk_mass + m * 4 * kBM + lrow;
+      int at = -1, last = -1;
+      float before = 0.f, tk = INFINITY;
+#pragma unroll
+      for (int k = 0; k < kCombWarps / 4; ++k) {
+        const float mk = cm[k * kBM];
+        if (mk > 0.f) {
+          last = k;
+          if (at < 0 && before + mk > target) { at = k; tk = target - before; }
+        }
+        before += mk;
+      }
+      mine = chunk == (at >= 0 ? at : last);
+      target = tk;
+    } else {
+      mine = mine && chunk == 0;
+    }
+    if (!__any_sync(0xffffffffu, mine)) continue;
+    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
+    const float Cp = ri.Cp, Cq = ri.Cq;
+    const int end = __any_sync(0xffffffffu, mine && from_p) ? kBN : kChunk;  // (then chunk is 0)
+    const int end_row = from_p ? kBN : kChunk;
     float cum = 0.f;
     int32_t pick = -1, lastpos = -1;
     // (8 entries per rolled step: it runs once, and an unrolled tile was fetched
     // cold, 9.5 us in the CTAs that hold a crossing)
 #pragma unroll 1
-    for (int ch = 0; ch < kBN; ch += 8) {
+    for (int ch = 0; ch < end; ch += 8) {
       float v[8], w[8];
       tmem_ld8(tp + ch, v);
       tmem_ld8(tq + ch, w);
+      if (ch < end_row) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float pv = ex2_approx(fmaf(v[i], c, -Cp));
-        const float wt = from_p ? pv : fmaxf(pv - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
-        cum += wt;
-        if (wt > 0.f) {
-          lastpos = v0 + ch + i;
-          if (pick < 0 && cum > tc) pick = lastpos;
+        for (int i = 0; i < 8; ++i) {
+          const float pv = ex2_approx(fmaf(v[i], c, -Cp));
+          const float wt = from_p ? pv : fmaxf(pv - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
+          cum += wt;
+          if (wt > 0.f) {
+            lastpos = v0 + chunk * kChunk + ch + i;
+            if (pick < 0 && cum > target) pick = lastpos;
+          }
         }
       }
+      __syncwarp();
     }
     if (mine) a.out_tok[row] = pick >= 0 ? pick : lastpos;
   }
@@ -616,9 +698,10 @@ int unit_k(int32_t rows, int32_t K) { return rows <= kBM && K % 128 == 0 ? 128 :
 
 size_t smem_bytes(int32_t rows, int ku, int stages) {
   const int mt = row_tiles(rows);
-  // + the first rejected draft of each sequence (at most one per row)
+  // + the first rejected draft of each sequence (at most one per row), and the
+  // list of the rows to draw
   return 1024 + (size_t)stages * (staged_rows(rows) + kBN) * ku * 2 + (2 * stages + 1) * 8 + 16 +
-         (size_t)mt * kBM * sizeof(LmSmemRow) + (size_t)mt * kBM * sizeof(int32_t);
+         (size_t)mt * kBM * sizeof(LmSmemRow) + (size_t)(2 * mt * kBM + 1) * sizeof(int32_t);
 }
 
 // As many stages as the shared memory holds, at most 8.
