@@ -25,9 +25,10 @@
 // a tile's whole K runs in its CTA: no partial sums, so between the phases
 // there is only the tile's epilogue, one counter and the next activations'
 // copies, at the price of every CTA reading all of X from L2 (24 rows: 1.2 MB
-// beside 3.1 MB of weights).  At d = 4096, m = 8192, V = 16384: 24 rows 89 us
-// (0.67 of the time at the measured copy bandwidth), 64 rows 97, 128 rows 121;
-// 92 rows at d = 896 43.  Splitting each tile's K over CTAs instead, with the
+// beside 3.1 MB of weights).  At d = 4096, m = 8192, V = 16384: 24 rows 85 us
+// (0.71 of the rate of the measured copy), 64 rows 92, 128 rows 117; 92 rows at
+// d = 896 38.  (With 4 epilogue warps of whole rows 89, 97, 120 and 42; with 16 of
+// them that each polled for the products 86, 93, 123 and 41.)  Splitting each tile's K over CTAs instead, with the
 // partials summed through L2 by the last contributor (~9 us per phase boundary,
 // 254 KB of code), took 113, 135, 147 and 93 us.
 //   * warp 0: weight producer, running ahead through all four phases into a
@@ -37,7 +38,7 @@
 //     final (a counter per phase), one copy per unit from z, Ag, G or Hg;
 //   * warp 2: issues the MMAs of each unit into one of two TMEM accumulators
 //     (a CTA's next tile overlaps the epilogue of the one before);
-//   * warps 4-7: the epilogue.  Each TMEM lane is one row: A, Ag and the row's
+//   * warps 4-19: the epilogue, four warps per TMEM lane quarter.  Each TMEM lane is one row: A, Ag and the row's
 //     sum of squares over the tile (P0); G (P1); h and Hg (P2); the tile's
 //     argmax, raised into one 64-bit key per row by a max reduction (P3).  The
 //     row scales s(A) are summed once per CTA, beside the P1 products; the last
@@ -53,13 +54,14 @@ namespace ssd {
 
 namespace {
 
-constexpr int kPThreads = 256;       // 8 warps
+constexpr int kPThreads = 640;       // 20 warps
 constexpr int kWarpW = 0;            // weight producer
 constexpr int kWarpX = 1;            // activation producer
 constexpr int kWarpMma = 2;
 constexpr int kWarpTmem = 3;         // allocates / frees tensor memory
-constexpr int kEpiWarp0 = 4;         // warps 4-7: TMEM lane quarters 0-3
-constexpr int kEpiThreads = 128;
+constexpr int kEpiWarp0 = 4;         // warps 4-19: TMEM lane quarter w % 4, column chunk (w - 4) / 4
+constexpr int kEpiChunks = 4;
+constexpr int kEpiThreads = 128 * kEpiChunks;
 constexpr int kMaxRows = 128;
 constexpr int kPhases = 4;
 constexpr int kBarEpi = 1;           // named barrier of the epilogue warps
@@ -171,6 +173,11 @@ __device__ __forceinline__ int32_t argmax_index(unsigned long long key) {
   return (int32_t)(0xffffffffu - (uint32_t)(key & 0xffffffffull));
 }
 
+// The four warps of one TMEM lane quarter.
+__device__ __forceinline__ void quarter_sync(int quarter) {
+  bar_named(kBarEpi + 1 + quarter, 32 * kEpiChunks);
+}
+
 __device__ __forceinline__ uint4 pack8(const float* y) {
   return make_uint4(pack_bf16x2(y[0], y[1]), pack_bf16x2(y[2], y[3]), pack_bf16x2(y[4], y[5]),
                     pack_bf16x2(y[6], y[7]));
@@ -178,9 +185,13 @@ __device__ __forceinline__ uint4 pack8(const float* y) {
 
 // The finishing step of tile t of phase p for one row (this thread's TMEM lane;
 // live: the row exists), 8 features at a time, in one rolled loop per phase: it
-// runs once per tile, so its instructions are fetched rather than reused.
+// runs once per tile, so its instructions are fetched rather than reused.  The
+// quarter's four warps take every fourth group of 8 (one warp per quarter took
+// 1.3 us per tile, the gate 3.8) and combine sums and keys through `xch`
+// (8 bytes per row: with 24 the ring lost a slot at 73 to 96 rows).
 __device__ __forceinline__ void finish_hidden(const PredLaunch& L, int p, int32_t t, int32_t row,
-                                              bool live, uint32_t acc) {
+                                              bool live, uint32_t acc, int chunk, int quarter,
+                                              float2* xch, float* srow) {
   const PredPhase& ph = L.ph[p];
   const int32_t f0 = t * ph.tn, n = min(ph.tn, ph.F - f0);
   float* hid = L.hid + (int64_t)row * L.d + f0;
@@ -188,7 +199,7 @@ __device__ __forceinline__ void finish_hidden(const PredLaunch& L, int p, int32_
   const float* gamma = (p == 0 ? L.gamma1 : L.gamma2) + f0;
   float sq = 0.f;
 #pragma unroll 1
-  for (int32_t c = 0; c < n; c += 8) {
+  for (int32_t c = 8 * chunk; c < n; c += 8 * kEpiChunks) {
     float y[8];
     tmem_ld8(acc + c, y);
     if (!live) continue;
@@ -208,16 +219,23 @@ __device__ __forceinline__ void finish_hidden(const PredLaunch& L, int p, int32_
     sq += ((y[0] * y[0] + y[1] * y[1]) + (y[2] * y[2] + y[3] * y[3])) +
           ((y[4] * y[4] + y[5] * y[5]) + (y[6] * y[6] + y[7] * y[7]));
   }
-  if (p == 0 && live) L.ss[(int64_t)t * kMaxRows + row] = sq;
+  if (p == 0) {
+    // (srow is free until P1)
+    if (chunk > 0 && live) (chunk == 1 ? xch[row].x : chunk == 2 ? xch[row].y : srow[row]) = sq;
+    quarter_sync(quarter);
+    if (chunk == 0 && live)
+      L.ss[(int64_t)t * kMaxRows + row] = sq + xch[row].x + xch[row].y + srow[row];
+    quarter_sync(quarter);  // (the CTA's next tile writes them again)
+  }
 }
 // P1: G = bf16(silu(U) * Vg) with U, Vg scaled by the row's s(A).
 __device__ __forceinline__ void finish_gate(const PredLaunch& L, int32_t t, int32_t row, bool live,
-                                            uint32_t acc, float sr) {
+                                            uint32_t acc, float sr, int chunk) {
   const PredPhase& ph = L.ph[1];
   const int32_t f0 = t * ph.tn, n = min(ph.tn, ph.F - f0);
   __nv_bfloat16* g = L.g + (int64_t)row * L.m + f0;
 #pragma unroll 1
-  for (int32_t c = 0; c < n; c += 8) {
+  for (int32_t c = 8 * chunk; c < n; c += 8 * kEpiChunks) {
     float u[8], v[8];
     tmem_ld8(acc + c, u);
     tmem_ld8(acc + kMaxN / 2 + c, v);
@@ -232,12 +250,13 @@ __device__ __forceinline__ void finish_gate(const PredLaunch& L, int32_t t, int3
 }
 // P3: the tile's argmax for the row (lowest index on ties) raised into the row's key.
 __device__ __forceinline__ void finish_argmax(const PredLaunch& L, int32_t t, int32_t row, bool live,
-                                              uint32_t acc) {
+                                              uint32_t acc, int chunk, int quarter,
+                                              unsigned long long* xch) {
   const PredPhase& ph = L.ph[3];
   const int32_t f0 = t * ph.tn;
   unsigned long long key = 0;
 #pragma unroll 1
-  for (int32_t c = 0; c < ph.tn; c += 8) {
+  for (int32_t c = 8 * chunk; c < ph.tn; c += 8 * kEpiChunks) {
     float v[8];
     tmem_ld8(acc + c, v);
     float bv = v[0];
@@ -248,9 +267,13 @@ __device__ __forceinline__ void finish_argmax(const PredLaunch& L, int32_t t, in
     const unsigned long long k = argmax_key(bv, f0 + c + bi);
     if (k > key) key = k;
   }
-  if (live)
-    asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;"
-                 ::"l"(L.best + (int64_t)row * kKeyStride), "l"(key) : "memory");
+  if (chunk > 0 && live) atomicMax(&xch[row], key);
+  quarter_sync(quarter);
+  if (chunk > 0 || !live) return;
+  key = max(key, xch[row]);
+  xch[row] = 0;  // for the CTA's next tile
+  asm volatile("red.relaxed.gpu.global.max.u64 [%0], %1;"
+               ::"l"(L.best + (int64_t)row * kKeyStride), "l"(key) : "memory");
 }
 
 // The row scales s(A) = 1 / sqrt(mean(A^2) + eps) of every row from the P0
@@ -298,6 +321,8 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
   float* srow = reinterpret_cast<float*>(tmem_slot + 4);  // [128]
   unsigned char* ring = smem + 1024;
   const int S = L.stages;
+  // past the ring: the epilogue's exchange, 8 bytes per row
+  unsigned long long* xch = reinterpret_cast<unsigned long long*>(ring + (size_t)S * L.slot_bytes);
 
   const int tid = threadIdx.x, warp = (int)warp_uniform(threadIdx.x >> 5), lane = tid & 31;
   const int32_t cta = blockIdx.x;
@@ -309,7 +334,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
     }
     for (int s = 0; s < 2; ++s) {
       mbar_init(&acc_full[s], 1);
-      mbar_init(&acc_empty[s], 4);  // one arrival per epilogue warp
+      mbar_init(&acc_empty[s], kEpiThreads / 32);  // one arrival per epilogue warp
     }
     mbar_init(mma_done, 1);
     *fail = 0;
@@ -452,16 +477,17 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
     if (leader) mma_commit(mma_done);  // arrives once every MMA issued above has completed
     __syncwarp();
   } else if (warp >= kEpiWarp0) {
-    // ---- epilogue (warps 4-7): TMEM lane = row
-    const int et = tid - kEpiWarp0 * 32, quarter = warp & 3;
+    // ---- epilogue (warps 4-19): TMEM lane = row
+    const int et = tid - kEpiWarp0 * 32, quarter = warp & 3, chunk = (warp - kEpiWarp0) >> 2;
     const uint32_t lane_base = (uint32_t)(quarter * 32) << 16;
-    const int32_t row = M == 128 ? et : quarter * 16 + lane;
+    const int32_t row = quarter * (M / 4) + lane;
     const bool live = row < L.rows && (M == 128 || lane < 16);
     uint32_t tc = 0;
     bool ok = true;
 #pragma unroll 1
     for (int p = 0; p < kPhases && ok; ++p) {
       const PredPhase& pp = L.ph[p];
+      if (p == 3 && chunk == 0 && live) xch[row] = 0;  // (read again after P3's first barrier)
       if (p == 1 && cta < pp.tiles) {
         // the row scales, beside the first P1 products: once every P0 tile is
         // final (a bounded wait by one thread)
@@ -481,7 +507,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
       for (int32_t t = cta; t < pp.tiles; t += L.ncta, ++tc) {
         const uint32_t buf = tc & 1u, acc = tmem + lane_base + buf * kMaxN;
         bool stop = false;
-        if (lane == 0)
+        if (et == 0)  // (one thread polls; the others wait at the barrier)
           stop = *fail != 0 || !mbar_wait(&acc_full[buf], (tc >> 1) & 1, L.status, L.max_polls);
         if (bar_or(kBarEpi, kEpiThreads, stop)) {
           ok = false;
@@ -491,11 +517,11 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
         // (a quarter without rows has nothing to read)
         if (quarter * (M / 4) < L.rows) {
           if (p == 1)
-            finish_gate(L, t, row, live, acc, live ? srow[row] : 0.f);
+            finish_gate(L, t, row, live, acc, live ? srow[row] : 0.f, chunk);
           else if (p == 3)
-            finish_argmax(L, t, row, live, acc);
+            finish_argmax(L, t, row, live, acc, chunk, quarter, xch);
           else
-            finish_hidden(L, p, t, row, live, acc);
+            finish_hidden(L, p, t, row, live, acc, chunk, quarter, reinterpret_cast<float2*>(xch), srow);
         }
         tc_fence_before();
         __syncwarp();
@@ -578,6 +604,7 @@ PredPlan make_plan(int32_t rows, int32_t d, int32_t m, int32_t V, int32_t sm_cou
     over = std::max(over, (size_t)(q.ku / 64 - 1) * P.rpad * 128 + (size_t)P.m_rows * 128);
   }
   over = over > P.slot ? over - P.slot : 0;
+  over = std::max(over, (size_t)P.rpad * 8);  // (or the epilogue's exchange, in the same place)
   const size_t budget = 232448;  // 227 KB of dynamic shared memory per CTA
   P.stages = (int32_t)std::min<size_t>(8, (budget - 2048 - over) / P.slot);
   P.smem = 2048 + (size_t)P.stages * P.slot + over;
