@@ -728,8 +728,8 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
     // leaves idle (24 of 152 with 16384 entries: its CTAs follow one another
     // there, and what is left runs when the lm_head ends); then the counts.  The
     // attention first, beside a side stream, held the lm_head's cooperative
-    // launch up until it had ended (five 24x24 images 91.6 -> 82.3 us per step, with
-    // 512 hidden entries 49.9 -> 40.9; two 64x64 images of 4200 keys, most of whose
+    // launch up until it had ended (five 24x24 images 91.6 -> 82.3 us per step at
+    // the time, with 512 hidden entries 49.9 -> 40.9; two 64x64 images of 4200 keys, most of whose
     // attention is left when the lm_head ends, 97.9 -> 97.6).
     e = launch_fused_accept(x, y, ws + attn_ws, workspace_bytes - attn_ws, stream,
                             /*early_dependents=*/1);

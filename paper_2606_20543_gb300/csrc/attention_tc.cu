@@ -184,17 +184,6 @@ __device__ __forceinline__ uint32_t cluster_size() {
   asm("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(n));
   return n;
 }
-// Every thread of every CTA of the cluster; orders shared-memory accesses.
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// The address of this CTA's shared-memory location `saddr` in CTA `rank` of the cluster.
-__device__ __forceinline__ uint32_t peer_addr(uint32_t saddr, uint32_t rank) {
-  uint32_t a;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(saddr), "r"(rank));
-  return a;
-}
 __device__ __forceinline__ float4 ld_peer4(uint32_t a) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"

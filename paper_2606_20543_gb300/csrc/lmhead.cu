@@ -8,13 +8,14 @@
 // with the logits never written to memory.
 //
 // Design (GB300, tcgen05 + TMEM):
-//  * one CTA per tile of 128 vocabulary entries; draft rows on the MMA's M
-//    dimension (TMEM lanes, padded to 128 per row tile), vocabulary on N, so
+//  * one CTA per tile of 128 vocabulary entries, above 128 rows a pair of CTAs
+//    (cta_group::2) per two tiles; draft rows on the MMA's M
+//    dimension (TMEM lanes, padded to 128 per CTA), vocabulary on N, so
 //    each epilogue thread owns 32 of one row's 128 logits of the tile;
 //  * A = hidden states (K-major), B = weights (MN-major: the vocabulary is
 //    contiguous in W[K][V]); both staged by TMA with the 128-byte swizzle
-//    through a 3-stage mbarrier ring, two threads producing (hidden states;
-//    weights, one copy per tile through a 3D view), one thread
+//    through an mbarrier ring of units of 64 or 128 K of one head, two warps
+//    producing (hidden states; weights; one copy each per unit), one thread
 //    issuing tcgen05.mma (bf16 x bf16 -> fp32) into two TMEM accumulators
 //    (target, draft), tcgen05.commit releasing each stage;
 //  * epilogue: tcgen05.ld of each row's tile, per-tile softmax partials to a
@@ -29,7 +30,7 @@
 //    in TMEM throughout.
 // Bound: the weights' bytes (each read once) in the main loop, then a chain of
 // three grid barriers, each followed by one cold pass over a little code: 48 rows x
-// 16384 x 4096 take 56.8 us, 36 of them the loop (7.4 TB/s), 1.6 the partials, 3 to
+// 16384 x 4096 take 56.4 us (256 rows 69.6), 36 of them the loop (7.4 TB/s), 1.6 the partials, 3 to
 // 4 each the combine, the masses and the search with their barriers, and 5 the
 // cooperative launch.  Small rolled code over all 16 warps took the chain after
 // the loop from 25 to 14 us.
@@ -47,7 +48,8 @@ constexpr int kThreadsL = 512;  // 16 warps: 4 TMEM lane quarters x 4 column chu
 constexpr int kCombWarps = kThreadsL / 32;
 constexpr int kChunk = kBN / (kCombWarps / 4);  // columns of a tile per warp in the epilogues
 constexpr int kMaxTilesPerLane = 8;  // vocabulary tiles per lane in the combines: V <= 32768
-constexpr int kMaxRowTiles = 2; // rows <= 256
+constexpr int kMaxRows = 2 * kBM;
+constexpr size_t kMaxSmem = 232448;  // 227 KB
 constexpr float kLog2eL = 1.4426950408889634f;
 constexpr float kLn2L = 0.6931471805599453f;
 
@@ -59,9 +61,10 @@ struct LmPartial {  // one row, one vocabulary tile (32 bytes)
   float pad;
 };
 
-// Instruction descriptor, kind::f16: fp32 D, bf16 A and B, A K-major,
-// B MN-major, N = 128, M = 128.
+// Instruction descriptors, kind::f16: fp32 D, bf16 A and B, A K-major,
+// B MN-major; N = M = 128 in one CTA, 256 over a pair.
 constexpr uint32_t kIdesc = idesc_bf16(kBM, kBN, false, true);
+constexpr uint32_t kIdescPair = idesc_bf16(2 * kBM, 2 * kBN, false, true);
 
 __device__ __forceinline__ bool better(float v, int32_t i, float bv, int32_t bi) {
   return v > bv || (v == bv && (uint32_t)i < (uint32_t)bi);
@@ -133,17 +136,25 @@ struct LmRowRec {   // one row's combine, for every CTA after the second barrier
 };
 
 struct LmLaunch {
-  int32_t ncta, mt, stages;
+  int32_t tiles, stages;   // vocabulary tiles; ring stages
   int32_t ku;           // K per stage (64 or 128)
-  int32_t rpad;         // staged rows: the rows in swizzle groups of 8
-  LmPartial* part;      // [rows][ncta]
-  float* mass;          // [rows][ncta]
+  int32_t rpad;         // staged rows of a CTA: its rows in swizzle groups of 8
+  LmPartial* part;      // [rows][tiles]
+  float* mass;          // [rows][tiles]
   LmRowRec* rec;        // [rows] each row's decision, written by the CTA that combined it
   unsigned int* barrier;
   uint32_t max_polls;   // limit of every bounded wait of the kernel
   uint32_t shortfall;   // extra arrivals each grid barrier waits for (0; > 0 in tests)
 };
 
+// PAIR: rows above 128.  Two CTAs (a cluster) share two vocabulary tiles: each
+// stages half of the rows and one tile of weights, the pair's MMAs (M = N = 256)
+// read both CTAs' halves, and each CTA ends up with its rows' logits of both
+// tiles.  A CTA staging all rows itself was bound by what an SM takes in: 240 rows
+// and 128 columns bring 47 KB per 64 K, 49 us of copies at 64 B per clock for 4096 K
+// of both heads, a pair 32 KB per CTA (256 rows x 16384 x 4096 84.9 -> 69.6 us, 136
+// rows x 8192 x 1024 39.3 -> 34.8).
+template <bool PAIR>
 __global__ void __launch_bounds__(kThreadsL, 1)
 lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_constant__ CUtensorMap tmHd,
                      const __grid_constant__ CUtensorMap tmWt, const __grid_constant__ CUtensorMap tmWd,
@@ -152,7 +163,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   if (a.early_dependents) pdl_launch_dependents();
-  const int mt = L.mt, S = L.stages;
+  constexpr int kTiles = PAIR ? 2 : 1;  // vocabulary tiles with accumulators in this CTA
+  const int S = L.stages;
   const int a_bytes = L.rpad * L.ku * 2, w_bytes = L.ku * kBN * 2;
   const int stage_bytes = a_bytes + w_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + S * stage_bytes);
@@ -161,13 +173,16 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
   int32_t* flag = reinterpret_cast<int32_t*>(tmem_slot + 1);
   int32_t* fail = flag + 1;
-  LmSmemRow* rowinfo = reinterpret_cast<LmSmemRow*>(fail + 2);  // [mt * 128]
+  LmSmemRow* rowinfo = reinterpret_cast<LmSmemRow*>(fail + 2);  // [128]: this CTA's rows
 
   const int tid = threadIdx.x, lane = tid & 31, warp = (int)warp_uniform(tid >> 5);
-  const int cta = blockIdx.x;
-  const int32_t v0 = cta * kBN;
+  const int cta = blockIdx.x, ncta = gridDim.x;
+  const int rank = PAIR ? cta & 1 : 0;
+  const int tile0 = cta - rank;              // the tiles of its accumulators: tile0, ...
+  const int32_t row0 = rank * L.rpad;        // its rows: row0 .. row0 + nrows - 1
+  const int32_t nrows = PAIR ? max(min(L.rpad, a.rows - row0), 0) : a.rows;
   const int32_t nunits = 2 * (a.K / L.ku);  // ring units: K step u / 2 of the target (even u) or draft head
-  const uint32_t ncols = (uint32_t)(mt * 2 * kBN);  // target + draft accumulators per row tile
+  constexpr uint32_t ncols = (uint32_t)(kTiles * 2 * kBN);  // target + draft accumulators
 
   // ---- set-up: barriers, TMEM
   if (tid == 0) {
@@ -180,29 +195,35 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     fence_barrier_init();
   }
   if (warp == 0) {
-    tmem_alloc(tmem_slot, ncols);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(tmem_slot, ncols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, ncols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR) cluster_sync_all();  // (the peer's barriers too are initialised)
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
 
-  // ---- main loop: warp 0 lane 0 copies the weights, warp 2 lane 0 the hidden
-  // states, warp 1 lane 0 issues the MMAs; the other threads wait at the
-  // block's barrier (not polling beside them).  The loop is bound by the copies'
-  // issue unless there are few of them: one thread issues a copy every ~0.37 us
-  // (several lanes of a warp in one instruction ~0.17 us each), so a unit of
-  // one head takes two copies of up to 32 KB, from two warps.  With four 16 KB
-  // copies per 64 K the loop took 0.75 us per step whatever the vocabulary.
+  // ---- main loop: warp 0 copies the weights, warp 2 the hidden states, warp 1
+  // issues the MMAs (one elected lane of each, in warp-uniform loops); the other
+  // threads wait at the block's barrier (not polling beside them).  A warp issues
+  // a copy every ~0.3 us, so a unit of one head takes two copies of up to 32 KB,
+  // from two warps.
   if (warp == 0 || warp == 2) {
     const bool w = warp == 0, leader = elect_one();
     const uint64_t pol = w ? policy_evict_first()   // weights: read once
                            : policy_evict_last();   // hidden states: read by every CTA
-    int s = 0;
+    int s = 0, u = 0;
     uint32_t ph = 1;
+    // a pair's bytes are counted by its even CTA's barriers
+    const uint32_t full0 = PAIR ? peer_addr(smem_u32(full), 0) : 0;
 #pragma unroll 1
-    for (int u = 0; u < nunits; ++u) {
+    for (; u < nunits; ++u) {
       const int k0 = (u >> 1) * L.ku;
       if (u >= S && !mbar_wait_warp(&empty[s], ph, a.status, L.max_polls)) {
         *fail = 1;
@@ -211,13 +232,13 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       if (leader) {
         unsigned char* st = smem + s * stage_bytes;
         // weights: 3D view {64, K, V / 64}; hidden states: {64, rows, K / 64}
-        if (w) {
-          mbar_arrive_expect_tx(&full[s], (uint32_t)w_bytes);
-          tma_load_3d(st + a_bytes, (u & 1) ? &tmWd : &tmWt, 0, k0, v0 / 64, &full[s], pol);
-        } else {
-          mbar_arrive_expect_tx(&full[s], (uint32_t)a_bytes);
-          tma_load_3d(st, (u & 1) ? &tmHd : &tmHt, 0, 0, k0 / kBK, &full[s], pol);
-        }
+        const CUtensorMap* map = w ? ((u & 1) ? &tmWd : &tmWt) : ((u & 1) ? &tmHd : &tmHt);
+        unsigned char* dst = w ? st + a_bytes : st;
+        const int32_t c1 = w ? k0 : row0, c2 = w ? cta * (kBN / 64) : k0 / kBK;
+        if (rank == 0)
+          mbar_arrive_expect_tx(&full[s], (uint32_t)(kTiles * (w ? w_bytes : a_bytes)));
+        if constexpr (PAIR) tma_load_3d_pair(dst, map, 0, c1, c2, full0 + 8 * s, pol);
+        else tma_load_3d(dst, map, 0, c1, c2, &full[s], pol);
       }
       __syncwarp();
       if (++s == S) {
@@ -225,8 +246,15 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
         ph ^= 1u;
       }
     }
+    // after a failure: this CTA's (the pair's) copies still in flight, among the last
+    // S units, land before it goes on (the pair's other CTA waits at the end)
+    if (u < nunits && rank == 0) {
+#pragma unroll 1
+      for (int x = max(u - S, 0); x < u; ++x)
+        mbar_wait(&full[x % S], (x / S) & 1, nullptr, L.max_polls);
+    }
     __syncwarp();
-  } else if (warp == 1) {
+  } else if (warp == 1 && rank == 0) {
     const uint32_t base = warp_uniform(smem_u32(smem)), tm = warp_uniform(tmem);
     const bool leader = elect_one();
     int s = 0;
@@ -244,24 +272,22 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       // row, 64 K a [rpad][128 B] block.  (A row tile is read to 128 rows, past
       // the staged ones: those rows of the accumulators are never used.)
       const uint64_t db0 = smem_desc(st + a_bytes, L.ku * 128, 1024), da0 = smem_desc(st, 16, 1024);
-      const uint32_t d = tm + (u & 1) * kBN;
+      const uint32_t d = tm + (u & 1) * (kTiles * kBN);
       const uint32_t acc0 = u > 1 ? 1u : 0u;
       if (leader) {
 #pragma unroll 1
         for (int sub = 0; sub < L.ku / kBK; ++sub) {
           const uint64_t da = smem_desc_at(da0, sub * L.rpad * 128), db = smem_desc_at(db0, sub * 8192);
 #pragma unroll
-          for (int kk = 0; kk < kBK / kMMAK; ++kk)
-            mma_ss(d, smem_desc_at(da, kk * 32), smem_desc_at(db, kk * 2048), kIdesc,
-                   kk > 0 || sub > 0 ? 1u : acc0);
-          if (mt > 1) {
-#pragma unroll
-            for (int kk = 0; kk < kBK / kMMAK; ++kk)
-              mma_ss(d + 2 * kBN, smem_desc_at(da, kBM * 128 + kk * 32), smem_desc_at(db, kk * 2048),
-                     kIdesc, kk > 0 || sub > 0 ? 1u : acc0);
+          for (int kk = 0; kk < kBK / kMMAK; ++kk) {
+            const uint64_t dak = smem_desc_at(da, kk * 32), dbk = smem_desc_at(db, kk * 2048);
+            const uint32_t acc = kk > 0 || sub > 0 ? 1u : acc0;
+            if constexpr (PAIR) mma_ss_pair(d, dak, dbk, kIdescPair, acc);
+            else mma_ss(d, dak, dbk, kIdesc, acc);
           }
         }
-        mma_commit(&empty[s]);
+        if constexpr (PAIR) mma_commit_pair(&empty[s]);
+        else mma_commit(&empty[s]);
       }
       __syncwarp();
       if (++s == S) {
@@ -269,9 +295,16 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
         ph ^= 1u;
       }
     }
-    if (leader) mma_commit(done);
+    if (leader) {
+      if constexpr (PAIR) mma_commit_pair(done);
+      else mma_commit(done);
+    }
     // the accumulators, for every thread at the barrier below
     if (!good || !mbar_wait_warp(done, 0, a.status, L.max_polls)) *fail = 1;
+    __syncwarp();
+  }
+  if (PAIR && warp == 1 && rank == 1) {  // (issued by the even CTA)
+    if (!mbar_wait_warp(done, 0, a.status, L.max_polls)) *fail = 1;
     __syncwarp();
   }
   tc_fence_before();
@@ -286,21 +319,23 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // [32 (w / 4), + 32) of the tile, and a quarter's four warps merge their
   // chunks through shared memory (the ring's, free now).
   const int quarter = warp & 3, chunk = warp >> 2;
-  const int lrow = quarter * 32 + lane;  // row of a row tile
+  const int lrow = quarter * 32 + lane;  // of this CTA's rows
+  const int32_t row_of = row0 + lrow;
+  const bool live = lrow < nrows;
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
-  float4* chunk_part = reinterpret_cast<float4*>(smem);  // [mt][4 chunks][2][128 rows]
-  float* chunk_mass = reinterpret_cast<float*>(chunk_part + mt * 8 * kBM);  // [mt][4 chunks][128]
+  float4* chunk_part = reinterpret_cast<float4*>(smem);  // [tiles][4 chunks][2][128 rows]
+  float* chunk_mass = reinterpret_cast<float*>(chunk_part + kTiles * 8 * kBM);  // [tiles][4 chunks][128]
 
   // ---- epilogue 1: per-tile softmax partials of every row (4 warps alone took
-  // 1.7 us per row tile)
+  // 1.7 us per tile)
 #pragma unroll 1
-  for (int m = 0; m < mt && ok; ++m) {
-    const int32_t row = m * kBM + lrow;
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
+  for (int m = 0; m < kTiles && ok; ++m) {
+    const int32_t row = row_of, tile = tile0 + m;
+    const uint32_t tp = tmem + lane_off + m * kBN + chunk * kChunk, tq = tp + kTiles * kBN;
     float xq_c = -INFINITY, xp_c = 0.f;
     int32_t cand = -1;
-    const int32_t given = (a.draft_tok != nullptr && row < rows) ? a.draft_tok[row] : -1;
-    const int32_t c0 = v0 + chunk * kChunk;
+    const int32_t given = (a.draft_tok != nullptr && live) ? a.draft_tok[row] : -1;
+    const int32_t c0 = tile * kBN + chunk * kChunk;
     float v[kChunk], w[kChunk];
     tmem_ld32(tp, v);
     tmem_ld32(tq, w);
@@ -332,7 +367,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     part[(2 * chunk) * kBM] = make_float4(cmp, lp, cmq, lq);
     part[(2 * chunk + 1) * kBM] = make_float4(xq_c, xp_c, __int_as_float(cand), 0.f);
     quarter_sync(quarter);
-    if (chunk == 0 && row < rows) {
+    if (chunk == 0 && live && tile < L.tiles) {
       float mp = -INFINITY, sp = 0.f, mq = -INFINITY, sq = 0.f, xq = -INFINITY, xp = 0.f;
       int32_t t = -1;
 #pragma unroll 1
@@ -346,19 +381,19 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
           t = __float_as_int(e1.z);
         }
       }
-      float4* out = reinterpret_cast<float4*>(L.part + (int64_t)row * L.ncta + cta);
+      float4* out = reinterpret_cast<float4*>(L.part + (int64_t)row * L.tiles + tile);
       out[0] = make_float4(mp, sp, mq, sq);
       out[1] = make_float4(xq, xp, __int_as_float(t), 0.f);
     }
   }
-  ok = grid_barrier(L.barrier, (unsigned)L.ncta + L.shortfall, a.status, flag, L.max_polls) && ok;
+  ok = grid_barrier(L.barrier, (unsigned)ncta + L.shortfall, a.status, flag, L.max_polls) && ok;
 
   // ---- epilogue 2: combine the partials of each row and decide.  Row r is
   // combined by CTA r % ncta alone (one warp per row; lane l merges tiles l,
   // l + 32, ... in order, then a xor tree), which writes its outputs and its
   // record for the other CTAs.  All loads of a row are issued before any merge.
 #pragma unroll 1
-  for (int32_t row = cta + L.ncta * warp; row < rows && ok; row += L.ncta * kCombWarps) {
+  for (int32_t row = cta + ncta * warp; row < rows && ok; row += ncta * kCombWarps) {
     bool pad = false;
     if (a.n_drafts != nullptr) {
       const int32_t b = row / a.D_max, j = row - b * a.D_max;
@@ -374,12 +409,12 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       }
       continue;
     }
-    const float4* prow = reinterpret_cast<const float4*>(L.part + (int64_t)row * L.ncta);
+    const float4* prow = reinterpret_cast<const float4*>(L.part + (int64_t)row * L.tiles);
     float4 q0[kMaxTilesPerLane], q1[kMaxTilesPerLane];
 #pragma unroll
     for (int j = 0; j < kMaxTilesPerLane; ++j) {
       const int k = lane + 32 * j;
-      if (k < L.ncta) {
+      if (k < L.tiles) {
         q0[j] = __ldcg(prow + 2 * k);
         q1[j] = __ldcg(prow + 2 * k + 1);
       }
@@ -388,7 +423,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     int32_t t = 0x7fffffff;
 #pragma unroll
     for (int j = 0; j < kMaxTilesPerLane; ++j) {
-      if (lane + 32 * j < L.ncta) {
+      if (lane + 32 * j < L.tiles) {
         Mp = fmaxf(Mp, q0[j].x);
         Mq = fmaxf(Mq, q0[j].z);
         const int32_t ck = __float_as_int(q1[j].z);
@@ -406,7 +441,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     }
 #pragma unroll
     for (int j = 0; j < kMaxTilesPerLane; ++j) {
-      if (lane + 32 * j < L.ncta) {  // (a tile of -inf alone has no sum)
+      if (lane + 32 * j < L.tiles) {  // (a tile of -inf alone has no sum)
         if (q0[j].x > -INFINITY) Sp = fmaf(q0[j].y, ex2_approx((q0[j].x - Mp) * c), Sp);
         if (q0[j].z > -INFINITY) Sq = fmaf(q0[j].w, ex2_approx((q0[j].z - Mq) * c), Sq);
       }
@@ -445,21 +480,22 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       }
     }
   }
-  ok = grid_barrier(L.barrier, 2u * ((unsigned)L.ncta + L.shortfall), a.status, flag,
+  ok = grid_barrier(L.barrier, 2u * ((unsigned)ncta + L.shortfall), a.status, flag,
                     L.max_polls) && ok;
 
   // ---- the rows to draw, in every CTA: every valid rejected row, or (lazy)
   // the first rejected row of each sequence among its drafts
-  int32_t* first = reinterpret_cast<int32_t*>(rowinfo + mt * kBM);  // [rows / D_max]
+  int32_t* first = reinterpret_cast<int32_t*>(rowinfo + kBM);  // [rows / D_max]
   const bool lazy = a.lazy != 0 && a.n_drafts != nullptr;
   const int32_t ngroups = lazy ? rows / a.D_max : 0;
-  int32_t* ndraw = first + mt * kBM;     // the rows to draw, in any order, and their count
-  int32_t* drawn = ndraw + 1;            // [mt * 128]
+  int32_t* ndraw = first + kMaxRows;     // of this CTA's rows those to draw, in any order
+  int32_t* drawn = ndraw + 1;            // [128]
   if (tid == 0) *ndraw = 0;
+  if (tid < kBM) rowinfo[tid].state = 0;
   for (int32_t g = tid; g < ngroups; g += kThreadsL) first[g] = 0x7fffffff;
   // the record of a row, written by another CTA, read from L2 (at most one row
   // per thread; its state says all that the choice needs)
-  static_assert(kMaxRowTiles * kBM <= kThreadsL, "one row per thread");
+  static_assert(kMaxRows <= kThreadsL, "one row per thread");
   float4 rv = make_float4(0.f, 0.f, 0.f, 0.f);
   if (tid < rows && ok) rv = __ldcg(reinterpret_cast<const float4*>(L.rec + tid));
   const int32_t state = __float_as_int(rv.w);
@@ -467,8 +503,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   __syncthreads();
   if (lazy && state != 0) atomicMin(&first[group], tid - group * a.D_max);
   __syncthreads();
-  if (tid < mt * kBM) {
-    LmSmemRow& ri = rowinfo[tid];
+  if (tid >= row0 && tid < row0 + nrows) {
+    LmSmemRow& ri = rowinfo[tid - row0];
     const bool pick = state == 1 && (!lazy || tid - group * a.D_max == first[group]);
     ri.Cp = rv.x;
     ri.Cq = rv.y;
@@ -476,21 +512,21 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     ri.state = pick ? 1 : 0;
     ri.from_p = 0;
     ri.cstar = -1;
-    if (pick) drawn[atomicAdd(ndraw, 1)] = tid;
+    if (pick) drawn[atomicAdd(ndraw, 1)] = tid - row0;
   }
   __syncthreads();
 
   // ---- epilogue 3: residual mass of this tile for every row to draw: chunk sums
   // in vocabulary order, then their sum
 #pragma unroll 1
-  for (int m = 0; m < mt && ok; ++m) {
-    const int32_t row = m * kBM + lrow;
-    const LmSmemRow& ri = rowinfo[m * kBM + lrow];
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
+  for (int m = 0; m < kTiles && ok; ++m) {
+    const int32_t row = row_of, tile = tile0 + m;
+    const LmSmemRow& ri = rowinfo[lrow];
+    const uint32_t tp = tmem + lane_off + m * kBN + chunk * kChunk, tq = tp + kTiles * kBN;
     float mass = 0.f;
     // every lane of the warp takes part in tcgen05.ld; rows that do not draw
     // simply discard the values
-    const bool draw = row < rows && ri.state == 1;
+    const bool draw = ri.state == 1;
     if (!__any_sync(0xffffffffu, draw)) continue;  // no row of this quarter draws
     const float Cp = ri.Cp, Cq = ri.Cq;
 #pragma unroll 1
@@ -505,16 +541,16 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     float* cm = chunk_mass + m * 4 * kBM + lrow;
     cm[chunk * kBM] = mass;
     quarter_sync(quarter);
-    if (draw && chunk == 0)
-      L.mass[(int64_t)row * L.ncta + cta] = mass + cm[kBM] + cm[2 * kBM] + cm[3 * kBM];
+    if (draw && chunk == 0 && tile < L.tiles)
+      L.mass[(int64_t)row * L.tiles + tile] = mass + cm[kBM] + cm[2 * kBM] + cm[3 * kBM];
   }
-  ok = grid_barrier(L.barrier, 3u * ((unsigned)L.ncta + L.shortfall), a.status, flag,
+  ok = grid_barrier(L.barrier, 3u * ((unsigned)ncta + L.shortfall), a.status, flag,
                     L.max_polls) && ok;
 
   // ---- epilogue 4: locate the tile holding u_res * Z (warp per row; lane l
   // owns tiles [l*per, (l+1)*per) and keeps their masses in registers; the
   // same arithmetic in every CTA)
-  const int32_t per = (L.ncta + 31) / 32;  // <= kMaxTilesPerLane
+  const int32_t per = (L.tiles + 31) / 32;  // <= kMaxTilesPerLane
   // (a row takes a warp ~1.1 us: from the list, since by row number the drawn rows
   // of images of 48 rows fell to one warp, 5 us)
   if (ok) {
@@ -523,16 +559,16 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
 #pragma unroll
       for (int q = 0; q < kMaxTilesPerLane; ++q) {
         const int k = lane * per + q;
-        mk[q] = q < per && k < L.ncta && i < nd
-                    ? __ldcg(L.mass + (int64_t)drawn[i] * L.ncta + k) : 0.f;
+        mk[q] = q < per && k < L.tiles && i < nd
+                    ? __ldcg(L.mass + (int64_t)(row0 + drawn[i]) * L.tiles + k) : 0.f;
       }
     };
     float mnext[kMaxTilesPerLane];  // of the warp's next row, in flight during this one
     tile_masses(warp, mnext);
 #pragma unroll 1
     for (int32_t i = warp; i < nd; i += kCombWarps) {
-      const int32_t row = drawn[i];
-      LmSmemRow& ri = rowinfo[row];
+      const int32_t row = row0 + drawn[i];
+      LmSmemRow& ri = rowinfo[drawn[i]];
       float mk[kMaxTilesPerLane];
 #pragma unroll
       for (int q = 0; q < kMaxTilesPerLane; ++q) mk[q] = mnext[q];
@@ -544,9 +580,9 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
           for (int q = 0; q < kMaxTilesPerLane; ++q) {
             const int k = lane * per + q;
             mk[q] = 0.f;
-            if (q < per && k < L.ncta) {
+            if (q < per && k < L.tiles) {
               const float4 p0 =
-                  __ldcg(reinterpret_cast<const float4*>(L.part + (int64_t)row * L.ncta + k));
+                  __ldcg(reinterpret_cast<const float4*>(L.part + (int64_t)row * L.tiles + k));
               mk[q] = p0.y * ex2_approx(p0.x * c - ri.Cp);
             }
           }
@@ -562,7 +598,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
         }
         const float Z = __shfl_sync(0xffffffffu, incl, 31);
         if (!(Z > 0.f)) {
-          if (fp == 1 && lane == 0 && cta == 0) {
+          if (fp == 1 && lane == 0 && tile0 == 0) {
             a.out_tok[row] = -1;
             record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
           }
@@ -579,7 +615,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
           float tk = INFINITY, cum = 0.f;
 #pragma unroll
           for (int q = 0; q < kMaxTilesPerLane; ++q) {
-            if (q < per && lane * per + q < L.ncta) {
+            if (q < per && lane * per + q < L.tiles) {
               if (mk[q] > 0.f) {
                 klast = lane * per + q;
                 if (ks < 0 && cum + mk[q] > t1) { ks = klast; tk = t1 - cum; }
@@ -603,10 +639,10 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // (its chunk masses say which) in order; a row drawn from p, whose chunk
   // masses are not kept, is scanned whole by the first chunk's warp
 #pragma unroll 1
-  for (int m = 0; m < mt && ok; ++m) {
-    const int32_t row = m * kBM + lrow;
-    const LmSmemRow& ri = rowinfo[m * kBM + lrow];
-    bool mine = row < rows && ri.state == 1 && ri.cstar == cta;
+  for (int m = 0; m < kTiles && ok; ++m) {
+    const int32_t row = row_of, tile = tile0 + m;
+    const LmSmemRow& ri = rowinfo[lrow];
+    bool mine = ri.state == 1 && ri.cstar == tile;
     if (!__any_sync(0xffffffffu, mine)) continue;  // warp-uniform
     const bool from_p = ri.from_p != 0;
     float target = ri.tc;
@@ -629,7 +665,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       mine = mine && chunk == 0;
     }
     if (!__any_sync(0xffffffffu, mine)) continue;
-    const uint32_t tp = tmem + lane_off + m * 2 * kBN + chunk * kChunk, tq = tp + kBN;
+    const uint32_t tp = tmem + lane_off + m * kBN + chunk * kChunk, tq = tp + kTiles * kBN;
     const float Cp = ri.Cp, Cq = ri.Cq;
     const int end = __any_sync(0xffffffffu, mine && from_p) ? kBN : kChunk;  // (then chunk is 0)
     const int end_row = from_p ? kBN : kChunk;
@@ -649,7 +685,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
           const float wt = from_p ? pv : fmaxf(pv - ex2_approx(fmaf(w[i], c, -Cq)), 0.f);
           cum += wt;
           if (wt > 0.f) {
-            lastpos = v0 + chunk * kChunk + ch + i;
+            lastpos = tile * kBN + chunk * kChunk + ch + i;
             if (pick < 0 && cum > target) pick = lastpos;
           }
         }
@@ -662,9 +698,11 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // ---- teardown: release TMEM (all MMAs have completed: `done` fired)
   tc_fence_before();
   __syncthreads();
+  if constexpr (PAIR) cluster_sync_all();  // (no copy or MMA of the pair is left)
   if (warp == 0) {
     tc_fence_after();
-    tmem_dealloc(tmem, ncols);
+    if constexpr (PAIR) tmem_dealloc_pair(tmem, ncols);
+    else tmem_dealloc(tmem, ncols);
   }
 }
 
@@ -689,25 +727,34 @@ bool make_weight_map(CUtensorMap* map, const void* base, uint64_t V, uint64_t K,
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
 
-int row_tiles(int32_t rows) { return (rows + kBM - 1) / kBM; }
-
-// Staged rows, and K per ring unit: 128 while a unit of all rows leaves room for
-// three stages (fewer, larger copies), else 64.
-int staged_rows(int32_t rows) { return (rows + 7) / 8 * 8; }
-int unit_k(int32_t rows, int32_t K) { return rows <= kBM && K % 128 == 0 ? 128 : kBK; }
-
+// Rows above one row tile run on CTA pairs, half of the rows (in swizzle groups of
+// 8) in each CTA.
+bool row_pairs(int32_t rows) { return rows > kBM; }
+int staged_rows(int32_t rows) { return ((row_pairs(rows) ? (rows + 1) / 2 : rows) + 7) / 8 * 8; }
+// CTAs of a launch: one per vocabulary tile, whole pairs.
+int32_t lm_ctas(int32_t rows, int32_t V) {
+  const int32_t tiles = V / kBN;
+  return row_pairs(rows) ? (tiles + 1) / 2 * 2 : tiles;
+}
 size_t smem_bytes(int32_t rows, int ku, int stages) {
-  const int mt = row_tiles(rows);
   // + the first rejected draft of each sequence (at most one per row), and the
   // list of the rows to draw
   return 1024 + (size_t)stages * (staged_rows(rows) + kBN) * ku * 2 + (2 * stages + 1) * 8 + 16 +
-         (size_t)mt * kBM * sizeof(LmSmemRow) + (size_t)(2 * mt * kBM + 1) * sizeof(int32_t);
+         (size_t)kBM * sizeof(LmSmemRow) + (size_t)(kMaxRows + 1 + kBM) * sizeof(int32_t);
+}
+
+// K per ring unit: 128 (fewer, larger copies) where it divides K and leaves four
+// stages (up to 88 staged rows), else 64.  With three stages of 128 too little is
+// in flight: 128 rows x 16384 x 4096 66.2 us against 64.1 with 64, 80 rows 59.7 and
+// 59.3; 48 rows x 2048 x 4096 42.1 against 47.3.
+int unit_k(int32_t rows, int32_t K) {
+  return K % 128 == 0 && smem_bytes(rows, 128, 4) <= kMaxSmem ? 128 : kBK;
 }
 
 // As many stages as the shared memory holds, at most 8.
 int stages_for(int32_t rows, int ku) {
   int s = 8;
-  while (s > 2 && smem_bytes(rows, ku, s) > 232448) --s;
+  while (s > 2 && smem_bytes(rows, ku, s) > kMaxSmem) --s;
   return s;
 }
 
@@ -720,7 +767,7 @@ size_t lmhead_workspace(int32_t rows, int32_t V) {
 }
 
 ssd_status lmhead_check(int32_t rows, int32_t V, int32_t K) {
-  if (rows < 1 || rows > kMaxRowTiles * kBM) return SSD_ERR_UNSUPPORTED;
+  if (rows < 1 || rows > kMaxRows) return SSD_ERR_UNSUPPORTED;
   if (K <= 0 || K % kBK != 0) return SSD_ERR_UNSUPPORTED;
   if (V <= 0 || V % kBN != 0) return SSD_ERR_UNSUPPORTED;
   if (V / kBN > 32 * kMaxTilesPerLane) return SSD_ERR_UNSUPPORTED;
@@ -728,22 +775,23 @@ ssd_status lmhead_check(int32_t rows, int32_t V, int32_t K) {
   int per_sm = 0;
   const int ku = unit_k(rows, K);
   const size_t smem = smem_bytes(rows, ku, stages_for(rows, ku));
-  if (cudaFuncSetAttribute(lmhead_accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem) != cudaSuccess)
+  auto occupancy = [&](auto kernel) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+               cudaSuccess &&
+           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreadsL, smem) ==
+               cudaSuccess;
+  };
+  if (!(row_pairs(rows) ? occupancy(lmhead_accept_kernel<true>)
+                        : occupancy(lmhead_accept_kernel<false>)))
     return SSD_ERR_CUDA;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, lmhead_accept_kernel, kThreadsL,
-                                                    smem) != cudaSuccess)
-    return SSD_ERR_CUDA;
-  if ((int64_t)(V / kBN) > (int64_t)per_sm * device_sm_count()) return SSD_ERR_UNSUPPORTED;
+  if ((int64_t)lm_ctas(rows, V) > (int64_t)per_sm * device_sm_count()) return SSD_ERR_UNSUPPORTED;
   return SSD_OK;
 }
 
 cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream) {
   if (a.rows == 0) return cudaSuccess;
-  const int mt = row_tiles(a.rows);
   LmLaunch L;
-  L.ncta = a.V / kBN;
-  L.mt = mt;
+  L.tiles = a.V / kBN;
   L.ku = unit_k(a.rows, a.K);
   L.rpad = staged_rows(a.rows);
   L.stages = stages_for(a.rows, L.ku);
@@ -753,9 +801,9 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
   L.barrier = reinterpret_cast<unsigned int*>(w);  // [0] arrivals, [1] abort flag
   w += al256(2 * sizeof(unsigned int));
   L.part = reinterpret_cast<LmPartial*>(w);
-  w += al256((size_t)a.rows * L.ncta * sizeof(LmPartial));
+  w += al256((size_t)a.rows * L.tiles * sizeof(LmPartial));
   L.mass = reinterpret_cast<float*>(w);
-  w += al256((size_t)a.rows * L.ncta * sizeof(float));
+  w += al256((size_t)a.rows * L.tiles * sizeof(float));
   L.rec = reinterpret_cast<LmRowRec*>(w);
   CUtensorMap ht, hd, wt, wd;
   const uint32_t ku = (uint32_t)L.ku, rpad = (uint32_t)L.rpad;
@@ -770,20 +818,26 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
     if (e != cudaSuccess) return e;
   }
   const size_t smem = smem_bytes(a.rows, L.ku, L.stages);
-  e = cudaFuncSetAttribute(lmhead_accept_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)smem);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)L.ncta, 1, 1);
-  cfg.blockDim = dim3(kThreadsL, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeCooperative;
-  attr[0].val.cooperative = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, lmhead_accept_kernel, ht, hd, wt, wd, a, L);
+  const bool pair = row_pairs(a.rows);
+  auto launch = [&](auto kernel) {
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)lm_ctas(a.rows, a.V), 1, 1);
+    cfg.blockDim = dim3(kThreadsL, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pair ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, ht, hd, wt, wd, a, L);
+  };
+  return pair ? launch(lmhead_accept_kernel<true>) : launch(lmhead_accept_kernel<false>);
 }
 
 }  // namespace ssd

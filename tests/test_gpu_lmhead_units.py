@@ -15,9 +15,10 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("rows,K,V", [
     (1, 64, 128),      # one unit of 64 K, one CTA, one staged group of 8 rows
     (41, 192, 384),    # K not a multiple of 128: units of 64; a ragged row group, three CTAs
-    (128, 384, 512),   # the most rows of 128-K units, an odd number of them
-    (129, 384, 512),   # the fewest of two row tiles: units of 64
-    (256, 128, 640),   # the most rows; five CTAs
+    (88, 384, 512),    # the most rows of 128-K units, an odd number of them
+    (128, 384, 512),   # the most rows of one CTA
+    (129, 384, 512),   # the fewest on CTA pairs
+    (256, 128, 640),   # the most rows; five tiles, the third pair half empty
 ])
 def test_unit_shapes_match_oracle(ssd, rows, K, V):  # noqa: F811
     ht, hd, wt, wd, u = make_inputs(rows, K, V, 60 + rows, 0.1)
@@ -76,3 +77,21 @@ def test_fused_step_is_its_parts(ssd, side, lens, V, hidden):  # noqa: F811
     for k in first:
         assert np.array_equal(first[k], parts[k]), k
         assert np.array_equal(first[k], replayed[k]), k
+
+
+def test_pair_gives_up_and_the_context_stays_usable(ssd):  # noqa: F811
+    """CTA pairs leave together when a grid barrier runs out."""
+    rows, K, V = 160, 256, 1024
+    ht, hd, wt, wd, u = make_inputs(rows, K, V, 23, 0.05)
+    ssd.ssd_set_wait_limit(1 << 12)
+    ssd.ssd_set_barrier_shortfall(1)
+    try:
+        tok, acc, _, _, st = run_fused(ssd, ht, hd, wt, wd, u)
+    finally:
+        ssd.ssd_set_barrier_shortfall(0)
+        ssd.ssd_set_wait_limit(0)
+    assert st == 5 and np.all(tok == -7) and np.all(acc == 7)  # SSD_ERR_TIMEOUT, nothing written
+    tok, acc, ratio, lse, st = run_fused(ssd, ht, hd, wt, wd, u)
+    assert st == 0
+    ref = olm.lmhead_accept(bf16_to_f64(ht), bf16_to_f64(hd), bf16_to_f64(wt), bf16_to_f64(wd), u)
+    compare_decisions(ref, tok, acc, ratio, lse, what="pair after a timeout", tol=FUSED_PROB_TOL)
