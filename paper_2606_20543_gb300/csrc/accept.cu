@@ -285,6 +285,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
     fence_barrier_init();
   }
   __syncthreads();
+  // (the dependent reads none of this kernel's results, but what precedes it must be
+  // complete for it too)
+  pdl_wait();
   if (a.early_dependents) pdl_launch_dependents();
 
   // (A) never draws and lazy (C) leaves its draws to launch_resolve: one pass
@@ -698,6 +701,7 @@ __device__ __forceinline__ void resolve_part_masses(const float4* tp, const floa
 
 __global__ void __launch_bounds__(32, 32) resolve_kernel(ResolveArgs a) {
   extern __shared__ __align__(16) float rmass[];  // [nblocks], last part only
+  if (a.wait) pdl_wait();
   const int32_t part = blockIdx.x, b = blockIdx.y, lane = threadIdx.x;
   const int32_t nblocks = ((a.V + kChunk - 1) / kChunk) * kBlocksPerChunk;  // resolve_blocks(V)
   const int32_t nv = a.V >> 2;
@@ -816,8 +820,7 @@ cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    kernel<<<(unsigned)grid, kThreads, smem, stream>>>(a);
-    return cudaGetLastError();
+    return launch_kernel(kernel, dim3((unsigned)grid), dim3(kThreads), smem, stream, /*pdl=*/true, a);
   };
   switch (a.strategy) {
     case SSD_STRATEGY_GREEDY: return launch(accept_kernel<SSD_STRATEGY_GREEDY, false>);
@@ -830,13 +833,15 @@ cudaError_t launch_accept(const AcceptArgs& a, cudaStream_t stream) {
 
 int32_t resolve_blocks(int32_t V) { return ((V + kChunk - 1) / kChunk) * kBlocksPerChunk; }
 
-cudaError_t launch_resolve(const ResolveArgs& a, bool pdl, cudaStream_t stream) {
-  if (a.B == 0) return cudaSuccess;
+cudaError_t launch_resolve(const ResolveArgs& a_, bool pdl, cudaStream_t stream) {
+  if (a_.B == 0) return cudaSuccess;
+  ResolveArgs a = a_;
+  a.wait = pdl ? 0 : 1;
   const int32_t nblocks = resolve_blocks(a.V);
   const size_t smem = (size_t)nblocks * sizeof(float);
   static_assert(kMaxV / 256 * sizeof(float) <= 48 * 1024, "within the default shared memory limit");
   const dim3 grid((unsigned)((nblocks + kRBlocks - 1) / kRBlocks), (unsigned)a.B);
-  return launch_kernel(resolve_kernel, grid, dim3(32), smem, stream, pdl, a);
+  return launch_kernel(resolve_kernel, grid, dim3(32), smem, stream, /*pdl=*/true, a);
 }
 
 }  // namespace ssd

@@ -317,6 +317,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     pdl_launch_dependents();
     return;
   }
+  if (L.order == 0) pdl_wait();  // on its own: what precedes it is complete
   pdl_launch_dependents();
   const int32_t cta = (int32_t)blockIdx.x - L.order, ncta = (int32_t)gridDim.x - L.order;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -1211,7 +1212,7 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
     const int64_t clusters = std::min<int64_t>(n_items, resident_clusters(kernel, smem));
     L.order = pdl ? kCluster : 0;
     return launch_clusters(kernel, dim3((unsigned)(clusters * kCluster + L.order)),
-                           dim3(kThreadsTC), smem, stream, pdl, kCluster, tq, tk, tv, a, L);
+                           dim3(kThreadsTC), smem, stream, /*pdl=*/true, kCluster, tq, tk, tv, a, L);
   };
   if (a.d == 128)
     return bm == 64 ? launch(frontier_attn_tc_kernel<128, 64>, tc_smem_bytes<128, 64>())

@@ -814,7 +814,7 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
     return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
   if (!a.counters_zeroed) {
-    e = cudaMemsetAsync(L.barrier, 0, kLmheadCounters * sizeof(unsigned int), stream);
+    e = launch_zero(L.barrier, kLmheadCounters, stream);
     if (e != cudaSuccess) return e;
   }
   const size_t smem = smem_bytes(a.rows, L.ku, L.stages);

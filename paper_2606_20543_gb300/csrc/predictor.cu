@@ -698,7 +698,7 @@ cudaError_t launch_rows(const PredictorArgs& a, void* ws, size_t ws_bytes, int32
       map(&tag, w.ag, R, d, P.rpad, q[1].ku / 64) && map(&tg, w.g, R, m, P.rpad, q[2].ku / 64) &&
       map(&thg, w.ag, R, d, P.rpad, q[3].ku / 64);
   if (!ok) return cudaErrorInvalidValue;
-  cudaError_t e = cudaMemsetAsync(w.ctr, 0, w.zero_bytes, stream);
+  cudaError_t e = launch_zero(w.ctr, (int32_t)(w.zero_bytes / 4), stream);
   if (e != cudaSuccess) return e;
   auto launch = [&](auto kernel) {
     cudaError_t err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
