@@ -864,7 +864,7 @@ def run_predictor(a, world, rank, dev, torch, ssd):
         "call_us_l2_flushed": flushed_ms * 1000.0,
         "e2e": {"value": world * 1000.0 / e2e_ms, "unit": "draft predictor calls/s",
                 "h2d_bytes_per_step": rows * 2 * d * 2, "d2h_bytes_per_step": rows * 4},
-        "gpu_launches": -(-rows // 128) * calls,  # one predictor kernel per 128 rows
+        "gpu_launches": 2 * -(-rows // 128) * calls,  # the counters' clearing and the predictor per 128 rows
         "device_status": int(st.item()), "cpu_baseline": cpu,
     }
     print(json.dumps(line))
