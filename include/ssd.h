@@ -15,7 +15,8 @@
  *    every buffer; the library allocates nothing on these paths.  Workspace,
  *    where needed, is sized by the matching *_workspace() query and passed in.
  *  - All work is enqueued asynchronously on `stream` (NULL = the legacy
- *    default stream).  Nothing synchronises.
+ *    default stream).  Nothing synchronises.  Kernels are launched as
+ *    programmatic dependents that wait for what precedes them on the stream.
  *  - Host-side checks (null pointers, unsupported shapes, too little
  *    workspace) return a status synchronously and enqueue nothing.
  *    SSD_ERR_CUDA reports a failed launch (cudaGetLastError).
@@ -147,7 +148,8 @@ ssd_status ssd_frontier(const ssd_grid* grid, int32_t B, const int32_t* cache_le
  *   lse        dev float32 [B][Hq][D_max] or NULL: log-sum-exp of the
  *              scaled scores (natural log)
  *   workspace  dev, >= ssd_verify_attention_workspace(...) bytes (split-KV
- *              partials and the schedule); may be NULL if that is 0.
+ *              partials above 128 query heads per KV head); may be NULL if
+ *              that is 0.
  * Supported: d in {64, 128}; Hq % Hkv == 0; 1 <= D_max <= 128;
  * D_max * (Hq / Hkv) <= 512.  Device errors: a draft position outside the
  * grid or a key count above L_max -> DEVICE_BOUNDS (rows left untouched).

@@ -9,14 +9,14 @@
 // clusters of kCluster, that walks work items (sequence, KV head, tile of 128
 // query rows = drafts x the Hq/Hkv heads sharing the KV head, up to 128 heads;
 // 64-row tiles with M = 64 products when a KV head's query rows fit in 64).
-// The horizontal stage's 6 rows per head run here too (20 images: 28.9 -> 20.7
-// us per step against the mma.sync kernel).  The kernel is
+// The horizontal stage's 6 rows per head run here too (20 images: 28.9 -> 17.8
+// us per step, 20.7 of it with this kernel in the mma.sync one's place).  The kernel is
 // bound by the K/V stream when its items fill the GPU and by the serial chain
 // of one item (load, S, softmax, PV per tile) when they do not, hence:
 //  * two CTAs per SM: one CTA's start-up, item boundaries and tile chain
 //    overlap the other's (one 202 KB CTA per SM with 128-key tiles before: the
 //    24x24 sweep's step 62.6 us, the 16 x 32x32 GQA step 51.6 us, 8 x 64x64 at
-//    2300-3800 keys 75.5 us; now 49.4, 40.9 and 73.2 us, the last 5.75 TB/s);
+//    2300-3800 keys 75.5 us; now 46.4, 34.8 and 69.2 us, the last 6.1 TB/s);
 //  * the producer warp alone sets up, plans and issues its first item's five
 //    copies, a lane each in one instruction, before the block's barrier.  What
 //    an SM waits for between that and the first P is instruction fetch once
@@ -31,7 +31,7 @@
 //    streaming a part of its keys, and merge their partial rows through
 //    distributed shared memory at the end: no partials in global memory and
 //    no second kernel (one image left of 8 x 64x64: the attention 40 -> 27 us;
-//    two rounds on 8 x 24x24: 86.5 -> 67.8 us with no combine launch).
+//    two rounds on 8 x 24x24: 86.5 -> 67.8 us at the time with no combine launch).
 //  * warp 4 (producer): decodes the next item, checks and converts its draft
 //    positions into an item slot (two slots), loads Q through a 3D tensor map
 //    and the item's K tiles of 64 keys; warp 5 streams its V tiles (TMA,

@@ -93,10 +93,6 @@ __device__ __forceinline__ void fence_barrier_init() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-__device__ __forceinline__ void fence_proxy_async() {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-}
-
 __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)),
                "r"(bytes)
@@ -151,39 +147,6 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, i
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, max_polls)) != 0;
 }
 
-__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n"
-      " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait on two mbarrier phases at once.  A poll of an mbarrier takes a
-// few hundred cycles even when the phase is long complete; both polls are
-// issued back to back so their latencies overlap.
-__device__ __forceinline__ bool mbar_wait2(uint64_t* bar1, uint32_t parity1, uint64_t* bar2,
-                                           uint32_t parity2, int32_t* status) {
-  bool done1 = false, done2 = false;
-  for (uint32_t i = 0; i < kMaxPolls; ++i) {
-    const bool t1 = done1 || mbar_test_wait(bar1, parity1);
-    const bool t2 = done2 || mbar_test_wait(bar2, parity2);
-    done1 = t1;
-    done2 = t2;
-    if (done1 && done2) return true;
-    if (i > 4096) {
-      __nanosleep(128);
-      if (give_up(i, status)) return false;
-    }
-  }
-  record_status(status, SSD_ERR_TIMEOUT);
-  return false;
-}
-
 // ------------------------------------------------------------- bulk copies
 // Untiled bulk copy global -> shared (TMA engine); both addresses 16-byte
 // aligned, bytes a multiple of 16.  Completion is signalled on `bar`.
@@ -193,16 +156,6 @@ __device__ __forceinline__ void bulk_g2s_at(uint32_t smem_dst, const void* gmem_
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
           smem_dst),
       "l"(gmem_src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-// Untiled bulk copy global -> shared with an L2 cache policy.
-__device__ __forceinline__ void bulk_g2s_hint(void* smem_dst, const void* gmem_src, uint32_t bytes,
-                                              uint64_t* bar, uint64_t policy) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint"
-      " [%0], [%1], %2, [%3], %4;" ::"r"(smem_u32(smem_dst)),
-      "l"(gmem_src), "r"(bytes), "r"(smem_u32(bar)), "l"(policy)
       : "memory");
 }
 
@@ -476,12 +429,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t*>(&v);
-}
-
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-  return v;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

@@ -34,8 +34,8 @@ __device__ __forceinline__ int32_t frontier_drafts(const ssd_grid& g, int32_t ca
 // before it on `stream` (cudaLaunchAttributeProgrammaticStreamSerialization).
 // Every kernel but the cooperative ones and the mma.sync attention is launched so.
 // Unless a schedule of several kernels orders it otherwise, it waits (pdl_wait)
-// before its first access to global memory and lets nothing after it start early,
-// so the order of the stream holds, while its CTAs are in place when the kernel
+// before its first access to global memory (and only the attention lets what follows
+// be scheduled early, which waits in its turn), so the order of the stream holds, while its CTAs are in place when the kernel
 // before it ends: back to back, a 24x24 step takes 11.8 us instead of 14.4, five
 // drafts of 20 images 18.2 for 20.5, an acceptance of 1024 rows x 65536 85.2 for
 // 89.9.  (Letting the next call's kernels in before the last draws were done saved
@@ -90,9 +90,9 @@ cudaError_t launch_frontier(const ssd_grid& g, int32_t B, const int32_t* cache_l
                             int32_t n_zero = 0);
 // Clears n words.
 cudaError_t launch_zero(unsigned int* p, int32_t n, cudaStream_t stream);
-// pdl: launched as a programmatic dependent of the kernel before it on the
-// stream (it may start while that kernel runs, needs none of its results and
-// waits for it before exiting, so stream order is kept).
+// pdl: in a step, after the attention: it may run beside that kernel, needs none of
+// its results and waits for it before exiting, so stream order is kept.  Otherwise it
+// waits for the kernel before it first.
 cudaError_t launch_counts(const ssd_grid& g, int32_t commit, int32_t B, int32_t D_max,
                           const int32_t* cache_len, const int32_t* n_drafts,
                           const uint8_t* accepted, int32_t* accepted_count,
