@@ -82,10 +82,14 @@ constexpr int kCtasPerSmTC = 2;   // 2 x 256 TMEM columns, 2 x ~107 KB of shared
 #define SSD_ATTN_CLUSTER 4
 #endif
 constexpr int kCluster = SSD_ATTN_CLUSTER;  // CTAs that can share one item
-// Fewest key tiles of a part of the longest item: merging parts takes ~3 us, a
-// tile 0.3-0.5 us (two rounds on 8 x 24x24, at most 11 tiles: 59.5 us with parts
-// of a tile or more, 51.6 whole; 16x16, 4 tiles: 12.3 and 12.0 us).
-constexpr int kMinTiles = 8;
+// Fewest key tiles of a part of the longest item, with 4 and with 2 parts, while every
+// part has an SM to itself (few) and beyond that (many): merging parts takes ~3 us
+// and a tile 0.3-0.5 us, and the parts of items that fill the SMs anyway only share
+// them.  With 8 throughout: one 32x32 GQA image (17 tiles, 16 items) 16.4 us per
+// step in 2 parts, 13.2 in 4; six of them (96 items) 24.4 in 2 parts, 22.6 whole; one
+// 48x48 image 16.0 and 13.0.  With 4 throughout two rounds on 8 x 24x24 (11 tiles,
+// 128 items) took 55.8 us, whole 47.8, and one 24x24 image 11.9 and 11.7.
+constexpr int kFew4 = 4, kMany4 = 8, kFew2 = 8, kMany2 = 12;
 constexpr float kLog2eTC = 1.4426950408889634f;
 constexpr float kRescale = 8.0f;  // log2 growth of the running max that forces a rescale
 
@@ -205,6 +209,7 @@ struct TcLaunch {
   int32_t mtiles;    // query tiles of a KV head with D_max drafts
   int32_t drafts;    // drafts per query tile (BM / G): its rows are drafts * G <= BM
   int32_t order;     // leading CTAs that only order the launches (programmatic launch), else 0
+  int32_t sms;       // of the device
   int32_t q_copies;  // copies per Q tile: 1, or one per 64 columns if the tile has fewer than BM rows
 };
 
@@ -452,9 +457,12 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     n_items = planned ? s_plan[0] : a.B * per_b;
     if (planned) {
       const int32_t cs = (int32_t)cluster_size(), most_tiles = (s_plan[1] + KTC - 1) / KTC;
-      while ((2 << ns_log) <= cs && ((2 << ns_log) * n_items) <= ncta &&
-             (2 << ns_log) * kMinTiles <= most_tiles)
-        ++ns_log;
+      auto fits = [&](int parts, int few, int many) {
+        const int n = parts * n_items;
+        return parts <= cs && n <= ncta && most_tiles >= parts * (n <= L.sms ? few : many);
+      };
+      if (fits(4, kFew4, kMany4)) ns_log = 2;
+      else if (fits(2, kFew2, kMany2)) ns_log = 1;
     }
   };
   uint32_t tmem = 0, tS = 0, tO = 0;
@@ -1186,6 +1194,7 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
   // a copy per block, so that every block starts on a swizzle atom (the rows
   // past it are never read back).
   TcLaunch L;
+  L.sms = device_sm_count();
   L.drafts = bm / G;
   L.mtiles = (a.D_max + L.drafts - 1) / L.drafts;
   L.q_copies = bm % G == 0 ? 1 : (int32_t)halves;

@@ -20,6 +20,13 @@ pytestmark = pytest.mark.gpu
     ("tail_gqa", 8, (32, 8), 128, 32, 64, [64 + 1024] * 5 + [64 + 300, 64 + 1024, 64 + 31 * 32 + 4]),
     # exactly as many live items as half the CTAs and fewer: 2 CTAs per item
     ("two_way", 8, (16, 16), 128, 24, 120, [120 + 72 * k for k in range(8)]),
+    # 16 items of 17 tiles: 4 parts, of 4 tiles and one of 5
+    ("four_short_parts", 1, (16, 16), 128, 32, 64, [64 + 975]),
+    # 48 items of 16 and 17 tiles: 2 parts of 8 (4 would not have an SM each)
+    ("two_parts_of_8", 3, (16, 16), 128, 32, 64, [64 + 940, 64 + 930, 64 + 960]),
+    # 96 items of 24 tiles: 2 parts of 12 beyond one CTA per SM, where 23 stay whole
+    ("two_parts_of_12", 6, (16, 16), 128, 40, 64, [64 + 1420] * 6),
+    ("whole_below_12", 6, (16, 16), 128, 40, 64, [64 + 1320] * 6),
     # more than 32 sequences: planned by the block (empty frontiers among them)
     ("block_plan", 40, (4, 4), 64, 16, 7, [7 + (37 * k) % 257 for k in range(40)]),
     # 3 and 20 query heads per KV head: tiles of 126 and 120 rows (42 and 6 drafts),
