@@ -30,10 +30,10 @@
 //    in TMEM throughout.
 // Bound: the weights' bytes (each read once) in the main loop, then a chain of
 // three grid barriers, each followed by one cold pass over a little code: 48 rows x
-// 16384 x 4096 take 56.4 us (256 rows 69.6), 36 of them the loop (7.4 TB/s), 1.6 the partials, 3 to
-// 4 each the combine, the masses and the search with their barriers, and 5 the
-// cooperative launch.  Small rolled code over all 16 warps took the chain after
-// the loop from 25 to 14 us.
+// 16384 x 4096 take 53.4 us (256 rows 69), 36 of them the loop (7.4 TB/s), 1.4 the
+// partials, 2 to 4 each the combine, the masses and the search with their barriers,
+// and 5 the launches.  Small rolled code over all 16 warps took the chain after the
+// loop from 25 to 12 us.
 #include "kernels.cuh"
 
 namespace ssd {
@@ -394,6 +394,19 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // record for the other CTAs.  All loads of a row are issued before any merge.
 #pragma unroll 1
   for (int32_t row = cta + ncta * warp; row < rows && ok; row += ncta * kCombWarps) {
+    const float4* prow = reinterpret_cast<const float4*>(L.part + (int64_t)row * L.tiles);
+    float4 q0[kMaxTilesPerLane], q1[kMaxTilesPerLane];
+#pragma unroll
+    for (int j = 0; j < kMaxTilesPerLane; ++j) {
+      const int k = lane + 32 * j;
+      if (k < L.tiles) {
+        q0[j] = __ldcg(prow + 2 * k);
+        q1[j] = __ldcg(prow + 2 * k + 1);
+      }
+    }
+    // (with the partials in flight)
+    const int32_t given = a.draft_tok != nullptr ? a.draft_tok[row] : -1;
+    const float2 u = row_uniforms(a.rng, row);
     bool pad = false;
     if (a.n_drafts != nullptr) {
       const int32_t b = row / a.D_max, j = row - b * a.D_max;
@@ -408,16 +421,6 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
         if (a.lse) { a.lse[2 * row] = 0.f; a.lse[2 * row + 1] = 0.f; }
       }
       continue;
-    }
-    const float4* prow = reinterpret_cast<const float4*>(L.part + (int64_t)row * L.tiles);
-    float4 q0[kMaxTilesPerLane], q1[kMaxTilesPerLane];
-#pragma unroll
-    for (int j = 0; j < kMaxTilesPerLane; ++j) {
-      const int k = lane + 32 * j;
-      if (k < L.tiles) {
-        q0[j] = __ldcg(prow + 2 * k);
-        q1[j] = __ldcg(prow + 2 * k + 1);
-      }
     }
     float Mp = -INFINITY, Sp = 0.f, Mq = -INFINITY, Sq = 0.f, xq = -INFINITY, xp = 0.f;
     int32_t t = 0x7fffffff;
@@ -452,11 +455,9 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       Sq += __shfl_xor_sync(0xffffffffu, Sq, o);
     }
     if (lane == 0) {
-      const int32_t given = a.draft_tok != nullptr ? a.draft_tok[row] : -1;
       const bool valid_t = (t >= 0 && t < a.V) && (given < 0 || t == given);
       float ratio = 0.f;
       bool acc = false;
-      const float2 u = row_uniforms(a.rng, row);
       if (valid_t) {
         const float l2p = (xp - Mp) * c - log2f(Sp);
         const float l2q = (xq - Mq) * c - log2f(Sq);
@@ -547,90 +548,105 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   ok = grid_barrier(L.barrier, 3u * ((unsigned)ncta + L.shortfall), a.status, flag,
                     L.max_polls) && ok;
 
-  // ---- epilogue 4: locate the tile holding u_res * Z (warp per row; lane l
-  // owns tiles [l*per, (l+1)*per) and keeps their masses in registers; the
-  // same arithmetic in every CTA)
-  const int32_t per = (L.tiles + 31) / 32;  // <= kMaxTilesPerLane
-  // (a row takes a warp ~1.1 us: from the list, since by row number the drawn rows
-  // of images of 48 rows fell to one warp, 5 us)
+  // ---- epilogue 4: locate the tile holding u_res * Z: half a warp per row up to 128
+  // tiles, else a warp; lane l of the row's lanes owns tiles [l*per, (l+1)*per) and
+  // keeps their masses in registers; the same arithmetic in every CTA.  (The rows come
+  // from the list: by row number the drawn rows of images of 48 rows fell to one
+  // warp, 5 us.  The pass is bound by its instructions, ~1 us for 16 warps, so 47 drawn
+  // rows took 3.4 us at a warp each.)
   if (ok) {
     const int32_t nd = *ndraw;
+    const int W = L.tiles <= 16 * kMaxTilesPerLane ? 16 : 32;
+    const int seg0 = lane & ~(W - 1), sl = lane & (W - 1);
+    const uint32_t seg_mask = W == 32 ? 0xffffffffu : 0xffffu << seg0;
+    const int32_t most = (L.tiles + W - 1) / W, per = most <= 2 ? most : most <= 4 ? 4 : 8;
+    static_assert(kMaxTilesPerLane == 8, "two 16-byte loads per lane");
+    const int32_t k0 = sl * per, own = min(per, L.tiles - k0);  // (own <= 0: none)
+    const bool vec = per >= 4 && L.tiles % 4 == 0;
     auto tile_masses = [&](int32_t i, float* mk) {
+      const int32_t n = i < nd ? own : 0;
+      const float* m = L.mass + (int64_t)(row0 + (i < nd ? drawn[i] : 0)) * L.tiles + k0;
+      if (vec) {
+        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        const float4 x = n > 0 ? __ldcg(reinterpret_cast<const float4*>(m)) : z;
+        const float4 y = n > 4 ? __ldcg(reinterpret_cast<const float4*>(m) + 1) : z;
+        mk[0] = x.x; mk[1] = x.y; mk[2] = x.z; mk[3] = x.w;
+        mk[4] = y.x; mk[5] = y.y; mk[6] = y.z; mk[7] = y.w;
+      } else {
 #pragma unroll
-      for (int q = 0; q < kMaxTilesPerLane; ++q) {
-        const int k = lane * per + q;
-        mk[q] = q < per && k < L.tiles && i < nd
-                    ? __ldcg(L.mass + (int64_t)(row0 + drawn[i]) * L.tiles + k) : 0.f;
+        for (int q = 0; q < kMaxTilesPerLane; ++q) mk[q] = q < n ? __ldcg(m + q) : 0.f;
       }
     };
-    float mnext[kMaxTilesPerLane];  // of the warp's next row, in flight during this one
-    tile_masses(warp, mnext);
+    const int32_t step = kCombWarps * (32 / W), i00 = warp * (32 / W);
+    float mnext[kMaxTilesPerLane];  // of the lane's next row, in flight during this one
+    tile_masses(i00 + seg0 / W, mnext);
 #pragma unroll 1
-    for (int32_t i = warp; i < nd; i += kCombWarps) {
-      const int32_t row = row0 + drawn[i];
-      LmSmemRow& ri = rowinfo[drawn[i]];
-      float mk[kMaxTilesPerLane];
+    for (int32_t i0 = i00; i0 < nd; i0 += step) {  // warp-uniform
+      const int32_t i = i0 + seg0 / W;
+      const bool valid = i < nd;
+      LmSmemRow& ri = rowinfo[drawn[valid ? i : i0]];
+      float mk[kMaxTilesPerLane], ls, incl, Z;
 #pragma unroll
       for (int q = 0; q < kMaxTilesPerLane; ++q) mk[q] = mnext[q];
-      tile_masses(i + kCombWarps, mnext);
+      tile_masses(i + step, mnext);
+      auto scan = [&]() {
+        ls = 0.f;
+#pragma unroll
+        for (int q = 0; q < kMaxTilesPerLane; ++q) ls += mk[q];
+        incl = ls;
 #pragma unroll 1
-      for (int fp = 0; fp < 2; ++fp) {
-        if (fp == 1) {  // masses of p itself, from the tile partials
+        for (int o = 1; o < W; o <<= 1) {
+          const float y = __shfl_up_sync(0xffffffffu, incl, o, W);
+          if (sl >= o) incl += y;
+        }
+        Z = __shfl_sync(0xffffffffu, incl, W - 1, W);
+      };
+      scan();
+      // zero residual mass: the draw is from p, whose tile masses are in the partials
+      const bool empty = valid && !(Z > 0.f);
+      if (__any_sync(0xffffffffu, empty)) {
+        if (empty) {
+          const float4* part = reinterpret_cast<const float4*>(
+              L.part + (int64_t)(row0 + drawn[i]) * L.tiles + k0);
 #pragma unroll
           for (int q = 0; q < kMaxTilesPerLane; ++q) {
-            const int k = lane * per + q;
             mk[q] = 0.f;
-            if (q < per && k < L.tiles) {
-              const float4 p0 =
-                  __ldcg(reinterpret_cast<const float4*>(L.part + (int64_t)row * L.tiles + k));
+            if (q < own) {
+              const float4 p0 = __ldcg(part + 2 * q);
               mk[q] = p0.y * ex2_approx(p0.x * c - ri.Cp);
             }
           }
         }
-        float ls = 0.f;
-#pragma unroll
-        for (int q = 0; q < kMaxTilesPerLane; ++q) ls += mk[q];
-        float incl = ls;
-#pragma unroll 1
-        for (int o = 1; o < 32; o <<= 1) {
-          const float y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const float Z = __shfl_sync(0xffffffffu, incl, 31);
-        if (!(Z > 0.f)) {
-          if (fp == 1 && lane == 0 && tile0 == 0) {
-            a.out_tok[row] = -1;
-            record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
-          }
-          continue;  // zero residual mass: try p
-        }
-        const float target = ri.u_res * Z;
-        const uint32_t pos = __ballot_sync(0xffffffffu, ls > 0.f);
-        const uint32_t cross = __ballot_sync(0xffffffffu, ls > 0.f && incl > target);
-        const int32_t lstar = cross ? (__ffs(cross) - 1) : (31 - __clz(pos));
-        float t1 = __shfl_sync(0xffffffffu, incl - ls, lstar);
-        t1 = cross ? target - t1 : INFINITY;
-        if (lane == lstar) {
-          int32_t ks = -1, klast = -1;
-          float tk = INFINITY, cum = 0.f;
-#pragma unroll
-          for (int q = 0; q < kMaxTilesPerLane; ++q) {
-            if (q < per && lane * per + q < L.tiles) {
-              if (mk[q] > 0.f) {
-                klast = lane * per + q;
-                if (ks < 0 && cum + mk[q] > t1) { ks = klast; tk = t1 - cum; }
-              }
-              cum += mk[q];
-            }
-          }
-          if (ks < 0) { ks = klast; tk = INFINITY; }
-          ri.cstar = ks;
-          ri.tc = tk;
-          ri.from_p = fp;
-        }
         __syncwarp();
-        break;
+        scan();
+        if (empty && !(Z > 0.f) && sl == 0 && tile0 == 0) {
+          a.out_tok[row0 + drawn[i]] = -1;
+          record_status(a.status, SSD_ERR_DEVICE_BOUNDS);
+        }
       }
+      const float target = ri.u_res * Z;
+      const uint32_t pos = __ballot_sync(0xffffffffu, ls > 0.f) & seg_mask;
+      const uint32_t cross = __ballot_sync(0xffffffffu, ls > 0.f && incl > target) & seg_mask;
+      const int32_t lstar = cross ? __ffs(cross) - 1 : pos ? 31 - __clz(pos) : lane;
+      float t1 = __shfl_sync(0xffffffffu, incl - ls, lstar);
+      t1 = cross ? target - t1 : INFINITY;
+      if (valid && Z > 0.f && lane == lstar) {
+        int32_t ks = -1, klast = -1;
+        float tk = INFINITY, cum = 0.f;
+#pragma unroll
+        for (int q = 0; q < kMaxTilesPerLane; ++q) {
+          if (mk[q] > 0.f) {  // (0 past the lane's tiles)
+            klast = k0 + q;
+            if (ks < 0 && cum + mk[q] > t1) { ks = klast; tk = t1 - cum; }
+          }
+          cum += mk[q];
+        }
+        if (ks < 0) { ks = klast; tk = INFINITY; }
+        ri.cstar = ks;
+        ri.tc = tk;
+        ri.from_p = empty ? 1 : 0;
+      }
+      __syncwarp();
     }
   }
   __syncthreads();
