@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
     # 128-row tiles (GQA): two query tiles for the first sequence's 256 rows, one
     # for the second's last grid row; every other image complete
     ("tail_gqa", 8, (32, 8), 128, 32, 64, [64 + 1024] * 5 + [64 + 300, 64 + 1024, 64 + 31 * 32 + 4]),
-    # exactly as many live items as half the CTAs and fewer: 2 CTAs per item
+    # 128 live items of at most 11 tiles: whole
     ("two_way", 8, (16, 16), 128, 24, 120, [120 + 72 * k for k in range(8)]),
     # 16 items of 17 tiles: 4 parts, of 4 tiles and one of 5
     ("four_short_parts", 1, (16, 16), 128, 32, 64, [64 + 975]),

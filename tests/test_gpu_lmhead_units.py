@@ -19,6 +19,9 @@ pytestmark = pytest.mark.gpu
     (128, 384, 512),   # the most rows of one CTA
     (129, 384, 512),   # the fewest on CTA pairs
     (256, 128, 640),   # the most rows; five tiles, the third pair half empty
+    # the search: 70 tiles (half a warp per row, 8 tiles per lane, one load each), 133
+    # and 148 tiles (a warp per row; 148 in 16-byte loads), more rows than one pass takes
+    (90, 64, 8960), (40, 64, 17024), (90, 64, 18944),
 ])
 def test_unit_shapes_match_oracle(ssd, rows, K, V):  # noqa: F811
     ht, hd, wt, wd, u = make_inputs(rows, K, V, 60 + rows, 0.1)
