@@ -208,7 +208,7 @@ class ClockSampler:
 MEASURED_TRAFFIC = {
     # (kernel, config): (source, sha256 prefix of the source the capture ran,
     # DRAM bytes read + written in one launch, rows of that launch or None)
-    ("lmhead_accept", 4): ("lmhead.cu", "4067185d518772ef", 269286656 + 115456, None),
+    ("lmhead_accept", 4): ("lmhead.cu", "26bbdea7ac53856b", 269286656 + 115456, None),
     # 8 x 64x64 replay, first step (1024 draft rows): accept_kernel alone; the
     # bench scales it to the rows of the replay states it sums
     ("accept", 5): ("accept.cu", "6c41882f517fa019", 536914176 + 67840, 1024),

@@ -352,9 +352,9 @@ struct LmHeadArgs {
   int32_t early_dependents = 0;
 };
 size_t lmhead_workspace(int32_t rows, int32_t V);
-// The grid-barrier words at the start of a workspace and their count.
+// The grid-barrier word at the start of a workspace (count 1).
 inline unsigned int* lmhead_counters(void* ws) { return static_cast<unsigned int*>(ws); }
-constexpr int32_t kLmheadCounters = 2;
+constexpr int32_t kLmheadCounters = 1;
 ssd_status lmhead_check(int32_t rows, int32_t V, int32_t K);
 cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream);
 

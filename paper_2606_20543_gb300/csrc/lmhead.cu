@@ -84,12 +84,14 @@ __device__ __forceinline__ uint32_t ld_acquire(const unsigned int* p) {
 }
 
 // Bounded grid barrier over `ncta` co-resident CTAs (cooperative launch).
-// ctr[0] counts arrivals over the kernel's barriers (cumulative targets);
-// ctr[1] is an abort flag: a CTA that gives up waiting (after max_polls polls,
-// SSD_ERR_TIMEOUT recorded) raises it before it arrives anywhere else, so a
-// slower CTA that later sees the count reached through that CTA's next
-// arrival fails too instead of going on with missing partials.  Returns false
-// in every thread if this CTA gave up or the kernel was aborted.
+// *ctr counts arrivals over the kernel's barriers (cumulative targets) in its low 31
+// bits; the top bit aborts the kernel: a CTA that gives up waiting (after max_polls
+// polls, SSD_ERR_TIMEOUT recorded) raises it before it arrives anywhere else, so a
+// slower CTA that later sees the count reached through that CTA's next arrival
+// fails too instead of going on with missing partials.  (One word, so that a wait ends
+// with the load that sees the count: a flag read after it cost ~0.6 us per barrier.)
+// Returns false in every thread if this CTA gave up or the kernel was aborted.
+constexpr unsigned int kAbort = 0x80000000u;
 __device__ __noinline__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* status,
                              int32_t* flag, uint32_t max_polls) {
   __syncthreads();
@@ -97,16 +99,16 @@ __device__ __noinline__ bool grid_barrier(unsigned int* ctr, unsigned int target
     // (a release and an acquire, ordered with the block by its barriers, instead of
     // two full fences: ~1 us per grid barrier)
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
-    bool ok = false;
+    bool ok = false, aborted = false;
 #pragma unroll 1
-    for (uint32_t i = 0; i < max_polls; ++i) {
-      if (ld_acquire(ctr) >= target) { ok = true; break; }
+    for (uint32_t i = 0; i < max_polls && !ok && !aborted; ++i) {
+      const uint32_t v = ld_acquire(ctr);
+      aborted = (v & kAbort) != 0;
+      ok = !aborted && v >= target;
       if (i > 256) __nanosleep(64);
     }
-    if (ok) {
-      ok = ld_acquire(ctr + 1) == 0u;
-    } else {
-      atomicExch(ctr + 1, 1u);
+    if (!ok && !aborted) {
+      atomicOr(ctr, kAbort);
       record_status(status, SSD_ERR_TIMEOUT);
     }
     *flag = ok ? 1 : 0;
@@ -814,7 +816,7 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
   L.max_polls = wait_poll_limit();
   L.shortfall = barrier_shortfall();
   unsigned char* w = static_cast<unsigned char*>(ws);
-  L.barrier = reinterpret_cast<unsigned int*>(w);  // [0] arrivals, [1] abort flag
+  L.barrier = reinterpret_cast<unsigned int*>(w);  // arrivals and the abort bit
   w += al256(2 * sizeof(unsigned int));
   L.part = reinterpret_cast<LmPartial*>(w);
   w += al256((size_t)a.rows * L.tiles * sizeof(LmPartial));

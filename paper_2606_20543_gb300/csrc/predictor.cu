@@ -25,10 +25,12 @@
 // a tile's whole K runs in its CTA: no partial sums, so between the phases
 // there is only the tile's epilogue, one counter and the next activations'
 // copies, at the price of every CTA reading all of X from L2 (24 rows: 1.2 MB
-// beside 3.1 MB of weights).  At d = 4096, m = 8192, V = 16384: 24 rows 85 us
-// (0.71 of the rate of the measured copy), 64 rows 92, 128 rows 117; 92 rows at
-// d = 896 38.  (With 4 epilogue warps of whole rows 89, 97, 120 and 42; with 16 of
-// them that each polled for the products 86, 93, 123 and 41.)  Splitting each tile's K over CTAs instead, with the
+// beside 3.1 MB of weights).  At d = 4096, m = 8192, V = 16384: 24 rows 79 us
+// (0.76 of the rate of the measured copy), 64 rows 86, 128 rows 110; 92 rows at
+// d = 896 33.  (In turn: with 4 epilogue warps of whole rows 89, 97, 120 and 42; 16
+// warps that each polled for the products 86, 93, 123 and 41, one of them polling 85,
+// 92, 117 and 38; started as a programmatic dependent's successor 82, 90, 114 and 37;
+// then without the GPU-wide fences.)  Splitting each tile's K over CTAs instead, with the
 // partials summed through L2 by the last contributor (~9 us per phase boundary,
 // 254 KB of code), took 113, 135, 147 and 93 us.
 //   * warp 0: weight producer, running ahead through all four phases into a
@@ -129,13 +131,6 @@ __device__ __forceinline__ void fence_proxy_async_global() {
   asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-// Release / acquire at GPU scope (lighter than a sequentially consistent
-// fence): orders this thread's earlier writes before, and its later reads
-// after, the ticket and counter atomics that publish and claim them.
-__device__ __forceinline__ void fence_acq_rel_gpu() {
-  asm volatile("fence.acq_rel.gpu;" ::: "memory");
-}
-
 // Counters, one per 128-byte line: tiles done per phase, abort.
 constexpr int kCtrStride = 32;
 __device__ __forceinline__ unsigned int* done_ctr(const PredLaunch& L, int p) {
@@ -150,7 +145,9 @@ __device__ __forceinline__ unsigned int* abort_flag(const PredLaunch& L) {
 __device__ __noinline__ bool wait_count(const PredLaunch& L, const unsigned int* ctr, uint32_t target) {
 #pragma unroll 1
   for (uint32_t i = 0; i < L.max_polls; ++i) {
-    if (ld_acquire_u32(ctr) >= target) return ld_acquire_u32(abort_flag(L)) == 0u;
+    // (the count alone says that every tile is final: a CTA that gives up counts no
+    // more of its own)
+    if (ld_acquire_u32(ctr) >= target) return true;
     if ((i & 1023u) == 1023u && ld_acquire_u32(abort_flag(L)) != 0u) return false;
     if (i > 64) __nanosleep(128);
   }
@@ -373,9 +370,8 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
                         lane != 0 || (*fail == 0 && wait_count(L, done_ctr(L, p - 1),
                                                                (uint32_t)L.ph[p - 1].tiles + L.shortfall))) != 0;
         if (!ok) break;
-        fence_acq_rel_gpu();
+        __syncwarp();  // what the waiting lane acquired, for the lane that copies
         fence_proxy_async_global();  // written by generic stores, loaded by TMA
-        __syncwarp();
       }
       const CUtensorMap* map = w ? (p == 0 ? &tmW0 : p == 1 ? &tmW1 : p == 2 ? &tmW2 : &tmWH)
                                  : (p == 0 ? &tmZ : p == 1 ? &tmAg : p == 2 ? &tmG : &tmHg);
@@ -499,7 +495,6 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
           ok = false;
           break;
         }
-        fence_acq_rel_gpu();
         row_scales(L, et, srow);
         bar_named(kBarEpi, kEpiThreads);
       }
@@ -527,17 +522,19 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
         __syncwarp();
         if (lane == 0) mbar_arrive(&acc_empty[buf]);
         fence_proxy_async_global();  // Ag, G, Hg are loaded by TMA in the next phase
-        fence_acq_rel_gpu();
         bar_named(kBarEpi, kEpiThreads);
-        if (p < 3) {  // the tile is final (a reduction: nothing waits for its result)
+        // One thread's release publishes the tile, ordered after the others' stores by
+        // the barrier, and a wait's acquire load needs no fence behind it either: a
+        // GPU-wide fence in every thread on both sides took 24 rows 81.4 us instead of
+        // 79.2, 92 rows at d = 896 35.8 instead of 33.0.
+        if (p < 3) {  // (a reduction: nothing waits for its result)
           if (et == 0)
-            asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(done_ctr(L, p)) : "memory");
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(done_ctr(L, p)) : "memory");
         } else {
-          if (et == 0) *bcast = atomicAdd(done_ctr(L, 3), 1u);
+          if (et == 0) *bcast = (uint32_t)atom_add_acq_rel(reinterpret_cast<int32_t*>(done_ctr(L, 3)), 1);
           bar_named(kBarEpi, kEpiThreads);
           if (*bcast == (uint32_t)(pp.tiles - 1)) {
             // the last tile of the vocabulary: every tile's key is in
-            fence_acq_rel_gpu();
             for (int32_t r = et; r < L.rows; r += kEpiThreads)
               L.out_tok[r] = argmax_index(__ldcg(L.best + (int64_t)r * kKeyStride));
           }
