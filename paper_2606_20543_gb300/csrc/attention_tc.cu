@@ -328,7 +328,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   __shared__ TcSeq s_seq[kLptMax];     // the plan: sequences longest first
   __shared__ int2 s_key[kLptMax];      // (keys, items) of each sequence
-  __shared__ int32_t s_plan[2];        // live items, most keys
+  __shared__ int32_t s_plan[3];        // live items, log2 of the CTAs per item, items shared by two
   __shared__ TcItem* s_merge;          // the item this CTA shares with its group (split mode)
   unsigned char* smem = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -378,6 +378,29 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       key = make_int2(c + n, a.Hkv * (L.mtiles == 1 ? 1 : (n + L.drafts - 1) / L.drafts));
     }
   }
+  // CTAs per item: as many of a cluster (a power of two) as leave one item or none per
+  // group of them, if the parts are long enough; by one thread, from the live items,
+  // the longest item's keys and all items' tiles
+  auto put_plan = [&](int32_t total, int32_t most, int32_t tiles) {
+    const int32_t cs = (int32_t)cluster_size(), most_tiles = (most + KTC - 1) / KTC;
+    auto fits = [&](int parts, int few, int many) {
+      const int n = parts * total;
+      return parts <= cs && n <= ncta && most_tiles >= parts * (n <= L.sms ? few : many);
+    };
+    int32_t log = 0, pairs = 0;
+    if (fits(4, kFew4, kMany4)) log = 2;
+    else if (fits(2, kFew2, kMany2)) log = 1;
+    else if (total < ncta && most_tiles >= 2 * kMany2 && 4 * most_tiles * total >= 5 * tiles)
+      // Whole items leave CTAs idle, fewer than a second one each, and the longest is
+      // a quarter longer than their mean: the longest items take those CTAs, two per
+      // item in the first clusters (five 64x64 sequences of 600 to 4100 keys 49.5
+      // -> 41.8 us, seven 56.7 -> 53.9; with items of one length the merges cost
+      // more: six of 3000 to 4000 61.1 -> 62.2).
+      pairs = min(ncta - total, total) & ~1;
+    s_plan[0] = total;
+    s_plan[1] = log;
+    s_plan[2] = pairs;
+  };
   TcSeq mine{0, 0, 0, 0x7fffffff};  // producer warp: this lane's sequence and first item (B <= 32)
   if (warp == kSoftWarps) {
     if (lane == 0) {
@@ -414,10 +437,8 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (key.y > 0) mine = TcSeq{lane, c, n, off};
       const int32_t total = __reduce_add_sync(0xffffffffu, key.y);
       const int32_t most = __reduce_max_sync(0xffffffffu, key.x);
-      if (lane == 0) {
-        s_plan[0] = total;
-        s_plan[1] = most;
-      }
+      const int32_t tiles = __reduce_add_sync(0xffffffffu, (key.x + KTC - 1) / KTC * key.y);
+      if (lane == 0) put_plan(total, most, tiles);
     }
     __syncwarp();
   } else if (warp == kSoftWarps + 1) {
@@ -431,7 +452,7 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     if (tid < a.B) s_key[tid] = key;
     __syncthreads();
     if (tid < a.B) {
-      int32_t r = 0, off = 0, total = 0, most = 0;
+      int32_t r = 0, off = 0, total = 0, most = 0, tiles = 0;
 #pragma unroll 1
       for (int32_t j = 0; j < a.B; ++j) {
         const int2 kj = s_key[j];
@@ -440,29 +461,20 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         off += ahead ? kj.y : 0;
         total += kj.y;
         most = max(most, kj.x);
+        tiles += (kj.x + KTC - 1) / KTC * kj.y;
       }
       s_seq[r] = TcSeq{tid, c, n, off};
-      if (tid == 0) {
-        s_plan[0] = total;
-        s_plan[1] = most;
-      }
+      if (tid == 0) put_plan(total, most, tiles);
     }
     __syncthreads();
   }
 
-  // CTAs per item: as many of a cluster (a power of two) as leave one item or
-  // none per group of them, but no more than the longest item has tiles
-  int32_t n_items = 0, ns_log = 0;
+  int32_t n_items = 0, ns_log = 0, shared = 0;
   auto read_plan = [&]() {
     n_items = planned ? s_plan[0] : a.B * per_b;
     if (planned) {
-      const int32_t cs = (int32_t)cluster_size(), most_tiles = (s_plan[1] + KTC - 1) / KTC;
-      auto fits = [&](int parts, int few, int many) {
-        const int n = parts * n_items;
-        return parts <= cs && n <= ncta && most_tiles >= parts * (n <= L.sms ? few : many);
-      };
-      if (fits(4, kFew4, kMany4)) ns_log = 2;
-      else if (fits(2, kFew2, kMany2)) ns_log = 1;
+      shared = s_plan[2];
+      ns_log = cta < 2 * shared ? 1 : s_plan[1];
     }
   };
   uint32_t tmem = 0, tS = 0, tO = 0;
@@ -491,7 +503,10 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const uint32_t q_bytes = (uint32_t)(L.drafts * G * 128) * (L.q_copies == 1 ? D / 64 : 1);  // per copy
     read_plan();
     const int32_t ns = 1 << ns_log;
-    const int32_t part = cta & (ns - 1), group = cta >> ns_log, ngroups = ncta >> ns_log;
+    const int32_t part = cta & (ns - 1);
+    // (shared items: one round, the pairs first)
+    const int32_t group = ns_log > 0 || shared == 0 ? cta >> ns_log : cta - shared;
+    const int32_t ngroups = shared > 0 ? n_items : ncta >> ns_log;
 #pragma unroll 1
     for (int32_t round = 0; ok; ++round) {
       const int32_t base = round * ngroups;

@@ -27,6 +27,10 @@ pytestmark = pytest.mark.gpu
     # 96 items of 24 tiles: 2 parts of 12 beyond one CTA per SM, where 23 stay whole
     ("two_parts_of_12", 6, (16, 16), 128, 40, 64, [64 + 1420] * 6),
     ("whole_below_12", 6, (16, 16), 128, 40, 64, [64 + 1320] * 6),
+    # 160 ragged items of 2 to 26 tiles: the 128 longest take two CTAs each, the rest one
+    ("longest_shared", 5, (32, 32), 64, 40, 0, [100, 400, 800, 1200, 1599]),
+    ("longest_shared_block_plan", 40, (4, 4), 64, 40, 0, [1590 if k % 3 == 0 else 60 + 9 * k
+                                                         for k in range(40)]),
     # more than 32 sequences: planned by the block (empty frontiers among them)
     ("block_plan", 40, (4, 4), 64, 16, 7, [7 + (37 * k) % 257 for k in range(40)]),
     # 3 and 20 query heads per KV head: tiles of 126 and 120 rows (42 and 6 drafts),
