@@ -16,7 +16,7 @@
 //  * two CTAs per SM: one CTA's start-up, item boundaries and tile chain
 //    overlap the other's (one 202 KB CTA per SM with 128-key tiles before: the
 //    24x24 sweep's step 62.6 us, the 16 x 32x32 GQA step 51.6 us, 8 x 64x64 at
-//    2300-3800 keys 75.5 us; now 46.4, 34.8 and 69.2 us, the last 6.1 TB/s);
+//    2300-3800 keys 75.5 us; now 46.4, 34.8 and 68.4 us, the last 6.15 TB/s);
 //  * the producer warp alone sets up, plans and issues its first item's five
 //    copies, a lane each in one instruction, before the block's barrier.  What
 //    an SM waits for between that and the first P is instruction fetch once
