@@ -176,7 +176,7 @@ cudaError_t launch_stage_shift(int32_t B, int32_t D_max, int32_t W, int32_t* tok
 }
 
 // (a kernel where a memset would do: as a programmatic dependent it starts sooner
-// after the kernel before it; the predictor of 24 rows 84.3 -> 81.1 us back to back)
+// after the kernel before it; the predictor of 24 rows 110.2 -> 108.4 us back to back)
 __global__ void zero_kernel(unsigned int* p, int32_t n) {
   pdl_wait();
   const int32_t i = blockIdx.x * blockDim.x + threadIdx.x;

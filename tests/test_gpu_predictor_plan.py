@@ -8,12 +8,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("rows,d,m,V", [
-    (64, 384, 640, 1152),    # the most rows of M = 64 products; a last unit of part of the K
-    (65, 384, 640, 1152),    # the fewest of M = 128
-    (7, 2432, 256, 640),     # a last tile of 128 of the 2432 features (tiles of 16 on <= 152 SMs)
-    (3, 128, 10240, 256),    # more gate tiles than CTAs: two rounds of one phase
-    (24, 128, 256, 20480),   # more GenHead tiles than CTAs, 128 wide
-    (40, 256, 384, 9856),    # 64-wide GenHead tiles against 128-wide ones
+    (64, 384, 640, 1152),    # four groups of 16 rows on N, and the first row of a fifth: two
+    (65, 384, 640, 1152),    # tensor-memory column blocks and three
+    (7, 2432, 256, 640),     # tiles of 38 units shared by 8 CTAs, which bounds the CTA count
+    (3, 128, 10240, 256),    # two CTAs (a phase of two units) for 80 gate tiles
+    (24, 128, 256, 20480),   # and for 160 GenHead tiles
+    (40, 256, 384, 9856),    # 77 GenHead tiles on 6 CTAs, whose ranges cut tiles
 ])
 def test_predictor_plan_shapes(ssd, rows, d, m, V):  # noqa: F811
     w, g1, g2 = _case(170 + rows, rows, d, m, V)
