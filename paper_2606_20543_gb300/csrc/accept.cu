@@ -765,11 +765,13 @@ __global__ void __launch_bounds__(32, 32) resolve_kernel(ResolveArgs a) {
     if (lane == 0) gmass[bk] = m;
   }
   // last part to finish: lane 0 stored this part's masses; its ticket releases
-  // them and, for the last part, acquires the others'
+  // them and, for the last part, acquires the others' (for the whole warp, by the
+  // warp barrier: a shuffle orders no memory)
   int32_t last = 0;
   if (lane == 0) last = atom_add_acq_rel(&a.tickets[b], 1) == (int32_t)gridDim.x - 1;
   const float u_res = row_uniforms(a.rng, r).y;
   last = __shfl_sync(0xffffffffu, last, 0);
+  __syncwarp();
   if (!last) {
     if (pdl_first_block()) pdl_wait();
     return;
