@@ -139,7 +139,8 @@ ssd_status ssd_frontier(const ssd_grid* grid, int32_t B, const int32_t* cache_le
  * over key slots s < cache_len[b] + n_drafts[b].  Slots [0, cache_len) are
  * the committed cache (flat position s); slot cache_len + j' holds draft
  * j''s own key/value (flat position of draft_pos[b][j']).  M = 0 iff
- * pos(key) <= pos(query), else -inf.  scale = 0 selects 1/sqrt(d).
+ * pos(key) <= pos(query), else -inf.  scale = 0 selects 1/sqrt(d).  Slots
+ * from cache_len + n_drafts on may hold anything, NaN and infinities too.
  *   q          dev bf16 [B][D_max][Hq][d]
  *   k, v       dev bf16 [B][Hkv][L_max][d]; cache_len + n_drafts <= L_max
  *   cache_len, n_drafts  dev int32 [B]

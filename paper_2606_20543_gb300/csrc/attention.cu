@@ -220,6 +220,17 @@ frontier_attn_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_const
     if (tid == 0 && t + kStages - 1 < ntiles) issue(t + kStages - 1);
     const int s = t % kStages;
     if (!mbar_wait(&full[s], (t / kStages) & 1, a.status)) ok = false;
+    const int32_t keys = k_hi - (k_lo + t * KT);  // from this tile on
+    if (keys < KT) {
+      // the slots behind the sequence's last key hold whatever the cache holds: their P
+      // of 0 must not meet a NaN or an infinity in V
+      for (int32_t i = tid; i < (KT - keys) * (D / 8); i += blockDim.x) {
+        const int32_t r = keys + i / (D / 8), ch = i % (D / 8);
+        *reinterpret_cast<uint4*>(sV + s * TILE_BYTES + (ch >> 3) * (KT * 128) + r * 128 +
+                                  (ch & 7) * 16) = make_uint4(0u, 0u, 0u, 0u);
+      }
+      __syncthreads();
+    }
     if (warp_active && ok) {
       const uint32_t kbase = smem_u32(sK + s * TILE_BYTES);
       const uint32_t vbase = smem_u32(sV + s * TILE_BYTES);

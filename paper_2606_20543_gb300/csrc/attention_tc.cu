@@ -266,6 +266,17 @@ __device__ __forceinline__ uint32_t part_off(int32_t r, int32_t ch) {
   return (uint32_t)r * (D * 4) + (uint32_t)((ch ^ (r & 7)) << 4);
 }
 
+// Rows r0 .. r1 - 1 of a K or V tile set to zero, by one warp.
+template <int D>
+__device__ __forceinline__ void clear_rows(unsigned char* tile, int32_t r0, int32_t r1, int lane) {
+#pragma unroll 1
+  for (int32_t i = lane; i < (r1 - r0) * (D / 8); i += 32) {
+    const int32_t r = r0 + i / (D / 8), ch = i % (D / 8);
+    *reinterpret_cast<uint4*>(tile + (ch >> 3) * (KTC * 128) + r * 128 + (ch & 7) * 16) =
+        make_uint4(0u, 0u, 0u, 0u);
+  }
+}
+
 // The keys c0 .. c0 + 63 a row may see, as a bit mask: cache keys are a prefix
 // of the window (visible up to qpos), draft keys come from the row's
 // visibility bits (vhi:vlo), keys past the part are dropped.
@@ -754,22 +765,33 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (!mbar_wait_warp(&it_full[s], (k >> 1) & 1, a.status)) break;
       const int32_t ntiles = (int32_t)warp_uniform((uint32_t)items[s].ntiles);
       if (ntiles < 0) break;
+      int32_t left = (int32_t)warp_uniform((uint32_t)(items[s].k_hi - items[s].k_lo));  // keys
       // the first product of the item overwrites O: the epilogue of the item before must be done
       if (k >= 1 && !mbar_wait_warp(o_empty, (k - 1) & 1, a.status)) break;
 #pragma unroll 1
-      for (int t = 0; t < ntiles; ++t, ++T) {
+      for (int t = 0; t < ntiles; ++t, ++T, left -= KTC) {
         const int sb = T % kNB;
         ok = mbar_wait_warp(&v_ready[sb], (T / kNB) & 1, a.status);
         if (!ok) break;
         tc_fence_after();
+        if (left < KTC) {
+          // The sequence's last keys: the slots behind them hold whatever the cache
+          // holds, and their P of 0 times a NaN or an infinity is a NaN in every row.
+          // Steps of 16 keys past the last are left out, and the rest of its step is
+          // cleared (whole rows of the tile, so the swizzle does not matter).
+          clear_rows<D>(sV + sb * KV_BYTES, left, (left + 15) & ~15, lane);
+          fence_proxy_async_shared();
+          __syncwarp();
+        }
         // A = P in TMEM (16 keys = 8 columns per step), B = V (MN-major: d
         // atoms KTC*128 bytes apart, 8-key groups 1 KB apart; 16 keys = 2 KB)
         const uint64_t dv = smem_desc(aV + sb * KV_BYTES, KTC * 128, 1024);
         if (leader) {
 #pragma unroll
           for (int kk = 0; kk < KTC / 16; ++kk)
-            mma_ts(tOu, tSu + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
-                    (t == 0 && kk == 0) ? 0u : 1u);
+            if (16 * kk < left)
+              mma_ts(tOu, tSu + sb * KTC + kk * 8, smem_desc_at(dv, kk * 2048), kIdescO,
+                     (t == 0 && kk == 0) ? 0u : 1u);
           mma_commit(&pv_done[sb]);
           mma_commit(&k_ready[sb]);  // S_{T+kNB} may start: the S/P buffer is free again
         }
