@@ -1186,14 +1186,14 @@ int32_t tc_tile_rows(const AttnArgs& a) {
   return attention_rows_hint(a.grid, a.D_max) * (a.Hq / a.Hkv) <= 64 ? 64 : kBM;
 }
 
-// Clusters of the kernel that the current device can hold at once (a device
+// Clusters of the kernel <D, BM> that the current device can hold at once (a device
 // constant, queried once per device and kernel), at least one.  The occupancy
 // calculator counts one CTA per SM for any kernel that allocates tensor
 // memory; kCtasPerSmTC of this kernel's CTAs, which share the 512 columns, do
 // run on an SM (304 of 304 CTAs of a probe started at once).
 constexpr int kMaxDevicesTC = 64;
-template <typename K>
-int resident_clusters(K kernel, size_t smem) {
+template <int D, int BM>
+int resident_clusters() {
   static std::atomic<int> known[kMaxDevicesTC];
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 1;
@@ -1203,20 +1203,38 @@ int resident_clusters(K kernel, size_t smem) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(kCluster);
   cfg.blockDim = dim3(kThreadsTC);
-  cfg.dynamicSmemBytes = smem;
+  cfg.dynamicSmemBytes = tc_smem_bytes<D, BM>();
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = kCluster;
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n < 1) {
-    cudaGetLastError();
-    n = std::max(1, device_sm_count() / kCluster / 2);
+  if (cudaOccupancyMaxActiveClusters(&n, frontier_attn_tc_kernel<D, BM>, &cfg) != cudaSuccess ||
+      n < 1) {
+    cudaGetLastError();  // (not kept: the next launch asks again)
+    return std::max(1, device_sm_count() / kCluster / 2) * kCtasPerSmTC;
   }
   n *= kCtasPerSmTC;
   if (slot) known[dev].store(n, std::memory_order_relaxed);
   return n;
+}
+
+// The launch of the kernel <D, BM>: persistent, whole clusters, as many as are
+// resident, at most one per item.
+template <int D, int BM>
+cudaError_t launch_tiles(const AttnArgs& a, TcLaunch L, const CUtensorMap& tq, const CUtensorMap& tk,
+                         const CUtensorMap& tv, cudaStream_t stream, bool pdl) {
+  constexpr size_t smem = tc_smem_bytes<D, BM>();
+  const cudaError_t e = cudaFuncSetAttribute(
+      frontier_attn_tc_kernel<D, BM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  const int64_t n_items = (int64_t)a.B * a.Hkv * L.mtiles;
+  const int64_t clusters = std::min<int64_t>(n_items, resident_clusters<D, BM>());
+  L.order = pdl ? kCluster : 0;
+  return launch_clusters(frontier_attn_tc_kernel<D, BM>,
+                         dim3((unsigned)(clusters * kCluster + L.order)), dim3(kThreadsTC), smem,
+                         stream, /*pdl=*/true, kCluster, tq, tk, tv, a, L);
 }
 }  // namespace
 
@@ -1249,22 +1267,11 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
          bf16_tensor_map(&tv, a.v, 4, dims, strides, box);
   }
   if (!ok) return cudaErrorInvalidValue;
-  // persistent: whole clusters, as many as are resident, at most one per item
-  const int64_t n_items = (int64_t)a.B * a.Hkv * L.mtiles;
-  auto launch = [&](auto kernel, size_t smem) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    const int64_t clusters = std::min<int64_t>(n_items, resident_clusters(kernel, smem));
-    L.order = pdl ? kCluster : 0;
-    return launch_clusters(kernel, dim3((unsigned)(clusters * kCluster + L.order)),
-                           dim3(kThreadsTC), smem, stream, /*pdl=*/true, kCluster, tq, tk, tv, a, L);
-  };
   if (a.d == 128)
-    return bm == 64 ? launch(frontier_attn_tc_kernel<128, 64>, tc_smem_bytes<128, 64>())
-                    : launch(frontier_attn_tc_kernel<128, 128>, tc_smem_bytes<128, 128>());
-  return bm == 64 ? launch(frontier_attn_tc_kernel<64, 64>, tc_smem_bytes<64, 64>())
-                  : launch(frontier_attn_tc_kernel<64, 128>, tc_smem_bytes<64, 128>());
+    return bm == 64 ? launch_tiles<128, 64>(a, L, tq, tk, tv, stream, pdl)
+                    : launch_tiles<128, 128>(a, L, tq, tk, tv, stream, pdl);
+  return bm == 64 ? launch_tiles<64, 64>(a, L, tq, tk, tv, stream, pdl)
+                  : launch_tiles<64, 128>(a, L, tq, tk, tv, stream, pdl);
 }
 
 }  // namespace ssd
