@@ -78,10 +78,9 @@ constexpr uint32_t kTmemCols = 256;  // S/P x 2 (64 columns each), O (up to 128 
 constexpr int kSoftWarps = 4;     // one per TMEM lane quarter
 constexpr int kThreadsTC = (kSoftWarps + 4) * 32;  // + K/Q producer, V producer, S, PV
 constexpr int kCtasPerSmTC = 2;   // 2 x 256 TMEM columns, 2 x ~107 KB of shared memory
-#ifndef SSD_ATTN_CLUSTER
-#define SSD_ATTN_CLUSTER 4
-#endif
-constexpr int kCluster = SSD_ATTN_CLUSTER;  // CTAs that can share one item
+constexpr int kCluster = 4;       // CTAs that can share one item
+// (the plan's pairs of CTAs, and its groups of two or four, lie inside one cluster)
+static_assert(kCluster == 2 || kCluster == 4, "cluster size");
 // Fewest key tiles of a part of the longest item, with 4 and with 2 parts, while every
 // part has an SM to itself (few) and beyond that (many): merging parts takes ~3 us
 // and a tile 0.3-0.5 us, and the parts of items that fill the SMs anyway only share
