@@ -153,6 +153,26 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, i
   return __all_sync(0xffffffffu, mbar_wait(bar, parity, status, max_polls)) != 0;
 }
 
+// After a wait that gave up: this CTA's copies and products still in flight land
+// within microseconds, so its shared and tensor memory are let go once `bar`'s phase
+// completes or ~5 ms have passed (a phase that lacks another arrival never completes),
+// whatever limit the launch's waits have.
+[[maybe_unused]] static __device__ __noinline__ void mbar_drain(uint64_t* bar, uint32_t parity) {
+#pragma unroll 1
+  for (int i = 0; i < (1 << 14); ++i) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n"
+        " mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return;
+    __nanosleep(256);
+  }
+}
+
 // ------------------------------------------------------------- bulk copies
 // Untiled bulk copy global -> shared (TMA engine); both addresses 16-byte
 // aligned, bytes a multiple of 16.  Completion is signalled on `bar`.

@@ -216,6 +216,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   // threads wait at the block's barrier (not polling beside them).  A warp issues
   // a copy every ~0.3 us, so a unit of one head takes two copies of up to 32 KB,
   // from two warps.
+  int issued = 0;  // units that this warp copied
   if (warp == 0 || warp == 2) {
     const bool w = warp == 0, leader = elect_one();
     const uint64_t pol = w ? policy_evict_first()   // weights: read once
@@ -248,14 +249,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
         ph ^= 1u;
       }
     }
-    // after a failure: this CTA's (the pair's) copies still in flight, among the last
-    // S units, land before it goes on (the pair's other CTA waits at the end)
-    if (u < nunits && rank == 0) {
-#pragma unroll 1
-      for (int x = max(u - S, 0); x < u; ++x)
-        mbar_wait(&full[x % S], (x / S) & 1, nullptr, L.max_polls);
-    }
-    __syncwarp();
+    issued = u;
   } else if (warp == 1 && rank == 0) {
     const uint32_t base = warp_uniform(smem_u32(smem)), tm = warp_uniform(tmem);
     const bool leader = elect_one();
@@ -312,7 +306,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  bool ok = *fail == 0;
+  const bool main_ok = *fail == 0;
+  bool ok = main_ok;
 
   const float c = kLog2eL / a.temperature;
   const int32_t rows = a.rows;
@@ -713,7 +708,22 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     if (mine) a.out_tok[row] = pick >= 0 ? pick : lastpos;
   }
 
-  // ---- teardown: release TMEM (all MMAs have completed: `done` fired)
+  // ---- teardown.  After a failure in the main loop: the copies still in flight, among
+  // each copying warp's last S units, and the products.  A pair's copies are counted
+  // by its even CTA; after any failure the odd one waits its time out on a barrier that
+  // nothing arrives at.
+  if (rank == 1) {
+    if (!ok && warp == 0) mbar_drain(&full[0], 0);
+  } else if (!main_ok) {
+    if (issued > 0) {
+#pragma unroll 1
+      for (int x = max(issued - S, 0); x < issued; ++x) mbar_drain(&full[x % S], (x / S) & 1);
+    } else if (warp == 1) {
+      mbar_drain(done, 0);
+    }
+  }
+  // release TMEM (all MMAs have completed: `done` fired)
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if constexpr (PAIR) cluster_sync_all();  // (no copy or MMA of the pair is left)

@@ -179,6 +179,11 @@ __device__ bool wait_count(const PredLaunch& L, const unsigned int* ctr, uint32_
   return false;
 }
 
+// The end of this CTA's own copies or products, also after a wait that gave up.
+__device__ __forceinline__ void land(uint64_t* bar, uint32_t parity, uint32_t max_polls) {
+  if (!mbar_wait(bar, parity, nullptr, max_polls)) mbar_drain(bar, parity);
+}
+
 __device__ __forceinline__ void warp_argmax(float& v, int32_t& i) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -512,7 +517,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
       // copies still in flight can only be among the last S units issued:
       // wait for those before the CTA may exit
       for (uint32_t x = gu > (uint32_t)S ? gu - S : 0; x < gu; ++x)
-        if ((int)(x & 1u) == warp) mbar_wait(&full[x % S], (x / S) & 1, nullptr, L.max_polls);
+        if ((int)(x & 1u) == warp) land(&full[x % S], (x / S) & 1, L.max_polls);
     }
     __syncwarp();
   } else if (warp == kWarpX) {
@@ -608,7 +613,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
     }
     if (lane == 0)
       for (uint32_t x = gu > (uint32_t)S ? gu - S : 0; x < gu; ++x)
-        mbar_wait(&full[x % S], (x / S) & 1, nullptr, L.max_polls);
+        land(&full[x % S], (x / S) & 1, L.max_polls);
     __syncwarp();
   } else if (warp == kWarpMma) {
     // ---- MMA issue (every lane in the loop, one elected around the products)
@@ -769,7 +774,7 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
   }
 
   // ---- teardown: every MMA complete before tensor memory is freed
-  if (warp == kWarpX && lane == 0) mbar_wait(mma_done, 0, nullptr, L.max_polls);
+  if (warp == kWarpX && lane == 0) land(mma_done, 0, L.max_polls);
   tc_fence_before();
   __syncthreads();
   if (warp == kWarpX) {

@@ -80,3 +80,56 @@ def test_predictor_wait_runs_out_and_the_context_stays_usable(ssd):
     tok, hid, st = call()
     assert st == 0
     _check(w, g1, g2, 1e-6, tok, hid)
+
+
+@pytest.mark.parametrize("limit", [1, 4, 64])
+@pytest.mark.parametrize("rows,K", [(48, 1024), (160, 1024)])
+def test_lmhead_short_limits_leave_nothing_in_flight(ssd, rows, K, limit):
+    """Limits that run out in the main loop: the copies and products in flight are
+    waited for all the same, and the next call is right."""
+    V = 2048
+    ht, hd, wt, wd, u = make_inputs(rows, K, V, 24, 0.05)
+    want = run_fused(ssd, ht, hd, wt, wd, u)
+    assert want[-1] == 0
+    for _ in range(4):
+        ssd.ssd_set_wait_limit(limit)
+        try:
+            st = run_fused(ssd, ht, hd, wt, wd, u)[-1]
+        finally:
+            ssd.ssd_set_wait_limit(0)
+        assert st in (0, SSD_ERR_TIMEOUT)
+        got = run_fused(ssd, ht, hd, wt, wd, u)
+        assert all(np.array_equal(a, b) for a, b in zip(want, got))
+
+
+@pytest.mark.parametrize("limit", [1, 4, 64])
+def test_predictor_short_limits_leave_nothing_in_flight(ssd, limit):
+    from tests.test_gpu_predictor import _case, _run
+    rows, d, m, V = 24, 512, 1024, 4096
+    w, g1, g2 = _case(32, rows, d, m, V)
+    want = _run(ssd, rows, d, m, V, w, g1, g2, 1e-6)
+    for _ in range(4):
+        ssd.ssd_set_wait_limit(limit)
+        try:
+            tok, st = _give_up(ssd, rows, d, m, V, w, g1, g2)
+        finally:
+            ssd.ssd_set_wait_limit(0)
+        assert (st == SSD_ERR_TIMEOUT and np.all(tok == -7)) or (
+            st == 0 and np.array_equal(tok, want[0]))
+        got = _run(ssd, rows, d, m, V, w, g1, g2, 1e-6)
+        assert np.array_equal(want[0], got[0]) and np.array_equal(want[1], got[1])
+
+
+def _give_up(ssd, rows, d, m, V, w, g1, g2):
+    from tests.test_gpu_predictor import _bf_dev
+    dev = {k: _bf_dev(v) for k, v in w.items()}
+    ws = torch.empty(ssd.ssd_draft_predict_workspace(rows, d, m, V), dtype=torch.uint8,
+                     device="cuda")
+    tok = torch.full((rows,), -7, dtype=torch.int32, device="cuda")
+    hid = torch.zeros((rows, d), dtype=torch.float32, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    ssd.ssd_draft_predict(rows, d, m, V, dev["z"], dev["w0"], dev["w1"], dev["w3"], dev["w2"],
+                          torch.from_numpy(g1).cuda(), torch.from_numpy(g2).cuda(), dev["wh"],
+                          1e-6, tok, hid, ws, ws.numel(), st)
+    torch.cuda.synchronize()
+    return tok.cpu().numpy(), int(st.item())
