@@ -85,21 +85,22 @@ __device__ __forceinline__ uint32_t ld_acquire(const unsigned int* p) {
 
 // Bounded grid barrier over `ncta` co-resident CTAs (cooperative launch).
 // *ctr counts arrivals over the kernel's barriers (cumulative targets) in its low 31
-// bits; the top bit aborts the kernel: a CTA that gives up waiting (after max_polls
-// polls, SSD_ERR_TIMEOUT recorded) raises it before it arrives anywhere else, so a
-// slower CTA that later sees the count reached through that CTA's next arrival
-// fails too instead of going on with missing partials.  (One word, so that a wait ends
-// with the load that sees the count: a flag read after it cost ~0.6 us per barrier.)
+// bits; the top bit aborts the kernel: a CTA that gave up, here (after max_polls
+// polls, SSD_ERR_TIMEOUT recorded) or before (good false: its partials are missing),
+// raises it and arrives nowhere any more, so that no CTA goes on with missing
+// partials.  (One word, so that a wait ends with the load that sees the count: a flag
+// read after it cost ~0.6 us per barrier.)
 // Returns false in every thread if this CTA gave up or the kernel was aborted.
 constexpr unsigned int kAbort = 0x80000000u;
 __device__ __noinline__ bool grid_barrier(unsigned int* ctr, unsigned int target, int32_t* status,
-                             int32_t* flag, uint32_t max_polls) {
+                             int32_t* flag, uint32_t max_polls, bool good) {
   __syncthreads();
   if (threadIdx.x == 0) {
     // (a release and an acquire, ordered with the block by its barriers, instead of
     // two full fences: ~1 us per grid barrier)
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
-    bool ok = false, aborted = false;
+    if (good) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(ctr) : "memory");
+    else atomicOr(ctr, kAbort);
+    bool ok = false, aborted = !good;
 #pragma unroll 1
     for (uint32_t i = 0; i < max_polls && !ok && !aborted; ++i) {
       const uint32_t v = ld_acquire(ctr);
@@ -383,7 +384,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       out[1] = make_float4(xq, xp, __int_as_float(t), 0.f);
     }
   }
-  ok = grid_barrier(L.barrier, (unsigned)ncta + L.shortfall, a.status, flag, L.max_polls) && ok;
+  ok = grid_barrier(L.barrier, (unsigned)ncta + L.shortfall, a.status, flag, L.max_polls, ok);
 
   // ---- epilogue 2: combine the partials of each row and decide.  Row r is
   // combined by CTA r % ncta alone (one warp per row; lane l merges tiles l,
@@ -478,8 +479,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
       }
     }
   }
-  ok = grid_barrier(L.barrier, 2u * ((unsigned)ncta + L.shortfall), a.status, flag,
-                    L.max_polls) && ok;
+  ok = grid_barrier(L.barrier, 2u * ((unsigned)ncta + L.shortfall), a.status, flag, L.max_polls, ok);
 
   // ---- the rows to draw, in every CTA: every valid rejected row, or (lazy)
   // the first rejected row of each sequence among its drafts
@@ -542,8 +542,7 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
     if (draw && chunk == 0 && tile < L.tiles)
       L.mass[(int64_t)row * L.tiles + tile] = mass + cm[kBM] + cm[2 * kBM] + cm[3 * kBM];
   }
-  ok = grid_barrier(L.barrier, 3u * ((unsigned)ncta + L.shortfall), a.status, flag,
-                    L.max_polls) && ok;
+  ok = grid_barrier(L.barrier, 3u * ((unsigned)ncta + L.shortfall), a.status, flag, L.max_polls, ok);
 
   // ---- epilogue 4: locate the tile holding u_res * Z: half a warp per row up to 128
   // tiles, else a warp; lane l of the row's lanes owns tiles [l*per, (l+1)*per) and
