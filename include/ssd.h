@@ -396,7 +396,8 @@ ssd_status ssd_lmhead_accept(int32_t rows, int32_t V, int32_t K, const void* h_t
  * Streams: on the logits path the acceptance pass computes the frontier itself
  * (and writes n_drafts and draft_pos) and the attention computes the same
  * frontier from cache_len; on the fused path the frontier comes first.  With at
- * most 128 query heads per KV head (the tcgen05 attention) everything runs on
+ * most 128 query heads per KV head, and q and o 16-byte aligned (4-byte aligned is
+ * required), the attention is the tcgen05 one and everything runs on
  * `stream`: the acceptance (or the lm_head acceptance); the attention as its
  * programmatic dependent (it reads none of its results and takes the SMs that
  * it leaves); then the counts (and committed draws) as one of the
@@ -448,8 +449,9 @@ typedef struct {
 } ssd_verify_out;
 
 size_t ssd_verify_step_workspace(const ssd_verify_args* args);
-/* Number of kernels one ssd_verify_step() with these arguments launches
- * (host query, no GPU work); -1 if the arguments would be rejected. */
+/* Number of kernels one ssd_verify_step() with these arguments (and a 16-byte
+ * aligned out->o) launches (host query, no GPU work); -1 if the arguments would be
+ * rejected. */
 int32_t ssd_verify_step_launches(const ssd_verify_args* args);
 ssd_status ssd_verify_step(const ssd_verify_args* args, const ssd_verify_out* out,
                            void* workspace, size_t workspace_bytes, ssd_stream_t stream);

@@ -627,7 +627,7 @@ int32_t ssd_verify_step_launches(const ssd_verify_args* x) {
   // logits: acceptance (with the frontier) + attention (+ split combine) + counts/draws;
   // fused: frontier + attention (+ combine) + lm_head acceptance + counts
   const int fixed = x->tgt_logits != nullptr ? 2 : 3;
-  return fixed + attention_launches(x->B, x->Hq, x->Hkv, x->d, x->D_max, x->L_max);
+  return fixed + attention_launches(x->B, x->Hq, x->Hkv, x->d, x->D_max, x->L_max, x->q);
 }
 
 ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, void* workspace,
@@ -641,6 +641,9 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
   if (x->B == 0) return SSD_OK;
   if (x->q == nullptr || x->k == nullptr || x->v == nullptr) return SSD_ERR_INVALID_ARG;
   if (y->draft_pos == nullptr || y->o == nullptr) return SSD_ERR_INVALID_ARG;
+  // (read and written in pairs of entries at least)
+  if (((reinterpret_cast<uintptr_t>(x->q) | reinterpret_cast<uintptr_t>(y->o)) & 3u) != 0)
+    return SSD_ERR_INVALID_ARG;
   s = check_accept_part(x, y);
   if (s != SSD_OK) return s;
   // The counts write next_cache_len while the attention (beside them, or as
@@ -686,7 +689,7 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
     // (16x16 step 17.0 -> 13.9 us, two rounds on 8 x 24x24 72 -> 62 us; 24x24
     // sweep under (A) 53.1 -> 50.8, GQA batch under (A) 45.4 -> 39.5 and (B)
     // 52.3 -> 46.4).
-    const bool serial = attention_tc_supported(x->Hq, x->Hkv, x->d);
+    const bool serial = attention_tc_runs(x->Hq, x->Hkv, x->d, x->q, y->o);
     if (serial) {
       // On `stream` alone: the acceptance; the attention, which reads none of
       // its results, as a programmatic dependent that lets the next kernel be
@@ -722,7 +725,7 @@ ssd_status ssd_verify_step(const ssd_verify_args* x, const ssd_verify_out* y, vo
   e = launch_frontier(x->grid, x->B, x->cache_len, x->D_max, y->n_drafts, y->draft_pos, y->status,
                       stream, lmhead_counters(ws + attn_ws), kLmheadCounters);
   if (e != cudaSuccess) return SSD_ERR_CUDA;
-  if (attention_tc_supported(x->Hq, x->Hkv, x->d)) {
+  if (attention_tc_runs(x->Hq, x->Hkv, x->d, x->q, y->o)) {
     // On `stream` alone: a1; the lm_head acceptance, one CTA per 128 vocabulary
     // entries; the attention as its programmatic dependent, on the SMs that it
     // leaves idle (24 of 152 with 16384 entries: its CTAs follow one another

@@ -509,10 +509,15 @@ size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_
 
 static cudaError_t launch_combine(const AttnArgs& a, const AttnLaunch& L, cudaStream_t stream);
 
+bool attention_tc_runs(int32_t Hq, int32_t Hkv, int32_t d, const void* q, const void* o) {
+  return attention_tc_supported(Hq, Hkv, d) &&
+         ((reinterpret_cast<uintptr_t>(q) | reinterpret_cast<uintptr_t>(o)) & 15u) == 0;
+}
+
 int attention_launches(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
-                       int32_t L_max) {
+                       int32_t L_max, const void* q) {
   if (B == 0) return 0;
-  if (attention_tc_supported(Hq, Hkv, d)) return 1;
+  if (attention_tc_runs(Hq, Hkv, d, q, nullptr)) return 1;
   return make_plan(B, Hq, Hkv, d, D_max, L_max).splits > 1 ? 2 : 1;
 }
 
@@ -543,7 +548,7 @@ AttnLaunch carve(const AttnArgs& a, const Plan& p, void* ws) {
 cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream,
                              bool pdl) {
   if (a.B == 0) return cudaSuccess;
-  if (attention_tc_supported(a.Hq, a.Hkv, a.d)) return launch_attention_tc(a, stream, pdl);
+  if (attention_tc_runs(a.Hq, a.Hkv, a.d, a.q, a.o)) return launch_attention_tc(a, stream, pdl);
   const Plan p = make_plan(a.B, a.Hq, a.Hkv, a.d, a.D_max, a.L_max);
   const AttnLaunch L = carve(a, p, ws);
   cudaError_t e;

@@ -309,8 +309,11 @@ size_t attention_workspace(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_
 // the mma.sync kernel is always launched plainly.
 cudaError_t launch_attention(const AttnArgs& a, void* ws, size_t ws_bytes, cudaStream_t stream,
                              bool pdl = false);
+// Whether launch_attention runs the tcgen05 kernel: its shapes, with Q and O 16-byte
+// aligned (TMA and 16-byte stores; the mma.sync kernel loads and stores 4 bytes).
+bool attention_tc_runs(int32_t Hq, int32_t Hkv, int32_t d, const void* q, const void* o);
 int attention_launches(int32_t B, int32_t Hq, int32_t Hkv, int32_t d, int32_t D_max,
-                       int32_t L_max);
+                       int32_t L_max, const void* q);
 // Most drafts one sequence can have under grid `g` (Sec. 3.3 frontier: at most
 // min(k_h, W) horizontal positions, or W - c with k_h = 0, then k_v rows of W),
 // clipped to D_max.

@@ -182,6 +182,10 @@ def test_verify_accept_and_step_host_validation(lib):
     for at in (fake, fake + 4, fake - 4):
         assert step(ctypes.byref(args()), ctypes.byref(out(next_cache_len=at)),
                     ctypes.c_void_p(fake), need, None) == 1
+    # q and o are read and written in pairs of entries
+    for bad_q, bad_o in ((fake + 2, fake), (fake, fake + 2)):
+        assert step(ctypes.byref(args(q=bad_q)), ctypes.byref(out(o=bad_o)), ctypes.c_void_p(fake),
+                    need, None) == 1
     # launch counts: acceptance + attention (+ combine) + counts on the logits path,
     # and one more (the frontier) on the fused path
     n_logits = so.ssd_verify_step_launches(ctypes.byref(args()))
