@@ -785,6 +785,26 @@ int stages_for(int32_t rows, int ku) {
   return s;
 }
 
+// The launch: cooperative, above one row tile in clusters of two.
+struct LmConfig {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[2];
+  LmConfig(int32_t rows, int32_t V, size_t smem, cudaStream_t stream) {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)lm_ctas(rows, V), 1, 1);
+    cfg.blockDim = dim3(kThreadsL, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = row_pairs(rows) ? 2 : 1;
+  }
+  LmConfig(const LmConfig&) = delete;  // (cfg points into it)
+};
+
 }  // namespace
 
 size_t lmhead_workspace(int32_t rows, int32_t V) {
@@ -798,20 +818,28 @@ ssd_status lmhead_check(int32_t rows, int32_t V, int32_t K) {
   if (K <= 0 || K % kBK != 0) return SSD_ERR_UNSUPPORTED;
   if (V <= 0 || V % kBN != 0) return SSD_ERR_UNSUPPORTED;
   if (V / kBN > 32 * kMaxTilesPerLane) return SSD_ERR_UNSUPPORTED;
-  // every CTA must be resident at once (one CTA per SM: TMEM and shared memory)
-  int per_sm = 0;
+  // every CTA must be resident at once (one per SM: TMEM and shared memory), above one
+  // row tile in pairs, fewer of which may fit than half of the SMs
   const int ku = unit_k(rows, K);
   const size_t smem = smem_bytes(rows, ku, stages_for(rows, ku));
-  auto occupancy = [&](auto kernel) {
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-               cudaSuccess &&
-           cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kThreadsL, smem) ==
-               cudaSuccess;
-  };
-  if (!(row_pairs(rows) ? occupancy(lmhead_accept_kernel<true>)
-                        : occupancy(lmhead_accept_kernel<false>)))
-    return SSD_ERR_CUDA;
-  if ((int64_t)lm_ctas(rows, V) > (int64_t)per_sm * device_sm_count()) return SSD_ERR_UNSUPPORTED;
+  int n = 0;
+  int64_t resident = 0;
+  if (row_pairs(rows)) {
+    LmConfig c(rows, V, smem, nullptr);
+    if (cudaFuncSetAttribute(lmhead_accept_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, lmhead_accept_kernel<true>, &c.cfg) != cudaSuccess)
+      return SSD_ERR_CUDA;
+    resident = 2 * (int64_t)n;
+  } else {
+    if (cudaFuncSetAttribute(lmhead_accept_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)smem) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, lmhead_accept_kernel<false>, kThreadsL,
+                                                      smem) != cudaSuccess)
+      return SSD_ERR_CUDA;
+    resident = (int64_t)n * device_sm_count();
+  }
+  if (lm_ctas(rows, V) > resident) return SSD_ERR_UNSUPPORTED;
   return SSD_OK;
 }
 
@@ -845,26 +873,13 @@ cudaError_t launch_lmhead(const LmHeadArgs& a, void* ws, size_t ws_bytes, cudaSt
     if (e != cudaSuccess) return e;
   }
   const size_t smem = smem_bytes(a.rows, L.ku, L.stages);
-  const bool pair = row_pairs(a.rows);
   auto launch = [&](auto kernel) {
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)lm_ctas(a.rows, a.V), 1, 1);
-    cfg.blockDim = dim3(kThreadsL, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = 2;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pair ? 2 : 1;
-    return cudaLaunchKernelEx(&cfg, kernel, ht, hd, wt, wd, a, L);
+    LmConfig c(a.rows, a.V, smem, stream);
+    return cudaLaunchKernelEx(&c.cfg, kernel, ht, hd, wt, wd, a, L);
   };
-  return pair ? launch(lmhead_accept_kernel<true>) : launch(lmhead_accept_kernel<false>);
+  return row_pairs(a.rows) ? launch(lmhead_accept_kernel<true>) : launch(lmhead_accept_kernel<false>);
 }
 
 }  // namespace ssd

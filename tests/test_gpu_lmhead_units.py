@@ -22,6 +22,8 @@ pytestmark = pytest.mark.gpu
     # the search: 70 tiles (half a warp per row, 8 tiles per lane, one load each), 133
     # and 148 tiles (a warp per row; 148 in 16-byte loads), more rows than one pass takes
     (90, 64, 8960), (40, 64, 17024), (90, 64, 18944),
+    # the most tiles, one per SM: single CTAs, pairs, and pairs of an odd number of tiles
+    (8, 64, 19456), (160, 64, 19456), (200, 128, 19328),
 ])
 def test_unit_shapes_match_oracle(ssd, rows, K, V):  # noqa: F811
     ht, hd, wt, wd, u = make_inputs(rows, K, V, 60 + rows, 0.1)
@@ -30,6 +32,15 @@ def test_unit_shapes_match_oracle(ssd, rows, K, V):  # noqa: F811
     ref = olm.lmhead_accept(bf16_to_f64(ht), bf16_to_f64(hd), bf16_to_f64(wt), bf16_to_f64(wd), u)
     assert compare_decisions(ref, tok, acc, ratio, lse, what=f"rows={rows} V={V}",
                              tol=FUSED_PROB_TOL) <= max_excused_rows(rows)
+
+
+@pytest.mark.parametrize("rows", [8, 160])
+def test_more_tiles_than_resident_ctas_are_refused(ssd, rows):  # noqa: F811
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ht, hd, wt, wd, u = make_inputs(rows, 64, 128 * (sms + 1), 5, 0.1)
+    with pytest.raises(ssd.SsdError) as e:
+        run_fused(ssd, ht, hd, wt, wd, u)
+    assert e.value.code == 3  # SSD_ERR_UNSUPPORTED
 
 
 @pytest.mark.parametrize("side,lens,V,hidden", [
