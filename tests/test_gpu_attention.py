@@ -105,10 +105,9 @@ def test_long_cache_many_splits(ssd):
 
 
 def test_split_merge_ignores_workspace_contents(ssd):
-    """A KV cache split over CTAs: partials in the workspace, merged by the
-    combine kernel.  Whatever the workspace held before (all ones, zeros, the
-    partials of earlier launches of this and of another case), the result is
-    the same, bit for bit."""
+    """A KV cache split over CTAs of a cluster, which merge without the workspace.
+    Whatever that held before (all ones, zeros, what earlier launches of this and
+    of another case left), the result is the same, bit for bit."""
     c = synth.make_case("long", grid_h=64, grid_w=64, prefix_len=256, cache_len=[256 + 64 * 40 + 9],
                         Hq=4, Hkv=4, d=128, V=64, seed=7, with_logits=False)
     other = synth.make_case("long2", grid_h=64, grid_w=64, prefix_len=256,
@@ -150,9 +149,9 @@ def test_head_dim_64_gqa_tensor_core_path(ssd):
 
 
 def test_mma_sync_and_tensor_core_paths_agree(ssd):
-    """Related problems on both kernels: 3 query heads per KV head (128 is not
-    a multiple of 3: mma.sync), and MHA and 2 heads per KV head on the same
-    caches (tcgen05); all must match the oracle."""
+    """Related problems in different tilings: 3 query heads per KV head (128 is not
+    a multiple of 3: tiles of 126 rows), MHA and 2 heads per KV head on the same
+    caches, and 150 heads on one KV head (mma.sync); all must match the oracle."""
     c = synth.make_case("gqa3", grid_h=24, grid_w=24, prefix_len=120, cache_len=[120, 408],
                         Hq=12, Hkv=4, d=128, V=64, seed=10, with_logits=False)
     check_case(ssd, c)
@@ -162,6 +161,9 @@ def test_mma_sync_and_tensor_core_paths_agree(ssd):
     c2 = synth.make_case("gqa96", grid_h=24, grid_w=24, prefix_len=120, cache_len=[120, 408],
                          Hq=16, Hkv=8, d=128, V=64, seed=10, with_logits=False)
     check_case(ssd, c2)
+    c3 = synth.make_case("mqa150", grid_h=24, grid_w=3, prefix_len=120, cache_len=[120, 157],
+                         Hq=150, Hkv=1, d=128, V=64, seed=10, k_v=0, with_logits=False)
+    check_case(ssd, c3)
 
 
 def _gqa_batch(B, seed):
@@ -238,11 +240,14 @@ def test_tensor_core_shuffled_draft_order(ssd):
 
 
 def test_mma_sync_shuffled_draft_order(ssd):
-    # 3 query heads per KV head: the mma.sync kernel
+    # 3 query heads per KV head: tiles of 126 rows; 150: the mma.sync kernel
     c = synth.make_case("gqa3_shuffled", grid_h=24, grid_w=24, prefix_len=120,
                         cache_len=[120, 144, 408, 672], Hq=12, Hkv=4, d=128, V=64, seed=15,
                         with_logits=False)
     _check_permuted_frontier(ssd, c)
+    _check_permuted_frontier(ssd, synth.make_case(
+        "mqa150_shuffled", grid_h=24, grid_w=3, prefix_len=120, cache_len=[120, 157], Hq=150,
+        Hkv=1, d=128, V=64, seed=15, k_v=0, with_logits=False))
 
 
 def test_sweep_shape_shuffled_draft_order(ssd):

@@ -20,6 +20,7 @@ SUBSET = [
     "tests/test_gpu_attention.py::test_long_cache_many_splits",
     "tests/test_gpu_attention.py::test_mma_sync_and_tensor_core_paths_agree",
     "tests/test_gpu_attention.py::test_split_merge_ignores_workspace_contents",
+    "tests/test_gpu_attention_mma_sync.py",
     "tests/test_gpu_step.py::test_committed_draw_is_the_full_draw_bit_for_bit",
     "tests/test_gpu_lmhead.py::test_fused_lmhead_matches_oracle",
     "tests/test_zz_no_alloc.py",

@@ -40,11 +40,15 @@ def _cases():
         synth.make_case("long_gqa", grid_h=64, grid_w=64, prefix_len=256,
                         cache_len=[256 + 64 * 30 + 5, 256 + 64 * 7], Hq=8, Hkv=4, d=128,
                         V=64, seed=3, with_logits=False),
-        # mma.sync kernel (a query group of 3 does not divide 128) with split-KV
-        # partials and the combine kernel, both in the scratch
-        synth.make_case("mma_sync_split", grid_h=32, grid_w=32, prefix_len=64,
+        # tcgen05 kernel, a query group of 3 (tiles of 126 rows)
+        synth.make_case("group_of_3", grid_h=32, grid_w=32, prefix_len=64,
                         cache_len=[64 + 32 * 29 + 3, 64 + 32 * 20 + 31], Hq=6, Hkv=2, d=128,
                         V=64, seed=4, with_logits=False),
+        # mma.sync kernel (150 query heads per KV head) with split-KV partials and the
+        # combine kernel, both in the scratch
+        synth.make_case("mma_sync_scratch", grid_h=10, grid_w=3, prefix_len=900,
+                        cache_len=[907, 925], Hq=150, Hkv=1, d=128, V=64, seed=5, k_v=0,
+                        with_logits=False),
     ]
 
 
@@ -91,15 +95,16 @@ def test_noalloc_matches_workspace_entry_point_two_calls_in_a_row(ssd):
     first = None
     for c in cases + [cases[0]]:
         r = _both(ssd, c)
-        assert r["wsb"] > 256  # the problem really uses split-KV scratch
+        assert r["wsb"] > 256  # a plan of the mma.sync kernel would split it
         _assert_same(c, r)
         if first is None:
             first = r
     assert np.array_equal(r["o_na"], first["o_na"]) and np.array_equal(r["lse_na"], first["lse_na"])
 
 
-def test_noalloc_matches_oracle(ssd):
-    c = _cases()[2]  # the mma.sync kernel with split-KV partials and the combine
+@pytest.mark.parametrize("i", [2, 3])
+def test_noalloc_matches_oracle(ssd, i):
+    c = _cases()[i]
     r = _both(ssd, c)
     att = ostep.attention_step(c.grid_h, c.grid_w, c.prefix_len, c.row_stride, c.k_v,
                                c.cache_len, bf16_to_f64(c.q), bf16_to_f64(c.k), bf16_to_f64(c.v),
