@@ -16,8 +16,8 @@
 // more (from L2, microseconds later) for the draw; it runs ahead into the next
 // row while the consumers finish the current one.  Under (A), and in a
 // one-round prefix-commit step (lazy: only the committed tokens are drawn, by
-// resolve_kernel below), every row is streamed once.  The consumers are latency-bound, so the arithmetic is kept
-// short: per first-pass chunk each thread folds its 8 entries of both rows
+// resolve_kernel below), every row is streamed once.  The consumers are
+// latency-bound, so the arithmetic is kept short: per first-pass chunk each thread folds its 8 entries of both rows
 // into online (max, sum of 2^x) statistics with a branch-free rescale,
 // three-input maxima and packed fp32 pairs (fma/add .f32x2) for the exponent
 // arguments and the sums, and tracks the first argmax of q with the target
@@ -108,8 +108,10 @@ __device__ __forceinline__ float2 exp_sum8(const float4& x0, const float4& x1, f
   const float2 a1 = ffma2(make_float2(x0.z, x0.w), cc, nmc);
   const float2 a2 = ffma2(make_float2(x1.x, x1.y), cc, nmc);
   const float2 a3 = ffma2(make_float2(x1.z, x1.w), cc, nmc);
-  const float2 e0 = make_float2(ex2_approx(a0.x), ex2_approx(a0.y)), e1 = make_float2(ex2_approx(a1.x), ex2_approx(a1.y));
-  const float2 e2 = make_float2(ex2_approx(a2.x), ex2_approx(a2.y)), e3 = make_float2(ex2_approx(a3.x), ex2_approx(a3.y));
+  const float2 e0 = make_float2(ex2_approx(a0.x), ex2_approx(a0.y));
+  const float2 e1 = make_float2(ex2_approx(a1.x), ex2_approx(a1.y));
+  const float2 e2 = make_float2(ex2_approx(a2.x), ex2_approx(a2.y));
+  const float2 e3 = make_float2(ex2_approx(a3.x), ex2_approx(a3.y));
   return fadd2(fadd2(e0, e1), fadd2(e2, e3));
 }
 
@@ -318,7 +320,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
         if (leader) {
           mbar_arrive_expect_tx(&sh.full[s], 2u * bytes);
           bulk_g2s_at(ring_a + s * (2 * kChunk * 4), trow + ch * kChunk, bytes, &sh.full[s]);
-          bulk_g2s_at(ring_a + s * (2 * kChunk * 4) + kChunk * 4, drow + ch * kChunk, bytes, &sh.full[s]);
+          bulk_g2s_at(ring_a + s * (2 * kChunk * 4) + kChunk * 4, drow + ch * kChunk, bytes,
+                      &sh.full[s]);
         }
         if (++s == kStages) {
           s = 0;
@@ -622,7 +625,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) accept_kernel(AcceptArgs
         if (bk >= 0 || from_p) break;
         // zero residual mass: the same draw from p (block masses of p itself)
         from_p = true;
-#pragma unroll 1
 #pragma unroll 1
         for (int32_t b0 = 0; b0 < nblocks; ++b0) {
           const int32_t i0 = b0 * 64 + lane, i1 = i0 + 32;

@@ -510,7 +510,8 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const bool leader = elect_one();
     int32_t k = 0;        // items handed out
     uint32_t T = 0;       // K tiles issued
-    const uint32_t q_bytes = (uint32_t)(L.drafts * G * 128) * (L.q_copies == 1 ? D / 64 : 1);  // per copy
+    // per copy
+    const uint32_t q_bytes = (uint32_t)(L.drafts * G * 128) * (L.q_copies == 1 ? D / 64 : 1);
     read_plan();
     const int32_t ns = 1 << ns_log;
     const int32_t part = cta & (ns - 1);
@@ -715,7 +716,8 @@ frontier_attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   } else if (warp == kSoftWarps + 2) {
     // ----------------------------------------------------------- S products
     // (every lane in the loop, one elected around the products: elect_one())
-    const uint32_t tSu = warp_uniform(tS), aQ = warp_uniform(smem_u32(sQ)), aK = warp_uniform(smem_u32(sK));
+    const uint32_t tSu = warp_uniform(tS), aQ = warp_uniform(smem_u32(sQ));
+    const uint32_t aK = warp_uniform(smem_u32(sK));
     const bool leader = elect_one();
     bool ok = true;
     uint32_t T = 0;
@@ -1255,7 +1257,8 @@ cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t stream, bool pdl
   {  // {64 columns, Hq, B * D_max, d / 64}, box {64, G, bm / G, d / 64 or 1}
     const uint64_t dims[4] = {64, (uint64_t)a.Hq, (uint64_t)a.B * a.D_max, halves};
     const uint64_t strides[3] = {row, (uint64_t)a.Hq * row, 128};
-    const uint32_t box[4] = {64, (uint32_t)G, (uint32_t)L.drafts, L.q_copies == 1 ? (uint32_t)halves : 1u};
+    const uint32_t box[4] = {64, (uint32_t)G, (uint32_t)L.drafts,
+                             L.q_copies == 1 ? (uint32_t)halves : 1u};
     ok = bf16_tensor_map(&tq, a.q, 4, dims, strides, box);
   }
   {  // {64 columns, rows, 1, d / 64}, box {64, KTC, 1, d / 64}

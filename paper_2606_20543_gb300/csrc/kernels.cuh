@@ -35,10 +35,10 @@ __device__ __forceinline__ int32_t frontier_drafts(const ssd_grid& g, int32_t ca
 // Every kernel but the cooperative ones and the mma.sync attention is launched so.
 // Unless a schedule of several kernels orders it otherwise, it waits (pdl_wait)
 // before its first access to global memory (and only the attention lets what follows
-// be scheduled early, which waits in its turn), so the order of the stream holds, while its CTAs are in place when the kernel
-// before it ends: back to back, a 24x24 step takes 11.8 us instead of 14.4, five
-// drafts of 20 images 18.2 for 20.5, an acceptance of 1024 rows x 65536 85.2 for
-// 89.9.  (Letting the next call's kernels in before the last draws were done saved
+// be scheduled early, which waits in its turn), so the order of the stream holds,
+// while its CTAs are in place when the kernel before it ends: back to back, a 24x24
+// step takes 11.8 us instead of 14.4, five drafts of 20 images 18.2 for 20.5, an
+// acceptance of 1024 rows x 65536 85.2 for 89.9.  (Letting the next call's kernels in before the last draws were done saved
 // no more, and their CTAs then took what SMs were free, four to one: one image left
 // of 8 x 64x64 33.5 -> 37.1.)
 template <typename... KArgs, typename... Args>

@@ -184,7 +184,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   const int tile0 = cta - rank;              // the tiles of its accumulators: tile0, ...
   const int32_t row0 = rank * L.rpad;        // its rows: row0 .. row0 + nrows - 1
   const int32_t nrows = PAIR ? max(min(L.rpad, a.rows - row0), 0) : a.rows;
-  const int32_t nunits = 2 * (a.K / L.ku);  // ring units: K step u / 2 of the target (even u) or draft head
+  // ring units: K step u / 2 of the target (even u) or draft head
+  const int32_t nunits = 2 * (a.K / L.ku);
   constexpr uint32_t ncols = (uint32_t)(kTiles * 2 * kBN);  // target + draft accumulators
 
   // ---- set-up: barriers, TMEM
@@ -322,7 +323,8 @@ lmhead_accept_kernel(const __grid_constant__ CUtensorMap tmHt, const __grid_cons
   const bool live = lrow < nrows;
   const uint32_t lane_off = (uint32_t)(quarter * 32) << 16;
   float4* chunk_part = reinterpret_cast<float4*>(smem);  // [tiles][4 chunks][2][128 rows]
-  float* chunk_mass = reinterpret_cast<float*>(chunk_part + kTiles * 8 * kBM);  // [tiles][4 chunks][128]
+  // [tiles][4 chunks][128]
+  float* chunk_mass = reinterpret_cast<float*>(chunk_part + kTiles * 8 * kBM);
 
   // ---- epilogue 1: per-tile softmax partials of every row (4 warps alone took
   // 1.7 us per tile)

@@ -89,7 +89,7 @@ struct PredLaunch {
   PredPhase ph[kPhases];
   int32_t ncta, rows, nn, nc;  // rows, MMA N (rows padded to 16), TMEM columns per accumulator
   int32_t stages;              // ring slots (weights + activations of one unit each)
-  int32_t d, m, V;
+  int32_t d, m;
   uint32_t max_polls, shortfall;
   int32_t tile_waits;          // activation copies wait per tile (else per phase)
   float eps;
@@ -317,7 +317,8 @@ __device__ void finish_tile_t(const PredLaunch& L, int p, int32_t f, int32_t cnt
       }
       as[b] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (p == 2 && i0 + b < my_rows)
-        as[b] = __ldcg(reinterpret_cast<const float4*>(L.hid + (int64_t)(w + 4 * (i0 + b)) * L.d + feat));
+        as[b] = __ldcg(reinterpret_cast<const float4*>(L.hid + (int64_t)(w + 4 * (i0 + b)) * L.d +
+                                                       feat));
     }
 #pragma unroll 1
     for (int b = 0; b < RB && i0 + b < my_rows; ++b) {  // the same in every lane of the warp
@@ -499,7 +500,8 @@ predictor_kernel(const __grid_constant__ CUtensorMap tmW0, const __grid_constant
       bool ok = true;
       for (int p = 0; p < kPhases && ok; ++p) {
         const PredPhase& ph = L.ph[p];
-        const int64_t lo = unit_start(cta, ph.units, L.ncta), hi = unit_start(cta + 1, ph.units, L.ncta);
+        const int64_t lo = unit_start(cta, ph.units, L.ncta);
+        const int64_t hi = unit_start(cta + 1, ph.units, L.ncta);
         for (int64_t u = lo; u < hi; ++u, ++gu) {
           if ((int)(gu & 1u) != warp) continue;
           const uint32_t s = gu % S;
@@ -922,7 +924,6 @@ cudaError_t launch_rows(const PredictorArgs& a, void* ws, size_t ws_bytes, int32
   L.stages = P.stages;
   L.d = a.d;
   L.m = a.m;
-  L.V = a.V;
   L.max_polls = wait_poll_limit();
   L.shortfall = barrier_shortfall();
   // measured (graphs of back-to-back calls): per-tile waits 136 vs 144 us at 72
