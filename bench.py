@@ -208,10 +208,10 @@ class ClockSampler:
 MEASURED_TRAFFIC = {
     # (kernel, config): (source, sha256 prefix of the source the capture ran,
     # DRAM bytes read + written in one launch, rows of that launch or None)
-    ("lmhead_accept", 4): ("lmhead.cu", "26bbdea7ac53856b", 269286656 + 115456, None),
+    ("lmhead_accept", 4): ("lmhead.cu", "e3d9a5a7c652ff8d", 269287808 + 137600, None),
     # 8 x 64x64 replay, first step (1024 draft rows): accept_kernel alone; the
     # bench scales it to the rows of the replay states it sums
-    ("accept", 5): ("accept.cu", "6c41882f517fa019", 536914176 + 67840, 1024),
+    ("accept", 5): ("accept.cu", "a9407478c494c2a9", 536913024 + 231552, 1024),
 }
 
 

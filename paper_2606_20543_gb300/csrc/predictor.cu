@@ -52,7 +52,11 @@
 //     P1 finish; the last tile of P3 to finish turns the keys into the tokens.
 // Numerics: every product input is bf16 (z, the weights, Ag, G, Hg); A, U,
 // Vg, h and the logits are fp32; every sum runs in a fixed order, so results
-// do not depend on timing.
+// do not depend on timing.  The order is part of the result: a tile's whole K in one
+// CTA (rows on M, no partials: 24 rows 79 us) moved h by 5.4e-4 at the same error
+// against 64 bits and changed 10 of 2304 tokens, all where two logits nearly tie.
+// d = 4096, m = 8192, V = 16384: 24 rows 108 us (0.56 of the measured copy's rate), 48
+// rows 119, 64 rows 125, 128 rows 134; the phase boundaries take ~9 us each.
 #include <algorithm>
 
 #include "kernels.cuh"
